@@ -107,13 +107,18 @@ def _check(code: int, where: str) -> None:
         raise D2DError(code, where)
 
 
+# Marshalling is on the path of every decode step: plain integers for pointers (ctypes converts them), the raw handle of
+# the current stream (70 ns; building a torch.cuda.Stream object around it takes 3 us) and workspace sizes looked up once.
+_raw_stream = torch._C._cuda_getCurrentRawStream
+_device_index = torch._C._cuda_getDevice
+
+
 def _ptr(t):
-    return None if t is None else c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return c_void_p(s.cuda_stream)
+    return _raw_stream(_device_index()) if stream is None else stream.cuda_stream
 
 
 def torch_dtype(name: str):
@@ -127,29 +132,37 @@ class Routing:
         """lists=False leaves out the per-expert lists (counts, offsets, perm, n_sel): d2d_layer_fwd then does not build them."""
         W = (E + 31) // 32
         cap = T * E if perm_capacity is None else int(perm_capacity)
-        i32 = dict(dtype=torch.int32, device=device)
-        self.T, self.E, self.W = T, E, W
-        self.mask = torch.zeros((max(T, 1), W), **i32)     # raw uint32 words kept in an int32 tensor
-        self.k = torch.zeros((max(T, 1),), **i32)
-        self.scalars = torch.zeros((2,), **i32)            # n_sel, status
-        self.lists = lists
-        if not lists:
-            self.counts = self.offsets = self.perm = self.tok_off = self.tok_exp = None
-            self.struct = RoutingStruct(mask=self.mask.data_ptr(), k=self.k.data_ptr(), counts=None, offsets=None, perm=None,
-                                        tok_off=None, tok_exp=None, n_sel=None, status=self.scalars.data_ptr() + 4,
-                                        perm_capacity=0)
-            return
-        self.counts = torch.zeros((E,), **i32)
-        self.offsets = torch.zeros((E + 1,), **i32)
-        self.perm = torch.zeros((max(cap, 1),), **i32)
-        self.tok_off = torch.zeros((T + 1,), **i32) if dual else None
-        self.tok_exp = torch.zeros((max(cap, 1),), **i32) if dual else None
-        self.struct = RoutingStruct(
-            mask=self.mask.data_ptr(), k=self.k.data_ptr(), counts=self.counts.data_ptr(),
-            offsets=self.offsets.data_ptr(), perm=self.perm.data_ptr(),
-            tok_off=self.tok_off.data_ptr() if dual else None,
-            tok_exp=self.tok_exp.data_ptr() if dual else None,
-            n_sel=self.scalars.data_ptr(), status=self.scalars.data_ptr() + 4, perm_capacity=cap)
+        self.T, self.E, self.W, self.lists = T, E, W, lists
+        # One zeroed allocation for all buffers, each on a 256-byte boundary; the tensors over it are made when asked for
+        # (mask: raw uint32 words kept in an int32 tensor; scalars: n_sel, status).
+        shapes = {"mask": (max(T, 1), W), "k": (max(T, 1),), "scalars": (2,)}
+        if lists:
+            shapes.update(counts=(E,), offsets=(E + 1,), perm=(max(cap, 1),))
+            if dual:
+                shapes.update(tok_off=(T + 1,), tok_exp=(max(cap, 1),))
+        at, n = {}, 0
+        for name, shape in shapes.items():
+            at[name] = n
+            n += (shape[0] * (shape[1] if len(shape) > 1 else 1) + 63) // 64 * 64
+        self._slab = torch.zeros((n,), dtype=torch.int32, device=device)
+        self._shapes, self._at = shapes, at
+        base = self._slab.data_ptr()
+        p = {name: base + 4 * o for name, o in at.items()}
+        self.struct = RoutingStruct(p["mask"], p["k"], p.get("counts"), p.get("offsets"), p.get("perm"), p.get("tok_off"), p.get("tok_exp"),
+                                    p["scalars"] if lists else None, p["scalars"] + 4, cap if lists else 0)
+
+    def __getattr__(self, name):
+        # the buffers' tensors, on first use (attributes that exist never come here)
+        if name in ("mask", "k", "scalars", "counts", "offsets", "perm", "tok_off", "tok_exp"):
+            shape = self._shapes.get(name)
+            if shape is None:
+                t = None
+            else:
+                o = self._at[name]
+                t = self._slab[o: o + shape[0]] if len(shape) == 1 else self._slab[o: o + shape[0] * shape[1]].view(shape)
+            setattr(self, name, t)
+            return t
+        raise AttributeError(name)
 
     @property
     def n_sel(self) -> int:
@@ -194,6 +207,7 @@ class Layer:
         self.handle = handle
         self.fp8_experts = bool(fp8_experts)
         self._ws = None
+        self._ws_bytes = {}
 
     @classmethod
     def from_config(cls, cfg, weights: dict, device="cuda:0", fp8_experts: bool = False) -> "Layer":
@@ -223,10 +237,19 @@ class Layer:
         return int(_lib.d2d_workspace_bytes(self.handle, T))
 
     def workspace(self, T: int):
-        need = self.workspace_bytes(T)
-        if self._ws is None or self._ws.numel() < need:
+        return self._workspace(T)[0]
+
+    def _workspace(self, T: int):
+        """The workspace tensor and its size in bytes."""
+        need = self._ws_bytes.get(T)
+        if need is None:
+            if len(self._ws_bytes) >= 256:
+                self._ws_bytes.clear()
+            need = self._ws_bytes[T] = self.workspace_bytes(T)
+        if self._ws is None or self._ws_size < need:
             self._ws = torch.empty((need,), dtype=torch.uint8, device=self.device)
-        return self._ws
+            self._ws_size = need
+        return self._ws, self._ws_size
 
     def new_routing(self, T: int, dual: bool = False, perm_capacity: int | None = None, lists: bool = True) -> Routing:
         return Routing(T, self.E, self.device, dual, perm_capacity, lists)
@@ -322,10 +345,11 @@ class Layer:
             y = torch.empty((T, self.d), dtype=self.tdtype, device=self.device)
         if routing is None:
             routing = self.new_routing(T)
-        ws = self.workspace(T)
-        _check(_lib.d2d_layer_fwd(self.handle, _ptr(x), T, c_float(tau), _ptr(y), _ptr(R_out),
-                                  ctypes.byref(routing.struct), _ptr(ws), ws.numel(), _stream(stream)),
-               "d2d_layer_fwd")
+        ws, ws_bytes = self._workspace(T)
+        rc = _lib.d2d_layer_fwd(self.handle, x.data_ptr(), T, tau, y.data_ptr(), None if R_out is None else R_out.data_ptr(),
+                                ctypes.byref(routing.struct), ws.data_ptr(), ws_bytes, _stream(stream))
+        if rc != D2D_OK:
+            raise D2DError(rc, "d2d_layer_fwd")
         return y, routing
 
     def host_workspace(self, T: int):
@@ -353,6 +377,7 @@ class LayerGroup:
             _check(_lib.d2d_group_create(arr, len(self.layers), _stream(), ctypes.byref(handle)), "d2d_group_create")
         self.handle = handle
         self._ws = None
+        self._ws_bytes = {}
 
     def close(self):
         if getattr(self, "handle", None):
@@ -366,10 +391,19 @@ class LayerGroup:
             pass
 
     def workspace(self, T: int):
-        need = int(_lib.d2d_group_workspace_bytes(self.handle, T))
-        if self._ws is None or self._ws.numel() < need:
+        return self._workspace(T)[0]
+
+    def _workspace(self, T: int):
+        """The workspace tensor and its size in bytes."""
+        need = self._ws_bytes.get(T)
+        if need is None:
+            if len(self._ws_bytes) >= 256:
+                self._ws_bytes.clear()
+            need = self._ws_bytes[T] = int(_lib.d2d_group_workspace_bytes(self.handle, T))
+        if self._ws is None or self._ws_size < need:
             self._ws = torch.empty((need,), dtype=torch.uint8, device=self.device)
-        return self._ws
+            self._ws_size = need
+        return self._ws, self._ws_size
 
     def group_fwd(self, x, tau: float, y=None, routings: list | None = None, stream=None):
         """y: [n_layers, T, d]; routings: one Routing per layer (outputs)."""
@@ -380,9 +414,10 @@ class LayerGroup:
         if routings is None:
             routings = [l.new_routing(T) for l in self.layers]
         arr = (RoutingStruct * n)(*[r.struct for r in routings])
-        ws = self.workspace(T)
-        _check(_lib.d2d_group_fwd(self.handle, _ptr(x), T, c_float(tau), _ptr(y), arr, _ptr(ws), ws.numel(),
-                                  _stream(stream)), "d2d_group_fwd")
+        ws, ws_bytes = self._workspace(T)
+        rc = _lib.d2d_group_fwd(self.handle, x.data_ptr(), T, tau, y.data_ptr(), arr, ws.data_ptr(), ws_bytes, _stream(stream))
+        if rc != D2D_OK:
+            raise D2DError(rc, "d2d_group_fwd")
         return y, routings
 
 
