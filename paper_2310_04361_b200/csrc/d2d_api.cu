@@ -7,6 +7,7 @@
 
 #include "d2d_common.cuh"
 #include <stdlib.h>
+#include "decode.cuh"
 #include "gemm_tc.cuh"
 #include "moe_gather.cuh"
 
@@ -88,10 +89,74 @@ static bool use_small_ffn(const d2d_layer *L, int T)
     return T <= lim && d2d_small_ffn_supports(L->desc);
 }
 
+// Batches of a few tokens of bf16 layers: cluster router and streaming expert kernel (decode_router.cu, decode_ffn.cu).
+// A path forced through d2d_layer_set_expert_path concerns the tensor-core batches: those keep it.
+bool d2d_use_decode_ffn(const d2d_layer *L, int n_layers, int T)
+{
+    if (T > d2d_decode_max_tokens(L->desc) && L->expert_path != D2D_PATH_AUTO) return false;
+    return L->dec_maps && d2d_decode_ffn_supports(L->desc, n_layers, T, L->q_w1 != nullptr);
+}
+
+d2d_decode_ffn_layer d2d_decode_ffn_args_for(const d2d_layer *L, const d2d_routing *r, float *y32, unsigned int *ticket, void *y)
+{
+    d2d_decode_ffn_layer a = {};
+    a.tm_w1 = L->tm_dec[0]; a.tm_wg = L->tm_dec[1]; a.tm_w2t_cl = L->tm_dec + 2;
+    a.b1 = (const __nv_bfloat16 *)L->b1; a.b2 = (const __nv_bfloat16 *)L->b2;
+    if (L->q_w1) {                                             // 8-bit expert weights: the kernel reads the codes
+        a.k1 = L->q_k1; a.kg = L->q_kg; a.k2 = L->q_k2;
+    }
+    a.mask = r->mask; a.y32 = y32; a.ticket = ticket; a.y = (__nv_bfloat16 *)y; a.status = r->status;
+    return a;
+}
+
+d2d_decode_router_layer d2d_decode_router_args_for(const d2d_layer *L, const d2d_routing *r, float *R, float *zero)
+{
+    d2d_decode_router_layer a = {};
+    a.w_r1 = (const __nv_bfloat16 *)L->w_r1; a.b_r1 = (const __nv_bfloat16 *)L->b_r1;
+    a.w_r2 = (const __nv_bfloat16 *)L->w_r2; a.b_r2 = (const __nv_bfloat16 *)L->b_r2;
+    a.R = R; a.zero = zero;
+    if (r) {
+        a.mask = r->mask; a.k = r->k; a.counts = r->counts; a.offsets = r->offsets; a.perm = r->perm;
+        a.tok_off = r->tok_off; a.tok_exp = r->tok_exp; a.n_sel = r->n_sel; a.status = r->status; a.capacity = (long long)r->perm_capacity;
+    }
+    return a;
+}
+
+// [ticket (256 bytes) | float32 accumulator [T, d] | list of units]
+size_t d2d_decode_scratch_bytes(const d2d_layer_desc &D, int T)
+{
+    return 256 + d2d_align_up((size_t)T * D.d * 4, 256) + d2d_align_up((size_t)(1 + D.d_ff / 16) * 4, 256);
+}
+
+d2d_status d2d_decode_layers(const d2d_layer *const *layers, int n, const void *x, int T, float tau, const d2d_routing *routing, float *R,
+                             void *const *scratch, void *y, cudaStream_t st)
+{
+    const d2d_layer_desc &D = layers[0]->desc;
+    d2d_decode_router_args ra = {};
+    d2d_decode_ffn_args fa = {};
+    // experts of whole units: the router lists the units the experts share out; otherwise they find them from the mask
+    const int U = D.d_ff / 16, upe = D.expert_size % 16 ? 0 : D.expert_size / 16;
+    const int u0 = upe ? d2d_decode_ffn_first_shared(D, n, T, layers[0]->q_w1 != nullptr) : U;
+    const bool list = u0 < U && u0 % upe == 0;
+    for (int l = 0; l < n; ++l) {
+        float *y32 = (float *)((char *)scratch[l] + 256);
+        ra.l[l] = d2d_decode_router_args_for(layers[l], &routing[l], R, y32);           // the router clears the accumulator
+        fa.l[l] = d2d_decode_ffn_args_for(layers[l], &routing[l], y32, layers[l]->tickets + 16, (char *)y + (size_t)l * T * D.d * 2);
+        if (list) {
+            ra.l[l].units = (int32_t *)((char *)y32 + d2d_align_up((size_t)T * D.d * 4, 256));
+            ra.l[l].u0 = u0; ra.l[l].upe = upe;
+            fa.l[l].units = ra.l[l].units;
+        }
+    }
+    const d2d_status rc = d2d_decode_router(D, n, ra, x, T, tau, 1, T * D.d, st);
+    return rc != D2D_OK ? rc : d2d_decode_ffn(D, n, fa, x, T, true, st);
+}
+
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 {
     size_t need = 256;
-    if (use_small_ffn(L, T)) need = d2d_small_ffn_ws_bytes(L, T);
+    if (d2d_decode_ffn_supports(L->desc, 1, T, L->q_w1 != nullptr)) need = d2d_decode_scratch_bytes(L->desc, T);
+    if (use_small_ffn(L, T) && d2d_small_ffn_ws_bytes(L, T) > need) need = d2d_small_ffn_ws_bytes(L, T);
     // hidden activations H [T, d_ff] bf16 of the dense-masked path
     if (L->desc.dtype == D2D_BF16 && T > d2d_decode_max_tokens(L->desc)) {
         size_t h = d2d_align_up((size_t)T * L->desc.d_ff * 2, 256);
@@ -245,6 +310,13 @@ d2d_status d2d_launch_moe_ffn(const d2d_layer *L, const void *x, int T, const d2
                               void *ws, size_t ws_bytes, cudaStream_t st, int *up_counter, int small_fused, const int32_t *n_sel)
 {
     if (ws_bytes < d2d_moe_ffn_ws_bytes(L, T)) return D2D_ERR_WORKSPACE;
+    if (d2d_use_decode_ffn(L, 1, T)) {
+        // the ticket and the float32 accumulator must start at zero
+        if (cudaMemsetAsync(ws, 0, 256 + (size_t)T * L->desc.d * 4, st) != cudaSuccess) return D2D_ERR_CUDA;
+        d2d_decode_ffn_args a = {};
+        a.l[0] = d2d_decode_ffn_args_for(L, r, (float *)((char *)ws + 256), (unsigned int *)ws, y);
+        return d2d_decode_ffn(L->desc, 1, a, x, T, false, st);
+    }
     if (use_small_ffn(L, T)) return has_lists(r) ? d2d_small_ffn(L, x, T, r, y, ws, st, small_fused) : D2D_ERR_INVALID_ARG;
     if (use_dense_masked(L, T)) return launch_tc_experts(L, x, T, r, y, ws, st, up_counter, n_sel ? n_sel : r->n_sel);
     return d2d_launch_moe_ffn_token(L, x, T, r, y, st);
@@ -368,6 +440,7 @@ d2d_status d2d_layer_create(const d2d_layer_desc *desc, const d2d_weights *w, vo
         L->w1g = (char *)L->slab + cat_off;
         rc = build_gate_cat(L, st);
     }
+    if (rc == D2D_OK) rc = d2d_decode_ffn_maps(L);
     if (rc == D2D_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = D2D_ERR_CUDA;
     if (rc == D2D_OK && (cudaStreamCreateWithFlags(&L->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
                          cudaEventCreateWithFlags(&L->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -442,6 +515,7 @@ d2d_status d2d_layer_create_fp8(const d2d_layer_desc *desc, const d2d_weights *w
     if (rc == D2D_OK && D.gated) rc = d2d_quantize_experts_e4m3(L->w_gate, L->q_wg, L->q_kg, D.n_experts, per, st);
     if (rc == D2D_OK) rc = d2d_launch_transpose(L->w2t, L->w2, D.d_ff, D.d, L->elem, st);      // W2 [d, d_ff] from the transposed copy
     if (rc == D2D_OK && L->w1g) rc = build_gate_cat(L, st);
+    if (rc == D2D_OK) rc = d2d_decode_ffn_maps(L);
     if (rc == D2D_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = D2D_ERR_CUDA;
     if (rc != D2D_OK) {
         d2d_layer_destroy(L);
@@ -683,6 +757,10 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     char *base = (char *)ws;
     float *R = R_out ? R_out : (float *)(base + w.r_off);
     d2d_status rc;
+    if (d2d_decode_router_supports(layer->desc, T) && d2d_use_decode_ffn(layer, 1, T)) {
+        void *scratch = base + w.ffn_off;
+        return d2d_decode_layers(&layer, 1, x, T, tau, routing, R_out, &scratch, y, st);
+    }
     if (d2d_router_fused_supports(layer->desc, T)) {
         // router and dynamic-k mask in one kernel; the selection step then only builds the per-expert metadata
         if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;

@@ -1,6 +1,7 @@
 // Shared declarations of the CUDA translation units behind include/d2d.h.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -21,6 +22,8 @@ struct d2d_layer {
     void *w1g;              // gated bf16 layers: W1 and W_gate interleaved in blocks of 128 rows (see d2d_gemm_args::b_cat)
     void *slab;             // one allocation backing all of the above
     size_t slab_bytes;
+    CUtensorMap tm_dec[5];  // W1, W_gate and W2T (three cuts; codes of an 8-bit layer) as the decode expert kernel reads them
+    int dec_maps;           // 1: the maps exist
     // side stream + events: the per-expert metadata (counts, offsets, token lists) is built beside the
     // expert GEMMs, which do not read it
     cudaStream_t side_stream;
@@ -84,6 +87,8 @@ struct d2d_group {
 // Host-side count of kernel launches (reported by d2d_launch_count()).
 extern unsigned long long d2d_launch_counter;
 #define D2D_LAUNCHED(n) __atomic_fetch_add(&d2d_launch_counter, (unsigned long long)(n), __ATOMIC_RELAXED)
+
+bool d2d_tc_pdl_enabled();      // gemm_tc.cu: false when D2D_GEMM_PDL=0 asks for fully serialised launches
 
 // Largest batch served by the decode kernels (cp.async CUDA-core kernels, two launches per layer call); larger bf16
 // batches take the tensor-core path.  4 by default, D2D_DECODE_MAX_TOKENS=n (0 .. 8) overrides it for tuning.

@@ -1,0 +1,841 @@
+// Expert step of a decode batch (Sec. 3.2, 3.4; gated form App. G): y = b2 + sum over kept experts, for a few tokens.
+//
+// Bound by the bytes of the kept experts' weights.  The unit of work is 16 adjacent neurons: their rows of W1 (and
+// W_gate) and of the transposed W2.  A cluster of CL CTAs takes CL units per round: CTA r forms the 16 hidden values of unit
+// r for all tokens, hands them (a few hundred bytes) to the other CTAs through distributed shared memory, and all CTAs
+// then add all CL units' contributions to their own d / CL output columns.  The output accumulators of those columns stay
+// in registers from the first round to the last, so a CTA adds T d / CL floats to the result, once (CTAs that kept all
+// columns added CL times as much: 6 us of reductions, fences and conversion behind 13 tokens of a d = 1024 layer).
+//
+// A producer warp streams the weights into a ring of 32 KB stages of [16 rows x 128 bytes] blocks, brought by TMA requests
+// for up to 16 blocks each (a 3-D box; one request per row piece measured 50 ns a piece, a third of the memory rate); 16
+// consumer warps compute.  The matrix instructions are the warp-level ones: at 8 to 32 tokens the tensor pipe is idle
+// either way, and these read weights as their 16-row operand with no padding to 128 rows.
+//
+// Which units: a cluster starts on `n_static` rounds fixed by its index before the selection is known (their copies and
+// up projections run beside the router), and takes its share of the others once the router's list of kept units is
+// there.  The up projection of the next round precedes the down projection of the current one, which hides the exchange.
+// The last CTA to add to its columns (a ticket per rank) adds b2 and writes y.
+#include <cuda_fp8.h>
+
+#include "decode.cuh"
+#include "tc_common.cuh"
+
+namespace {
+
+using namespace d2d_decode;
+
+constexpr int NCW = 16, NC = NCW * 32, NT = NC + 32;      // consumer warps / threads, all threads
+constexpr int SUB_BYTES = 16 * 128;                       // a block: 16 rows x 128 bytes, 128-byte swizzle
+constexpr int STAGE_BLOCKS = 16, STAGE_BYTES = STAGE_BLOCKS * SUB_BYTES;
+constexpr int MAX_STAGES = 6;
+constexpr int MAX_UNITS = 4096, MAX_LIST = 128;
+constexpr int H_ROW = 48;                                 // bytes between tokens' rows of 16 hidden values: free of bank conflicts
+constexpr unsigned FULL = 0xffffffffu;
+
+template <typename WT> __host__ __device__ constexpr int sub_cols() { return 128 / (int)sizeof(WT); }       // columns per warp and stage
+template <typename WT> __host__ __device__ constexpr int seg_cols() { return NCW * sub_cols<WT>(); }        // columns per stage
+// Token rows in shared memory: 16 bytes beyond a multiple of 128, so that eight rows' 16-byte pieces do not meet in a bank
+__host__ __device__ constexpr int x_pitch(int d) { return (d * 2 + 127) / 128 * 128 + 16; }
+
+// One stage: 16 rows from `row` on, the 128-byte column blocks from `block` on (3-D map: column in block, row, block)
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int row, int block, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+        ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(block), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void red_add4(float *p, float4 v)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, uint4 v)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void consumer_bar() { asm volatile("bar.sync 1, %0;" ::"n"(NC) : "memory"); }
+
+// Two e4m3 codes as a bf16 pair.  t holds them in the upper bytes of its halves (lower bytes: anything).  Sign and the
+// seven exponent and mantissa bits are moved to where bf16 has them; the exponent's bias differs by 127 - 7, which one
+// exact multiplication by 2^120 makes up (also for the codes below the normal range).
+__device__ __forceinline__ uint32_t e4m3_to_bf16x2(uint32_t t)
+{
+    const uint32_t v = ((t >> 4) & 0x07f007f0u) | (t & 0x80008000u);
+    const uint32_t scale = 0x7b807b80u;                   // 2^120 twice
+    uint32_t r;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(scale));
+    return r;
+}
+
+// Shared-memory offset of byte `col` of row `row` inside a warp's sub-tile (16-byte pieces XORed with the row)
+__device__ __forceinline__ uint32_t swz(int row, int col) { return (uint32_t)(row * 128 + (col ^ ((row & 7) << 4))); }
+
+// Four 8 x 8 matrices of bf16; lane i gives the row address of row i % 8 of matrix i / 8.  TRANS: each is transposed.
+template <bool TRANS> __device__ __forceinline__ void ldmatrix4(uint32_t (&o)[4], uint32_t addr)
+{
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]) : "r"(addr) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]) : "r"(addr) : "memory");
+}
+// Two columns of two rows of codes -> two bf16x2 words, lower half = first row
+__device__ __forceinline__ void load_pairs(const unsigned char *r0, const unsigned char *r1, uint32_t &o0, uint32_t &o1)
+{
+    const uint32_t a = *reinterpret_cast<const uint16_t *>(r0), b = *reinterpret_cast<const uint16_t *>(r1);
+    o0 = e4m3_to_bf16x2(__byte_perm(a, b, 0x4404));
+    o1 = e4m3_to_bf16x2(__byte_perm(a, b, 0x5414));
+}
+// Sixteen codes -> eight bf16x2 words
+__device__ __forceinline__ void widen16(const uint4 &r, uint32_t (&o)[8])
+{
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o[2 * i] = e4m3_to_bf16x2(__byte_perm(w[i], 0, 0x1404));
+        o[2 * i + 1] = e4m3_to_bf16x2(__byte_perm(w[i], 0, 0x3424));
+    }
+}
+
+__device__ __forceinline__ float act_accurate(int act, float z)
+{
+    return act == D2D_ACT_RELU ? d2d_activate<D2D_ACT_RELU>(z) : act == D2D_ACT_GELU_ERF ? d2d_activate<D2D_ACT_GELU_ERF>(z)
+         : act == D2D_ACT_GELU_TANH ? d2d_activate<D2D_ACT_GELU_TANH>(z) : d2d_activate<D2D_ACT_SILU>(z);
+}
+__device__ __forceinline__ float act_fast(int act, float z)
+{
+    return act == D2D_ACT_RELU ? d2d_tc::fast_act<D2D_ACT_RELU>(z) : act == D2D_ACT_GELU_ERF ? d2d_tc::fast_act<D2D_ACT_GELU_ERF>(z)
+         : act == D2D_ACT_GELU_TANH ? d2d_tc::fast_act<D2D_ACT_GELU_TANH>(z) : d2d_tc::fast_act<D2D_ACT_SILU>(z);
+}
+
+struct FfnShape {
+    int T, d, d_ff, E, s, W, act, gated;
+    uint32_t inv_s;          // ceil(2^32 / s): neuron / s = umulhi(neuron, inv_s) for neurons < 2^16
+    int planes;              // 3: hidden values kept to float32 precision and exact activations; 1: bf16 and the fast ones
+    int cl, clusters;        // CTAs per cluster, clusters per layer
+    int n_static, stages;    // rounds fixed by the cluster's index; stages of the ring
+    int up_blocks;           // blocks one request of the up matrices brings
+    int nb, sps;             // blocks of a unit's rows of W2T one CTA reads (its d / cl columns); units per stage of those
+};
+
+// TPW: 16-column output tiles per warp (d / cl <= 256 TPW); NT8: tokens / 8.
+template <typename WT, int TPW, int NT8>
+__global__ void __launch_bounds__(NT, 1)
+decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const __grid_constant__ d2d_decode_ffn_args args)
+{
+    constexpr int T8 = 8 * NT8;
+    constexpr bool Q8 = sizeof(WT) == 1;
+    constexpr int SUB = sub_cols<WT>(), SEG = seg_cols<WT>();
+    constexpr int TPS = SUB / 16, PARTS = TPW > TPS ? TPW / TPS : 1, TPP = TPW > TPS ? TPS : TPW;      // tiles per warp: of a full stage; stages per unit; per stage
+    const d2d_decode_ffn_layer &P = args.l[blockIdx.y];
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);       // swizzle atoms are 1024 bytes
+    __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], h_full[3], h_empty[2];
+    __shared__ int unit_list[MAX_LIST], unit_list_p[MAX_LIST], n_units;
+    __shared__ uint32_t keep_bits[MAX_UNITS / 32];
+    __shared__ int keep_pre[MAX_UNITS / 32];
+    __shared__ unsigned int my_ticket;
+    const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c = lane & 3;
+    const int warp = __shfl_sync(FULL, tid >> 5, 0);           // warp-uniform for the compiler: see mma16816
+    const int d = S.d, T = S.T, U = S.d_ff / 16, CL = S.cl, NCL = S.clusters;
+    const int rank = (int)blockIdx.x % CL, cid = (int)blockIdx.x / CL;
+    const int n_mat = S.gated ? 2 : 1, nq = (d + SEG - 1) / SEG;
+    const int xp = x_pitch(d);
+    unsigned char *ring = smem;
+    unsigned char *xs = ring + (size_t)S.stages * STAGE_BYTES;
+    float *red = reinterpret_cast<float *>(xs + (size_t)T8 * xp);              // [n_mat][16 warps][16][T8]
+    float *zs = red + (size_t)n_mat * NCW * 16 * T8;                           // [n_static + 1][3][16 * T8] up, gate, scale of a round
+    unsigned char *hs = reinterpret_cast<unsigned char *>(zs + (size_t)(S.n_static + 1) * 3 * 16 * T8);     // [n_static + 2][CL][planes][T8] rows
+    uint32_t *smask = reinterpret_cast<uint32_t *>(hs + (size_t)(S.n_static + 2) * CL * S.planes * T8 * H_ROW);     // [T][W], then the union [W]
+
+    if (tid == 0) {
+        for (int i = 0; i < S.stages; ++i) {
+            d2d_tc::mbar_init(smem_addr(&bar_full[i]), 1);
+            d2d_tc::mbar_init(smem_addr(&bar_empty[i]), NCW);
+        }
+        for (int i = 0; i < 3; ++i) d2d_tc::mbar_init(smem_addr(&h_full[i]), CL);
+        for (int i = 0; i < 2; ++i) d2d_tc::mbar_init(smem_addr(&h_empty[i]), NCW * CL);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();                                            // the barriers of every CTA of the cluster exist
+    pdl_trigger();
+
+    // Rounds: the first `my_static` take units (cid + r * NCL) * CL + slot, the others the list's entries in the same order.
+    // `n`: entries of the list.  Slots are filled from 0 on: `slots` of a round hold a unit.
+    const int my_static = min(S.n_static, cid * CL < U ? (U - cid * CL + NCL * CL - 1) / (NCL * CL) : 0);
+    auto rounds_for = [&](int n) { return my_static + (n > cid * CL ? (n - cid * CL + NCL * CL - 1) / (NCL * CL) : 0); };
+    auto slots = [&](int r, int n) { return min(CL, r < my_static ? U - (cid + r * NCL) * CL : n - (cid + (r - my_static) * NCL) * CL); };
+    auto unit_of = [&](int r, int k, const int *list) { return r < my_static ? (cid + r * NCL) * CL + k : list[(r - my_static) * CL + k]; };
+    // whether, after the static rounds' up projections, round ru's comes before round rd's down projection
+    auto up_next = [&](int ru, int rd, int R) { return ru < R && ru <= rd + 1 && !(ru == my_static && rd < my_static); };
+    // this cluster's entries of the router's list
+    auto load_list = [&](int *list, int i0, int step) {
+        for (int i = i0; i < MAX_LIST; i += step) {
+            const int j = (cid + i / CL * NCL) * CL + i % CL;
+            if (j >= U) break;
+            list[i] = __ldcg(P.units + 1 + j);
+        }
+    };
+
+    if (warp == NCW) {
+        // ------------------------------------------------------------------ producer
+        uint32_t it = 0, phase = 1;                                            // stages requested; parity of "free" at `slot`
+        int slot = -1;
+        bool ok = true;
+        // waits for the next stage, announces `blocks` blocks for it and returns its address
+        auto next_stage = [&](int blocks) -> uint32_t {
+            if (++slot == S.stages) slot = 0;
+            if (slot == 0) phase ^= 1u;
+            if (it >= (uint32_t)S.stages) ok = ok && d2d_tc::mbar_wait_warp(smem_addr(&bar_empty[slot]), phase ^ 1u, P.status);
+            if (ok && lane == 0) d2d_tc::mbar_expect_tx(smem_addr(&bar_full[slot]), (uint32_t)(blocks * SUB_BYTES));
+            ++it;
+            return smem_addr(ring + (size_t)slot * STAGE_BYTES);
+        };
+        auto full_bar = [&]() { return smem_addr(&bar_full[slot]); };
+        auto up = [&](int r, int n) {
+            if (rank >= slots(r, n)) return;
+            const int u = unit_of(r, rank, unit_list_p);
+            for (int q = 0; q < nq && ok; ++q)
+                for (int m = 0; m < n_mat && ok; ++m) {
+                    const uint32_t dst = next_stage(S.up_blocks);
+                    if (ok && lane == 0) tma_load_3d(dst, m ? &P.tm_wg : &P.tm_w1, u * 16, q * STAGE_BLOCKS, full_bar());
+                    __syncwarp();
+                }
+        };
+        // the down stages of round r from number `from` on, while fewer than `limit` stages have been requested (0: all)
+        auto down = [&](int r, int from, uint32_t limit, int n) -> int {
+            int st = 0;
+            const int nv = slots(r, n);
+            for (int k0 = 0; k0 < nv; k0 += S.sps)
+                for (int part = 0; part < PARTS; ++part, ++st) {
+                    if (st < from) continue;
+                    if ((limit > 0 && it >= limit) || !ok) return st;
+                    const int k1 = min(nv, k0 + S.sps);
+                    const uint32_t dst = next_stage((k1 - k0) * (PARTS > 1 ? STAGE_BLOCKS : S.nb));
+                    if (ok && lane == 0)
+                        for (int k = k0; k < k1; ++k)
+                            tma_load_3d(dst + (k - k0) * S.nb * SUB_BYTES, &P.tm_w2t, unit_of(r, k, unit_list_p) * 16, rank * S.nb + part * STAGE_BLOCKS, full_bar());
+                    __syncwarp();
+                }
+            return -1;
+        };
+        // Before anything is known about the selection: the up stages of the static rounds, which the consumers use up
+        // before they wait for it, and of the down stages what the ring holds.
+        for (int r = 0; r < my_static; ++r) up(r, 0);
+        int r = 0, from = 0;
+        const uint32_t early = it + (uint32_t)S.stages;
+        for (; r < my_static; ++r) {
+            from = down(r, 0, early, 0);
+            if (from >= 0) break;
+            from = 0;
+        }
+        int n = 0;
+        if (P.units) {
+            pdl_wait();
+            n = __ldcg(P.units);
+            load_list(unit_list_p, lane, 32);
+            __syncwarp();
+        } else {
+            asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");           // the consumers have built unit_list
+            n = n_units;
+            for (int i = lane; i < MAX_LIST; i += 32) unit_list_p[i] = unit_list[i];
+            __syncwarp();
+        }
+        const int R = rounds_for(n);
+        for (int ru = my_static; r < R && ok; ) {
+            if (up_next(ru, r, R)) {
+                up(ru, n);
+                ++ru;
+            } else {
+                down(r, from, 0, n);
+                ++r;
+                from = 0;
+            }
+        }
+        // nothing may be in flight when the CTA exits: the consumers wait for every stage they use, so only a run that
+        // gave up needs this
+        if (!ok)
+            for (uint32_t k = it > (uint32_t)S.stages ? it - S.stages : 0; k + 1 < it; ++k)
+                d2d_tc::mbar_wait_warp(smem_addr(&bar_full[k % S.stages]), (k / S.stages) & 1u, P.status);
+        cluster_arrive();
+    } else {
+        // ------------------------------------------------------------------ consumers
+        // x does not depend on the router (the kernel behind which this one may start early waits for its own
+        // predecessor before it lets this one start)
+        for (int i = tid, t = 0; t < T; ) {
+            if (i >= d / 8) { i -= d / 8; ++t; continue; }
+            cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
+            i += NC;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        consumer_bar();
+
+        int slot = 0, n = 0;
+        uint32_t phase = 0;
+        bool ok = true;
+        auto stage_wait = [&]() {
+            if (ok) ok = d2d_tc::mbar_wait_warp(smem_addr(&bar_full[slot]), phase, P.status);
+        };
+        auto stage_done = [&]() {
+            __syncwarp();
+            if (lane == 0) d2d_tc::mbar_arrive(smem_addr(&bar_empty[slot]));
+            if (++slot == S.stages) { slot = 0; phase ^= 1u; }
+        };
+        // this thread's hidden value in a round: neuron nr of its unit, token tok
+        const int nr = tid / T8, tok = tid % T8;
+        const bool mine = tid < 16 * T8 && tok < T;
+        // ldmatrix addresses: row of this lane inside a 16-row operand tile, and which 16-byte piece of a pair
+        const int lrow = (lane & 7) + ((lane >> 3) & 1) * 8, lhalf = lane >> 4;
+        const uint32_t xs_addr = smem_addr(xs);
+
+        // ---- up projection (and gate) of this CTA's unit of round r; the sums, bias added, go to this thread's places in
+        // zs[place].  A warp takes one 128-byte column block.
+        auto up = [&](int r, int place) {
+            if (rank >= slots(r, n)) return;
+            const int u = unit_of(r, rank, unit_list);
+            float bias = 0.0f;
+            int sc[3] = {0, 0, 0};                                // exponents of the scales of W1, W_gate and W2
+            if (mine) {
+                if (P.b1) bias = __bfloat162float(P.b1[u * 16 + nr]);
+                if (Q8) {
+                    const int e = __umulhi((uint32_t)(u * 16 + nr), S.inv_s);
+                    sc[0] = P.k1[e]; sc[2] = P.k2[e];
+                    if (S.gated) sc[1] = P.kg[e];
+                }
+            }
+            constexpr int CH = NT8 == 1 ? 2 : 1;                  // chains of matrix instructions per accumulator
+            float s[2][NT8 * CH][4];
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int t = 0; t < NT8 * CH; ++t) s[m][t][0] = s[m][t][1] = s[m][t][2] = s[m][t][3] = 0.0f;
+#pragma unroll 1
+            for (int q = 0; q < nq; ++q) {
+                const int k0 = q * SEG + warp * SUB;
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    if (m == 1 && !S.gated) break;
+                    stage_wait();
+                    if (k0 < d) {                                 // warp-uniform: d is a multiple of a block's columns
+                        unsigned char *st = ring + (size_t)slot * STAGE_BYTES + warp * SUB_BYTES;
+                        if (!Q8) {
+                            const uint32_t sa = smem_addr(st);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {                     // 32 columns at a time
+                                uint32_t a0[4], a1[4];
+                                ldmatrix4<false>(a0, sa + swz(lrow, h * 64 + lhalf * 16));
+                                ldmatrix4<false>(a1, sa + swz(lrow, h * 64 + 32 + lhalf * 16));
+#pragma unroll
+                                for (int t = 0; t < NT8; ++t) {
+                                    uint32_t b[4];
+                                    ldmatrix4<false>(b, xs_addr + min(t * 8 + (lane & 7), T - 1) * xp + (k0 + h * 32) * 2 + (lane >> 3) * 16);
+                                    mma16816(s[m][t * CH], a0[0], a0[1], a0[2], a0[3], b[0], b[1]);
+                                    mma16816(s[m][t * CH + CH - 1], a1[0], a1[1], a1[2], a1[3], b[2], b[3]);
+                                }
+                            }
+                        } else {
+                            // lane = rows g, g + 8.  A row is eight 16-byte pieces; lane c takes pieces c and c + 4, odd rows in the other
+                            // order, so that eight lanes (two rows) do not meet in a bank
+                            const int flip = (g & 1) * 64;
+                            uint4 a[2][2];                        // [piece c / c + 4][row g / g + 8]
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) a[h][i] = *reinterpret_cast<const uint4 *>(st + swz(g + 8 * i, c * 16 + (h * 64 ^ flip)));
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                const uint4 p = a[0][i], o = a[1][i];
+                                a[0][i] = flip ? o : p;
+                                a[1][i] = flip ? p : o;
+                            }
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const unsigned char *xr = xs + min(g, T - 1) * xp + (k0 + h * (SUB / 2)) * 2 + c * 32;
+                                uint32_t wa[2][8];
+                                widen16(a[h][0], wa[0]);
+                                widen16(a[h][1], wa[1]);
+#pragma unroll
+                                for (int t = 0; t < NT8; ++t)
+#pragma unroll
+                                    for (int p = 0; p < 2; ++p) {
+                                        const uint4 xb = *reinterpret_cast<const uint4 *>(xr + t * 8 * xp + p * 16);
+                                        mma16816(s[m][t * CH], wa[0][4 * p], wa[1][4 * p], wa[0][4 * p + 1], wa[1][4 * p + 1], xb.x, xb.y);
+                                        mma16816(s[m][t * CH + CH - 1], wa[0][4 * p + 2], wa[1][4 * p + 2], wa[0][4 * p + 3], wa[1][4 * p + 3], xb.z, xb.w);
+                                    }
+                            }
+                        }
+                    }
+                    stage_done();
+                }
+            }
+            // the warps' partial sums meet
+            consumer_bar();                                       // the sums of the previous round have been read
+#pragma unroll
+            for (int m = 0; m < 2; ++m) {
+                if (m == 1 && !S.gated) break;
+#pragma unroll
+                for (int t = 0; t < NT8; ++t) {
+                    if (CH == 2) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) s[m][0][i] += s[m][CH - 1][i];
+                    }
+                    float *r = red + (size_t)((m * NCW + warp) * 16 + g) * T8 + t * 8 + 2 * c;
+                    *reinterpret_cast<float2 *>(r) = make_float2(s[m][t * CH][0], s[m][t * CH][1]);
+                    *reinterpret_cast<float2 *>(r + 8 * T8) = make_float2(s[m][t * CH][2], s[m][t * CH][3]);
+                }
+            }
+            consumer_bar();
+            if (mine) {
+                float *z = zs + (size_t)place * 3 * 16 * T8 + tid;
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    if (m == 1 && !S.gated) break;
+                    const float *p = red + (size_t)m * NCW * 16 * T8 + tid;
+                    float v = 0.0f;
+#pragma unroll
+                    for (int w = 0; w < NCW; ++w) v += p[w * 16 * T8];
+                    if (Q8) v = ldexpf(v, sc[m]);
+                    z[m * 16 * T8] = m == 0 ? v + bias : v;
+                }
+                if (Q8) z[2 * 16 * T8] = ldexpf(1.0f, sc[2]);
+            }
+        };
+
+        // Waits for the router and brings mask and list of kept units into shared memory (the list is found here, from the
+        // mask, where the router does not make it).
+        auto mask_ready = [&]() {
+            pdl_wait();
+            if (P.units) {
+                load_list(unit_list, tid, NC);
+                n = __ldcg(P.units);
+            }
+            for (int i = tid; i < T * S.W; i += NC) smask[i] = __ldcg(P.mask + i);
+            consumer_bar();
+            if (P.units) return;
+            const int u0 = min(S.n_static * NCL * CL, U), nu = U - u0;
+            if (nu > 0) {
+                uint32_t *un = smask + T * S.W;
+                for (int w = tid; w < S.W; w += NC) {
+                    uint32_t v = 0u;
+                    for (int t = 0; t < T; ++t) v |= smask[t * S.W + w];
+                    un[w] = v;
+                }
+                consumer_bar();
+                const int nw = (nu + 31) / 32;
+                for (int w = warp; w < nw; w += NCW) {
+                    const int u = u0 + w * 32 + lane;
+                    bool keep = false;
+                    if (u < U)
+                        for (int e = u * 16 / S.s; e <= (u * 16 + 15) / S.s; ++e) keep |= (un[e >> 5] >> (e & 31)) & 1u;
+                    const uint32_t bits = __ballot_sync(FULL, keep);
+                    if (lane == 0) keep_bits[w] = bits;
+                }
+                consumer_bar();
+                if (warp == 0) {
+                    int run = 0;
+                    for (int w0 = 0; w0 < nw; w0 += 32) {
+                        const int v = w0 + lane < nw ? __popc(keep_bits[w0 + lane]) : 0;
+                        int inc = v;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int m = __shfl_up_sync(FULL, inc, o);
+                            if (lane >= o) inc += m;
+                        }
+                        if (w0 + lane < nw) keep_pre[w0 + lane] = run + inc - v;
+                        run += __shfl_sync(FULL, inc, 31);
+                    }
+                    if (lane == 0) n_units = run;
+                }
+                consumer_bar();
+                for (int i = tid; i < nu; i += NC)
+                    if ((keep_bits[i >> 5] >> (i & 31)) & 1u) {
+                        const int r = keep_pre[i >> 5] + __popc(keep_bits[i >> 5] & ((1u << (i & 31)) - 1u)), j = r / CL;
+                        if (j % NCL == cid) unit_list[j / NCL * CL + r % CL] = u0 + i;
+                    }
+            } else if (tid == 0) {
+                n_units = 0;
+            }
+            asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
+            n = n_units;
+        };
+
+        // Hidden values live in buffers [static round, or n_static + the parity of a shared round][slot]; the static rounds' are
+        // exchanged together, once.
+        auto buffer = [&](int r) { return hs + (size_t)(r < my_static ? r : S.n_static + ((r - my_static) & 1)) * CL * S.planes * T8 * H_ROW; };
+
+        // ---- hidden values of rounds [r0, r1): activation and selection on this CTA's sums into its own buffers, from there to
+        // the other CTAs of the cluster, a warp per receiver (16-byte stores and one arrival; 4-byte asynchronous stores by
+        // the threads that have the values took 2.6 us)
+        auto finish = [&](int r0, int r1) {
+            const int j = r0 - my_static;                                      // shared rounds: their number
+            for (int r = r0; r < r1; ++r) {
+                if (rank >= slots(r, n) || !mine) continue;
+                const int e = __umulhi((uint32_t)(unit_of(r, rank, unit_list) * 16 + nr), S.inv_s);
+                const float *z = zs + (size_t)min(r, my_static) * 3 * 16 * T8 + tid;
+                const float up = z[0], pre = S.gated ? z[16 * T8] : up;
+                float h = 0.0f;
+                if ((smask[tok * S.W + (e >> 5)] >> (e & 31)) & 1u) {
+                    h = S.planes == 3 ? act_accurate(S.act, pre) : act_fast(S.act, pre);
+                    if (S.gated) h *= up;
+                }
+                // the scale of W2 is a power of two: applied to the hidden value, after its rounding
+                __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(buffer(r) + (size_t)(rank * S.planes * T8 + tok) * H_ROW) + nr;
+                if (S.planes == 3) {
+                    __nv_bfloat16 t[3];
+                    split3(Q8 ? h * z[2 * 16 * T8] : h, t);
+                    o[0] = t[0]; o[T8 * H_ROW / 2] = t[1]; o[2 * T8 * H_ROW / 2] = t[2];
+                } else {
+                    const __nv_bfloat16 hb = __float2bfloat16_rn(h);
+                    o[0] = Q8 ? __float2bfloat16_rn(__bfloat162float(hb) * z[2 * 16 * T8]) : hb;
+                }
+            }
+            consumer_bar();
+            if (CL > 1 && warp < CL) {
+                if (j >= 2 && ok) ok = mbar_wait_cluster(smem_addr(&h_empty[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
+                if (warp != rank) {
+                    for (int r = r0; r < r1; ++r) {
+                        if (rank >= slots(r, n)) break;
+                        const unsigned char *own = buffer(r) + (size_t)rank * S.planes * T8 * H_ROW;
+                        const uint32_t to = cluster_addr(smem_addr(own), warp);
+                        for (int i = lane; i < 2 * T8 * S.planes; i += 32) {
+                            const int off = (i >> 1) * H_ROW + (i & 1) * 16;
+                            if (NT8 == 1 || (i >> 1) < T) st_cluster4(to + off, *reinterpret_cast<const uint4 *>(own + off));
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) arrive_cluster(cluster_addr(smem_addr(&h_full[j < 0 ? 2 : j & 1]), warp));
+            }
+        };
+        // (A CTA's own slot of a shared round's buffer is written again two rounds later, behind the barriers of that round's up
+        // projection, which every warp reaches after it has read the buffer.)
+
+        // ---- down projection of round r onto this CTA's columns.  A tile's 16 columns: bf16 weights g and g + 8 of lane (g, c),
+        // codes 2 g and 2 g + 1.
+        float acc[TPW][NT8][4];
+#pragma unroll
+        for (int i = 0; i < TPW; ++i)
+#pragma unroll
+            for (int t = 0; t < NT8; ++t) acc[i][t][0] = acc[i][t][1] = acc[i][t][2] = acc[i][t][3] = 0.0f;
+        const int DC = d / CL;
+        auto down = [&](int r, int R) {
+            const int j = r - my_static, nv = slots(r, n);
+            if (ok && CL > 1) ok = mbar_wait_cluster(smem_addr(&h_full[j < 0 ? 2 : j & 1]), j < 0 ? 0u : (j >> 1) & 1u, P.status);
+            const unsigned char *hb0 = buffer(r) + g * H_ROW + c * 4;
+            for (int k0 = 0; k0 < nv; k0 += S.sps) {
+                const int k1 = min(nv, k0 + S.sps);
+#pragma unroll
+                for (int part = 0; part < PARTS; ++part) {
+                    stage_wait();
+                    unsigned char *stage = ring + (size_t)slot * STAGE_BYTES;
+#pragma unroll(PARTS == 1 ? 4 : 1)
+                    for (int k = k0; k < k1; ++k) {
+                        uint32_t hb[3][NT8][2];
+#pragma unroll
+                        for (int p = 0; p < 3; ++p)
+#pragma unroll
+                            for (int t = 0; t < NT8; ++t) {
+                                if (p > 0 && (NT8 > 1 || S.planes == 1)) break;
+                                const unsigned char *hr = hb0 + ((k * S.planes + p) * T8 + t * 8) * H_ROW;
+                                hb[p][t][0] = *reinterpret_cast<const uint32_t *>(hr);
+                                hb[p][t][1] = *reinterpret_cast<const uint32_t *>(hr + 16);
+                            }
+#pragma unroll
+                        for (int i = 0; i < TPP; ++i) {
+                            const int tile = warp + NCW * i;
+                            if (PARTS == 1 && tile * 16 >= DC) break;
+                            unsigned char *st = stage + ((k - k0) * S.nb + tile * 16 / SUB) * SUB_BYTES;
+                            const int col = tile * 16 % SUB * (int)sizeof(WT);
+                            uint32_t a[4];
+                            if (!Q8) {
+                                // matrices: neurons 0-7 and 8-15 (lane / 16), columns 0-7 and 8-15 (lane / 8 % 2)
+                                ldmatrix4<true>(a, smem_addr(st) + swz((lane & 7) + lhalf * 8, col + ((lane >> 3) & 1) * 16));
+                            } else {
+                                load_pairs(st + swz(2 * c, col + g * 2), st + swz(2 * c + 1, col + g * 2), a[0], a[1]);
+                                load_pairs(st + swz(2 * c + 8, col + g * 2), st + swz(2 * c + 9, col + g * 2), a[2], a[3]);
+                            }
+#pragma unroll
+                            for (int t = 0; t < NT8; ++t) mma16816(acc[part * TPP + i][t], a[0], a[1], a[2], a[3], hb[0][t][0], hb[0][t][1]);
+                            if (NT8 == 1 && S.planes == 3) {
+                                mma16816(acc[part * TPP + i][0], a[0], a[1], a[2], a[3], hb[1][0][0], hb[1][0][1]);
+                                mma16816(acc[part * TPP + i][0], a[0], a[1], a[2], a[3], hb[2][0][0], hb[2][0][1]);
+                            }
+                        }
+                    }
+                    stage_done();
+                }
+            }
+            // the buffer's next use is the shared round after the next: every CTA of the cluster hears from every warp that has
+            // read it
+            if (CL > 1 && j >= 0 && r + 2 < R && lane == 0)
+                for (int q = 0; q < CL; ++q) arrive_cluster(cluster_addr(smem_addr(&h_empty[j & 1]), q));
+        };
+
+        // Order of work: the up projections of the static rounds; then, with the selection there, hidden values one round
+        // ahead of the down projections.  The up projection of the first shared round waits until the static rounds are
+        // done: their down stages can then be requested before the list is known.
+        int R = 0;
+        bool ready = false;
+        for (int ru = 0, rf = 0, rd = 0;;) {                                   // next round's up / finish / down
+            if (!ready && ru == my_static) {
+                mask_ready();
+                ready = true;
+                R = rounds_for(n);
+            }
+            if (ready && rd == R) break;
+            if (!ready || (rf == ru && up_next(ru, rd, R))) {
+                up(ru, min(ru, my_static));
+                ++ru;
+            } else if (rf < ru && rf <= rd + 1) {
+                const int to = rf < my_static ? my_static : rf + 1;
+                finish(rf, to);
+                rf = to;
+            } else {
+                down(rd, R);
+                ++rd;
+            }
+        }
+        cluster_arrive();                                                      // this CTA sends nothing to the others any more
+        // ---- this CTA's sums.  Codes: two lanes put their column pairs together; bf16: four lanes (g of a group of four) exchange
+        // their four values each, so that every lane has four adjacent columns of one token: 16 bytes per reduction.
+        if (R > 0) {
+#pragma unroll
+            for (int i = 0; i < TPW; ++i) {
+                const int tile = (i % TPP) * NCW + warp, col0 = (i / TPP) * STAGE_BLOCKS * SUB + tile * 16;
+#pragma unroll
+                for (int t = 0; t < NT8; ++t) {
+                    const float(&v)[4] = acc[i][t];
+                    const bool o1 = g & 1, o2 = g & 2;
+                    float4 o;
+                    int tk, col;
+                    if (Q8) {
+                        const float p0 = __shfl_xor_sync(FULL, o1 ? v[0] : v[1], 4), p1 = __shfl_xor_sync(FULL, o1 ? v[2] : v[3], 4);
+                        o = o1 ? make_float4(p0, p1, v[1], v[3]) : make_float4(v[0], v[2], p0, p1);
+                        tk = 2 * c + (o1 ? 1 : 0);
+                        col = (g & ~1) * 2;
+                    } else {
+                        // 4 x 4 transpose over the lanes: value j of all four goes to lane j of the group
+                        const float x0 = __shfl_xor_sync(FULL, o1 ? v[0] : v[1], 4), x1 = __shfl_xor_sync(FULL, o1 ? v[2] : v[3], 4);
+                        const float a0 = o1 ? x0 : v[0], a1 = o1 ? v[1] : x0, b0 = o1 ? x1 : v[2], b1 = o1 ? v[3] : x1;   // (a0, a1): value o1, (b0, b1): value 2 + o1 of the lane pair
+                        const float y0 = __shfl_xor_sync(FULL, o2 ? a0 : b0, 8), y1 = __shfl_xor_sync(FULL, o2 ? a1 : b1, 8);
+                        o = o2 ? make_float4(y0, y1, b0, b1) : make_float4(a0, a1, y0, y1);
+                        tk = 2 * c + (o1 ? 1 : 0);
+                        col = (o2 ? 8 : 0) + (g & 4);
+                    }
+                    tk += t * 8;
+                    if (tk < T && col0 + col < DC) red_add4(P.y32 + (size_t)tk * d + rank * DC + col0 + col, o);
+                }
+            }
+        }
+        // ---- the CTA that is last to add to these columns finishes them: + b2, bf16
+        consumer_bar();
+        if (tid == 0) {
+            __threadfence();                                                   // orders the whole CTA's additions (the barrier before it)
+            my_ticket = atomicAdd(P.ticket + rank, 1u);
+            if (my_ticket == (unsigned)NCL - 1) P.ticket[rank] = 0u;
+            __threadfence();
+        }
+        consumer_bar();
+        const int per_row = my_ticket == (unsigned)NCL - 1 ? DC / 4 : 0;
+#pragma unroll 4
+        for (int i = tid; i < T * per_row; i += NC) {
+            const int t = i / per_row, col = rank * DC + (i - t * per_row) * 4;
+            const float4 v = __ldcg(reinterpret_cast<const float4 *>(P.y32 + (size_t)t * d + col));
+            float bb[4] = {0.f, 0.f, 0.f, 0.f};
+            if (P.b2) {
+                const uint2 q = __ldg(reinterpret_cast<const uint2 *>(P.b2 + col));
+                bb[0] = __uint_as_float(q.x << 16); bb[1] = __uint_as_float(q.x & 0xffff0000u);
+                bb[2] = __uint_as_float(q.y << 16); bb[3] = __uint_as_float(q.y & 0xffff0000u);
+            }
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x + bb[0], v.y + bb[1]), hi = __floats2bfloat162_rn(v.z + bb[2], v.w + bb[3]);
+            *reinterpret_cast<uint2 *>(P.y + (size_t)t * d + col) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        }
+    }
+    cluster_wait();                                                            // nobody leaves while another CTA may still send to it
+}
+
+constexpr size_t kSmemLimit = 218 * 1024;
+
+int nt8_for(int T) { return T <= 8 ? 1 : T <= 16 ? 2 : 4; }
+
+template <typename WT> size_t fixed_smem(const FfnShape &S)
+{
+    const size_t t8 = 8 * (size_t)nt8_for(S.T);
+    return 1024 + t8 * x_pitch(S.d) + (size_t)(S.gated ? 2 : 1) * NCW * 16 * t8 * 4 + (size_t)(S.n_static + 1) * 3 * 16 * t8 * 4 +
+           (size_t)(S.n_static + 2) * S.cl * S.planes * t8 * H_ROW + (size_t)(S.T + 1) * S.W * 4;
+}
+
+// Output tiles per warp for clusters of cl CTAs; 0: the shape cannot be cut that way.  A unit's rows of W2T are cut into
+// cl pieces of whole 128-byte blocks, several pieces to a stage or whole stages to a piece, and 16 x 8-token tiles of
+// output accumulators take at most 32 registers.
+template <typename WT> int tiles_per_warp(int d, int cl, int T)
+{
+    const int blocks = d / sub_cols<WT>();
+    if (d % sub_cols<WT>() || blocks % cl) return 0;
+    const int nb = blocks / cl, n = d2d_cdiv(d / cl, NCW * 16), tpw = n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : n <= 8 ? 8 : 0;
+    if (nb > STAGE_BLOCKS && nb != STAGE_BLOCKS * (tpw / (sub_cols<WT>() / 16))) return 0;
+    return tpw * nt8_for(T) <= 8 ? tpw : 0;
+}
+
+// Fills in the launch parameters for n layers; false: no cluster size fits the shape.
+template <typename WT> bool plan(FfnShape &S, int n_layers)
+{
+    const int U = S.d_ff / 16, sms = d2d_tc_sm_count();
+    int best = 0;
+    // Fewest rounds first (the rounds stream the weights), then the larger cluster (fewer sums to merge).  Clusters of four
+    // reach 132 of 148 SMs, smaller ones all of them.  One or two rows of sums are cheaper to merge than hidden values to
+    // exchange (1.2 us).
+    for (int cl = S.T * S.d <= 2048 && tiles_per_warp<WT>(S.d, 1, S.T) ? 1 : 4; cl >= 1; cl /= 2) {
+        const int clusters = (cl == 4 ? sms * 33 / 37 : sms) / n_layers / cl;
+        if (clusters < 1 || tiles_per_warp<WT>(S.d, cl, S.T) == 0) continue;
+        const int rounds = d2d_cdiv(d2d_cdiv(U, cl), clusters);
+        if (best == 0 || rounds < best) {
+            best = rounds;
+            S.cl = cl;
+            S.clusters = d2d_cdiv(d2d_cdiv(U, cl), rounds);
+        }
+    }
+    if (best == 0) return false;
+    const int blocks = S.d / sub_cols<WT>();
+    S.up_blocks = blocks < STAGE_BLOCKS ? blocks : STAGE_BLOCKS;
+    S.nb = blocks / S.cl;
+    S.sps = S.nb >= STAGE_BLOCKS ? 1 : STAGE_BLOCKS / S.nb < S.cl ? STAGE_BLOCKS / S.nb : S.cl;
+    // Rounds a cluster starts on before the selection is known: what the ring holds beside the up stages, which are used up
+    // by then.  None for the smallest batches, which keep a fraction of the experts: most of what would be fetched early
+    // would be thrown away.
+    const int per_up = d2d_cdiv(S.d, seg_cols<WT>()) * (S.gated ? 2 : 1), per_down = d2d_cdiv(S.d, seg_cols<WT>());
+    const int most = nt8_for(S.T) > 2 ? 2 : 4;
+    S.n_static = most;                                       // (the largest, while the ring is sized)
+    const size_t f = fixed_smem<WT>(S);
+    S.stages = f >= kSmemLimit ? 0 : (int)((kSmemLimit - f) / STAGE_BYTES);
+    if (S.stages > MAX_STAGES) S.stages = MAX_STAGES;
+    const int fit = (S.stages + per_up) / (per_up + per_down);
+    S.n_static = S.planes == 3 ? 0 : fit < 1 ? 1 : fit < most ? fit : most;
+    return S.stages >= 3;
+}
+
+FfnShape shape_for(const d2d_layer_desc &D, int T)
+{
+    FfnShape S = {};
+    S.T = T; S.d = D.d; S.d_ff = D.d_ff; S.E = D.n_experts; S.s = D.expert_size; S.inv_s = (uint32_t)((0x100000000ull + D.expert_size - 1) / D.expert_size); S.W = (D.n_experts + 31) / 32;
+    S.act = D.act; S.gated = D.gated ? 1 : 0;
+    S.planes = T <= d2d_decode_max_tokens(D) ? 3 : 1;
+    return S;
+}
+
+template <typename WT, int TPW, int NT8>
+d2d_status launch(const FfnShape &S, int n_layers, const d2d_decode_ffn_args &a, const void *x, bool after_router, cudaStream_t st)
+{
+    auto kern = decode_ffn_kernel<WT, TPW, NT8>;
+    static bool attr_set[64] = {};                          // the attribute is per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return D2D_ERR_CUDA;
+    if (!__atomic_load_n(&attr_set[dev], __ATOMIC_ACQUIRE)) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess) return D2D_ERR_CUDA;
+        __atomic_store_n(&attr_set[dev], true, __ATOMIC_RELEASE);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S.clusters * S.cl, n_layers, 1);
+    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.dynamicSmemBytes = fixed_smem<WT>(S) + (size_t)S.stages * STAGE_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S.cl; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = after_router && d2d_tc_pdl_enabled() ? 2 : 1;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, (const __nv_bfloat16 *)x, S, a);
+    D2D_LAUNCHED(1);
+    return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+}
+
+template <typename WT>
+d2d_status dispatch(FfnShape S, int n, const d2d_decode_ffn_args &a, const void *x, bool after, cudaStream_t st)
+{
+    if (!plan<WT>(S, n)) return D2D_ERR_UNSUPPORTED;
+    d2d_decode_ffn_args b = a;
+    for (int l = 0; l < n; ++l) b.l[l].tm_w2t = a.l[l].tm_w2t_cl[S.cl == 4 ? 2 : S.cl == 2 ? 1 : 0];
+    const int tpw = tiles_per_warp<WT>(S.d, S.cl, S.T), nt = nt8_for(S.T);
+    switch (tpw * 10 + nt) {
+    case 11: return launch<WT, 1, 1>(S, n, b, x, after, st);
+    case 12: return launch<WT, 1, 2>(S, n, b, x, after, st);
+    case 14: return launch<WT, 1, 4>(S, n, b, x, after, st);
+    case 21: return launch<WT, 2, 1>(S, n, b, x, after, st);
+    case 22: return launch<WT, 2, 2>(S, n, b, x, after, st);
+    case 24: return launch<WT, 2, 4>(S, n, b, x, after, st);
+    case 41: return launch<WT, 4, 1>(S, n, b, x, after, st);
+    case 42: return launch<WT, 4, 2>(S, n, b, x, after, st);
+    case 81: return launch<WT, 8, 1>(S, n, b, x, after, st);
+    }
+    return D2D_ERR_UNSUPPORTED;
+}
+
+template <typename WT> bool make_map(CUtensorMap *m, const void *w, int rows, int d, int blocks)
+{
+    const cuuint64_t dims[3] = {(cuuint64_t)sub_cols<WT>(), (cuuint64_t)rows, (cuuint64_t)(d / sub_cols<WT>())};
+    const cuuint64_t strides[2] = {(cuuint64_t)d * sizeof(WT), 128};
+    const cuuint32_t box[3] = {(cuuint32_t)sub_cols<WT>(), 16, (cuuint32_t)(blocks < STAGE_BLOCKS ? blocks : STAGE_BLOCKS)};
+    return d2d_tc_encode_map(m, sizeof(WT) == 1, 3, w, dims, strides, box);
+}
+
+template <typename WT> d2d_status make_maps(d2d_layer *L, const void *w1, const void *wg, const void *w2t)
+{
+    const int d = L->desc.d, rows = L->desc.d_ff, blocks = d / sub_cols<WT>();
+    if (d % sub_cols<WT>() || rows % 16) return D2D_OK;
+    bool ok = make_map<WT>(&L->tm_dec[0], w1, rows, d, blocks) && (!wg || make_map<WT>(&L->tm_dec[1], wg, rows, d, blocks));
+    for (int i = 0; i < 3; ++i)
+        if (blocks % (1 << i) == 0) ok = ok && make_map<WT>(&L->tm_dec[2 + i], w2t, rows, d, blocks >> i);
+    L->dec_maps = ok;
+    return ok ? D2D_OK : D2D_ERR_CUDA;
+}
+
+}  // namespace
+
+// The layer's tensor maps (its weights stay where they are for the layer's lifetime): W1, W_gate, and W2T as clusters of
+// 1, 2 and 4 CTAs read it.  L->dec_maps stays 0 for shapes the kernel does not take.
+d2d_status d2d_decode_ffn_maps(d2d_layer *L)
+{
+    L->dec_maps = 0;
+    if (L->desc.dtype != D2D_BF16) return D2D_OK;
+    return L->q_w1 ? make_maps<uint8_t>(L, L->q_w1, L->q_wg, L->q_w2t) : make_maps<__nv_bfloat16>(L, L->w1, L->w_gate, L->w2t);
+}
+
+// Whole 16-neuron units, rows of whole 128-byte blocks, a batch whose rows fit shared memory beside three stages.
+bool d2d_decode_ffn_supports(const d2d_layer_desc &D, int n_layers, int T, bool fp8)
+{
+    if (D.dtype != D2D_BF16 || T < 1 || T > 32 || D.d_ff % 16 || D.d_ff / 16 > MAX_UNITS) return false;
+    FfnShape S = shape_for(D, T);
+    return fp8 ? plan<uint8_t>(S, n_layers) : plan<__nv_bfloat16>(S, n_layers);
+}
+
+int d2d_decode_ffn_first_shared(const d2d_layer_desc &D, int n_layers, int T, bool fp8)
+{
+    FfnShape S = shape_for(D, T);
+    if (!(fp8 ? plan<uint8_t>(S, n_layers) : plan<__nv_bfloat16>(S, n_layers))) return 0;
+    return S.n_static * S.clusters * S.cl;
+}
+
+d2d_status d2d_decode_ffn(const d2d_layer_desc &D, int n_layers, const d2d_decode_ffn_args &a, const void *x, int T, bool after_router,
+                          cudaStream_t st)
+{
+    const bool fp8 = a.l[0].k1 != nullptr;
+    if (n_layers < 1 || n_layers > D2D_MAX_GROUP) return D2D_ERR_UNSUPPORTED;
+    const FfnShape S = shape_for(D, T);
+    return fp8 ? dispatch<uint8_t>(S, n_layers, a, x, after_router, st) : dispatch<__nv_bfloat16>(S, n_layers, a, x, after_router, st);
+}

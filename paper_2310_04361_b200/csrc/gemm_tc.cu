@@ -750,6 +750,16 @@ bool d2d_tc_make_map(CUtensorMap *map, const void *base, int rows, int cols, int
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool d2d_tc_encode_map(CUtensorMap *map, bool bytes, int rank, const void *base, const cuuint64_t *dims, const cuuint64_t *strides,
+                       const cuuint32_t *box)
+{
+    encode_tiled_fn enc = get_encode();
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return enc && enc(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base),
+                      dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int d2d_tc_sm_count()
 {
     static int cached = 0;

@@ -14,6 +14,7 @@
 #include <string.h>
 
 #include "d2d_common.cuh"
+#include "decode.cuh"
 #include "gemm_tc.cuh"
 
 namespace {
@@ -31,6 +32,16 @@ bool routing_full(const d2d_routing *r)
     if (!r->mask || !r->k || !r->counts || !r->offsets || !r->perm || !r->n_sel || !r->status) return false;
     if ((r->tok_off == nullptr) != (r->tok_exp == nullptr)) return false;
     return r->perm_capacity >= 0;
+}
+
+// Batches the cluster router and the streaming expert kernel take: every layer by the rule of d2d_layer_fwd, bf16 weights
+// in all of them or codes in all of them.
+bool decode_kernels(const d2d_group *g, int T)
+{
+    if (!d2d_decode_router_supports(g->desc, T)) return false;
+    for (int l = 0; l < g->n; ++l)
+        if (!d2d_use_decode_ffn(g->layers[l], g->n, T) || (g->layers[l]->q_w1 != nullptr) != (g->layers[0]->q_w1 != nullptr)) return false;
+    return true;
 }
 
 // Workspace of d2d_group_fwd.
@@ -54,10 +65,10 @@ group_layout layout_for(const d2d_group *g, int T)
     group_layout w;
     size_t off = 0;
     w.sel_off = off; w.sel_each = d2d_align_up(d2d_select_ws_bytes((int)Tn, D.n_experts), 256); off += n * w.sel_each;
-    const bool decode = (int)Tn <= 8;
+    const bool decode = (int)Tn <= 8 || decode_kernels(g, (int)Tn);
     w.r_off = off; w.r_each = decode ? d2d_align_up(Tn * D.n_experts * 4, 256) : 0; off += n * w.r_each;
     w.u_off = off; w.u_each = decode ? d2d_align_up(Tn * D.d_h * 4, 256) : 0; off += n * w.u_each;
-    w.y32_off = off; w.y32_each = decode ? d2d_align_up(Tn * D.d * 4, 256) : 0; off += n * w.y32_each;
+    w.y32_off = off; w.y32_each = decode ? d2d_decode_scratch_bytes(D, (int)Tn) : 0; off += n * w.y32_each;
     w.mask_off = off;
     if (g->merged) off += d2d_align_up(Tn * n * W * 4, 256);
     w.h_off = off;
@@ -179,6 +190,11 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
     char *base = (char *)ws;
 
     // ---- decode batches: two launches for the whole group
+    if (decode_kernels(g, T)) {
+        void *scratch[D2D_MAX_GROUP];
+        for (int l = 0; l < n; ++l) scratch[l] = base + w.y32_off + (size_t)l * w.y32_each;
+        return d2d_decode_layers(g->layers, n, x, T, tau, routing, nullptr, scratch, y, st);
+    }
     if (d2d_small_router_supports(D, T) && d2d_small_ffn_supports(D) && T <= (D.dtype == D2D_BF16 ? d2d_decode_max_tokens(D) : 8)) {
         float *R[D2D_MAX_GROUP], *u[D2D_MAX_GROUP], *y32[D2D_MAX_GROUP];
         for (int l = 0; l < n; ++l) {

@@ -5,6 +5,7 @@
 // in float32 in the workspace.  It covers every dtype and shape (fp32 layers must not
 // go through reduced-precision tensor-core formats to stay within 1e-4).
 #include "d2d_common.cuh"
+#include "decode.cuh"
 #include "gemm_tc.cuh"
 
 namespace {
@@ -82,6 +83,11 @@ d2d_status d2d_launch_router(const d2d_layer *L, const void *x, int T, float *R,
     if (T == 0) return D2D_OK;
     // u_ws points at [256-byte ticket area | T*d_h floats]
     float *u = (float *)((char *)u_ws + 256);
+    if (d2d_decode_router_supports(L->desc, T)) {
+        d2d_decode_router_args a = {};
+        a.l[0] = d2d_decode_router_args_for(L, nullptr, R, nullptr);
+        return d2d_decode_router(L->desc, 1, a, x, T, 0.0f, 0, 0, st);
+    }
     if (d2d_small_router_supports(L->desc, T)) return d2d_small_router(L, x, T, R, u_ws, st);
     if (d2d_router_fused_supports(L->desc, T)) return d2d_router_fused(L, x, T, 0.0f, 0, R, nullptr, nullptr, nullptr, st);
     if (L->desc.dtype == D2D_F32) return run_router<float>(L, x, T, R, u, st);

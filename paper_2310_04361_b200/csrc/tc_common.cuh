@@ -248,6 +248,9 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&r)[16
 // [rows, cols] bf16 row-major matrix as a TMA tensor map: box = box_rows x 64 columns, 128-byte swizzle, zero fill
 // outside the matrix.  False when the driver entry point for tensor-map encoding is unavailable or the encode fails.
 bool d2d_tc_make_map(CUtensorMap *map, const void *base, int rows, int cols, int box_rows);
+// The same with any rank, strides and box, for bf16 elements or bytes.
+bool d2d_tc_encode_map(CUtensorMap *map, bool bytes, int rank, const void *base, const cuuint64_t *dims, const cuuint64_t *strides,
+                       const cuuint32_t *box);
 // Number of SMs of the current device (148 when the query fails).
 int d2d_tc_sm_count();
 // False when D2D_GEMM_PDL=0 asks for fully serialised launches.

@@ -663,3 +663,45 @@ def test_small_fp32_layer_runs_in_one_launch(api, T, act, gated, lists):
         y_self = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[cfg.act], G)
         assert _rel_err(y.cpu().numpy(), y_self) <= TOL_Y["f32"]
     layer.close()
+
+
+# decode batches (cluster router + streaming expert kernel) at the edges of their tiles: token blocks of 8 / 16 / 32, the
+# last batch they take and the first they do not, experts of one unit (16 neurons), of two, and not of whole units (24: the
+# kept units are found from the mask), a width of 12 column blocks, output tiles of 1 / 2 / 4 / 8 per warp, fewer units than
+# CTAs, several scorers (E > 256), codes; a row of b1-less gated neurons
+DECODE_CASES = [(dict(d=1024, d_ff=4096, E=256), t, False) for t in (1, 7, 8, 9, 16, 17, 32, 33)] + [
+    (dict(d=768, d_ff=3072, E=128), 1, False), (dict(d=768, d_ff=3072, E=128), 12, False), (dict(d=768, d_ff=768, E=24), 20, False),
+    (dict(d=2048, d_ff=1600, E=100), 5, False), (dict(d=2048, d_ff=1600, E=100), 16, False), (dict(d=2048, d_ff=1600, E=100), 1, False),
+    (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 8, False),
+    (dict(d=4096, d_ff=5504, E=344, d_h=256), 3, False), (dict(d=64, d_ff=48, E=3, d_h=16), 6, False),
+    (dict(d=1024, d_ff=4096, E=256), 6, True), (dict(d=1024, d_ff=4096, E=128, act="relu"), 2, True),
+    (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 4, True)]
+
+
+@pytest.mark.parametrize("shape,T,fp8", DECODE_CASES)
+def test_decode_batches_at_the_edges_of_their_tiles(api, shape, T, fp8):
+    cfg = wl.LayerConfig("edge", "bf16", **{**dict(d_h=128, act="gelu_erf", token_sigma=0.5, b1_shift=-0.3), **shape}, T=T, seed=31)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w, fp8_experts=fp8)
+    if fp8:
+        w = dict(w)
+        for name in ("w1", "w_gate"):
+            w[name] = w[name] if w[name] is None else oracle.quantize_experts_e4m3(w[name], cfg.E)[2]
+        w["w2"] = np.ascontiguousarray(oracle.quantize_experts_e4m3(np.ascontiguousarray(w["w2"].T), cfg.E)[2].T)
+    act, xd = oracle.ACT_BY_NAME[cfg.act], api.to_device(x, cfg.dtype)
+    for tau in (0.9, 0.3, 0.0):
+        R = _poison(torch.empty((T, cfg.E), dtype=torch.float32, device="cuda"))
+        y = _poison(torch.empty((T, cfg.d), dtype=torch.bfloat16, device="cuda"))
+        _poison(layer.workspace(T))
+        y, r = layer.layer_fwd(xd, tau, y=y, R_out=R, routing=layer.new_routing(T, dual=True))
+        torch.cuda.synchronize()
+        assert r.status == 0
+        assert _rel_err(R.cpu().numpy(), oracle.router(x, w["w_r1"], w["b_r1"], w["w_r2"], w["b_r2"])) <= TOL_R["bf16"]
+        G = oracle.unpack_mask(r.mask_u32(), cfg.E)
+        assert np.array_equal(G, oracle.select(R.cpu().numpy(), tau)[0])
+        _check_routing(r, G, dual=True)
+        y_ref = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], act, G)
+        assert _rel_err(y.float().cpu().numpy(), y_ref) <= TOL_Y["bf16"]
+        y2 = layer.moe_ffn_fwd(xd, r)                      # the expert step on its own: no list of kept units from the router
+        assert _rel_err(y2.float().cpu().numpy(), y_ref) <= TOL_Y["bf16"]
+    layer.close()
