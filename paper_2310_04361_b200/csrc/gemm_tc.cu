@@ -60,7 +60,7 @@ __device__ __forceinline__ void tile_coords(int tile, int rows, int cols, int ba
 // 16 accumulator columns -> 16 output values: bias (float32, staged in shared memory), activation, selection mask.
 template <int EPI, int ACT, bool GATED>
 __device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint32_t (&g)[16], float (&v)[16],
-                                            const float *bias_f, bool has_bias, int col0, uint32_t keep, bool halves)
+                                            const float *bias_f, bool has_bias, int col0)
 {
     float bias[16];
     if (has_bias) {
@@ -73,9 +73,9 @@ __device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint3
 #pragma unroll
         for (int j = 0; j < 16; ++j) bias[j] = 0.0f;
     }
-    if (EPI == D2D_EPI_UP_MASKED && halves) {
-        // the common case of the up projection: math on pairs; the selection is applied by the caller on the packed
-        // bf16 words (each 8-column half belongs to one expert)
+    if (EPI == D2D_EPI_UP_MASKED) {
+        // math on pairs; the selection is applied by the caller on the packed bf16 words (each 8-column half belongs to one
+        // expert)
 #pragma unroll
         for (int j = 0; j < 16; j += 2) {
             // first accumulator = up projection (+ bias), second = gate
@@ -91,10 +91,6 @@ __device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint3
         float z = __uint_as_float(r[j]) + bias[j];
         if (EPI == D2D_EPI_RELU_BF16) z = fmaxf(z, 0.0f);
         if (EPI == D2D_EPI_ABS_F32) z = fabsf(z);
-        if (EPI == D2D_EPI_UP_MASKED) {
-            const float h = GATED ? fast_act<ACT>(__uint_as_float(g[j])) * z : fast_act<ACT>(z);
-            z = ((keep >> j) & 1u) ? h : 0.0f;
-        }
         v[j] = z;
     }
 }
@@ -151,18 +147,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // swizzle atoms are 1024-byte aligned
     __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t tmem_base_holder;
-    __shared__ volatile int epi_ok[2];                               // outcome of the epilogue's accumulator wait (per buffer parity)
+    // what the epilogue's leader publishes (per buffer parity): go on (or the work is done, or a wait ran out), tile coordinates
+    __shared__ volatile int epi_go[2], epi_m0[2], epi_n0[2], epi_prob[2];
     // dynamic scheduling: the producer draws work items from a global counter and hands them to the MMA thread and
     // to the epilogue through a two-slot ring (a CTA that starts late, or gets slow tiles, simply draws fewer)
     __shared__ uint64_t sched_full[2], sched_empty[2];
-    __shared__ volatile int sched_item[2], epi_item[2];
-    constexpr int MASK_REGS = 8;                                     // selection words of a row kept in registers (E <= 256; wider masks are read through L1)
+    __shared__ volatile int sched_item[2];
     // the whole bias vector is staged once, as float32, behind the operand stages when it fits
     float *bias_f = reinterpret_cast<float *>(smem + (size_t)STAGES * STAGE_BYTES);
     const int NB = N * ep.batch;                                     // bias entries of all problems
     const bool bias_cached = ep.bias != nullptr && NB <= BIAS_CACHE_ELEMS && (N & 3) == 0;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // warp-uniform: roles, columns
     const int nkb = (K + BK - 1) / BK;
     const int n_tiles = (N + BN - 1) / BN;
     // work item = (output tile, K split); with k_splits > 1 every item accumulates a slice of K and the
@@ -384,64 +380,60 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         const int quad = warp & 3;                          // TMEM lanes this warp may touch
         const int part = ew >> 2;                           // which quarter of the tile's columns
         constexpr int N_UNITS = COLS_PER_WARP / 16;
-        uint32_t local = 0;
-        bool ok = true;
-        for (;; ++local) {
+        for (uint32_t local = 0;; ++local) {
             const uint32_t buf = local & 1u, use = local >> 1;
-            int item = worker + (int)local * n_workers;
-            if (dyn) {
-                // the leader takes the item from the ring and publishes it to the sixteen warps
-                if (ew == 0 && lane == 0) {
-                    int got = -2;                            // -2: the wait ran out
-                    if (mbar_wait(smem_u32(&sched_full[buf]), use & 1u, ep.status)) {
-                        got = sched_item[buf];
+            // ONE thread takes the item from the ring, works out its coordinates (integer divisions), waits for the accumulator
+            // and publishes the outcome; the other epilogue warps sleep on a hardware barrier.  Sixteen pollers measurably slow
+            // the producer and MMA threads, whose own barrier tests share the same unit.
+            if (ew == 0 && lane == 0) {
+                int item = worker + (int)local * n_workers;
+                bool go = true;
+                if (dyn) {
+                    go = mbar_wait(smem_u32(&sched_full[buf]), use & 1u, ep.status);
+                    if (go) {
+                        item = sched_item[buf];
                         mbar_arrive(smem_u32(&sched_empty[buf]));
                     }
-                    epi_item[buf] = got;
                 }
-                asm volatile("bar.sync 1, %0;" ::"r"(N_EPI_WARPS * 32) : "memory");
-                item = epi_item[buf];
-                if (item < 0) break;
+                go = go && item >= 0 && item < total_tiles;
+                if (go) {
+                    int tile = (!GATED && k_splits == 1) ? item : item / k_splits;
+                    int prob = 0, tr, tc;
+                    if (ep.batch > 1) { prob = tile / tiles_pp; tile -= prob * tiles_pp; }
+                    tile_coords(tile, (M + TM - 1) / TM, n_tiles, ep.band_rows, tr, tc);
+                    epi_m0[buf] = tr * TM; epi_n0[buf] = tc * BN; epi_prob[buf] = prob;
+                    go = mbar_wait(smem_u32(&bar_acc_full[buf]), use & 1u, ep.status);
+                }
+                epi_go[buf] = go ? 1 : 0;
             }
-            if (item >= total_tiles) break;
-            int tile = (!GATED && k_splits == 1) ? item : item / k_splits;
-            int prob = 0;
-            if (ep.batch > 1) { prob = tile / tiles_pp; tile -= prob * tiles_pp; }
-            int tr, tc;
-            tile_coords(tile, (M + TM - 1) / TM, n_tiles, ep.band_rows, tr, tc);
-            const int m0 = tr * TM, n0 = tc * BN;
+            asm volatile("bar.sync 1, %0;" ::"r"(N_EPI_WARPS * 32) : "memory");
+            if (!epi_go[buf]) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const int m0 = epi_m0[buf], n0 = epi_n0[buf], prob = epi_prob[buf];
             // this problem's bias entries and output matrix
             const float *bias_p = bias_f + prob * N;
             const __nv_bfloat16 *bias_g = ep.bias ? ep.bias + prob * N : nullptr;
             void *out_p = (char *)ep.out + (size_t)prob * M * N * ((EPI == D2D_EPI_ABS_F32 || EPI == D2D_EPI_PARTIAL_F32) ? 4 : 2);
             const int row = m0 + quad * 32 + lane;
-            // this row's selection words go to registers before the wait, so their latency is hidden
-            uint32_t mw[MASK_REGS];
+            // Selection of this row, for the 8-column groups of this warp's columns (expert sizes that are multiples of 8: a group
+            // belongs to one expert): the experts of the range are consecutive bits of at most two mask words, loaded here and
+            // looked at after the first unit's math; bit h of kbits = group h.  Which expert a group belongs to is the same for
+            // all rows.  (Selecting among all words of the row in registers, group by group, was 3 of 18 instructions per
+            // element.)
+            const int colw = n0 + part * COLS_PER_WARP;
             const uint32_t *mrow = nullptr;
+            uint32_t kbits = 0xffffffffu, mw0 = 0u, mw1 = 0u, e0 = 0u;
             if (EPI == D2D_EPI_UP_MASKED && ep.mask && row < M) {
                 mrow = ep.mask + (size_t)row * ep.mask_words;
-                if (ep.mask_words <= MASK_REGS) {
-#pragma unroll
-                    for (int i = 0; i < MASK_REGS; ++i) mw[i] = i < ep.mask_words ? __ldg(mrow + i) : 0u;
+                if ((ep.expert_size & 7) == 0 && colw < N) {
+                    e0 = __umulhi((uint32_t)colw, ep.inv_expert_size);
+                    const int wi = (int)(e0 >> 5);
+                    mw0 = __ldg(mrow + wi);
+                    mw1 = wi + 1 < ep.mask_words ? __ldg(mrow + wi + 1) : 0u;
                 }
             }
-            // ONE thread polls the accumulator barrier and the other epilogue warps sleep on a hardware barrier: sixteen
-            // pollers measurably slow the producer and MMA threads, whose own barrier tests share the same unit
-            if (ew == 0 && lane == 0) epi_ok[local & 1u] = mbar_wait(smem_u32(&bar_acc_full[buf]), use & 1u, ep.status) ? 1 : 0;
-            asm volatile("bar.sync 1, %0;" ::"r"(N_EPI_WARPS * 32) : "memory");
-            ok = epi_ok[local & 1u] != 0;
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t tbase = tmem_base + buf * BUF_COLS + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * COLS_PER_WARP);
 
-            // expert that owns the first column of this warp's range (one division per tile; advanced incrementally)
-            const int colw = n0 + part * COLS_PER_WARP;
-            int e = 0, lo = 0, widx = -1;
-            uint32_t word = 0u;
-            if (EPI == D2D_EPI_UP_MASKED && mrow) {
-                e = colw / ep.expert_size;
-                lo = e * ep.expert_size - colw;             // first column of expert e relative to the current unit (<= 0)
-            }
             const bool bias_fast = ep.bias == nullptr || bias_cached;
             const bool wide_store = (N & 15) == 0 && (reinterpret_cast<uintptr_t>(out_p) & 31) == 0;   // 32-byte aligned rows
             const bool mask_on = EPI == D2D_EPI_UP_MASKED && ep.mask != nullptr;                         // CTA-uniform
@@ -456,27 +448,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 // two accumulators per column; a second set would spill, so each unit is loaded when it is needed and
                 // the other epilogue warps of the SM sub-partition cover the latency.
                 if (!GATED) tmem_ld16_issue(tbase, ra);
-                // selection bits of this row, one per 8-column group of the warp's columns (each group belongs to one
-                // expert; e = col / s by a multiply-high with the precomputed reciprocal); done once per tile so that the
-                // unrolled units below stay small
-                uint32_t kbits = 0xffffffffu;
-                if (mask_on && mrow) {
-                    kbits = 0u;
-#pragma unroll
-                    for (int h = 0; h < COLS_PER_WARP / 8; ++h) {
-                        const uint32_t ee = __umulhi((uint32_t)(colw + 8 * h), ep.inv_expert_size);
-                        const int wi = (int)(ee >> 5);
-                        uint32_t wd;
-                        if (ep.mask_words <= MASK_REGS) {
-                            wd = mw[0];
-#pragma unroll
-                            for (int i = 1; i < MASK_REGS; ++i) wd = (i == wi) ? mw[i] : wd;
-                        } else {
-                            wd = __ldg(mrow + wi);
-                        }
-                        kbits |= ((wd >> (ee & 31)) & 1u) << h;
-                    }
-                }
 #pragma unroll
                 for (int u = 0; u < N_UNITS; ++u) {             // at most 4 units
                     const int col0 = colw + u * 16;
@@ -486,13 +457,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                         tmem_ld16_issue(tbase + u * 16, ra);
                         tmem_ld16_issue(tbase + u * 16 + BN, reinterpret_cast<uint32_t (&)[16]>(ga));
                     }
-                    const uint32_t keep = ((kbits >> (2 * u)) & 1u ? 0x00ffu : 0u) | ((kbits >> (2 * u + 1)) & 1u ? 0xff00u : 0u);
                     tmem_ld_wait();                                               // this unit's accumulators have landed
                     if (!GATED && u + 1 < N_UNITS)                                // the next unit's load overlaps the math below
                         tmem_ld16_issue(tbase + (u + 1) * 16, (u & 1) ? ra : reinterpret_cast<uint32_t (&)[16]>(rb));
 
                     float v[16];
-                    epilogue_16<EPI, ACT, GATED>(r, g, v, bias_p, ep.bias != nullptr, col0, keep, EPI == D2D_EPI_UP_MASKED);
+                    epilogue_16<EPI, ACT, GATED>(r, g, v, bias_p, ep.bias != nullptr, col0);
+                    if (EPI == D2D_EPI_UP_MASKED && u == 0 && mask_on) {
+                        const uint32_t bits = __funnelshift_r(mw0, mw1, e0 & 31u);
+                        kbits = 0u;
+#pragma unroll
+                        for (int h = 0; h < COLS_PER_WARP / 8; ++h)
+                            kbits |= ((bits >> (__umulhi((uint32_t)(colw + 8 * h), ep.inv_expert_size) - e0)) & 1u) << h;
+                    }
+                    // all ones where the token keeps the expert of the unit's first / second eight columns
+                    const uint32_t keep2[2] = {(uint32_t)((int)(kbits << (31 - 2 * u)) >> 31), (uint32_t)((int)(kbits << (30 - 2 * u)) >> 31)};
                     if (row < M) {
                         if (EPI == D2D_EPI_PARTIAL_F32) {
                             float *o = (float *)out_p + (size_t)row * N + col0;
@@ -513,7 +492,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                                 pk[j] = *reinterpret_cast<uint32_t *>(&t);
                                 // selection: an expert the token did not keep contributes zeros (also when its
                                 // pre-activations are not finite)
-                                if (EPI == D2D_EPI_UP_MASKED) pk[j] = (keep >> (2 * j)) & 1u ? pk[j] : 0u;
+                                if (EPI == D2D_EPI_UP_MASKED) pk[j] &= keep2[j >> 2];
                             }
                             if (wide_store) {
                                 // one 32-byte store per row and unit: a whole sector per lane, half as many store instructions
@@ -528,6 +507,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 }
             } else {
                 // generic loop: one unit at a time, every bound checked, any expert size
+                // expert that owns the first column of this warp's range (one division per tile; advanced incrementally)
+                int e = 0, lo = 0, widx = -1;
+                uint32_t word = 0u;
+                if (EPI == D2D_EPI_UP_MASKED && mrow) {
+                    e = colw / ep.expert_size;
+                    lo = e * ep.expert_size - colw;         // first column of expert e relative to the current unit (<= 0)
+                }
                 uint32_t (&g)[16] = reinterpret_cast<uint32_t (&)[16]>(ga);
 #pragma unroll 1
                 for (int u = 0; u < N_UNITS; ++u) {
