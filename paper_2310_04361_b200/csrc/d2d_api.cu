@@ -763,8 +763,8 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     }
     if (d2d_router_fused_supports(layer->desc, T)) {
         // router and dynamic-k mask in one kernel; the selection step then only builds the per-expert metadata
-        if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
         const bool dense = use_dense_masked(layer, T) && !use_small_ffn(layer, T);
+        if (!dense && cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
         // tile counter of the up projection: layer-owned, zero at creation and reset by the kernel that used it, so no
         // memset node sits in front of the router (the up projection may begin while the router is still running)
         int *up_counter = dense ? (int *)(layer->tickets + 32) : nullptr;
@@ -780,7 +780,7 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
                 if (cudaEventRecord(layer->ev_fork, st) != cudaSuccess ||
                     cudaStreamWaitEvent(layer->side_stream, layer->ev_fork, 0) != cudaSuccess)
                     return D2D_ERR_CUDA;
-                rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1);
+                rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1, layer->tickets + 48);
                 if (rc != D2D_OK) return rc;
             }
             rc = d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, up_counter, 0, ksum + 4);
@@ -815,7 +815,7 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
         if (lists) {
             if (cudaEventRecord(layer->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(layer->side_stream, layer->ev_fork, 0) != cudaSuccess)
                 return D2D_ERR_CUDA;
-            rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1);
+            rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1, layer->tickets + 48);
             if (rc != D2D_OK) return rc;
         }
         rc = d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, nullptr, 0, ksum + 4);

@@ -41,9 +41,9 @@ struct d2d_layer {
     cudaEvent_t ev_in[kHostChunks], ev_done[kHostChunks], ev_begin, ev_end;
     // layer-owned "last CTA" tickets of the decode kernels used by d2d_layer_fwd (zero at creation, reset by the kernel
     // that used them): word 0 decode router, word 16 decode experts, word 32 tile counter of the up projection, words
-    // 40 / 41 sum of k and exit ticket of the fused router, word 44 the number of selected pairs the fused router
-    // publishes for the density-adaptive dispatch of the expert step, word 52 exit ticket of the one-launch layer
-    // kernel of small float32 problems.  Like the side stream, they make concurrent
+    // 40 / 41 / 42 sum of k, exit ticket and largest condition of the fused router, word 44 the number of selected pairs the fused router
+    // publishes for the density-adaptive dispatch of the expert step, word 48 ticket of the lists built on the side stream, word
+    // 52 exit ticket of the one-launch layer kernel of small float32 problems.  Like the side stream, they make concurrent
     // d2d_layer_fwd calls on ONE layer object from several streams unsafe; use one layer object per stream for that.
     // A call that ended in D2D_ERR_TIMEOUT may leave them non-zero: d2d_layer_reset_counters clears them.
     unsigned int *tickets;
@@ -106,7 +106,7 @@ size_t d2d_select_ws_bytes(int T, int E);
 // (fused router), only the per-expert metadata is built.
 d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d2d_routing *out, int32_t *ksum, cudaStream_t st);
 d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, const d2d_routing *out,
-                             void *ws, cudaStream_t st, int mask_ready = 0);
+                             void *ws, cudaStream_t st, int mask_ready = 0, unsigned int *zero_ticket = nullptr);
 
 // up_counter: see launch_tc_experts (NULL unless the fused router was launched just before on `st`)
 // n_sel: device word that holds the number of selected pairs when the expert kernels start (NULL: r->n_sel)
@@ -126,8 +126,9 @@ bool d2d_small_select_supports(int T, int E);
 d2d_status d2d_small_select(const float *R, int T, int E, float tau, const d2d_routing *out, cudaStream_t st,
                             int mask_ready = 0);
 bool d2d_router_fused_supports(const d2d_layer_desc &D, int T);
-// ksum (optional, 8 device ints, words 0 and 1 zero at launch and left at zero): the kernel adds up k over all tokens
-// and its last CTA publishes the total, the number of selected (token, expert) pairs, in ksum[4]
+// ksum (optional, 8 device ints, words 0 to 2 zero at launch and left at zero): the kernel adds up k over all tokens
+// and its last CTA publishes the total, the number of selected (token, expert) pairs, in ksum[4], and writes *status
+// (which the caller must have cleared otherwise)
 d2d_status d2d_router_fused(const d2d_layer *L, const void *x, int T, float tau, int do_mask, float *R, uint32_t *mask,
                             int32_t *k, int32_t *status, cudaStream_t st, int32_t *ksum = nullptr);
 d2d_status d2d_router_fused_group(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T,

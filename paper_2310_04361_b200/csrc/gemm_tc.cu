@@ -57,21 +57,16 @@ __device__ __forceinline__ void tile_coords(int tile, int rows, int cols, int ba
 }
 
 
-// 16 accumulator columns -> 16 output values: bias (float32, staged in shared memory), activation, selection mask.
+// 16 accumulator columns -> 16 output values: bias (16 consecutive bf16 entries, zeros if there is none), activation.
 template <int EPI, int ACT, bool GATED>
-__device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint32_t (&g)[16], float (&v)[16],
-                                            const float *bias_f, bool has_bias, int col0)
+__device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint32_t (&g)[16], float (&v)[16], const uint4 (&bias_w)[2])
 {
     float bias[16];
-    if (has_bias) {
+    const uint32_t w[8] = {bias_w[0].x, bias_w[0].y, bias_w[0].z, bias_w[0].w, bias_w[1].x, bias_w[1].y, bias_w[1].z, bias_w[1].w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 b4 = *reinterpret_cast<const float4 *>(bias_f + col0 + 4 * q);
-            bias[4 * q] = b4.x; bias[4 * q + 1] = b4.y; bias[4 * q + 2] = b4.z; bias[4 * q + 3] = b4.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) bias[j] = 0.0f;
+    for (int j = 0; j < 8; ++j) {
+        bias[2 * j] = __uint_as_float(w[j] << 16);
+        bias[2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
     }
     if (EPI == D2D_EPI_UP_MASKED) {
         // math on pairs; the selection is applied by the caller on the packed bf16 words (each 8-column half belongs to one
@@ -95,7 +90,7 @@ __device__ __forceinline__ void epilogue_16(const uint32_t (&r)[16], const uint3
     }
 }
 
-// Same result with every bound checked (ragged last column tile, odd leading dimension, bias too long for the cache).
+// Same result with every bound checked (ragged last column tile, odd leading dimension, odd expert sizes).
 // Statically indexed and inlined: an out-of-line version forced the accumulator registers onto the stack.
 template <int EPI, int ACT, bool GATED>
 __device__ __forceinline__ void epilogue_16_slow(const uint32_t (&r)[16], const uint32_t (&g)[16], const __nv_bfloat16 *bias,
@@ -120,7 +115,8 @@ __device__ __forceinline__ void epilogue_16_slow(const uint32_t (&r)[16], const 
 }
 
 constexpr int N_EPI_WARPS = 16;
-constexpr int BIAS_CACHE_ELEMS = 6144;           // 24 KB of float32 in shared memory behind the operand stages
+constexpr int OUT_BUF_BYTES = BM * 128;          // 128 rows x 64 bf16 columns of output on their way to a TMA store, two buffers
+constexpr int STAGE_BUDGET = 192 * 1024;         // shared memory for operand stages beside them
 constexpr int NTHREADS_V2 = 64 + 32 * N_EPI_WARPS;
 
 __host__ __device__ constexpr int pow2_at_least(int v) { return v <= 32 ? 32 : v <= 64 ? 64 : v <= 128 ? 128 : v <= 256 ? 256 : 512; }
@@ -129,9 +125,9 @@ __host__ __device__ constexpr int pow2_at_least(int v) { return v <= 32 ? 32 : v
 // fastest).  Two accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the
 // next.  GATED: two B tiles (up, gate) share the A tile; the epilogue forms A(gate) * (up + bias).
 template <int BN, int STAGES, int EPI, int ACT, bool GATED>
-__global__ void __launch_bounds__(NTHREADS_V2, 1)
+__global__ void __launch_bounds__(NTHREADS_V2) __maxnreg__(GATED ? 96 : 80)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-               const __grid_constant__ CUtensorMap tm_b2, EpiParams ep, int M, int N, int K, int k_splits)
+               const __grid_constant__ CUtensorMap tm_b2, const __grid_constant__ CUtensorMap tm_out, EpiParams ep, int M, int N, int K, int k_splits)
 {
     constexpr int TM = BM;                                // rows of the tile a CTA computes
     constexpr int B_ROWS = BN;                            // rows of B this CTA stages
@@ -143,8 +139,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     constexpr int COLS_PER_WARP = BN / 4;                            // four epilogue warps share a TMEM lane quadrant
     static_assert(TMEM_COLS <= 512 && BN % 64 == 0 && BN <= 256, "tile width");
 
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);   // swizzle atoms are 1024-byte aligned
+    // Swizzle atoms are 1024-byte aligned.  224 KB at most, so that a small CTA of the list-building kernels, which run beside
+    // this one, still finds 2 KB (and, with 80 registers per thread here, its registers) on the SM.
+    extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_acc_full[2], bar_acc_empty[2];
     __shared__ uint32_t tmem_base_holder;
     // what the epilogue's leader publishes (per buffer parity): go on (or the work is done, or a wait ran out), tile coordinates
@@ -153,11 +150,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // to the epilogue through a two-slot ring (a CTA that starts late, or gets slow tiles, simply draws fewer)
     __shared__ uint64_t sched_full[2], sched_empty[2];
     __shared__ volatile int sched_item[2];
-    // the whole bias vector is staged once, as float32, behind the operand stages when it fits
-    float *bias_f = reinterpret_cast<float *>(smem + (size_t)STAGES * STAGE_BYTES);
-    const int NB = N * ep.batch;                                     // bias entries of all problems
-    const bool bias_cached = ep.bias != nullptr && NB <= BIAS_CACHE_ELEMS && (N & 3) == 0;
-
+    uint8_t *out_s = smem + (size_t)STAGES * STAGE_BYTES;            // two output buffers behind the operand stages
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // warp-uniform: roles, columns
     const int nkb = (K + BK - 1) / BK;
     const int n_tiles = (N + BN - 1) / BN;
@@ -191,28 +184,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
-    // Programmatic dependent launch: everything above (barriers, TMEM, the bias vector: parameters, not activations)
+    // Programmatic dependent launch: everything above (barriers, TMEM)
     // may run while the previous kernel of the stream drains; nothing below starts before that kernel has completed
     // and its writes are visible.  The next kernel of the stream may be scheduled onto SMs as this grid frees them.
     // With late_wait only the epilogue depends on that kernel (the selection mask written by the router): the
     // operand loads and the MMAs of the first tiles then overlap it, and only the epilogue warps wait.
     const bool dyn = ep.tile_counter != nullptr;
-    if (bias_cached && warp >= 2) {
-        // The epilogue warps stage the bias (a parameter: no need to wait for the previous kernel) while the producer
-        // and the MMA thread are already at work.  16-byte loads, all issued before the first use: the fill costs one
-        // memory latency, not N / threads of them.
-        for (int i = ((int)threadIdx.x - 64) * 8; i < NB; i += N_EPI_WARPS * 32 * 8) {
-            float b8[8];
-            if (i + 8 <= NB) {
-                d2d_load8(ep.bias + i, b8);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) bias_f[i + q] = b8[q];
-            } else {
-                for (int q = 0; i + q < NB; ++q) bias_f[i + q] = __bfloat162float(ep.bias[i + q]);
-            }
-        }
-        asm volatile("bar.sync 1, %0;" ::"r"(N_EPI_WARPS * 32) : "memory");
-    }
     // early_b: the B operand (weights) does not depend on the previous kernel either, so the producer requests the B
     // tiles of its first k-blocks BEFORE it waits for that kernel and only the A tiles after (static schedule only)
     const bool early_b = !dyn && !ep.late_wait && ep.n_sel == nullptr;
@@ -378,8 +355,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         // everything-inline version of this epilogue was instruction-fetch bound).
         const int ew = warp - 2;
         const int quad = warp & 3;                          // TMEM lanes this warp may touch
-        const int part = ew >> 2;                           // which quarter of the tile's columns
+        const int part = ew >> 2;                           // which 16 of every 64 columns of the tile
         constexpr int N_UNITS = COLS_PER_WARP / 16;
+        uint32_t out_n = 0;                                 // output buffers used so far
         for (uint32_t local = 0;; ++local) {
             const uint32_t buf = local & 1u, use = local >> 1;
             // ONE thread takes the item from the ring, works out its coordinates (integer divisions), waits for the accumulator
@@ -411,7 +389,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int m0 = epi_m0[buf], n0 = epi_n0[buf], prob = epi_prob[buf];
             // this problem's bias entries and output matrix
-            const float *bias_p = bias_f + prob * N;
             const __nv_bfloat16 *bias_g = ep.bias ? ep.bias + prob * N : nullptr;
             void *out_p = (char *)ep.out + (size_t)prob * M * N * ((EPI == D2D_EPI_ABS_F32 || EPI == D2D_EPI_PARTIAL_F32) ? 4 : 2);
             const int row = m0 + quad * 32 + lane;
@@ -420,7 +397,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             // looked at after the first unit's math; bit h of kbits = group h.  Which expert a group belongs to is the same for
             // all rows.  (Selecting among all words of the row in registers, group by group, was 3 of 18 instructions per
             // element.)
-            const int colw = n0 + part * COLS_PER_WARP;
+            const int colw = n0 + part * 16;                // unit u: columns colw + 64 u + 0..15
             const uint32_t *mrow = nullptr;
             uint32_t kbits = 0xffffffffu, mw0 = 0u, mw1 = 0u, e0 = 0u;
             if (EPI == D2D_EPI_UP_MASKED && ep.mask && row < M) {
@@ -432,16 +409,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     mw1 = wi + 1 < ep.mask_words ? __ldg(mrow + wi + 1) : 0u;
                 }
             }
-            const uint32_t tbase = tmem_base + buf * BUF_COLS + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * COLS_PER_WARP);
+            const uint32_t tbase = tmem_base + buf * BUF_COLS + ((uint32_t)(quad * 32) << 16) + (uint32_t)(part * 16);
 
-            const bool bias_fast = ep.bias == nullptr || bias_cached;
-            const bool wide_store = (N & 15) == 0 && (reinterpret_cast<uintptr_t>(out_p) & 31) == 0;   // 32-byte aligned rows
             const bool mask_on = EPI == D2D_EPI_UP_MASKED && ep.mask != nullptr;                         // CTA-uniform
             // The common case gets a loop of its own with nothing else in it (the epilogue is sensitive to its
-            // instruction-cache footprint): a full-width tile, the bias in shared memory, vector-aligned rows and
-            // expert sizes that are multiples of 8.  Everything else (ragged last column tile, odd sizes, a bias too
-            // long for the cache) goes through the compact generic loop below.
-            const bool fast_tile = bias_fast && (N & 7) == 0 && n0 + BN <= N && (!mask_on || (ep.expert_size & 7) == 0);
+            // instruction-cache footprint): a full-width tile, vector-aligned rows and expert sizes that are multiples of 8.
+            // Everything else (ragged last column tile, odd sizes) goes through the compact generic loop below.
+            const bool fast_tile = (N & 7) == 0 && n0 + BN <= N && (!mask_on || (ep.expert_size & 7) == 0);
             uint32_t ra[16], rb[GATED ? 1 : 16], ga[GATED ? 16 : 1];
             if (fast_tile) {
                 // Non-gated: the next unit's accumulators are prefetched into a second register set.  Gated tiles need
@@ -450,59 +424,80 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (!GATED) tmem_ld16_issue(tbase, ra);
 #pragma unroll
                 for (int u = 0; u < N_UNITS; ++u) {             // at most 4 units
-                    const int col0 = colw + u * 16;
+                    const int col0 = colw + u * 64;
+                    uint4 bias_w[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};       // the same for all lanes, out of L1
+                    if (EPI != D2D_EPI_PARTIAL_F32 && ep.bias) {
+                        bias_w[0] = __ldg(reinterpret_cast<const uint4 *>(bias_g + col0));
+                        bias_w[1] = __ldg(reinterpret_cast<const uint4 *>(bias_g + col0 + 8));
+                    }
                     uint32_t (&r)[16] = GATED ? ra : ((u & 1) ? reinterpret_cast<uint32_t (&)[16]>(rb) : ra);
                     uint32_t (&g)[16] = reinterpret_cast<uint32_t (&)[16]>(ga);
                     if (GATED) {
-                        tmem_ld16_issue(tbase + u * 16, ra);
-                        tmem_ld16_issue(tbase + u * 16 + BN, reinterpret_cast<uint32_t (&)[16]>(ga));
+                        tmem_ld16_issue(tbase + u * 64, ra);
+                        tmem_ld16_issue(tbase + u * 64 + BN, reinterpret_cast<uint32_t (&)[16]>(ga));
                     }
                     tmem_ld_wait();                                               // this unit's accumulators have landed
                     if (!GATED && u + 1 < N_UNITS)                                // the next unit's load overlaps the math below
-                        tmem_ld16_issue(tbase + (u + 1) * 16, (u & 1) ? ra : reinterpret_cast<uint32_t (&)[16]>(rb));
+                        tmem_ld16_issue(tbase + (u + 1) * 64, (u & 1) ? ra : reinterpret_cast<uint32_t (&)[16]>(rb));
 
                     float v[16];
-                    epilogue_16<EPI, ACT, GATED>(r, g, v, bias_p, ep.bias != nullptr, col0);
+                    epilogue_16<EPI, ACT, GATED>(r, g, v, bias_w);
                     if (EPI == D2D_EPI_UP_MASKED && u == 0 && mask_on) {
                         const uint32_t bits = __funnelshift_r(mw0, mw1, e0 & 31u);
                         kbits = 0u;
 #pragma unroll
-                        for (int h = 0; h < COLS_PER_WARP / 8; ++h)
-                            kbits |= ((bits >> (__umulhi((uint32_t)(colw + 8 * h), ep.inv_expert_size) - e0)) & 1u) << h;
+                        for (int h = 0; h < 2 * N_UNITS; ++h)
+                            kbits |= ((bits >> (__umulhi((uint32_t)(colw + 64 * (h >> 1) + 8 * (h & 1)), ep.inv_expert_size) - e0)) & 1u) << h;
                     }
                     // all ones where the token keeps the expert of the unit's first / second eight columns
                     const uint32_t keep2[2] = {(uint32_t)((int)(kbits << (31 - 2 * u)) >> 31), (uint32_t)((int)(kbits << (30 - 2 * u)) >> 31)};
-                    if (row < M) {
-                        if (EPI == D2D_EPI_PARTIAL_F32) {
+                    if (u == N_UNITS - 1) {
+                        // all of this warp's TMEM reads of the buffer are complete: hand it back to the MMA warp
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
+                    }
+                    if (EPI == D2D_EPI_PARTIAL_F32) {
+                        if (row < M) {
                             float *o = (float *)out_p + (size_t)row * N + col0;
 #pragma unroll
                             for (int j = 0; j < 16; j += 4)
                                 asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(o + j), "f"(v[j]), "f"(v[j + 1]),
                                              "f"(v[j + 2]), "f"(v[j + 3]) : "memory");
-                        } else if (EPI == D2D_EPI_ABS_F32) {
+                        }
+                    } else if (EPI == D2D_EPI_ABS_F32) {
+                        if (row < M) {
                             float *o = (float *)out_p + (size_t)row * N + col0;
 #pragma unroll
                             for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4 *>(o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                        } else {
-                            __nv_bfloat16 *o = (__nv_bfloat16 *)out_p + (size_t)row * N + col0;
-                            uint32_t pk[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                                pk[j] = *reinterpret_cast<uint32_t *>(&t);
-                                // selection: an expert the token did not keep contributes zeros (also when its
-                                // pre-activations are not finite)
-                                if (EPI == D2D_EPI_UP_MASKED) pk[j] &= keep2[j >> 2];
-                            }
-                            if (wide_store) {
-                                // one 32-byte store per row and unit: a whole sector per lane, half as many store instructions
-                                asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o), "r"(pk[0]), "r"(pk[1]),
-                                             "r"(pk[2]), "r"(pk[3]), "r"(pk[4]), "r"(pk[5]), "r"(pk[6]), "r"(pk[7]) : "memory");
-                            } else {
-                                *reinterpret_cast<uint4 *>(o) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                                *reinterpret_cast<uint4 *>(o + 8) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-                            }
                         }
+                    } else {
+                        uint32_t pk[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            __nv_bfloat162 t = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+                            pk[j] = *reinterpret_cast<uint32_t *>(&t);
+                            // selection: an expert the token did not keep contributes zeros (also when its
+                            // pre-activations are not finite)
+                            if (EPI == D2D_EPI_UP_MASKED) pk[j] &= keep2[j >> 2];
+                        }
+                        // The sixteen warps put 128 rows x 64 columns into a buffer (128-byte rows, swizzled as the TMA expects) and one
+                        // thread stores it: whole 128-byte lines.  (Every thread storing 32 bytes of its own row took 15 % of the
+                        // kernel: 112 us against 96 us without stores on the ViT-shaped up projection.)
+                        uint8_t *o = out_s + (out_n & 1u) * OUT_BUF_BYTES + (quad * 32 + lane) * 128;
+                        *reinterpret_cast<uint4 *>(o + (((2 * part) ^ (lane & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        *reinterpret_cast<uint4 *>(o + (((2 * part + 1) ^ (lane & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        // the store before this one has read the other buffer: free for everybody behind the barrier
+                        if (part == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                        asm volatile("bar.sync %0, 128;" ::"r"(2 + quad) : "memory");
+                        if (part == 0 && lane == 0) {
+                            asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+                                         ::"l"(&tm_out), "r"(n0 + u * 64), "r"(m0 + quad * 32), "r"(prob),
+                                         "r"(smem_u32(out_s + (out_n & 1u) * OUT_BUF_BYTES + quad * 32 * 128)) : "memory");
+                            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                        }
+                        ++out_n;
                     }
                 }
             } else {
@@ -517,10 +512,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 uint32_t (&g)[16] = reinterpret_cast<uint32_t (&)[16]>(ga);
 #pragma unroll 1
                 for (int u = 0; u < N_UNITS; ++u) {
-                    const int col0 = colw + u * 16;
+                    const int col0 = colw + u * 64;
                     if (col0 >= N) break;                       // warp-uniform (ragged last column tile)
-                    tmem_ld16_issue(tbase + u * 16, ra);
-                    if (GATED) tmem_ld16_issue(tbase + u * 16 + BN, g);
+                    tmem_ld16_issue(tbase + u * 64, ra);
+                    if (GATED) tmem_ld16_issue(tbase + u * 64 + BN, g);
                     uint32_t keep = 0xffffu;
                     if (mask_on && mrow) {
                         keep = 0u;
@@ -540,19 +535,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                             ++ee;
                         }
                         // advance to the expert that owns the first column of the next unit
-                        lo -= 16;
+                        lo -= 64;
                         while (lo + s <= 0) { lo += s; ++e; }
                     }
                     tmem_ld_wait();
                     epilogue_16_slow<EPI, ACT, GATED>(ra, g, bias_g, out_p, row, M, col0, N, keep);
                 }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
             }
-            // all of this warp's TMEM reads of the buffer are complete: hand it back to the MMA warp
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
-
         }
+        // the buffers may not go away, nor the kernel count as finished, before the last stores are done
+        if (part == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -594,9 +589,10 @@ template <int BN, int EPI, int ACT, bool GATED>
 d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
 {
     constexpr int STAGE_BYTES = BM * BK * 2 + (GATED ? 2 : 1) * BN * BK * 2;
-    constexpr int STAGES = (200 * 1024) / STAGE_BYTES > 8 ? 8 : (200 * 1024) / STAGE_BYTES;   // 200 KB of operand stages (+ 24 KB bias cache)
-    constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + (size_t)BIAS_CACHE_ELEMS * 4;
-    CUtensorMap ta, tb, tb2;
+    constexpr int STAGES = STAGE_BUDGET / STAGE_BYTES > 8 ? 8 : STAGE_BUDGET / STAGE_BYTES;
+    constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 2 * (size_t)OUT_BUF_BYTES;
+    static_assert(SMEM <= 224 * 1024, "shared memory per CTA");
+    CUtensorMap ta, tb, tb2, to = {};
     const bool gate_cat = GATED && g.b_cat != nullptr && g.b_cat_block == BN;
     const int batch = g.batch > 1 ? g.batch : 1;
     if (batch > 1 && (GATED || g.K % BK != 0)) return D2D_ERR_UNSUPPORTED;
@@ -611,6 +607,12 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
         } else {
             tb2 = tb;
         }
+    }
+    if (EPI != D2D_EPI_PARTIAL_F32 && EPI != D2D_EPI_ABS_F32 && g.N % 8 == 0) {       // (other widths: every tile takes the generic loop)
+        const cuuint64_t dims[3] = {(cuuint64_t)g.N, (cuuint64_t)g.M, (cuuint64_t)batch};
+        const cuuint64_t strides[2] = {(cuuint64_t)g.N * 2, (cuuint64_t)g.N * g.M * 2};
+        const cuuint32_t box[3] = {64, 32, 1};
+        if (!d2d_tc_encode_map(&to, false, 3, g.out, dims, strides, box)) return D2D_ERR_CUDA;
     }
     auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED>;
     static bool attr_set[64] = {};
@@ -636,7 +638,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, ep, g.M, g.N, g.K, k_splits);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits);
     D2D_LAUNCHED(1);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }

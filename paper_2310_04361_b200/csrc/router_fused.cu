@@ -45,8 +45,9 @@ struct RouterGroupIO {
     RouterLayerIO l[D2D_MAX_GROUP];
     uint32_t *mask_cat;    // merged mask [T, cat_words] or NULL
     int cat_words;
-    int32_t *ksum;         // single layer only, or NULL: [0] running sum of k, [1] CTA exit ticket (both zero at launch and
-                           // left at zero), [4] receives the total = number of selected (token, expert) pairs
+    int32_t *ksum;         // single layer only, or NULL: [0] running sum of k, [1] CTA exit ticket, [2] largest condition (all
+                           // zero at launch and left at zero), [4] receives the total = number of selected (token, expert)
+                           // pairs; the last CTA then writes *status
 };
 
 // Shared memory (dynamic, 1024-byte aligned):
@@ -72,7 +73,8 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     float *__restrict__ R = io.l[layer].R;
     uint32_t *__restrict__ mask = io.l[layer].mask;
     int32_t *__restrict__ k = io.l[layer].k;
-    int32_t *__restrict__ status = io.l[layer].status;
+    // conditions are collected in a word of the layer and published once (no memset in front of the kernel)
+    int32_t *__restrict__ status = io.ksum ? io.ksum + 2 : io.l[layer].status;
     constexpr int KB2 = DH / BK;                          // k-blocks of the second GEMM
     constexpr int A_BYTES = BM * BK * 2, B1_BYTES = DH * BK * 2;
     constexpr int STAGE_BYTES = A_BYTES + B1_BYTES;
@@ -119,6 +121,8 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
     const uint32_t tmem_r = tmem_base + 256;
+    // the set-up above may overlap the tail of the previous kernel of the stream
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // the expert up projection that follows on the stream may start its operand loads and MMAs on the SMs this
     // grid leaves idle (T / 128 CTAs); its epilogue waits for this kernel to complete before it reads the mask
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -338,6 +342,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                         if (atomicAdd(io.ksum + 1, 1) == (int)(gridDim.x * gridDim.y) - 1) {
                             __threadfence();
                             io.ksum[4] = atomicExch(io.ksum, 0);         // the CTA that finishes last publishes and resets
+                            *io.l[layer].status = atomicExch(io.ksum + 2, 0);
                             io.ksum[1] = 0;
                         }
                     }
@@ -378,10 +383,20 @@ d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_la
         __atomic_store_n(&attr_set[dev], true, __ATOMIC_RELEASE);
     }
     const int EN = (D.n_experts + 15) / 16 * 16;
-    kern<<<dim3(d2d_cdiv(T, BM), n_layers), NTHREADS, SMEM, st>>>(tx, tw1, tw2, (const __nv_bfloat16 *)w.b_r1, (const __nv_bfloat16 *)w.b_r2,
-                                                                 T, D.d, D.n_experts, EN, tau, do_mask, io);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(d2d_cdiv(T, BM), n_layers, 1);
+    cfg.blockDim = dim3(NTHREADS, 1, 1);
+    cfg.dynamicSmemBytes = SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, tx, tw1, tw2, (const __nv_bfloat16 *)w.b_r1, (const __nv_bfloat16 *)w.b_r2,
+                                               T, D.d, D.n_experts, EN, tau, do_mask, io);
     D2D_LAUNCHED(1);
-    return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+    return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
 }  // namespace

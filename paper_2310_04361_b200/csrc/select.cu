@@ -23,8 +23,9 @@ __device__ __forceinline__ bool is_finite_f32(float v) { return (__float_as_uint
 
 // ---------------------------------------------------------------------------- mask kernels
 
-// ksum (optional): [0] running sum of k over the CTAs, [1] exit ticket (both zero at launch and left at zero), [4]
-// receives the total = number of selected (token, expert) pairs, for the density-adaptive dispatch of the expert step.
+// ksum (optional): [0] running sum of k over the CTAs, [1] exit ticket, [2] largest condition (all zero at launch and left at
+// zero), [4] receives the total = number of selected (token, expert) pairs, for the density-adaptive dispatch of the
+// expert step; the last CTA then also writes *status (otherwise the caller has cleared it).
 __global__ void __launch_bounds__(256)
 dynk_mask_kernel(const float *__restrict__ R, int T, int E, int W, float tau,
                  uint32_t *__restrict__ mask, int32_t *__restrict__ k, int32_t *__restrict__ status, int32_t *ksum)
@@ -62,7 +63,7 @@ dynk_mask_kernel(const float *__restrict__ R, int T, int E, int W, float tau,
         }
         if (lane == 0) {
             k[t] = kt;
-            if (bad) atomicMax(status, (int32_t)D2D_ERR_NONFINITE);
+            if (bad) atomicMax(ksum ? ksum + 2 : status, (int32_t)D2D_ERR_NONFINITE);
             if (ksum) atomicAdd(&block_k, kt);
         }
     }
@@ -74,6 +75,7 @@ dynk_mask_kernel(const float *__restrict__ R, int T, int E, int W, float tau,
         if (atomicAdd(ksum + 1, 1) == (int)gridDim.x - 1) {          // the last CTA publishes the total and resets
             __threadfence();
             ksum[4] = atomicExch(ksum, 0);
+            *status = atomicExch(ksum + 2, 0);
             ksum[1] = 0;
         }
     }
@@ -188,13 +190,19 @@ __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, i
 // counter) then scans: per expert the exclusive prefix over the blocks, and over the experts the
 // exclusive prefix of the totals -> counts, offsets, n_sel.  Integer sums only: the result does
 // not depend on which CTA is last.
-__global__ void __launch_bounds__(TOKB)
+// The scan is a chain of L2 latencies: a thread takes an expert and reads eight blocks' counts at a time before it writes
+// their prefixes back (one at a time: 25 us for 197 blocks); few experts (at most 64) are cut into segments of blocks, a
+// thread per (expert, segment).  Shared memory is kept below 700 bytes: these CTAs run beside the persistent GEMM CTAs,
+// which leave 1.8 KB of an SM's shared memory (1 KB of it reserved per CTA) and 10 K registers (40 per thread here).
+constexpr int SCAN_BATCH = 8, SCAN_SEGS = 128;
+
+__global__ void __launch_bounds__(TOKB, 6)
 bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W, int nblk,
                          int32_t *__restrict__ blockcounts, unsigned int *__restrict__ ticket,
                          int32_t *__restrict__ counts, int32_t *__restrict__ offsets, int32_t *__restrict__ n_sel,
                          int32_t *__restrict__ status, long long capacity)
 {
-    __shared__ int32_t cnt[TOKB / 32][33];
+    __shared__ union { uint16_t cnt[TOKB / 32][33]; int seg[SCAN_SEGS]; } sh;
     __shared__ int warp_sums[8];
     __shared__ int chunk_total;
     __shared__ unsigned int my_ticket;
@@ -203,37 +211,75 @@ bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     {
         const int w = blockIdx.y;                // one 32-expert mask word per CTA
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        cnt[warp][lane] = __popc(transpose_bits(word, lane));
+        sh.cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
         __syncthreads();
         if (warp == 0) {
             int total = 0;
 #pragma unroll
-            for (int i = 0; i < TOKB / 32; ++i) total += cnt[i][lane];
+            for (int i = 0; i < TOKB / 32; ++i) total += sh.cnt[i][lane];
             const int e = w * 32 + lane;
             if (e < E) blockcounts[(size_t)blockIdx.x * E + e] = total;
         }
         __syncthreads();
     }
-    __threadfence();
-    if (threadIdx.x == 0) my_ticket = atomicAdd(ticket, 1u);
+    if (threadIdx.x == 0) {
+        __threadfence();                         // the whole CTA's counts (the barrier before it)
+        my_ticket = atomicAdd(ticket, 1u);
+        if (my_ticket == (unsigned int)(nblk * W - 1)) *ticket = 0u;      // ready for the next call
+        __threadfence();                         // the last one: every other CTA's block counts are visible now
+    }
     __syncthreads();
     if (my_ticket != (unsigned int)(nblk * W - 1)) return;
-    __threadfence();                         // every other CTA's block counts are visible now
-    if (threadIdx.x == 0) *ticket = 0u;      // ready for the next call
+    const int nseg = E * 2 <= SCAN_SEGS ? SCAN_SEGS / E : 1, per = (nblk + nseg - 1) / nseg;
+    const int sg = nseg > 1 ? (int)threadIdx.x / E : 0;
+    const int b_begin = sg * per, b_end = min(nblk, b_begin + per);
     int carry = 0;
     for (int e0 = 0; e0 < E; e0 += TOKB) {
-        const int e = e0 + threadIdx.x;
+        const int e = nseg > 1 ? (int)threadIdx.x % E : e0 + (int)threadIdx.x;
+        const bool on = e < E && sg < nseg;
         int run = 0;
-        if (e < E) {
-            for (int b = 0; b < nblk; ++b) {
-                const int c = __ldcg(blockcounts + (size_t)b * E + e);
-                blockcounts[(size_t)b * E + e] = run;      // exclusive prefix over the token blocks
-                run += c;
-            }
-            counts[e] = run;
+        if (nseg > 1) {
+            // totals of the segments before this one
+            if (on)
+                for (int b0 = b_begin; b0 < b_end; b0 += SCAN_BATCH) {
+#pragma unroll
+                    for (int i = 0; i < SCAN_BATCH; ++i)
+                        if (b0 + i < b_end) run += __ldcg(blockcounts + (size_t)(b0 + i) * E + e);
+                }
+            if (on) sh.seg[sg * E + e] = run;
+            __syncthreads();
+            run = 0;
+            if (on)
+                for (int i = 0; i < sg; ++i) run += sh.seg[i * E + e];
+            __syncthreads();
         }
-        const int ex = block_exscan_256(run, warp_sums, &chunk_total);
-        if (e < E) offsets[e] = carry + ex;
+        if (on) {
+            for (int b0 = b_begin; b0 < b_end; b0 += SCAN_BATCH) {
+                int c[SCAN_BATCH];
+#pragma unroll
+                for (int i = 0; i < SCAN_BATCH; ++i) c[i] = b0 + i < b_end ? __ldcg(blockcounts + (size_t)(b0 + i) * E + e) : 0;
+#pragma unroll
+                for (int i = 0; i < SCAN_BATCH; ++i) {
+                    if (b0 + i < b_end) blockcounts[(size_t)(b0 + i) * E + e] = run;      // exclusive prefix over the token blocks
+                    run += c[i];
+                }
+            }
+        }
+        // the last segment's run is the expert's total; experts in the order of their threads
+        int total = run;
+        if (nseg > 1) {
+            if (on && sg == nseg - 1) sh.seg[e] = run;
+            __syncthreads();
+            total = (int)threadIdx.x < E ? sh.seg[threadIdx.x] : 0;
+        } else if (!on) {
+            total = 0;
+        }
+        const int ee = nseg > 1 ? (int)threadIdx.x : e;
+        const int ex = block_exscan_256(total, warp_sums, &chunk_total);
+        if (ee < E) {
+            counts[ee] = total;
+            offsets[ee] = carry + ex;
+        }
         carry += chunk_total;
         __syncthreads();
     }
@@ -253,7 +299,7 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
                    const int32_t *__restrict__ blockbase, const int32_t *__restrict__ offsets,
                    int32_t *__restrict__ perm, long long capacity)
 {
-    __shared__ int32_t cnt[TOKB / 32][33];
+    __shared__ uint16_t cnt[TOKB / 32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = blockIdx.x * TOKB + threadIdx.x;
     const uint32_t lower = (1u << lane) - 1u;
@@ -263,7 +309,7 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
         // start of this CTA's run inside expert e's list (lane = expert); issued early to hide the latency
         const long long cta_base = e < E ? (long long)__ldg(offsets + e) + __ldg(blockbase + (size_t)blockIdx.x * E + e) : 0;
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        cnt[warp][lane] = __popc(transpose_bits(word, lane));
+        cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
         __syncthreads();
         int before = 0;
         for (int i = 0; i < warp; ++i) before += cnt[i][lane];
@@ -359,14 +405,13 @@ size_t d2d_select_ws_bytes(int T, int E)
 // lists can be built afterwards, on any stream ordered behind this one, with d2d_launch_select(nullptr, ..., mask_ready = 1).
 d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d2d_routing *out, int32_t *ksum, cudaStream_t st)
 {
-    D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
     dynk_mask_kernel<<<d2d_cdiv(T, 8), 256, 0, st>>>(R, T, E, (E + 31) / 32, tau, out->mask, out->k, out->status, ksum);
     D2D_LAUNCHED(1);
     return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
 d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, const d2d_routing *out,
-                             void *ws, cudaStream_t st, int mask_ready)
+                             void *ws, cudaStream_t st, int mask_ready, unsigned int *zero_ticket)
 {
     const int W = (E + 31) / 32;
     if (!mask_ready) D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
@@ -389,9 +434,10 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         k_from_mask_kernel<<<d2d_cdiv(T, 256), 256, 0, st>>>(out->mask, T, W, out->k);
     }
     const int nblk = d2d_cdiv(T, TOKB);
-    unsigned int *ticket = (unsigned int *)ws;                    // must start at zero: cleared on every call
+    // the ticket must start at zero (the kernel leaves it there): a word the caller keeps, or cleared on every call
+    unsigned int *ticket = zero_ticket ? zero_ticket : (unsigned int *)ws;
     int32_t *blockcounts = (int32_t *)((char *)ws + 256);
-    D2D_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st));
+    if (!zero_ticket) D2D_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st));
     bucket_count_scan_kernel<<<dim3(nblk, W), TOKB, 0, st>>>(out->mask, T, E, W, nblk, blockcounts, ticket, out->counts,
                                                     out->offsets, out->n_sel, out->status,
                                                     (long long)out->perm_capacity);
