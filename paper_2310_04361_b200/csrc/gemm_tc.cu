@@ -122,18 +122,22 @@ constexpr int NTHREADS_V2 = 64 + 32 * N_EPI_WARPS;
 __host__ __device__ constexpr int pow2_at_least(int v) { return v <= 32 ? 32 : v <= 64 ? 64 : v <= 128 ? 128 : v <= 256 ? 256 : 512; }
 
 // Persistent kernel: CTA c computes tiles c, c + gridDim.x, ... (128 x BN each, column tiles
-// fastest).  Two accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the
+// fastest).  PAIR: two CTAs of a cluster compute 256 x BN tiles with tcgen05.mma.cta_group::2: each stages its own 128 rows
+// of A and HALF of the BN rows of B, the leader (rank 0) issues the MMAs, each CTA's tensor memory receives its own 128 rows.
+// A k-block then brings 16 + BN / 16 KB into an SM instead of 16 + BN / 8: the fill from L2 (about 117 GB/s per SM), not
+// the tensor pipe, bounds the single-CTA main loop.  Two accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the
 // next.  GATED: two B tiles (up, gate) share the A tile; the epilogue forms A(gate) * (up + bias).
-template <int BN, int STAGES, int EPI, int ACT, bool GATED>
+template <int BN, int STAGES, int EPI, int ACT, bool GATED, bool PAIR>
 __global__ void __launch_bounds__(NTHREADS_V2) __maxnreg__(GATED ? 96 : 80)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                const __grid_constant__ CUtensorMap tm_b2, const __grid_constant__ CUtensorMap tm_out, EpiParams ep, int M, int N, int K, int k_splits)
 {
-    constexpr int TM = BM;                                // rows of the tile a CTA computes
-    constexpr int B_ROWS = BN;                            // rows of B this CTA stages
+    constexpr int TM = PAIR ? 2 * BM : BM;                // rows of the tile a CTA (pair) computes
+    // rows of B this CTA stages (of each matrix; a gated pair: the leader the up rows, its peer the gate rows, all BN of them)
+    constexpr int B_ROWS = PAIR && !GATED ? BN / 2 : BN;
     constexpr int A_BYTES = BM * BK * 2;
     constexpr int B_BYTES = B_ROWS * BK * 2;
-    constexpr int STAGE_BYTES = A_BYTES + (GATED ? 2 : 1) * B_BYTES;
+    constexpr int STAGE_BYTES = A_BYTES + (GATED && !PAIR ? 2 : 1) * B_BYTES;
     constexpr int BUF_COLS = pow2_at_least(GATED ? 2 * BN : BN);    // TMEM columns per accumulator buffer
     constexpr int TMEM_COLS = 2 * BUF_COLS;
     constexpr int COLS_PER_WARP = BN / 4;                            // four epilogue warps share a TMEM lane quadrant
@@ -158,8 +162,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // epilogue adds its partial sums to a float32 buffer (small-M problems that would leave most SMs idle)
     const int tiles_pp = ((M + TM - 1) / TM) * n_tiles;            // output tiles per problem
     const int total_tiles = tiles_pp * ep.batch * k_splits;
-    const int worker = (int)blockIdx.x;
-    const int n_workers = (int)gridDim.x;
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;              // 0: the CTA that issues the MMAs
+    const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -168,20 +173,28 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&bar_acc_full[b]), 1);
-            mbar_init(smem_u32(&bar_acc_empty[b]), N_EPI_WARPS);
+            mbar_init(smem_u32(&bar_acc_empty[b]), PAIR ? 2 * N_EPI_WARPS : N_EPI_WARPS);
             mbar_init(smem_u32(&sched_full[b]), 1);
-            mbar_init(smem_u32(&sched_empty[b]), 2);          // read by the MMA thread and by the epilogue's leader
+            // a slot's readers: the MMA thread and the epilogue's leader; of a pair also the peer's producer and epilogue leader
+            mbar_init(smem_u32(&sched_empty[b]), PAIR ? 4 : 2);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
-                     "r"((uint32_t)TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if (PAIR) {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
+                         "r"((uint32_t)TMEM_COLS) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
+                         "r"((uint32_t)TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) cluster_sync_all();          // the peer's barriers are initialised before anything signals them
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
     // Programmatic dependent launch: everything above (barriers, TMEM)
@@ -192,7 +205,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     const bool dyn = ep.tile_counter != nullptr;
     // early_b: the B operand (weights) does not depend on the previous kernel either, so the producer requests the B
     // tiles of its first k-blocks BEFORE it waits for that kernel and only the A tiles after (static schedule only)
-    const bool early_b = !dyn && !ep.late_wait && ep.n_sel == nullptr;
+    const bool early_b = !PAIR && !dyn && !ep.late_wait && ep.n_sel == nullptr;
     if (warp >= 2 || (!ep.late_wait && !(early_b && warp == 0))) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // density-adaptive dispatch: below the crossover the gathered kernel, launched next to this one, does the work
@@ -221,18 +234,32 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 int item = worker + (int)local * n_workers;
                 if (dyn) {
                     const uint32_t sl = local & 1u, use = local >> 1;
-                    ok = mbar_wait(smem_u32(&sched_empty[sl]), (use & 1u) ^ 1u, ep.status);
-                    if (!ok) break;
-                    // A CTA's first item is its own index (no round trip to the counter before the first loads); the
-                    // counter hands out the items from gridDim.x on.  Every CTA draws exactly one value past the end,
-                    // total_tiles draws in all: whoever gets the last one leaves the counter at zero for the next launch.
-                    if (local > 0) {
-                        const int c = atomicAdd(ep.tile_counter, 1);
-                        if (c == total_tiles - 1) *ep.tile_counter = 0;
-                        item = (int)gridDim.x + c;
+                    if (rank != 0) {
+                        // the leader draws for the pair
+                        ok = mbar_wait(smem_u32(&sched_full[sl]), use & 1u, ep.status);
+                        if (!ok) break;
+                        item = sched_item[sl];
+                        mbar_arrive_cluster(map_to_cta(smem_u32(&sched_empty[sl]), 0));
+                        if (item < 0) break;
+                    } else {
+                        ok = mbar_wait(smem_u32(&sched_empty[sl]), (use & 1u) ^ 1u, ep.status);
+                        if (!ok) break;
+                        // A worker's first item is its own index (no round trip to the counter before the first loads); the
+                        // counter hands out the items from n_workers on.  Every worker draws exactly one value past the end,
+                        // total_tiles draws in all: whoever gets the last one leaves the counter at zero for the next launch.
+                        if (local > 0) {
+                            const int c = atomicAdd(ep.tile_counter, 1);
+                            if (c == total_tiles - 1) *ep.tile_counter = 0;
+                            item = n_workers + c;
+                        }
+                        const int got = item < total_tiles ? item : -1;
+                        sched_item[sl] = got;
+                        if (PAIR) {
+                            st_cluster_u32(map_to_cta(smem_u32((const void *)&sched_item[sl]), 1), (uint32_t)got);
+                            mbar_arrive_cluster(map_to_cta(smem_u32(&sched_full[sl]), 1));
+                        }
+                        mbar_arrive(smem_u32(&sched_full[sl]));   // release: the slot's content is visible to whoever sees the phase
                     }
-                    sched_item[sl] = item < total_tiles ? item : -1;
-                    mbar_arrive(smem_u32(&sched_full[sl]));       // release: the slot's content is visible to whoever sees the phase
                 }
                 if (item >= total_tiles) break;
                 int tile = (!GATED && k_splits == 1) ? item : item / k_splits;
@@ -245,7 +272,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (ep.batch > 1) { prob = tile / tiles_pp; tile -= prob * tiles_pp; }
                 int tr, tc;
                 tile_coords(tile, (M + TM - 1) / TM, n_tiles, ep.band_rows, tr, tc);
-                const int m0 = tr * TM, n0 = prob * N + tc * BN;
+                const int m0 = tr * TM + rank * BM, n0 = prob * N + tc * BN + (GATED ? 0 : rank * B_ROWS);
                 const int ka = prob * K;                      // problem p reads columns [p*K, (p+1)*K) of A
                 if (early_b && local == 0) {
                     // arm the first stages and request their B tiles, then wait for the previous kernel (A may be its output)
@@ -268,6 +295,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     ok = mbar_wait(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, ep.status);
                     if (!ok) break;
                     const uint32_t dst = smem_u32(smem + (size_t)s * STAGE_BYTES);
+                    if (PAIR) {
+                        // both CTAs' bytes are credited to the leader's barrier (where the MMAs are issued)
+                        const uint32_t full = map_to_cta(smem_u32(&bar_full[s]), 0);
+                        if (rank == 0) mbar_expect_tx(smem_u32(&bar_full[s]), 2u * (uint32_t)STAGE_BYTES);
+                        tma_load_2d_pair(dst, &tm_a, ka + kb * BK, m0, full);
+                        tma_load_2d_pair(dst + A_BYTES, GATED && rank ? &tm_b2 : &tm_b, kb * BK, n0, full);
+                        continue;
+                    }
                     const uint32_t full = smem_u32(&bar_full[s]);
                     mbar_expect_tx(full, (uint32_t)STAGE_BYTES);
                     tma_load_2d(dst, &tm_a, ka + kb * BK, m0, full);
@@ -275,6 +310,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 }
             }
         }
+    } else if (warp == 1 && rank != 0) {
+        // the leader's MMA warp works for both CTAs
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
         // The whole warp walks the loop, so that waits, indices and descriptors are warp-uniform (the tensor-core
@@ -327,7 +364,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     auto issue = [&](int k) {
                         const uint64_t koff = (uint64_t)((k * UMMA_K * 2) >> 4);    // 32 bytes per K step inside the swizzle row
                         const uint32_t accum = (kb > kb0 || k != 0) ? 1u : 0u;
-                        umma_bf16(acc, da + koff, db + koff, idesc, accum);
+                        if (PAIR) umma_bf16_pair(acc, da + koff, db + koff, idesc, accum);
+                        else umma_bf16(acc, da + koff, db + koff, idesc, accum);
                     };
                     if (elect_one()) {
 #pragma unroll
@@ -337,12 +375,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     have = __all_sync(0xffffffffu, mbar_test(smem_u32(&bar_full[s_next]), round_next & 1u));
                     if (elect_one()) {
                         issue(BK / UMMA_K - 1);
-                        umma_commit(smem_u32(&bar_empty[s]));        // stage reusable once these MMAs have read it
+                        if (PAIR) umma_commit_pair(smem_u32(&bar_empty[s]));
+                        else umma_commit(smem_u32(&bar_empty[s]));   // stage reusable once these MMAs have read it
                     }
                     __syncwarp();
                 }
                 if (!ok) break;
-                if (elect_one()) umma_commit(smem_u32(&bar_acc_full[buf]));   // accumulator of this tile complete
+                if (elect_one()) {                           // accumulator of this tile complete
+                    if (PAIR) umma_commit_pair(smem_u32(&bar_acc_full[buf]));
+                    else umma_commit(smem_u32(&bar_acc_full[buf]));
+                }
                 __syncwarp();
             }
         }
@@ -357,6 +399,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         const int quad = warp & 3;                          // TMEM lanes this warp may touch
         const int part = ew >> 2;                           // which 16 of every 64 columns of the tile
         constexpr int N_UNITS = COLS_PER_WARP / 16;
+        auto acc_release = [&](uint32_t b) {                // to the MMA warp (the leader's)
+            if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[b]), 0));
+            else mbar_arrive(smem_u32(&bar_acc_empty[b]));
+        };
         uint32_t out_n = 0;                                 // output buffers used so far
         for (uint32_t local = 0;; ++local) {
             const uint32_t buf = local & 1u, use = local >> 1;
@@ -370,7 +416,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     go = mbar_wait(smem_u32(&sched_full[buf]), use & 1u, ep.status);
                     if (go) {
                         item = sched_item[buf];
-                        mbar_arrive(smem_u32(&sched_empty[buf]));
+                        if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&sched_empty[buf]), 0));
+                        else mbar_arrive(smem_u32(&sched_empty[buf]));
                     }
                 }
                 go = go && item >= 0 && item < total_tiles;
@@ -379,7 +426,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     int prob = 0, tr, tc;
                     if (ep.batch > 1) { prob = tile / tiles_pp; tile -= prob * tiles_pp; }
                     tile_coords(tile, (M + TM - 1) / TM, n_tiles, ep.band_rows, tr, tc);
-                    epi_m0[buf] = tr * TM; epi_n0[buf] = tc * BN; epi_prob[buf] = prob;
+                    epi_m0[buf] = tr * TM + rank * BM; epi_n0[buf] = tc * BN; epi_prob[buf] = prob;
                     go = mbar_wait(smem_u32(&bar_acc_full[buf]), use & 1u, ep.status);
                 }
                 epi_go[buf] = go ? 1 : 0;
@@ -455,7 +502,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                         // all of this warp's TMEM reads of the buffer are complete: hand it back to the MMA warp
                         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
+                        if (lane == 0) acc_release(buf);
                     }
                     if (EPI == D2D_EPI_PARTIAL_F32) {
                         if (row < M) {
@@ -543,7 +590,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 }
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
+                if (lane == 0) acc_release(buf);
             }
         }
         // the buffers may not go away, nor the kernel count as finished, before the last stores are done
@@ -552,7 +599,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 1)
+    if (PAIR) cluster_sync_all();          // neither CTA releases shared memory or TMEM while the other may still use it
+    if (PAIR && warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
+    if (!PAIR && warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_COLS) : "memory");
 }
 
@@ -585,15 +635,16 @@ template <typename K> bool ensure_smem_attr(K kern, size_t smem, bool (&done)[64
     return true;
 }
 
-template <int BN, int EPI, int ACT, bool GATED>
+template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false>
 d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
 {
-    constexpr int STAGE_BYTES = BM * BK * 2 + (GATED ? 2 : 1) * BN * BK * 2;
+    constexpr int B_ROWS = PAIR && !GATED ? BN / 2 : BN, TM = PAIR ? 2 * BM : BM;
+    constexpr int STAGE_BYTES = BM * BK * 2 + (GATED && !PAIR ? 2 : 1) * B_ROWS * BK * 2;
     constexpr int STAGES = STAGE_BUDGET / STAGE_BYTES > 8 ? 8 : STAGE_BUDGET / STAGE_BYTES;
     constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 2 * (size_t)OUT_BUF_BYTES;
     static_assert(SMEM <= 224 * 1024, "shared memory per CTA");
     CUtensorMap ta, tb, tb2, to = {};
-    const bool gate_cat = GATED && g.b_cat != nullptr && g.b_cat_block == BN;
+    const bool gate_cat = GATED && !PAIR && g.b_cat != nullptr && g.b_cat_block == BN;
     const int batch = g.batch > 1 ? g.batch : 1;
     if (batch > 1 && (GATED || g.K % BK != 0)) return D2D_ERR_UNSUPPORTED;
     if (!d2d_tc_make_map(&ta, g.a, g.M, g.K * batch, BM)) return D2D_ERR_CUDA;
@@ -601,9 +652,9 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
         if (!d2d_tc_make_map(&tb, g.b_cat, 2 * BN * d2d_cdiv(g.N, BN), g.K, 2 * BN)) return D2D_ERR_CUDA;
         tb2 = tb;
     } else {
-        if (!d2d_tc_make_map(&tb, g.b, g.N * batch, g.K, BN)) return D2D_ERR_CUDA;
+        if (!d2d_tc_make_map(&tb, g.b, g.N * batch, g.K, B_ROWS)) return D2D_ERR_CUDA;
         if (GATED) {
-            if (!d2d_tc_make_map(&tb2, g.b_gate, g.N, g.K, BN)) return D2D_ERR_CUDA;
+            if (!d2d_tc_make_map(&tb2, g.b_gate, g.N, g.K, B_ROWS)) return D2D_ERR_CUDA;
         } else {
             tb2 = tb;
         }
@@ -614,50 +665,63 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
         const cuuint32_t box[3] = {64, 32, 1};
         if (!d2d_tc_encode_map(&to, false, 3, g.out, dims, strides, box)) return D2D_ERR_CUDA;
     }
-    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED>;
+    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED, PAIR>;
     static bool attr_set[64] = {};
     if (!ensure_smem_attr(kern, SMEM, attr_set)) return D2D_ERR_CUDA;
     const int es = g.expert_size > 0 ? g.expert_size : 1;
     EpiParams ep{(const __nv_bfloat16 *)g.bias, g.out, g.mask, g.mask_words, es, g.status,
                  (uint32_t)((0x100000000ull + (unsigned long long)es - 1) / (unsigned long long)es),
                  g.tile_counter, (g.pdl_late_wait && !g.n_sel && d2d_tc_pdl_enabled()) ? 1 : 0, gate_cat ? 1 : 0,
-                 band_rows_for(g.M, g.N, g.K, BM, GATED), batch, g.n_sel, g.n_sel_max,
+                 band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max,
                  (g.test_skip_load && !g.tile_counter && !g.pdl_late_wait && !g.n_sel) ? 1 : 0};
     const int k_splits = g.k_splits > 1 ? g.k_splits : 1;
-    const int tiles = d2d_cdiv(g.N, BN) * d2d_cdiv(g.M, BM) * k_splits * batch;
-    const int workers = d2d_tc_sm_count();
-    const int grid = tiles < workers ? tiles : workers;
+    const int tiles = d2d_cdiv(g.N, BN) * d2d_cdiv(g.M, TM) * k_splits * batch;
+    const int workers = PAIR ? d2d_tc_sm_count() / 2 : d2d_tc_sm_count();
+    const int grid = (tiles < workers ? tiles : workers) * (PAIR ? 2 : 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid, 1, 1);
     cfg.blockDim = dim3(NTHREADS_V2, 1, 1);
     cfg.dynamicSmemBytes = SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = PAIR ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     // the kernel's prologue may overlap the tail of the previous kernel in the stream (see griddepcontrol.wait in the kernel)
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 2 : 1;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits);
     D2D_LAUNCHED(1);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
-// Tile width with the least modelled time: rounds over the SMs x the time of one 64-deep k-block of a 128 x bn tile.
-// That time is not proportional to bn: every k-block brings 16 KB of A and bn / 8 KB of B into the SM, and the SM's
-// path from L2 is what a 128-row tile saturates, so a narrow tile pays almost as much as a wide one for fewer columns.
-// Measured on B200 (K = 11008, T = 4096 and 8192): 0.40 us per k-block at bn = 256, 0.31 us at bn = 128, i.e. about
-// 0.13 us + 0.7 ns per row of A and B staged.  Wider tiles win ties.
-int pick_bn(int M, int N, int tile_m, int workers, const int *cands, int n_cands, int batch = 1)
+// Tile with the least modelled time: rounds over the SMs (pairs of SMs) x the time of one 64-deep k-block.  That time is not
+// proportional to the width bn: every k-block brings 16 KB of A and bn / 8 KB of B (a pair's CTA: half of them) into an SM,
+// and the fill from L2 is what bounds it.  Measured on B200 under sustained load (us per k-block, K = 3072 .. 11008):
+// single CTAs 0.457 / 0.40 / 0.345 at bn = 256 / 192 / 128, pairs 0.42 / 0.345 / 0.29.  Wider tiles win ties.
+// Pairs: not for one row tile, nor for K below 2048, where their coarser tiles and set-up cost more than the fill saves
+// (BERT-shaped layer with pairs in both projections / in the down projection / none: 55.6 / 51.7 / 52.4 us; ViT-shaped
+// 252 / 248.5 / 249; Llama-shaped down projection 506-533 us with pairs, 550 without).
+struct tile_choice { int bn; bool pair; };
+tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok)
 {
-    int best = cands[0];
+    const int sms = d2d_tc_sm_count();
+    const int bns[4] = {256, 192, 128, 64};
+    const double t1[4] = {0.457, 0.40, 0.345, 0.28}, t2[3] = {0.42, 0.345, 0.29};
+    tile_choice best = {256, false};
     double best_cost = 1e300;
-    for (int i = 0; i < n_cands; ++i) {
-        const int bn = cands[i];
-        const long tiles = (long)d2d_cdiv(N, bn) * d2d_cdiv(M, tile_m) * batch;
-        const long rounds = (tiles + workers - 1) / workers;
-        const double cost = (double)rounds * (0.13 + 0.0007 * (double)(tile_m + bn));
-        if (cost < best_cost - 1e-9) { best_cost = cost; best = bn; }
+    for (int i = 0; i < 4; ++i) {
+        const long tiles = (long)d2d_cdiv(N, bns[i]) * d2d_cdiv(M, BM) * batch;
+        const double cost = (double)((tiles + sms - 1) / sms) * t1[i];
+        if (cost < best_cost - 1e-9) { best_cost = cost; best = {bns[i], false}; }
+    }
+    if (!pairs_ok || M <= BM || K < 2048) return best;
+    const int pairs = sms / 2;
+    for (int i = 0; i < 3; ++i) {
+        const long tiles = (long)d2d_cdiv(N, bns[i]) * d2d_cdiv(M, 2 * BM) * batch;
+        const double cost = (double)((tiles + pairs - 1) / pairs) * t2[i];
+        if (cost < best_cost - 1e-9) { best_cost = cost; best = {bns[i], true}; }
     }
     return best;
 }
@@ -665,13 +729,22 @@ int pick_bn(int M, int N, int tile_m, int workers, const int *cands, int n_cands
 template <int EPI, int ACT, bool GATED>
 d2d_status launch_bn(const d2d_gemm_args &g, cudaStream_t st)
 {
-    if (GATED) return launch<128, EPI, ACT, true>(g, st);
-    const int cands[4] = {256, 192, 128, 64};
-    switch (pick_bn(g.M, g.N, BM, d2d_tc_sm_count(), cands, 4, g.batch > 1 ? g.batch : 1)) {
-    case 256: return launch<256, EPI, ACT, false>(g, st);
-    case 192: return launch<192, EPI, ACT, false>(g, st);
-    case 128: return launch<128, EPI, ACT, false>(g, st);
-    default: return launch<64, EPI, ACT, false>(g, st);
+    const bool pairs_ok = !g.test_skip_load && EPI != D2D_EPI_ABS_F32;
+    if (GATED) {
+        if (pairs_ok && g.M > BM) return launch<128, EPI, ACT, GATED, true>(g, st);
+        return launch<128, EPI, ACT, GATED>(g, st);
+    }
+    const tile_choice c = pick_tile(g.M, g.N, g.K, g.batch > 1 ? g.batch : 1, pairs_ok);
+    if (c.pair) {
+        if (c.bn == 256) return launch<GATED ? 128 : 256, EPI, ACT, GATED, EPI != D2D_EPI_ABS_F32>(g, st);
+        if (c.bn == 192) return launch<GATED ? 128 : 192, EPI, ACT, GATED, EPI != D2D_EPI_ABS_F32>(g, st);
+        return launch<128, EPI, ACT, GATED, EPI != D2D_EPI_ABS_F32>(g, st);
+    }
+    switch (c.bn) {
+    case 256: return launch<GATED ? 128 : 256, EPI, ACT, GATED>(g, st);
+    case 192: return launch<GATED ? 128 : 192, EPI, ACT, GATED>(g, st);
+    case 128: return launch<128, EPI, ACT, GATED>(g, st);
+    default: return launch<GATED ? 128 : 64, EPI, ACT, GATED>(g, st);
     }
 }
 
