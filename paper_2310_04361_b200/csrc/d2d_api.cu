@@ -791,6 +791,9 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
         }
         if (!lists) return D2D_ERR_INVALID_ARG;               // the expert kernels of this shape walk the per-expert lists
         rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, st, 1);
+    } else if (d2d_layer_f32_small_supports(layer->desc, T, lists)) {
+        // float32 layers that fit one SM's shared memory: router, rule, experts and lists in one launch
+        return d2d_layer_f32_small(layer, x, T, tau, y, R_out, routing, lists, layer->tickets + 52, st);
     } else if (T > 8 && d2d_layer_token_fused_supports(layer->desc, T, lists)) {
         // small float32 problems: router, rule, experts and lists in one launch
         if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;

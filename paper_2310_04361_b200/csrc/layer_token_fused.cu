@@ -71,6 +71,7 @@ layer_token_fused_kernel(const FusedArgs a)
     uint32_t *smask = words + a.W;                      // [T * W] all tokens' words (last CTA, lists only)
     __shared__ int n_kept;
     __shared__ int is_last;
+    __shared__ int sk[d2d_small::MAX_T];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int t = blockIdx.x, d = a.d, s = a.s;
     const T *x = (const T *)a.x;
@@ -210,7 +211,7 @@ layer_token_fused_kernel(const FusedArgs a)
     if (!is_last) return;
     __threadfence();
     d2d_small::select_cta(nullptr, a.T, a.E, a.W, a.tau, a.r.mask, a.r.k, a.r.counts, a.r.offsets, a.r.perm, a.r.tok_off, a.r.tok_exp,
-                          a.r.n_sel, a.r.status, a.r.perm_capacity, 1, smask);
+                          a.r.n_sel, a.r.status, a.r.perm_capacity, 1, smask, sk);
 }
 
 template <typename T, int ACT>

@@ -20,8 +20,9 @@ small_select_kernel(const float *__restrict__ R, int T, int E, int W, float tau,
                     long long capacity, int keep_status)
 {
     extern __shared__ uint32_t smask[];          // [T][W]
+    __shared__ int sk[d2d_small::MAX_T];
     d2d_small::select_cta(R, T, E, W, tau, mask, k, counts, offsets, perm, tok_off, tok_exp, n_sel, status, capacity,
-                          keep_status, smask);
+                          keep_status, smask, sk);
 }
 
 }  // namespace

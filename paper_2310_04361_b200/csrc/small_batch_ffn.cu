@@ -228,8 +228,9 @@ small_router_kernel(const TT *__restrict__ x, int T, int d, int d_h, int E, int 
         // the scores of all (at most 8) tokens were written by this CTA: select from them right here
         __syncthreads();
         uint32_t *smask = reinterpret_cast<uint32_t *>(us + (size_t)T * d_h);
+        __shared__ int sk[8];
         d2d_small::select_cta(R, T, E, (E + 31) / 32, sel.tau, sel.mask, sel.k, sel.counts, sel.offsets, sel.perm, sel.tok_off,
-                              sel.tok_exp, sel.n_sel, sel.status, sel.capacity, 0, smask);
+                              sel.tok_exp, sel.n_sel, sel.status, sel.capacity, 0, smask, sk);
     }
 }
 

@@ -9,21 +9,21 @@
 namespace d2d_small {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int MAX_T = 256;          // tokens select_cta can take (per-token k staged in shared memory)
+constexpr int MAX_T = 256;          // tokens the kernels with a fixed array for select_cta's per-token k take
 
 __device__ __forceinline__ bool finite_f32(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
 
-// Called by every thread of the CTA (blockDim.x a multiple of 32, at most 1024).  smask: shared memory, T * W words.
+// Called by every thread of the CTA (blockDim.x a multiple of 32, at most 1024).  smask: shared memory, T * W words; sk: T ints.
 // R == nullptr: the mask words are an input (override protocol), otherwise they are computed.  R may have been
 // written earlier by this very CTA (after a __syncthreads), hence the plain (coherent) loads.
 __device__ __forceinline__ void select_cta(const float *R, int T, int E, int W, float tau, uint32_t *mask, int32_t *k,
                                            int32_t *counts, int32_t *offsets, int32_t *perm, int32_t *tok_off,
                                            int32_t *tok_exp, int32_t *n_sel, int32_t *status, long long capacity,
-                                           int keep_status, uint32_t *smask)
+                                           int keep_status, uint32_t *smask, int *sk)
 {
     __shared__ int warp_sums[32];
     __shared__ int chunk_total;
-    __shared__ int sk[MAX_T];
+    __shared__ int k_total;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nthreads = blockDim.x, nwarps = nthreads >> 5;
     if (threadIdx.x == 0 && !keep_status) *status = 0;
@@ -166,7 +166,6 @@ __device__ __forceinline__ void select_cta(const float *R, int T, int E, int W, 
     }
     // token-major dual: exclusive scan of k by warp 0, then one thread per token
     if (tok_off && tok_exp) {
-        __shared__ int stok[MAX_T];
         __syncthreads();
         if (warp == 0) {
             int run = 0;
@@ -179,15 +178,16 @@ __device__ __forceinline__ void select_cta(const float *R, int T, int E, int W, 
                     const int n = __shfl_up_sync(FULL, inc, o);
                     if (lane >= o) inc += n;
                 }
-                if (t < T) stok[t] = run + inc - c;
+                if (t < T) sk[t] = run + inc - c;                  // now the token's offset
                 run += __shfl_sync(FULL, inc, 31);
             }
+            if (lane == 0) k_total = run;
         }
         __syncthreads();
         for (int t = threadIdx.x; t < T; t += nthreads) {
-            long long base = stok[t];
+            long long base = sk[t];
             tok_off[t] = (int32_t)base;
-            if (t == T - 1) tok_off[T] = (int32_t)(base + sk[t]);
+            if (t == T - 1) tok_off[T] = k_total;
             for (int w = 0; w < W; ++w) {
                 uint32_t word = smask[t * W + w];
                 while (word) {

@@ -705,3 +705,26 @@ def test_decode_batches_at_the_edges_of_their_tiles(api, shape, T, fp8):
         y2 = layer.moe_ffn_fwd(xd, r)                      # the expert step on its own: no list of kept units from the router
         assert _rel_err(y2.float().cpu().numpy(), y_ref) <= TOL_Y["bf16"]
     layer.close()
+
+
+@pytest.mark.parametrize("T,act,gated,lists", [(1, "relu", False, True), (8, "silu", True, True), (149, "relu", False, True),
+                                               (1000, "gelu_erf", False, True), (600, "gelu_tanh", True, False)])
+def test_fp32_layer_in_shared_memory_one_or_several_tokens_per_cta(api, T, act, gated, lists):
+    """Layers whose weights fit one SM: one token, one token per CTA and a few left over, several per CTA; twice."""
+    import dataclasses
+    cfg = dataclasses.replace(wl.with_tokens(wl.CONFIGS["tiny"], T), act=act, gated=gated)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    for tau in (0.5, 0.0):
+        r = layer.new_routing(T, dual=lists, lists=lists)
+        R_out = _poison(torch.empty((T, cfg.E), dtype=torch.float32, device="cuda"))
+        y, _ = layer.layer_fwd(api.to_device(x, cfg.dtype), tau, R_out=R_out, routing=r)
+        torch.cuda.synchronize()
+        assert _rel_err(R_out.cpu().numpy(), oracle.router(x, w["w_r1"], w["b_r1"], w["w_r2"], w["b_r2"])) <= TOL_R["f32"]
+        G = oracle.unpack_mask(r.mask_u32(), cfg.E)
+        assert np.array_equal(G, oracle.select(R_out.cpu().numpy(), tau)[0])
+        if lists:
+            _check_routing(r, G, dual=True)
+        y_ref = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[act], G)
+        assert r.status == 0 and _rel_err(y.cpu().numpy(), y_ref) <= TOL_Y["f32"]
+    layer.close()
