@@ -45,9 +45,9 @@ struct RouterGroupIO {
     RouterLayerIO l[D2D_MAX_GROUP];
     uint32_t *mask_cat;    // merged mask [T, cat_words] or NULL
     int cat_words;
-    int32_t *ksum;         // single layer only, or NULL: [0] running sum of k, [1] CTA exit ticket, [2] largest condition (all
-                           // zero at launch and left at zero), [4] receives the total = number of selected (token, expert)
-                           // pairs; the last CTA then writes *status
+    int32_t *ksum;         // single layer only, or NULL: [0..1] running sum of k and exit count (64 bits), [2] largest condition
+                           // (all zero at launch and left at zero), [4] receives the total = number of selected (token,
+                           // expert) pairs; the last CTA then writes *status
 };
 
 // Shared memory (dynamic, 1024-byte aligned):
@@ -89,9 +89,10 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     constexpr int W2_STAGES = (KB2 * W2_KB_BYTES + STAGE_BYTES - 1) / STAGE_BYTES;      // stages W_r2 overwrites
     __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_w2, bar_acc1, bar_u_ready, bar_acc2;
     __shared__ uint32_t tmem_base_holder;
-    __shared__ float b1_s[DH], b2_s[256];                  // biases as float32
-    __shared__ float pmax_s[4 * BM];                       // per column-part row maxima
-    __shared__ int pbad_s[4 * BM], pk_s[4 * BM];
+    __shared__ __align__(16) float b1_s[DH], b2_s[256];    // biases as float32
+    __shared__ uint32_t pmax_s[4 * BM];                    // per column-part row maxima (bit patterns of non-negative floats)
+    __shared__ int pk_s[4 * BM];
+    __shared__ int warp_k[4], warp_bad[4];
     for (int i = threadIdx.x; i < DH; i += NTHREADS) b1_s[i] = b_r1 ? __bfloat162float(b_r1[i]) : 0.0f;
     for (int i = threadIdx.x; i < 256; i += NTHREADS) b2_s[i] = (b_r2 && i < E) ? __bfloat162float(b_r2[i]) : 0.0f;
 
@@ -198,6 +199,29 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         const int r_local = quad * 32 + lane;
         const int row = m0 + r_local;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+        // Number of selected pairs of the whole batch, for the density-adaptive dispatch of the expert step, and the status
+        // word: one 64-bit addition per CTA carries its sum (36 bits), its exit (14 bits) and whether it saw a condition
+        // (14 bits); whoever completes the count publishes and resets.  Called by the four warps of part 0.
+        auto publish = [&](int k_warp, bool cond_warp) {
+            if (lane == 0) { warp_k[quad] = k_warp; warp_bad[quad] = cond_warp; }
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+            if (quad != 0 || lane != 0) return;
+            const int cond = warp_bad[0] | warp_bad[1] | warp_bad[2] | warp_bad[3];
+            if (cond) __threadfence();                       // its entry in the condition word comes first
+            const unsigned long long add = (unsigned long long)(warp_k[0] + warp_k[1] + warp_k[2] + warp_k[3]) + (1ull << 36) +
+                                           (cond ? 1ull << 50 : 0ull);
+            unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(io.ksum);
+            const unsigned long long tot = atomicAdd(acc64, add) + add;
+            if (((tot >> 36) & 0x3fffu) != (unsigned long long)(gridDim.x * gridDim.y)) return;
+            *acc64 = 0ull;
+            io.ksum[4] = (int32_t)(tot & 0xfffffffffull);
+            int32_t st = 0;
+            if (tot >> 50) {
+                __threadfence();
+                st = atomicExch(io.ksum + 2, 0);
+            }
+            *io.l[layer].status = st;
+        };
         int okw = 1;
         if (lane == 0) okw = mbar_wait(smem_u32(&bar_acc1), 0, status) ? 1 : 0;
         bool ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
@@ -235,13 +259,15 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int W = (E + 31) / 32;
             float v[2][32];
-            float m = -INFINITY;
-            bool bad = false;
+            // Scores are non-negative, so their bit patterns order like the values, with infinities and NaNs on top: ONE integer
+            // maximum per element yields the row maximum and whether a score is not finite.
+            uint32_t mb = 0u;
             if (ok) {
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
                     const int w = part + 4 * q;
                     if (w < W) {
+                        const bool whole = w * 32 + 32 <= E;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int c0 = w * 32 + h * 16;
@@ -249,14 +275,20 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                                 uint32_t acc[16];
                                 tmem_ld16(tmem_r + lane_base + (uint32_t)c0, acc);
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) {
-                                    const int i = c0 + j;
-                                    const float val = fabsf(__uint_as_float(acc[j]) + b2_s[i]);
-                                    v[q][h * 16 + j] = val;
-                                    if (i < E) {
-                                        bad |= (__float_as_uint(val) & 0x7f800000u) == 0x7f800000u;
-                                        m = val > m ? val : m;
-                                    }
+                                for (int j = 0; j < 16; j += 4) {
+                                    const float4 b = *reinterpret_cast<const float4 *>(b2_s + c0 + j);
+                                    v[q][h * 16 + j] = fabsf(__uint_as_float(acc[j]) + b.x);
+                                    v[q][h * 16 + j + 1] = fabsf(__uint_as_float(acc[j + 1]) + b.y);
+                                    v[q][h * 16 + j + 2] = fabsf(__uint_as_float(acc[j + 2]) + b.z);
+                                    v[q][h * 16 + j + 3] = fabsf(__uint_as_float(acc[j + 3]) + b.w);
+                                }
+                                if (whole) {
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j) mb = max(mb, __float_as_uint(v[q][h * 16 + j]));
+                                } else {
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j)
+                                        if (c0 + j < E) mb = max(mb, __float_as_uint(v[q][h * 16 + j]));
                                 }
                                 if (R && row < T) {
                                     float *o = R + (size_t)row * E + c0;
@@ -288,19 +320,15 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 }
             }
             if (do_mask) {
-                // row maximum across the four column parts (and the non-finite flag), through shared memory
-                pmax_s[part * BM + r_local] = m;
-                pbad_s[part * BM + r_local] = bad ? 1 : 0;
+                // row maximum across the four column parts, through shared memory
+                pmax_s[part * BM + r_local] = mb;
                 asm volatile("bar.sync 1, 512;" ::: "memory");           // the 16 epilogue warps only
-                float mm = pmax_s[r_local];
-                int anybad = pbad_s[r_local];
+                uint32_t mm = pmax_s[r_local];
 #pragma unroll
-                for (int p = 1; p < 4; ++p) {
-                    const float o = pmax_s[p * BM + r_local];
-                    mm = o > mm ? o : mm;
-                    anybad |= pbad_s[p * BM + r_local];
-                }
-                const float thr = __fmul_rn(tau, mm);
+                for (int p = 1; p < 4; ++p) mm = max(mm, pmax_s[p * BM + r_local]);
+                const bool bad = mm >= 0x7f800000u;
+                // a row with a score that is not finite keeps every expert: no score is below a negative threshold
+                const float thr = bad ? -1.0f : __fmul_rn(tau, __uint_as_float(mm));
                 int kt = 0;
                 if (ok) {
 #pragma unroll
@@ -309,10 +337,8 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                         if (w < W) {
                             uint32_t word = 0u;
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const int i = w * 32 + j;
-                                if (i < E && (anybad || v[q][j] >= thr)) word |= 1u << j;
-                            }
+                            for (int j = 0; j < 32; ++j) word |= !(v[q][j] < thr) ? 1u << j : 0u;
+                            if (w * 32 + 32 > E) word &= (1u << (E - w * 32)) - 1u;
                             if (row < T) {
                                 mask[(size_t)row * W + w] = word;
                                 if (io.mask_cat) io.mask_cat[(size_t)row * io.cat_words + layer * W + w] = word;
@@ -323,28 +349,18 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                 }
                 pk_s[part * BM + r_local] = kt;
                 asm volatile("bar.sync 1, 512;" ::: "memory");
-                int k_row = 0;
-                if (part == 0 && row < T) {
-                    k_row = pk_s[r_local] + pk_s[BM + r_local] + pk_s[2 * BM + r_local] + pk_s[3 * BM + r_local];
-                    k[row] = k_row;
-                    if (anybad) atomicMax(status, (int32_t)D2D_ERR_NONFINITE);
-                }
-                if (io.ksum) {
-                    // number of selected pairs of the whole batch, for the density-adaptive dispatch of the expert step
-                    if (part == 0) {
+                if (part == 0) {
+                    int k_row = 0;
+                    if (row < T) {
+                        k_row = pk_s[r_local] + pk_s[BM + r_local] + pk_s[2 * BM + r_local] + pk_s[3 * BM + r_local];
+                        k[row] = k_row;
+                        if (bad) atomicMax(status, (int32_t)D2D_ERR_NONFINITE);
+                    }
+                    if (io.ksum) {
+                        const bool any = __any_sync(0xffffffffu, bad && row < T);
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) k_row += __shfl_xor_sync(0xffffffffu, k_row, o);
-                        if (lane == 0) atomicAdd(io.ksum, k_row);
-                    }
-                    asm volatile("bar.sync 1, 512;" ::: "memory");
-                    if (warp == 2 && lane == 0) {
-                        __threadfence();
-                        if (atomicAdd(io.ksum + 1, 1) == (int)(gridDim.x * gridDim.y) - 1) {
-                            __threadfence();
-                            io.ksum[4] = atomicExch(io.ksum, 0);         // the CTA that finishes last publishes and resets
-                            *io.l[layer].status = atomicExch(io.ksum + 2, 0);
-                            io.ksum[1] = 0;
-                        }
+                        publish(k_row, any || !ok);
                     }
                 }
             }
@@ -352,7 +368,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             // keep the named barrier balanced when a bounded wait ran out
             asm volatile("bar.sync 1, 512;" ::: "memory");
             asm volatile("bar.sync 1, 512;" ::: "memory");
-            if (io.ksum) asm volatile("bar.sync 1, 512;" ::: "memory");
+            if (io.ksum && part == 0) publish(0, true);
         }
     }
 
@@ -404,7 +420,8 @@ d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_la
 bool d2d_router_fused_supports(const d2d_layer_desc &D, int T)
 {
     // d_h = 128 (the paper's router width) and E <= 256: operand ring, u and W_r2 then fit in shared memory together
-    return D.dtype == D2D_BF16 && T > d2d_decode_max_tokens(D) && D.d_h == 128 && D.n_experts <= 256 && D.d % 8 == 0 && d2d_gemm_tc_available();
+    return D.dtype == D2D_BF16 && T > d2d_decode_max_tokens(D) && D.d_h == 128 && D.n_experts <= 256 && D.d % 8 == 0 &&
+           T <= 16000 * BM && d2d_gemm_tc_available();          // (the exit count has 14 bits)
 }
 
 // R may be NULL when only the mask is wanted; mask / k / status are used when do_mask != 0.
