@@ -807,13 +807,16 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
         if (rc != D2D_OK) return rc;
         return d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, nullptr, small ? 1 : 0);
     } else if (use_dense_masked(layer, T) && !use_small_ffn(layer, T) && !d2d_small_select_supports(T, E)) {
-        // router shapes the fused kernel does not take, tensor-core expert step: scores by two GEMMs, then mask, k and
-        // the number of selected pairs by one kernel; the per-expert lists (when wanted) are built on the side stream
-        // while the experts, which read only the mask, run
-        rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
-        if (rc != D2D_OK) return rc;
+        // router shapes the fused kernel does not take, tensor-core expert step: the hidden layer by a GEMM, then scores,
+        // mask, k and the number of selected pairs by one kernel (two where the scores do not fit it); the per-expert lists
+        // (when wanted) are built on the side stream while the experts, which read only the mask, run
         int32_t *ksum = (int32_t *)(layer->tickets + 40);
-        rc = d2d_launch_dynk_mask(R, T, E, tau, routing, ksum, st);
+        if (d2d_router_scores_supports(layer->desc, T)) {
+            rc = d2d_router_scores(layer, x, base + w.u_off + 256, T, tau, R_out, routing->mask, routing->k, routing->status, st, ksum);
+        } else {
+            rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
+            if (rc == D2D_OK) rc = d2d_launch_dynk_mask(R, T, E, tau, routing, ksum, st);
+        }
         if (rc != D2D_OK) return rc;
         if (lists) {
             if (cudaEventRecord(layer->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(layer->side_stream, layer->ev_fork, 0) != cudaSuccess)

@@ -137,6 +137,10 @@ bool d2d_router_fused_supports(const d2d_layer_desc &D, int T);
 // (which the caller must have cleared otherwise)
 d2d_status d2d_router_fused(const d2d_layer *L, const void *x, int T, float tau, int do_mask, float *R, uint32_t *mask,
                             int32_t *k, int32_t *status, cudaStream_t st, int32_t *ksum = nullptr);
+// The same in two launches (hidden layer, then scores and selection) for d_h up to 256 and E up to 384; u: scratch [T, d_h] bf16
+bool d2d_router_scores_supports(const d2d_layer_desc &D, int T);
+d2d_status d2d_router_scores(const d2d_layer *L, const void *x, void *u, int T, float tau, float *R, uint32_t *mask,
+                             int32_t *k, int32_t *status, cudaStream_t st, int32_t *ksum);
 d2d_status d2d_router_fused_group(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T,
                                   float tau, const d2d_routing *routing, uint32_t *mask_cat, int cat_words, cudaStream_t st);
 d2d_status d2d_small_group_fwd(const d2d_layer *const *layers, int n, const void *x, int T, float tau, const d2d_routing *routing,

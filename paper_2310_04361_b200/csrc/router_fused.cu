@@ -50,6 +50,52 @@ struct RouterGroupIO {
                            // expert) pairs; the last CTA then writes *status
 };
 
+// Number of selected pairs of the whole batch, for the density-adaptive dispatch of the expert step, and the status word: one
+// 64-bit addition per CTA carries its sum (36 bits), its exit (14 bits) and whether it saw a condition (14 bits); whoever
+// completes the count publishes and resets.  Called by four warps (one per TMEM lane quadrant) with their sums of k.
+__device__ __forceinline__ void publish_batch(int32_t *ksum, int32_t *status_out, int quad, int lane, int k_warp, bool cond_warp,
+                                              int *warp_k, int *warp_bad)
+{
+    if (lane == 0) { warp_k[quad] = k_warp; warp_bad[quad] = cond_warp; }
+    asm volatile("bar.sync 2, 128;" ::: "memory");
+    if (quad != 0 || lane != 0) return;
+    const int cond = warp_bad[0] | warp_bad[1] | warp_bad[2] | warp_bad[3];
+    if (cond) __threadfence();                       // its entry in the condition word comes first
+    const unsigned long long add = (unsigned long long)(warp_k[0] + warp_k[1] + warp_k[2] + warp_k[3]) + (1ull << 36) +
+                                   (cond ? 1ull << 50 : 0ull);
+    unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(ksum);
+    const unsigned long long tot = atomicAdd(acc64, add) + add;
+    if (((tot >> 36) & 0x3fffu) != (unsigned long long)(gridDim.x * gridDim.y)) return;
+    *acc64 = 0ull;
+    ksum[4] = (int32_t)(tot & 0xfffffffffull);
+    int32_t st = 0;
+    if (tot >> 50) {
+        __threadfence();
+        st = atomicExch(ksum + 2, 0);
+    }
+    *status_out = st;
+}
+
+// 16 consecutive scores of one row, from column c0
+__device__ __forceinline__ void store_scores16(float *__restrict__ R, int row, int E, int c0, const float *v)
+{
+    float *o = R + (size_t)row * E + c0;
+    if (c0 + 16 <= E && (E & 7) == 0 && (reinterpret_cast<uintptr_t>(R) & 31) == 0) {
+        // 32-byte stores: a whole sector per lane and instruction
+#pragma unroll
+        for (int j = 0; j < 16; j += 8)
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + j), "f"(v[j]), "f"(v[j + 1]),
+                         "f"(v[j + 2]), "f"(v[j + 3]), "f"(v[j + 4]), "f"(v[j + 5]), "f"(v[j + 6]), "f"(v[j + 7]) : "memory");
+    } else if (c0 + 16 <= E && (E & 3) == 0) {
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) *reinterpret_cast<float4 *>(o + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (c0 + j < E) o[j] = v[j];
+    }
+}
+
 // Shared memory (dynamic, 1024-byte aligned):
 //   [ STAGES x (x tile 128x64 | W_r1 tile DH x 64) ]        first GEMM operand ring
 //   [ u: DH/64 k-blocks x (128 rows x 128 B) ]              A operand of the second GEMM (written by epilogue 1)
@@ -199,29 +245,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         const int r_local = quad * 32 + lane;
         const int row = m0 + r_local;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-        // Number of selected pairs of the whole batch, for the density-adaptive dispatch of the expert step, and the status
-        // word: one 64-bit addition per CTA carries its sum (36 bits), its exit (14 bits) and whether it saw a condition
-        // (14 bits); whoever completes the count publishes and resets.  Called by the four warps of part 0.
-        auto publish = [&](int k_warp, bool cond_warp) {
-            if (lane == 0) { warp_k[quad] = k_warp; warp_bad[quad] = cond_warp; }
-            asm volatile("bar.sync 2, 128;" ::: "memory");
-            if (quad != 0 || lane != 0) return;
-            const int cond = warp_bad[0] | warp_bad[1] | warp_bad[2] | warp_bad[3];
-            if (cond) __threadfence();                       // its entry in the condition word comes first
-            const unsigned long long add = (unsigned long long)(warp_k[0] + warp_k[1] + warp_k[2] + warp_k[3]) + (1ull << 36) +
-                                           (cond ? 1ull << 50 : 0ull);
-            unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(io.ksum);
-            const unsigned long long tot = atomicAdd(acc64, add) + add;
-            if (((tot >> 36) & 0x3fffu) != (unsigned long long)(gridDim.x * gridDim.y)) return;
-            *acc64 = 0ull;
-            io.ksum[4] = (int32_t)(tot & 0xfffffffffull);
-            int32_t st = 0;
-            if (tot >> 50) {
-                __threadfence();
-                st = atomicExch(io.ksum + 2, 0);
-            }
-            *io.l[layer].status = st;
-        };
+        auto publish = [&](int k_warp, bool cond_warp) { publish_batch(io.ksum, io.l[layer].status, quad, lane, k_warp, cond_warp, warp_k, warp_bad); };
         int okw = 1;
         if (lane == 0) okw = mbar_wait(smem_u32(&bar_acc1), 0, status) ? 1 : 0;
         bool ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
@@ -290,27 +314,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                                     for (int j = 0; j < 16; ++j)
                                         if (c0 + j < E) mb = max(mb, __float_as_uint(v[q][h * 16 + j]));
                                 }
-                                if (R && row < T) {
-                                    float *o = R + (size_t)row * E + c0;
-                                    if (c0 + 16 <= E && (E & 7) == 0 && (reinterpret_cast<uintptr_t>(R) & 31) == 0) {
-                                        // 32-byte stores: a whole sector per lane and instruction
-#pragma unroll
-                                        for (int j = 0; j < 16; j += 8)
-                                            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(o + j),
-                                                         "f"(v[q][h * 16 + j]), "f"(v[q][h * 16 + j + 1]), "f"(v[q][h * 16 + j + 2]),
-                                                         "f"(v[q][h * 16 + j + 3]), "f"(v[q][h * 16 + j + 4]), "f"(v[q][h * 16 + j + 5]),
-                                                         "f"(v[q][h * 16 + j + 6]), "f"(v[q][h * 16 + j + 7]) : "memory");
-                                    } else if (c0 + 16 <= E && (E & 3) == 0) {
-#pragma unroll
-                                        for (int j = 0; j < 16; j += 4)
-                                            *reinterpret_cast<float4 *>(o + j) = make_float4(v[q][h * 16 + j], v[q][h * 16 + j + 1],
-                                                                                             v[q][h * 16 + j + 2], v[q][h * 16 + j + 3]);
-                                    } else {
-#pragma unroll
-                                        for (int j = 0; j < 16; ++j)
-                                            if (c0 + j < E) o[j] = v[q][h * 16 + j];
-                                    }
-                                }
+                                if (R && row < T) store_scores16(R, row, E, c0, &v[q][h * 16]);
                             } else {
 #pragma unroll
                                 for (int j = 0; j < 16; ++j) v[q][h * 16 + j] = 0.0f;
@@ -379,6 +383,197 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     }
 }
 
+// Second router layer and selection for the shapes the kernel above has no room for (d_h up to 256, E up to 384): u comes from
+// a GEMM of its own, and this kernel reads it once, keeps the scores in TMEM and writes mask and k (and R when wanted).
+// One CTA per 128 tokens.  All of u's tile (d_h / 64 k-blocks of 16 KB) and three k-blocks of W_r2 (128-row boxes, up to
+// 48 KB each) are in flight at once; a fourth k-block takes the first one's place.  The scores fill up to 384 TMEM columns, too
+// many for registers, so the epilogue reads them twice: once for the row maxima, once for the mask words.
+// Bound by latency (one CTA per SM at most, one tile each): loads, 4 k-blocks of MMAs, two passes over TMEM.  Measured at
+// d = 4096, d_h = 256, E = 344, 8192 tokens, from the router's start to the up projection: 92 us against 124 us for a GEMM
+// that wrote R and a kernel that read it twice (11 MB each way); the whole layer 1668 -> 1626 us, at 128 tokens 121 -> 114.
+constexpr int S_MAX_KB = 4, S_STAGES = 3, S_STAGE_BYTES = 384 * 128, S_WORDS = 3;      // a part owns mask words p, p + 4, p + 8
+__global__ void __launch_bounds__(NTHREADS, 1)
+router_scores_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_w2,
+                     const __nv_bfloat16 *__restrict__ b_r2, int T, int kb2, int E, int EN /* E rounded up to 16 */, float tau,
+                     const __grid_constant__ RouterGroupIO io)
+{
+    float *__restrict__ R = io.l[0].R;
+    int32_t *__restrict__ status = io.ksum + 2;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *u_s = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t *w2_s = u_s + (size_t)S_MAX_KB * BM * 128;
+    __shared__ uint64_t bar_u, bar_w[S_MAX_KB], bar_free, bar_acc;
+    __shared__ uint32_t tmem_base_holder;
+    __shared__ __align__(16) float b2_s[384];
+    __shared__ uint32_t pmax_s[4 * BM];
+    __shared__ int pk_s[4 * BM];
+    __shared__ int warp_k[4], warp_bad[4];
+    for (int i = threadIdx.x; i < 384; i += NTHREADS) b2_s[i] = (b_r2 && i < E) ? __bfloat162float(b_r2[i]) : 0.0f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m0 = blockIdx.x * BM;
+    const int boxes = (E + 127) / 128;
+    auto load_w2 = [&](int kb) {
+        mbar_expect_tx(smem_u32(&bar_w[kb]), (uint32_t)boxes * 128 * 128);
+        for (int i = 0; i < boxes; ++i)
+            tma_load_2d(smem_u32(w2_s + (size_t)(kb % S_STAGES) * S_STAGE_BYTES + (size_t)i * 128 * 128), &tm_w2, kb * BK, i * 128,
+                        smem_u32(&bar_w[kb]));
+    };
+    if (threadIdx.x == 0) {
+        for (int kb = 0; kb < S_MAX_KB; ++kb) mbar_init(smem_u32(&bar_w[kb]), 1);
+        mbar_init(smem_u32(&bar_u), 1);
+        mbar_init(smem_u32(&bar_free), 1);
+        mbar_init(smem_u32(&bar_acc), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // the weights do not depend on the previous kernel of the stream
+        for (int kb = 0; kb < kb2 && kb < S_STAGES; ++kb) load_w2(kb);
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = tmem_base_holder;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    if (warp == 0) {
+        if (lane == 0) {
+            mbar_expect_tx(smem_u32(&bar_u), (uint32_t)kb2 * BM * 128);
+            for (int kb = 0; kb < kb2; ++kb) tma_load_2d(smem_u32(u_s + (size_t)kb * BM * 128), &tm_u, kb * BK, m0, smem_u32(&bar_u));
+            if (kb2 > S_STAGES && mbar_wait(smem_u32(&bar_free), 0, status)) load_w2(S_STAGES);
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            bool ok = mbar_wait(smem_u32(&bar_u), 0, status);
+            for (int kb = 0; kb < kb2 && ok; ++kb) {
+                ok = mbar_wait(smem_u32(&bar_w[kb]), 0, status);
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t da = smem_desc_sw128(smem_u32(u_s + (size_t)kb * BM * 128));
+                const uint32_t w_addr = smem_u32(w2_s + (size_t)(kb % S_STAGES) * S_STAGE_BYTES);
+                for (int n0 = 0; n0 < EN; n0 += 256) {       // one instruction takes at most 256 columns
+                    const uint64_t db = smem_desc_sw128(w_addr + (uint32_t)n0 * 128);
+                    const uint32_t idesc = instr_desc_bf16(BM, min(EN - n0, 256));
+#pragma unroll
+                    for (int q = 0; q < BK / UMMA_K; ++q) {
+                        const uint64_t koff = (uint64_t)((q * UMMA_K * 2) >> 4);
+                        umma_bf16(tmem_base + (uint32_t)n0, da + koff, db + koff, idesc, (kb | q) != 0 ? 1u : 0u);
+                    }
+                }
+                if (kb == 0) umma_commit(smem_u32(&bar_free));
+            }
+            umma_commit(smem_u32(&bar_acc));
+        }
+    } else {
+        const int quad = warp & 3, part = (warp - 2) >> 2;
+        const int r_local = quad * 32 + lane, row = m0 + r_local;
+        const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
+        const int W = (E + 31) / 32;
+        int okw = 1;
+        if (lane == 0) okw = mbar_wait(smem_u32(&bar_acc), 0, status) ? 1 : 0;
+        const bool ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        auto scores16 = [&](int c0, float (&v)[16]) {
+            uint32_t acc[16];
+            tmem_ld16(tmem_base + lane_base + (uint32_t)c0, acc);
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) {
+                const float4 b = *reinterpret_cast<const float4 *>(b2_s + c0 + j);
+                v[j] = fabsf(__uint_as_float(acc[j]) + b.x);
+                v[j + 1] = fabsf(__uint_as_float(acc[j + 1]) + b.y);
+                v[j + 2] = fabsf(__uint_as_float(acc[j + 2]) + b.z);
+                v[j + 3] = fabsf(__uint_as_float(acc[j + 3]) + b.w);
+            }
+        };
+        uint32_t mb = 0u;                                    // integer maximum of the bit patterns, as above
+        for (int q = 0; q < S_WORDS && ok; ++q) {
+            const int w = part + 4 * q;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c0 = w * 32 + h * 16;
+                if (c0 >= EN) break;
+                float v[16];
+                scores16(c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) mb = max(mb, c0 + j < E ? __float_as_uint(v[j]) : 0u);
+                if (R && row < T) store_scores16(R, row, E, c0, v);
+            }
+        }
+        pmax_s[part * BM + r_local] = mb;
+        asm volatile("bar.sync 1, 512;" ::: "memory");
+        uint32_t mm = pmax_s[r_local];
+#pragma unroll
+        for (int p = 1; p < 4; ++p) mm = max(mm, pmax_s[p * BM + r_local]);
+        const bool bad = mm >= 0x7f800000u;
+        const float thr = bad ? -1.0f : __fmul_rn(tau, __uint_as_float(mm));
+        int kt = 0;
+        for (int q = 0; q < S_WORDS && ok; ++q) {
+            const int w = part + 4 * q;
+            if (w >= W) break;
+            uint32_t word = 0u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c0 = w * 32 + h * 16;
+                if (c0 >= EN) break;
+                float v[16];
+                scores16(c0, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) word |= !(v[j] < thr) ? 1u << (h * 16 + j) : 0u;
+            }
+            if (w * 32 + 32 > E) word &= (1u << (E - w * 32)) - 1u;
+            if (row < T) io.l[0].mask[(size_t)row * W + w] = word;
+            kt += __popc(word);
+        }
+        pk_s[part * BM + r_local] = kt;
+        asm volatile("bar.sync 1, 512;" ::: "memory");
+        if (part == 0) {
+            int k_row = 0;
+            if (row < T) {
+                k_row = pk_s[r_local] + pk_s[BM + r_local] + pk_s[2 * BM + r_local] + pk_s[3 * BM + r_local];
+                io.l[0].k[row] = k_row;
+                if (bad) atomicMax(status, (int32_t)D2D_ERR_NONFINITE);
+            }
+            const bool any = __any_sync(0xffffffffu, bad && row < T);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) k_row += __shfl_xor_sync(0xffffffffu, k_row, o);
+            publish_batch(io.ksum, io.l[0].status, quad, lane, k_row, any || !ok, warp_k, warp_bad);
+        }
+    }
+
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+}
+
+// Launch with programmatic dependent launch; `done` remembers per device that the kernel's shared memory limit is set.
+template <typename K, typename... A>
+d2d_status launch_kernel(K kern, bool (&done)[64], dim3 grid, size_t smem, cudaStream_t st, A... args)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return D2D_ERR_CUDA;
+    if (!__atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return D2D_ERR_CUDA;
+        __atomic_store_n(&done[dev], true, __ATOMIC_RELEASE);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NTHREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, args...);
+    D2D_LAUNCHED(1);
+    return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+}
+
 template <int DH>
 d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T, float tau, int do_mask,
                   const RouterGroupIO &io, cudaStream_t st)
@@ -390,29 +585,10 @@ d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_la
     if (!d2d_tc_make_map(&tx, x, T, D.d, BM) || !d2d_tc_make_map(&tw1, w.w_r1, D.d_h * n_layers, D.d, DH) ||
         !d2d_tc_make_map(&tw2, w.w_r2, D.n_experts * n_layers, D.d_h, 256))
         return D2D_ERR_CUDA;
-    auto kern = router_fused_kernel<DH>;
     static bool attr_set[64] = {};                         // the attribute is per device
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return D2D_ERR_CUDA;
-    if (!__atomic_load_n(&attr_set[dev], __ATOMIC_ACQUIRE)) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM) != cudaSuccess) return D2D_ERR_CUDA;
-        __atomic_store_n(&attr_set[dev], true, __ATOMIC_RELEASE);
-    }
-    const int EN = (D.n_experts + 15) / 16 * 16;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(d2d_cdiv(T, BM), n_layers, 1);
-    cfg.blockDim = dim3(NTHREADS, 1, 1);
-    cfg.dynamicSmemBytes = SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, tx, tw1, tw2, (const __nv_bfloat16 *)w.b_r1, (const __nv_bfloat16 *)w.b_r2,
-                                               T, D.d, D.n_experts, EN, tau, do_mask, io);
-    D2D_LAUNCHED(1);
-    return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+    return launch_kernel(router_fused_kernel<DH>, attr_set, dim3(d2d_cdiv(T, BM), n_layers, 1), SMEM, st, tx, tw1, tw2,
+                         (const __nv_bfloat16 *)w.b_r1, (const __nv_bfloat16 *)w.b_r2, T, D.d, D.n_experts,
+                         (D.n_experts + 15) / 16 * 16, tau, do_mask, io);
 }
 
 }  // namespace
@@ -445,4 +621,31 @@ d2d_status d2d_router_fused_group(const d2d_layer_desc &D, const d2d_router_weig
     io.mask_cat = mask_cat;
     io.cat_words = cat_words;
     return launch<128>(D, w, n_layers, x, T, tau, 1, io, st);
+}
+
+bool d2d_router_scores_supports(const d2d_layer_desc &D, int T)
+{
+    // u's tile and three k-blocks of W_r2 fill the shared memory at d_h = 256 and E = 384
+    return D.dtype == D2D_BF16 && T > d2d_decode_max_tokens(D) && D.d_h <= S_MAX_KB * BK && D.d_h % 8 == 0 && D.n_experts <= S_STAGE_BYTES / 128 &&
+           D.d % 8 == 0 && T <= 16000 * BM && d2d_gemm_tc_available();
+}
+
+d2d_status d2d_router_scores(const d2d_layer *L, const void *x, void *u, int T, float tau, float *R, uint32_t *mask,
+                             int32_t *k, int32_t *status, cudaStream_t st, int32_t *ksum)
+{
+    const d2d_layer_desc &D = L->desc;
+    d2d_gemm_args l1 = {};
+    l1.a = x; l1.b = L->w_r1; l1.bias = L->b_r1; l1.out = u;
+    l1.M = T; l1.N = D.d_h; l1.K = D.d; l1.epilogue = D2D_EPI_RELU_BF16;
+    const d2d_status rc = d2d_gemm_tc(l1, st);
+    if (rc != D2D_OK) return rc;
+    RouterGroupIO io = {};
+    io.l[0] = {R, mask, k, status};
+    io.ksum = ksum;
+    CUtensorMap tu, tw2;
+    if (!d2d_tc_make_map(&tu, u, T, D.d_h, BM) || !d2d_tc_make_map(&tw2, L->w_r2, D.n_experts, D.d_h, 128)) return D2D_ERR_CUDA;
+    static bool attr_set[64] = {};
+    return launch_kernel(router_scores_kernel, attr_set, dim3(d2d_cdiv(T, BM), 1, 1),
+                         (size_t)S_MAX_KB * BM * 128 + (size_t)S_STAGES * S_STAGE_BYTES + 1024, st, tu, tw2, (const __nv_bfloat16 *)L->b_r2, T,
+                         d2d_cdiv(D.d_h, BK), D.n_experts, (D.n_experts + 15) / 16 * 16, tau, io);
 }

@@ -728,3 +728,26 @@ def test_fp32_layer_in_shared_memory_one_or_several_tokens_per_cta(api, T, act, 
         y_ref = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[act], G)
         assert r.status == 0 and _rel_err(y.cpu().numpy(), y_ref) <= TOL_Y["f32"]
     layer.close()
+
+
+# scores and selection in a kernel of their own: hidden widths of one to four k-blocks (whole and ragged), expert counts around
+# one, two and three boxes of 128 rows and 256 columns, ragged last tiles of tokens
+@pytest.mark.parametrize("E,d_h,T", [(257, 128, 65), (344, 256, 129), (384, 200, 256), (272, 72, 1000), (100, 192, 333), (256, 256, 700),
+                                     (128, 40, 127)])
+def test_router_with_separate_hidden_layer(api, E, d_h, T):
+    cfg = wl.LayerConfig("edge", "bf16", d=256, d_ff=E * 16, E=E, d_h=d_h, act="gelu_erf", T=T, token_sigma=0.5, b1_shift=-0.3, seed=37)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    x[T // 2, 3] = np.inf                                      # one token with scores that are not finite keeps every expert
+    layer = api.Layer.from_config(cfg, w)
+    good = np.arange(T) != T // 2
+    for tau in (0.6, 0.0):
+        R = _poison(torch.empty((T, E), dtype=torch.float32, device="cuda"))
+        _, r = layer.layer_fwd(api.to_device(x, cfg.dtype), tau, R_out=R, routing=layer.new_routing(T, dual=True))
+        torch.cuda.synchronize()
+        assert r.status == 5                                   # D2D_ERR_NONFINITE
+        R = R.cpu().numpy()
+        assert _rel_err(R[good], oracle.router(x[good], w["w_r1"], w["b_r1"], w["w_r2"], w["b_r2"])) <= TOL_R["bf16"]
+        G = oracle.unpack_mask(r.mask_u32(), E)
+        assert np.array_equal(G[good], oracle.select(R[good], tau)[0]) and G[T // 2].all()
+        assert np.array_equal(r.counts.cpu().numpy(), oracle.metadata(G)["counts"]) and np.array_equal(r.k.cpu().numpy(), G.sum(1))
+    layer.close()
