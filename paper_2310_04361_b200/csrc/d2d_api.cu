@@ -60,8 +60,10 @@ ws_layout layout_for(const d2d_layer *L, int T)
 
 }  // namespace
 
-// Up to this many tokens a bf16 layer takes the decode kernels.  Measured (us per layer call, decode kernels /
-// tensor-core path): GPT-2-medium-shaped FFN (64 KB of weights per expert) T = 3: 31 / 39, T = 4: 33 / 39, T = 5:
+// Up to this many tokens a bf16 layer takes CUDA-core arithmetic (the streaming decode kernels then carry float32 hidden
+// activations as three bf16 terms, so that results are as precise as those of small_batch_ffn.cu), above it tensor-core
+// arithmetic with bf16 hidden activations.  Measured with small_batch_ffn.cu, which still serves the shapes the streaming
+// kernels do not take (us per layer call, decode kernels / tensor-core path): GPT-2-medium-shaped FFN (64 KB of weights per expert) T = 3: 31 / 39, T = 4: 33 / 39, T = 5:
 // 41 / 40, T = 8: 43 / 39; Llama-shaped layer (786 KB per expert) T = 1: 84 / 129, T = 2: 108 / 133, T = 3: 221 / 133,
 // T = 4: 229 / 127.  So 4 tokens for small experts, 2 for large ones; D2D_DECODE_MAX_TOKENS overrides both.
 int d2d_decode_max_tokens(const d2d_layer_desc &D)
@@ -82,7 +84,6 @@ static bool use_dense_masked(const d2d_layer *L, int T)
 }
 
 // Up to this many tokens the expert-per-CTA kernel (each kept expert's slice read once) is used.
-
 static bool use_small_ffn(const d2d_layer *L, int T)
 {
     const int lim = L->desc.dtype == D2D_BF16 ? d2d_decode_max_tokens(L->desc) : 8;      // fp32 layers have no tensor-core path
