@@ -254,6 +254,9 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     } else if (path == D2D_PATH_FUSED) {
         return D2D_ERR_UNSUPPORTED;
     }
+    // decode-sized batches: split K of the down projection over the SMs, partial sums in the float32 scratch behind H
+    const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff);
+    float *partial = k_splits > 1 ? (float *)((char *)ws + d2d_align_up((size_t)T * D.d_ff * 2, 256)) : nullptr;
     if (path != D2D_PATH_GATHER) {
         d2d_gemm_args up = {};
         const bool forced = path == D2D_PATH_DENSE;
@@ -263,6 +266,7 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
         up.a = x; up.b = L->w1; up.b_gate = D.gated ? L->w_gate : nullptr; up.b_cat = L->w1g; up.b_cat_block = 128; up.bias = L->b1; up.out = ws;
         up.M = T; up.N = D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
         up.mask = r->mask; up.mask_words = (D.n_experts + 31) / 32; up.expert_size = D.expert_size; up.status = r->status;
+        if (forced && k_splits > 1) { up.zero = partial; up.zero_floats = (long long)T * D.d; }
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
     }
@@ -301,9 +305,9 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     dn.n_sel = path == D2D_PATH_AUTO && (!zero_fill || n_sel_fused >= 0) ? n_sel : nullptr;
     dn.n_sel_max = zero_fill ? n_sel_fused : n_sel_max;
     dn.M = T; dn.N = D.d; dn.K = D.d_ff; dn.epilogue = D2D_EPI_BIAS_BF16; dn.status = r->status;
-    // decode-sized batches: split K over the SMs, partial sums in the float32 scratch behind H
-    dn.k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff);
-    dn.partial = dn.k_splits > 1 ? (float *)((char *)ws + d2d_align_up((size_t)T * D.d_ff * 2, 256)) : nullptr;
+    dn.k_splits = k_splits;
+    dn.partial = partial;
+    dn.partial_zero = path == D2D_PATH_DENSE;
     return d2d_gemm_tc(dn, st);
 }
 

@@ -39,6 +39,8 @@ struct EpiParams {
     int batch;                       // >= 1 problems of one shape: A columns, B rows, bias entries and out advance per problem
     const int32_t *n_sel;            // density-adaptive dispatch: do nothing when *n_sel <= n_sel_max (NULL: always run)
     long long n_sel_max;
+    float4 *zero;                    // optional: cleared by the epilogue warps before their first tile (see d2d_gemm_args)
+    int zero_n;                      // 16-byte pieces
     int test_skip_load;              // test aid: CTA 0 never requests the A tile of its first k-block (see d2d_gemm_args)
 };
 
@@ -404,6 +406,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             else mbar_arrive(smem_u32(&bar_acc_empty[b]));
         };
         uint32_t out_n = 0;                                 // output buffers used so far
+        for (int i = (int)blockIdx.x * (N_EPI_WARPS * 32) + (int)threadIdx.x - 64; i < ep.zero_n; i += (int)gridDim.x * (N_EPI_WARPS * 32))
+            ep.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         for (uint32_t local = 0;; ++local) {
             const uint32_t buf = local & 1u, use = local >> 1;
             // ONE thread takes the item from the ring, works out its coordinates (integer divisions), waits for the accumulator
@@ -672,7 +676,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
     EpiParams ep{(const __nv_bfloat16 *)g.bias, g.out, g.mask, g.mask_words, es, g.status,
                  (uint32_t)((0x100000000ull + (unsigned long long)es - 1) / (unsigned long long)es),
                  g.tile_counter, (g.pdl_late_wait && !g.n_sel && d2d_tc_pdl_enabled()) ? 1 : 0, gate_cat ? 1 : 0,
-                 band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max,
+                 band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max, (float4 *)g.zero, g.zero ? (int)(g.zero_floats / 4) : 0,
                  (g.test_skip_load && !g.tile_counter && !g.pdl_late_wait && !g.n_sel) ? 1 : 0};
     const int k_splits = g.k_splits > 1 ? g.k_splits : 1;
     const int tiles = d2d_cdiv(g.N, BN) * d2d_cdiv(g.M, TM) * k_splits * batch;
@@ -767,6 +771,8 @@ __global__ void __launch_bounds__(256)
 splitk_finalize_kernel(const float *__restrict__ partial, const __nv_bfloat16 *__restrict__ bias, __nv_bfloat16 *__restrict__ out,
                        int M, int N, int batch)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t per = (size_t)M * N, total = per * batch;
     for (size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4; i < total; i += (size_t)gridDim.x * 1024) {
         const float4 v = __ldcg(reinterpret_cast<const float4 *>(partial + i));
@@ -868,7 +874,7 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
     case D2D_EPI_BIAS_BF16:
         if (g.k_splits > 1 && g.partial) {
             const int batch = g.batch > 1 ? g.batch : 1;
-            if (cudaMemsetAsync(g.partial, 0, (size_t)batch * g.M * g.N * sizeof(float), st) != cudaSuccess) return D2D_ERR_CUDA;
+            if (!g.partial_zero && cudaMemsetAsync(g.partial, 0, (size_t)batch * g.M * g.N * sizeof(float), st) != cudaSuccess) return D2D_ERR_CUDA;
             d2d_gemm_args p = g;
             p.epilogue = D2D_EPI_PARTIAL_F32;
             p.bias = nullptr;
@@ -876,10 +882,19 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
             const d2d_status rc = launch<64, D2D_EPI_PARTIAL_F32, 0, false>(p, st);
             if (rc != D2D_OK) return rc;
             const int blocks = d2d_cdiv(batch * g.M * g.N, 1024);
-            splitk_finalize_kernel<<<blocks < 148 ? blocks : 148, 256, 0, st>>>(g.partial, (const __nv_bfloat16 *)g.bias,
-                                                                                 (__nv_bfloat16 *)g.out, g.M, g.N, batch);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(blocks < 148 ? blocks : 148, 1, 1);
+            cfg.blockDim = dim3(256, 1, 1);
+            cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+            const cudaError_t err = cudaLaunchKernelEx(&cfg, splitk_finalize_kernel, (const float *)g.partial, (const __nv_bfloat16 *)g.bias,
+                                                       (__nv_bfloat16 *)g.out, g.M, g.N, batch);
             D2D_LAUNCHED(1);
-            return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+            return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
         }
         return launch_bn<D2D_EPI_BIAS_BF16, 0, false>(g, st);
     case D2D_EPI_UP_MASKED: return g.b_gate ? launch_up<true>(g, st) : launch_up<false>(g, st);

@@ -228,13 +228,17 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         up.a = x; up.b = g->w1; up.bias = g->b1; up.out = H;
         up.M = T; up.N = n * D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
         up.mask = mask_cat; up.mask_words = n * W; up.expert_size = D.expert_size; up.status = routing[0].status;
+        const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff, n);
+        float *partial = k_splits > 1 ? (float *)(base + w.partial_off) : nullptr;
+        up.zero = partial; up.zero_floats = (long long)n * T * D.d;
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
         d2d_gemm_args dn = {};
         dn.a = H; dn.b = g->w2; dn.bias = g->b2; dn.out = y;
         dn.M = T; dn.N = D.d; dn.K = D.d_ff; dn.batch = n; dn.epilogue = D2D_EPI_BIAS_BF16; dn.status = routing[0].status;
-        dn.k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff, n);
-        dn.partial = dn.k_splits > 1 ? (float *)(base + w.partial_off) : nullptr;
+        dn.k_splits = k_splits;
+        dn.partial = partial;
+        dn.partial_zero = 1;
         rc = d2d_gemm_tc(dn, st);
         if (cudaEventRecord(g->ev_join, g->side_stream) != cudaSuccess || cudaStreamWaitEvent(st, g->ev_join, 0) != cudaSuccess)
             return D2D_ERR_CUDA;
