@@ -105,6 +105,7 @@ size_t d2d_select_ws_bytes(int T, int E);
 // R == nullptr: the mask is an input.  mask_ready != 0: mask, k and the status word were already written
 // (fused router), only the per-expert metadata is built.
 d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d2d_routing *out, int32_t *ksum, cudaStream_t st);
+d2d_status d2d_launch_lists(const d2d_routing *r, int n, int T, int E, void *ws, size_t ws_each, cudaStream_t st);
 d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, const d2d_routing *out,
                              void *ws, cudaStream_t st, int mask_ready = 0, unsigned int *zero_ticket = nullptr);
 
@@ -141,7 +142,7 @@ d2d_status d2d_router_fused(const d2d_layer *L, const void *x, int T, float tau,
 bool d2d_router_scores_supports(const d2d_layer_desc &D, int T);
 d2d_status d2d_router_scores(const d2d_layer *L, const void *x, void *u, int T, float tau, float *R, uint32_t *mask,
                              int32_t *k, int32_t *status, cudaStream_t st, int32_t *ksum);
-d2d_status d2d_router_fused_group(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T,
+d2d_status d2d_router_fused_group(const d2d_layer *const *layers, int n_layers, const d2d_router_weights &w, const void *x, int T,
                                   float tau, const d2d_routing *routing, uint32_t *mask_cat, int cat_words, cudaStream_t st);
 d2d_status d2d_small_group_fwd(const d2d_layer *const *layers, int n, const void *x, int T, float tau, const d2d_routing *routing,
                                float *const *R, float *const *u, float *const *y32, void *y, cudaStream_t st);

@@ -208,19 +208,15 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
     // ---- merged tensor-core path
     if (g->merged && d2d_router_fused_supports(D, T)) {
         const int W = E / 32;
-        for (int l = 0; l < n; ++l)
-            if (cudaMemsetAsync(routing[l].status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
         uint32_t *mask_cat = (uint32_t *)(base + w.mask_off);
         const d2d_router_weights rw = {g->w_r1, g->b_r1, g->w_r2, g->b_r2};
-        d2d_status rc = d2d_router_fused_group(D, rw, n, x, T, tau, routing, mask_cat, n * W, st);
+        d2d_status rc = d2d_router_fused_group(g->layers, n, rw, x, T, tau, routing, mask_cat, n * W, st);
         if (rc != D2D_OK) return rc;
         // per-expert metadata of every layer on the side stream, beside the GEMMs (which read only the merged mask)
         if (cudaEventRecord(g->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(g->side_stream, g->ev_fork, 0) != cudaSuccess)
             return D2D_ERR_CUDA;
-        for (int l = 0; l < n; ++l) {
-            rc = d2d_launch_select(nullptr, T, E, tau, 0, &routing[l], base + w.sel_off + (size_t)l * w.sel_each, g->side_stream, 1);
-            if (rc != D2D_OK) return rc;
-        }
+        rc = d2d_launch_lists(routing, n, T, E, base + w.sel_off, w.sel_each, g->side_stream);
+        if (rc != D2D_OK) return rc;
         void *H = base + w.h_off;
         d2d_gemm_args up = {};
         up.tile_counter = g->up_counter;

@@ -45,7 +45,7 @@ struct RouterGroupIO {
     RouterLayerIO l[D2D_MAX_GROUP];
     uint32_t *mask_cat;    // merged mask [T, cat_words] or NULL
     int cat_words;
-    int32_t *ksum;         // single layer only, or NULL: [0..1] running sum of k and exit count (64 bits), [2] largest condition
+    int32_t *ksum[D2D_MAX_GROUP];      // all or none NULL, per layer: [0..1] running sum of k and exit count (64 bits), [2] largest condition
                            // (all zero at launch and left at zero), [4] receives the total = number of selected (token,
                            // expert) pairs; the last CTA then writes *status
 };
@@ -65,7 +65,7 @@ __device__ __forceinline__ void publish_batch(int32_t *ksum, int32_t *status_out
                                    (cond ? 1ull << 50 : 0ull);
     unsigned long long *acc64 = reinterpret_cast<unsigned long long *>(ksum);
     const unsigned long long tot = atomicAdd(acc64, add) + add;
-    if (((tot >> 36) & 0x3fffu) != (unsigned long long)(gridDim.x * gridDim.y)) return;
+    if (((tot >> 36) & 0x3fffu) != (unsigned long long)gridDim.x) return;
     *acc64 = 0ull;
     ksum[4] = (int32_t)(tot & 0xfffffffffull);
     int32_t st = 0;
@@ -120,7 +120,8 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     uint32_t *__restrict__ mask = io.l[layer].mask;
     int32_t *__restrict__ k = io.l[layer].k;
     // conditions are collected in a word of the layer and published once (no memset in front of the kernel)
-    int32_t *__restrict__ status = io.ksum ? io.ksum + 2 : io.l[layer].status;
+    int32_t *const ksum = io.ksum[layer];
+    int32_t *__restrict__ status = ksum ? ksum + 2 : io.l[layer].status;
     constexpr int KB2 = DH / BK;                          // k-blocks of the second GEMM
     constexpr int A_BYTES = BM * BK * 2, B1_BYTES = DH * BK * 2;
     constexpr int STAGE_BYTES = A_BYTES + B1_BYTES;
@@ -245,7 +246,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         const int r_local = quad * 32 + lane;
         const int row = m0 + r_local;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
-        auto publish = [&](int k_warp, bool cond_warp) { publish_batch(io.ksum, io.l[layer].status, quad, lane, k_warp, cond_warp, warp_k, warp_bad); };
+        auto publish = [&](int k_warp, bool cond_warp) { publish_batch(ksum, io.l[layer].status, quad, lane, k_warp, cond_warp, warp_k, warp_bad); };
         int okw = 1;
         if (lane == 0) okw = mbar_wait(smem_u32(&bar_acc1), 0, status) ? 1 : 0;
         bool ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
@@ -360,7 +361,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                         k[row] = k_row;
                         if (bad) atomicMax(status, (int32_t)D2D_ERR_NONFINITE);
                     }
-                    if (io.ksum) {
+                    if (ksum) {
                         const bool any = __any_sync(0xffffffffu, bad && row < T);
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) k_row += __shfl_xor_sync(0xffffffffu, k_row, o);
@@ -372,7 +373,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             // keep the named barrier balanced when a bounded wait ran out
             asm volatile("bar.sync 1, 512;" ::: "memory");
             asm volatile("bar.sync 1, 512;" ::: "memory");
-            if (io.ksum && part == 0) publish(0, true);
+            if (ksum && part == 0) publish(0, true);
         }
     }
 
@@ -398,7 +399,7 @@ router_scores_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_cons
                      const __grid_constant__ RouterGroupIO io)
 {
     float *__restrict__ R = io.l[0].R;
-    int32_t *__restrict__ status = io.ksum + 2;
+    int32_t *__restrict__ status = io.ksum[0] + 2;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *u_s = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *w2_s = u_s + (size_t)S_MAX_KB * BM * 128;
@@ -539,7 +540,7 @@ router_scores_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_cons
             const bool any = __any_sync(0xffffffffu, bad && row < T);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) k_row += __shfl_xor_sync(0xffffffffu, k_row, o);
-            publish_batch(io.ksum, io.l[0].status, quad, lane, k_row, any || !ok, warp_k, warp_bad);
+            publish_batch(io.ksum[0], io.l[0].status, quad, lane, k_row, any || !ok, warp_k, warp_bad);
         }
     }
 
@@ -606,21 +607,24 @@ d2d_status d2d_router_fused(const d2d_layer *L, const void *x, int T, float tau,
 {
     RouterGroupIO io = {};
     io.l[0] = {R, mask, k, status};
-    io.ksum = do_mask ? ksum : nullptr;
+    io.ksum[0] = do_mask ? ksum : nullptr;
     const d2d_router_weights w = {L->w_r1, L->b_r1, L->w_r2, L->b_r2};
     return launch<128>(L->desc, w, 1, x, T, tau, do_mask, io, st);
 }
 
 // n routers of one shape with stacked weights, one grid; routing[l] receives mask, k and status of router l.
-d2d_status d2d_router_fused_group(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T,
+d2d_status d2d_router_fused_group(const d2d_layer *const *layers, int n_layers, const d2d_router_weights &w, const void *x, int T,
                                   float tau, const d2d_routing *routing, uint32_t *mask_cat, int cat_words, cudaStream_t st)
 {
     if (n_layers < 1 || n_layers > D2D_MAX_GROUP) return D2D_ERR_INVALID_ARG;
     RouterGroupIO io = {};
-    for (int l = 0; l < n_layers; ++l) io.l[l] = {nullptr, routing[l].mask, routing[l].k, routing[l].status};
+    for (int l = 0; l < n_layers; ++l) {
+        io.l[l] = {nullptr, routing[l].mask, routing[l].k, routing[l].status};
+        io.ksum[l] = (int32_t *)(layers[l]->tickets + 40);
+    }
     io.mask_cat = mask_cat;
     io.cat_words = cat_words;
-    return launch<128>(D, w, n_layers, x, T, tau, 1, io, st);
+    return launch<128>(layers[0]->desc, w, n_layers, x, T, tau, 1, io, st);
 }
 
 bool d2d_router_scores_supports(const d2d_layer_desc &D, int T)
@@ -641,7 +645,7 @@ d2d_status d2d_router_scores(const d2d_layer *L, const void *x, void *u, int T, 
     if (rc != D2D_OK) return rc;
     RouterGroupIO io = {};
     io.l[0] = {R, mask, k, status};
-    io.ksum = ksum;
+    io.ksum[0] = ksum;
     CUtensorMap tu, tw2;
     if (!d2d_tc_make_map(&tu, u, T, D.d_h, BM) || !d2d_tc_make_map(&tw2, L->w_r2, D.n_experts, D.d_h, 128)) return D2D_ERR_CUDA;
     static bool attr_set[64] = {};

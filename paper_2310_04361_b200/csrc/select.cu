@@ -185,6 +185,98 @@ __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, i
     return res;
 }
 
+// Lists of a batch small enough for every CTA to look at all of the mask: one CTA per mask word (32 experts) and layer, no
+// order between CTAs, so counts, offsets and lists take one launch and no scratch.  A CTA adds up the pairs of the words
+// before its own (what its first list starts at), counts its 32 experts per warp (a warp has a contiguous range of 32-token
+// groups), scans, and writes.  k != NULL: k and the status word are wanted too.  Bound by latency; as small as
+// bucket_count_scan_kernel, for the same reason.  What it saves is the host's time (two launches, a memset and, for a mask that
+// is given, two more): see d2d_launch_select for the line.
+struct ListsIO {
+    const uint32_t *mask;
+    int32_t *k, *counts, *offsets, *perm, *n_sel, *status;
+    long long capacity;
+};
+struct ListsGroup { ListsIO l[D2D_MAX_GROUP]; };
+constexpr int LISTS_GROUPS = 4, LISTS_MAX_T = LISTS_GROUPS * TOKB;      // 32-token groups of a warp, held in registers
+
+__global__ void __launch_bounds__(TOKB, 6)
+lists_kernel(const __grid_constant__ ListsGroup g, int T, int E, int W)
+{
+    constexpr int NWARP = TOKB / 32;
+    __shared__ uint16_t cnt[NWARP][32];
+    __shared__ int sums[NWARP];
+    const ListsIO &io = g.l[blockIdx.y];
+    const uint32_t *__restrict__ mask = io.mask;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x;
+    int before = 0;
+    for (int t = threadIdx.x; t < T; t += TOKB) {
+        const uint32_t *row = mask + (size_t)t * W;
+        int n = 0;
+        for (int i = 0; i < w; ++i) n += __popc(__ldg(row + i));
+        before += n;
+        if (io.k && w == W - 1) io.k[t] = n + __popc(__ldg(row + w));
+    }
+    before = __reduce_add_sync(FULL, before);
+    const int per = (T + TOKB - 1) / TOKB * 32;                 // tokens of a warp
+    const int t0 = warp * per, e = w * 32 + lane;
+    uint32_t col[LISTS_GROUPS];                                 // per group of 32 tokens: which of them keep expert e
+#pragma unroll
+    for (int i = 0; i < LISTS_GROUPS; ++i) {
+        const int t = t0 + i * 32 + lane;
+        col[i] = i * 32 < per && t < T ? __ldg(mask + (size_t)t * W + w) : 0u;
+    }
+    int mine = 0;
+#pragma unroll
+    for (int i = 0; i < LISTS_GROUPS; ++i) {
+        col[i] = transpose_bits(col[i], lane);
+        if (e >= E) col[i] = 0u;
+        mine += __popc(col[i]);
+    }
+    cnt[warp][lane] = (uint16_t)mine;
+    if (lane == 0) sums[warp] = before;
+    __syncthreads();
+    int total = 0, earlier = 0;
+    before = 0;
+#pragma unroll
+    for (int i = 0; i < NWARP; ++i) {
+        const int c = cnt[i][lane];
+        if (i < warp) earlier += c;
+        total += c;
+        before += sums[i];
+    }
+    int inc = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += v;
+    }
+    const int first = before + inc - total;
+    if (warp == 0 && e < E) {
+        io.counts[e] = total;
+        io.offsets[e] = first;
+        if (e == E - 1) {
+            const int all = first + total;
+            io.offsets[E] = all;
+            *io.n_sel = all;
+            const int over = (long long)all > io.capacity ? (int)D2D_ERR_CAPACITY : 0;
+            if (io.k) *io.status = over;
+            else if (over) atomicMax(io.status, over);
+        }
+    }
+    int pos = first + earlier;
+#pragma unroll
+    for (int i = 0; i < LISTS_GROUPS; ++i) {
+        if (i * 32 >= per) break;
+#pragma unroll 4
+        for (int j = 0; j < 32; ++j) {
+            const uint32_t b = __shfl_sync(FULL, col[i], j);
+            const int at = __shfl_sync(FULL, pos, j) + __popc(b & ((1u << lane) - 1u));
+            if (((b >> lane) & 1u) && at < io.capacity) io.perm[at] = t0 + i * 32 + lane;
+        }
+        pos += __popc(col[i]);
+    }
+}
+
 // Per-expert token counts of each 256-token block (8 warps x 32 tokens; a warp turns its
 // 32 x 32 bit tile into per-expert bitmaps with 32 ballots).  The CTA that finishes last (ticket
 // counter) then scans: per expert the exclusive prefix over the blocks, and over the experts the
@@ -401,6 +493,48 @@ size_t d2d_select_ws_bytes(int T, int E)
     return 256 + d2d_align_up(nblk * (size_t)E * sizeof(int32_t), 256);
 }
 
+// One launch for the lists of batches whose time is the host's.  A CTA's work grows with the whole mask: up to 1024 tokens
+// where nothing runs beside it, up to 512 beside the experts, whose persistent CTAs it competes with for issue slots in longer
+// batches (at 1749 tokens it took the BERT-shaped layer from 41 to 57 us, at 1000 the Llama-shaped one from 231 to 244).
+static bool lists_in_one_launch(int T, int E, bool alone)
+{
+    return T <= (alone ? LISTS_MAX_T : LISTS_MAX_T / 2) && (long long)T * ((E + 31) / 32) <= 16384;
+}
+
+static void launch_lists(const d2d_routing *r, int n, int T, int E, bool with_k, cudaStream_t st)
+{
+    ListsGroup g = {};
+    for (int l = 0; l < n; ++l)
+        g.l[l] = {r[l].mask, with_k ? r[l].k : nullptr, r[l].counts, r[l].offsets, r[l].perm, r[l].n_sel, r[l].status,
+                  (long long)r[l].perm_capacity};
+    lists_kernel<<<dim3((E + 31) / 32, n), TOKB, 0, st>>>(g, T, E, (E + 31) / 32);
+    D2D_LAUNCHED(1);
+}
+
+// Token-major dual, where the caller wants it
+static void launch_dual(const d2d_routing *out, int T, int W, cudaStream_t st)
+{
+    if (!out->tok_off || !out->tok_exp) return;
+    D2D_LAUNCHED(2);
+    tok_scan_kernel<<<1, 1024, 0, st>>>(out->k, T, out->tok_off);
+    tok_fill_kernel<<<d2d_cdiv(T, 8), 256, 0, st>>>(out->mask, T, W, out->tok_off, out->tok_exp, (long long)out->perm_capacity);
+}
+
+// Lists of n layers of one shape whose masks, k and status words are there.  ws: n workspaces of ws_each bytes
+d2d_status d2d_launch_lists(const d2d_routing *r, int n, int T, int E, void *ws, size_t ws_each, cudaStream_t st)
+{
+    if (lists_in_one_launch(T, E, false)) {
+        launch_lists(r, n, T, E, false, st);
+        for (int l = 0; l < n; ++l) launch_dual(&r[l], T, (E + 31) / 32, st);
+        return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+    }
+    for (int l = 0; l < n; ++l) {
+        const d2d_status rc = d2d_launch_select(nullptr, T, E, 0.0f, 0, &r[l], (char *)ws + (size_t)l * ws_each, st, 1);
+        if (rc != D2D_OK) return rc;
+    }
+    return D2D_OK;
+}
+
 // Mask, k and status only (Eq. 4), T > 0; the sum of k is published through ksum (see the kernel).  The per-expert
 // lists can be built afterwards, on any stream ordered behind this one, with d2d_launch_select(nullptr, ..., mask_ready = 1).
 d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d2d_routing *out, int32_t *ksum, cudaStream_t st)
@@ -414,7 +548,10 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
                              void *ws, cudaStream_t st, int mask_ready, unsigned int *zero_ticket)
 {
     const int W = (E + 31) / 32;
-    if (!mask_ready) D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
+    // a mask that is given, lists in one launch: that kernel writes k and the status word as well
+    const bool one = T > 0 && lists_in_one_launch(T, E, !mask_ready), given = !R && !mask_ready;
+    const bool small = topk == 0 && d2d_small_select_supports(T, E);
+    if (!mask_ready && !(given && one && !small)) D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
     if (T == 0) {
         D2D_CUDA_TRY(cudaMemsetAsync(out->counts, 0, sizeof(int32_t) * (size_t)E, st));
         D2D_CUDA_TRY(cudaMemsetAsync(out->offsets, 0, sizeof(int32_t) * (size_t)(E + 1), st));
@@ -422,7 +559,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         if (out->tok_off) D2D_CUDA_TRY(cudaMemsetAsync(out->tok_off, 0, sizeof(int32_t), st));
         return D2D_OK;
     }
-    if (topk == 0 && d2d_small_select_supports(T, E)) return d2d_small_select(R, T, E, tau, out, st, mask_ready);
+    if (small) return d2d_small_select(R, T, E, tau, out, st, mask_ready);
     const int warps_per_cta = 8;
     const int grid_tok = d2d_cdiv(T, warps_per_cta);
     if (R) {
@@ -430,8 +567,14 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
             topk_mask_kernel<<<grid_tok, 256, 0, st>>>(R, T, E, W, topk, out->mask, out->k, out->status);
         else
             dynk_mask_kernel<<<grid_tok, 256, 0, st>>>(R, T, E, W, tau, out->mask, out->k, out->status, nullptr);
-    } else if (!mask_ready) {
+    } else if (given && !one) {
         k_from_mask_kernel<<<d2d_cdiv(T, 256), 256, 0, st>>>(out->mask, T, W, out->k);
+    }
+    if (one) {
+        D2D_LAUNCHED(R ? 1 : 0);
+        launch_lists(out, 1, T, E, given, st);
+        launch_dual(out, T, W, st);
+        return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
     }
     const int nblk = d2d_cdiv(T, TOKB);
     // the ticket must start at zero (the kernel leaves it there): a word the caller keeps, or cleared on every call
@@ -444,12 +587,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
     bucket_fill_kernel<<<dim3(nblk, W), TOKB, 0, st>>>(out->mask, T, E, W, blockcounts, out->offsets, out->perm,
                                               (long long)out->perm_capacity);
     D2D_LAUNCHED(mask_ready ? 2 : 3);
-    if (out->tok_off && out->tok_exp) {
-        D2D_LAUNCHED(2);
-        tok_scan_kernel<<<1, 1024, 0, st>>>(out->k, T, out->tok_off);
-        tok_fill_kernel<<<grid_tok, 256, 0, st>>>(out->mask, T, W, out->tok_off, out->tok_exp,
-                                                  (long long)out->perm_capacity);
-    }
+    launch_dual(out, T, W, st);
     return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 

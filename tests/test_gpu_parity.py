@@ -751,3 +751,15 @@ def test_router_with_separate_hidden_layer(api, E, d_h, T):
         assert np.array_equal(G[good], oracle.select(R[good], tau)[0]) and G[T // 2].all()
         assert np.array_equal(r.counts.cpu().numpy(), oracle.metadata(G)["counts"]) and np.array_equal(r.k.cpu().numpy(), G.sum(1))
     layer.close()
+
+
+# lists in one launch: one warp group and the limits of 256-token ranges, around 1024 tokens and 16384 mask words; ragged last words
+@pytest.mark.parametrize("T,E", [(65, 33), (256, 1), (257, 128), (700, 500), (1024, 512), (1023, 24), (1025, 24), (400, 1056)])
+def test_lists_from_a_given_mask(api, T, E):
+    G = (np.random.default_rng(T).random((T, E)) < 0.3).astype(np.uint8)
+    G[T // 3] = 0
+    words = torch.from_numpy(oracle.pack_mask(G).view(np.int32)).cuda()
+    for dual in (True, False):
+        r = api.routing_from_mask(words, E, dual=dual)
+        _check_routing(r, G, dual=dual)
+        assert np.array_equal(r.k.cpu().numpy(), G.sum(1))
