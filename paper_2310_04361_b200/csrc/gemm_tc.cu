@@ -708,8 +708,11 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
 // (BERT-shaped layer with pairs in both projections / in the down projection / none: 55.6 / 51.7 / 52.4 us; ViT-shaped
 // 252 / 248.5 / 249; Llama-shaped down projection 506-533 us with pairs, 550 without).
 struct tile_choice { int bn; bool pair; };
-tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok)
+tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok, bool gated)
 {
+    // A ragged last column tile takes the epilogue's generic loop, about 15 us that nothing hides in short problems (N = 8192,
+    // 300 tokens: 34 us with 192-column tiles against 18 us with 256-column ones).  Gated tiles always have 128 columns.
+    const auto ragged = [&](int bn) { return !gated && N % bn ? 15.0 / d2d_cdiv(K, BK) : 0.0; };
     const int sms = d2d_tc_sm_count();
     const int bns[4] = {256, 192, 128, 64};
     const double t1[4] = {0.457, 0.40, 0.345, 0.28}, t2[3] = {0.42, 0.345, 0.29};
@@ -717,14 +720,14 @@ tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok)
     double best_cost = 1e300;
     for (int i = 0; i < 4; ++i) {
         const long tiles = (long)d2d_cdiv(N, bns[i]) * d2d_cdiv(M, BM) * batch;
-        const double cost = (double)((tiles + sms - 1) / sms) * t1[i];
+        const double cost = (double)((tiles + sms - 1) / sms) * t1[i] + ragged(bns[i]);
         if (cost < best_cost - 1e-9) { best_cost = cost; best = {bns[i], false}; }
     }
     if (!pairs_ok || M <= BM || K < 2048) return best;
     const int pairs = sms / 2;
     for (int i = 0; i < 3; ++i) {
         const long tiles = (long)d2d_cdiv(N, bns[i]) * d2d_cdiv(M, 2 * BM) * batch;
-        const double cost = (double)((tiles + pairs - 1) / pairs) * t2[i];
+        const double cost = (double)((tiles + pairs - 1) / pairs) * t2[i] + ragged(bns[i]);
         if (cost < best_cost - 1e-9) { best_cost = cost; best = {bns[i], true}; }
     }
     return best;
@@ -738,7 +741,7 @@ d2d_status launch_bn(const d2d_gemm_args &g, cudaStream_t st)
         if (pairs_ok && g.M > BM) return launch<128, EPI, ACT, GATED, true>(g, st);
         return launch<128, EPI, ACT, GATED>(g, st);
     }
-    const tile_choice c = pick_tile(g.M, g.N, g.K, g.batch > 1 ? g.batch : 1, pairs_ok);
+    const tile_choice c = pick_tile(g.M, g.N, g.K, g.batch > 1 ? g.batch : 1, pairs_ok, GATED);
     if (c.pair) {
         if (c.bn == 256) return launch<GATED ? 128 : 256, EPI, ACT, GATED, EPI != D2D_EPI_ABS_F32>(g, st);
         if (c.bn == 192) return launch<GATED ? 128 : 192, EPI, ACT, GATED, EPI != D2D_EPI_ABS_F32>(g, st);
