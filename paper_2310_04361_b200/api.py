@@ -125,41 +125,52 @@ def torch_dtype(name: str):
     return torch.float32 if name == "f32" else torch.bfloat16
 
 
+_routing_plans = {}
+
+
+def _routing_plan(T: int, E: int, cap: int, dual: bool, lists: bool):
+    """Layout of a Routing's slab, each buffer on a 256-byte boundary (mask: raw uint32 words kept in an int32 tensor;
+    scalars: n_sel, status): (size, stride, offset) of every tensor, words in all, byte offsets in the order of
+    RoutingStruct's pointers."""
+    W = (E + 31) // 32
+    shapes = {"mask": (max(T, 1), W), "k": (max(T, 1),), "scalars": (2,)}
+    if lists:
+        shapes.update(counts=(E,), offsets=(E + 1,), perm=(max(cap, 1),))
+        if dual:
+            shapes.update(tok_off=(T + 1,), tok_exp=(max(cap, 1),))
+    views, n = {}, 0
+    for name, shape in shapes.items():
+        views[name] = (shape, (W, 1) if len(shape) > 1 else (1,), n)
+        n += (shape[0] * (W if len(shape) > 1 else 1) + 63) // 64 * 64
+    at = {name: 4 * v[2] for name, v in views.items()}
+    return views, n, [at["mask"], at["k"], at.get("counts"), at.get("offsets"), at.get("perm"), at.get("tok_off"), at.get("tok_exp"),
+                      at["scalars"] if lists else None, at["scalars"] + 4]
+
+
 class Routing:
     """Caller-owned device buffers for the routing of one batch (d2d_routing)."""
 
     def __init__(self, T: int, E: int, device, dual: bool = False, perm_capacity: int | None = None, lists: bool = True):
         """lists=False leaves out the per-expert lists (counts, offsets, perm, n_sel): d2d_layer_fwd then does not build them."""
-        W = (E + 31) // 32
         cap = T * E if perm_capacity is None else int(perm_capacity)
-        self.T, self.E, self.W, self.lists = T, E, W, lists
-        # One zeroed allocation for all buffers, each on a 256-byte boundary; the tensors over it are made when asked for
-        # (mask: raw uint32 words kept in an int32 tensor; scalars: n_sel, status).
-        shapes = {"mask": (max(T, 1), W), "k": (max(T, 1),), "scalars": (2,)}
-        if lists:
-            shapes.update(counts=(E,), offsets=(E + 1,), perm=(max(cap, 1),))
-            if dual:
-                shapes.update(tok_off=(T + 1,), tok_exp=(max(cap, 1),))
-        at, n = {}, 0
-        for name, shape in shapes.items():
-            at[name] = n
-            n += (shape[0] * (shape[1] if len(shape) > 1 else 1) + 63) // 64 * 64
-        self._slab = torch.zeros((n,), dtype=torch.int32, device=device)
-        self._shapes, self._at = shapes, at
+        key = (T, E, cap, dual, lists)
+        plan = _routing_plans.get(key)
+        if plan is None:
+            if len(_routing_plans) >= 256:
+                _routing_plans.clear()
+            plan = _routing_plans[key] = _routing_plan(*key)
+        self._shapes, words, off = plan
+        self.T, self.E, self.W, self.lists = T, E, (E + 31) // 32, lists
+        # One zeroed allocation for all buffers; the tensors over it are made when asked for
+        self._slab = torch.zeros((words,), dtype=torch.int32, device=device)
         base = self._slab.data_ptr()
-        p = {name: base + 4 * o for name, o in at.items()}
-        self.struct = RoutingStruct(p["mask"], p["k"], p.get("counts"), p.get("offsets"), p.get("perm"), p.get("tok_off"), p.get("tok_exp"),
-                                    p["scalars"] if lists else None, p["scalars"] + 4, cap if lists else 0)
+        self.struct = RoutingStruct(*[None if o is None else base + o for o in off], cap if lists else 0)
 
     def __getattr__(self, name):
         # the buffers' tensors, on first use (attributes that exist never come here)
         if name in ("mask", "k", "scalars", "counts", "offsets", "perm", "tok_off", "tok_exp"):
-            shape = self._shapes.get(name)
-            if shape is None:
-                t = None
-            else:
-                o = self._at[name]
-                t = self._slab[o: o + shape[0]] if len(shape) == 1 else self._slab[o: o + shape[0] * shape[1]].view(shape)
+            view = self._shapes.get(name)
+            t = None if view is None else self._slab.as_strided(*view)
             setattr(self, name, t)
             return t
         raise AttributeError(name)
