@@ -457,7 +457,8 @@ d2d_status d2d_layer_create(const d2d_layer_desc *desc, const d2d_weights *w, vo
         bool ok = cudaStreamCreateWithFlags(&L->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
                   cudaStreamCreateWithFlags(&L->copy_out, cudaStreamNonBlocking) == cudaSuccess &&
                   cudaEventCreateWithFlags(&L->ev_begin, cudaEventDisableTiming) == cudaSuccess &&
-                  cudaEventCreateWithFlags(&L->ev_end, cudaEventDisableTiming) == cudaSuccess;
+                  cudaEventCreateWithFlags(&L->ev_end, cudaEventDisableTiming) == cudaSuccess &&
+                  cudaMallocHost((void **)&L->status_host, sizeof(int32_t) * d2d_layer::kHostChunks) == cudaSuccess;
         for (int c = 0; c < d2d_layer::kHostChunks && ok; ++c)
             ok = cudaEventCreateWithFlags(&L->ev_in[c], cudaEventDisableTiming) == cudaSuccess &&
                  cudaEventCreateWithFlags(&L->ev_done[c], cudaEventDisableTiming) == cudaSuccess;
@@ -487,6 +488,7 @@ d2d_status d2d_layer_destroy(d2d_layer *layer)
     if (layer->ev_end) cudaEventDestroy(layer->ev_end);
     if (layer->copy_in) cudaStreamDestroy(layer->copy_in);
     if (layer->copy_out) cudaStreamDestroy(layer->copy_out);
+    if (layer->status_host) cudaFreeHost(layer->status_host);
     if (layer->q_slab) cudaFree(layer->q_slab);
     cudaError_t e = cudaFree(layer->slab);
     delete layer;
@@ -844,15 +846,26 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     return d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st);
 }
 
-// Data-dependent conditions of a finished host call: the largest device status word (0 = ok).
-static d2d_status host_status(const int32_t *status_dev, int n)
+// Ends a host call: its n status words come back with everything else queued on `st` (a blocking copy after the
+// synchronisation was a second round trip of 10 us); returns the largest (0 = ok).
+static d2d_status finish_host_call(const d2d_layer *layer, const int32_t *status_dev, int n, cudaStream_t st)
 {
-    int32_t h[d2d_layer::kHostChunks] = {0, 0, 0, 0};
-    if (n > d2d_layer::kHostChunks) n = d2d_layer::kHostChunks;
-    if (cudaMemcpy(h, status_dev, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost) != cudaSuccess) return D2D_ERR_CUDA;
+    D2D_CUDA_TRY(cudaMemcpyAsync(layer->status_host, status_dev, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, st));
+    D2D_CUDA_TRY(cudaStreamSynchronize(st));
     int32_t worst = 0;
-    for (int i = 0; i < n; ++i) worst = h[i] > worst ? h[i] : worst;
+    for (int i = 0; i < n; ++i) worst = layer->status_host[i] > worst ? layer->status_host[i] : worst;
     return (d2d_status)worst;
+}
+
+// Whether d2d_layer_fwd takes a batch without the per-expert lists (the order of its branches)
+static bool lists_optional(const d2d_layer *L, int T)
+{
+    const d2d_layer_desc &D = L->desc;
+    const bool masked = use_dense_masked(L, T) && !use_small_ffn(L, T);
+    if (d2d_decode_router_supports(D, T) && d2d_use_decode_ffn(L, 1, T)) return true;
+    if (d2d_router_fused_supports(D, T)) return masked;
+    return d2d_layer_f32_small_supports(D, T, false) || (T > 8 && d2d_layer_token_fused_supports(D, T, false)) ||
+           (masked && !d2d_small_select_supports(T, D.n_experts));
 }
 
 // Carves routing buffers + x/y staging + the layer workspace out of one device buffer.
@@ -934,12 +947,12 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     }
     if (n_chunks == 1) {
         D2D_CUDA_TRY(cudaMemcpyAsync(base + h.x_off, x_host, row_bytes, cudaMemcpyHostToDevice, st));
+        if (lists_optional(layer, T)) r.counts = r.offsets = r.perm = r.n_sel = nullptr;      // nobody sees them
         d2d_status rc = d2d_layer_fwd(layer, base + h.x_off, T, tau, base + h.y_off, nullptr, &r,
                                       base + h.ws_off, h.total - h.ws_off, st);
         if (rc != D2D_OK) return rc;
         D2D_CUDA_TRY(cudaMemcpyAsync(y_host, base + h.y_off, row_bytes, cudaMemcpyDeviceToHost, st));
-        D2D_CUDA_TRY(cudaStreamSynchronize(st));
-        return host_status(r.status, 1);
+        return finish_host_call(layer, r.status, 1, st);
     }
     // the copies may not start before work already queued on `stream` (which may still use ws) has finished
     D2D_CUDA_TRY(cudaEventRecord(layer->ev_begin, st));
@@ -953,13 +966,18 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
         D2D_CUDA_TRY(cudaEventRecord(layer->ev_in[c], layer->copy_in));
     }
     d2d_status rc = D2D_OK;
-    int32_t *const status0 = r.status;
+    int32_t *const status0 = r.status, *const counts = r.counts, *const offsets = r.offsets, *const perm = r.perm, *const n_sel = r.n_sel;
     int n_used = 0;
     for (int c = 0; c < n_chunks; ++c) {
         const int t0 = bounds[c], tc = bounds[c + 1] - bounds[c];
         if (tc <= 0) continue;
         r.status = status0 + n_used;                         // one status word per chunk (the layer call clears its own)
         ++n_used;
+        const bool lists = !lists_optional(layer, tc);       // nobody sees them
+        r.counts = lists ? counts : nullptr;
+        r.offsets = lists ? offsets : nullptr;
+        r.perm = lists ? perm : nullptr;
+        r.n_sel = lists ? n_sel : nullptr;
         D2D_CUDA_TRY(cudaStreamWaitEvent(st, layer->ev_in[c], 0));
         rc = d2d_layer_fwd(layer, base + h.x_off + (size_t)t0 * tok_bytes, tc, tau, base + h.y_off + (size_t)t0 * tok_bytes,
                            nullptr, &r, base + h.ws_off, h.total - h.ws_off, st);
@@ -975,8 +993,7 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     cudaEventRecord(layer->ev_end, layer->copy_in);
     cudaStreamWaitEvent(st, layer->ev_end, 0);
     if (rc != D2D_OK) return rc;
-    D2D_CUDA_TRY(cudaStreamSynchronize(st));
-    return host_status(status0, n_used);
+    return finish_host_call(layer, status0, n_used, st);
 }
 
 }  // extern "C"

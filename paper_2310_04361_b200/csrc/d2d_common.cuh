@@ -38,6 +38,7 @@ struct d2d_layer {
     // chunk of tokens, the layer on the previous chunk and the device -> host copy of the one before overlap
     static const int kHostChunks = 4;
     cudaStream_t copy_in, copy_out;
+    int32_t *status_host;                    // page-locked: the status words of a host call
     cudaEvent_t ev_in[kHostChunks], ev_done[kHostChunks], ev_begin, ev_end;
     // layer-owned "last CTA" tickets of the decode kernels used by d2d_layer_fwd (zero at creation, reset by the kernel
     // that used them): word 0 decode router, word 16 decode experts, word 32 tile counter of the up projection, words
