@@ -930,12 +930,19 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     // are short, the ones in between long (a short chunk costs more per token, so there are few of them).
     int bounds[d2d_layer::kHostChunks + 1] = {0, T, T, T, T};
     int n_chunks = 1;
-    if (T >= 8192) {
+    if (T >= 3584) {
         // sizes 3T/16, 5T/16, 5T/16, 3T/16 in multiples of 128 tokens (measured on the Llama-shaped layer, 8192 tokens:
         // 2.50 ms; T/8, 3T/8, 3T/8, T/8: 2.64; four equal chunks: 2.62; two equal chunks: 3.04)
         const int a = d2d_cdiv(3 * (T / 16), 128) * 128, b = d2d_cdiv((T - 2 * a) / 2, 128) * 128;
         bounds[1] = a; bounds[2] = a + b; bounds[3] = T - a > a + b ? T - a : a + b; bounds[4] = T;
         n_chunks = 4;
+    } else if (T >= 1024 && row_bytes >= ((size_t)3 << 20)) {
+        // Equal chunks, as many as pay for their launches and partly filled rounds.  Measured with 1 / 2 / 3 / 4 (us), Llama-shaped
+        // layer at 1000 tokens: 535 / 483 / 554 / 626, 2000: 1007 / 747 / 731 / 781, 4000: 1932 / 1421 / 1361 / 1168;
+        // GPT-2-medium-shaped at 1000: 146 / 153 / 153 / 172, 2000: 227 / 190 / 197 / 218, 4000: 392 / 328 / 298 / 297.
+        n_chunks = T >= 2560 ? 3 : 2;
+        const int chunk = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
+        for (int c = 1; c < n_chunks; ++c) bounds[c] = c * chunk;
     }
     if (const char *e = getenv("D2D_HOST_CHUNKS")) {          // 1 .. 4 equal chunks, for tuning
         const int n = atoi(e);

@@ -763,3 +763,20 @@ def test_lists_from_a_given_mask(api, T, E):
         r = api.routing_from_mask(words, E, dual=dual)
         _check_routing(r, G, dual=dual)
         assert np.array_equal(r.k.cpu().numpy(), G.sum(1))
+
+
+@pytest.mark.parametrize("T", [1023, 1024, 2559, 2560, 3583, 3585])
+def test_layer_fwd_host_two_to_four_chunks(api, T):
+    cfg, w, x, layer = _setup(api, "bert", T)
+    if T < 2048:                                     # 3 MB of rows: a wider layer
+        cfg = wl.LayerConfig("wide", "bf16", d=2048, d_ff=1024, E=32, d_h=128, act="gelu_erf", T=T, b1_shift=-0.3, seed=41)
+        w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+        layer = api.Layer.from_config(cfg, w)
+    xh = torch.from_numpy(x).to(torch.bfloat16).pin_memory()
+    yh = _poison(torch.empty_like(xh)).pin_memory()
+    layer.layer_fwd_host(xh, 0.3, yh, layer.host_workspace(T))
+    y, _ = layer.layer_fwd(xh.cuda(), 0.3)
+    torch.cuda.synchronize()
+    # a chunk may sum K in another order than the whole batch, which moves bf16 roundings
+    assert _rel_err(yh.float().numpy(), y.float().cpu().numpy()) <= TOL_Y["bf16"]
+    layer.close()
