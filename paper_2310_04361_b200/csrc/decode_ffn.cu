@@ -125,13 +125,20 @@ __device__ __forceinline__ float act_fast(int act, float z)
 
 struct FfnShape {
     int T, d, d_ff, E, s, W, act, gated;
-    uint32_t inv_s;          // ceil(2^32 / s): neuron / s = umulhi(neuron, inv_s) for neurons < 2^16
+    uint32_t inv_s;          // ceil(2^32 / s) for s > 1, see expert_of
     int planes;              // 3: hidden values kept to float32 precision and exact activations; 1: bf16 and the fast ones
     int cl, clusters;        // CTAs per cluster, clusters per layer
     int n_static, stages;    // rounds fixed by the cluster's index; stages of the ring
     int up_blocks;           // blocks one request of the up matrices brings
     int nb, sps;             // blocks of a unit's rows of W2T one CTA reads (its d / cl columns); units per stage of those
 };
+
+// neuron / s.  The rounded-up reciprocal is exact for neurons below 2^16 (its error, less than s, times the neuron stays
+// below 2^32); that of s = 1 does not fit 32 bits.
+__device__ __forceinline__ int expert_of(const FfnShape &S, int neuron)
+{
+    return S.s == 1 ? neuron : (int)__umulhi((uint32_t)neuron, S.inv_s);
+}
 
 // TPW: 16-column output tiles per warp (d / cl <= 256 TPW); NT8: tokens / 8.
 template <typename WT, int TPW, int NT8>
@@ -316,7 +323,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             if (mine) {
                 if (P.b1) bias = __bfloat162float(P.b1[u * 16 + nr]);
                 if (Q8) {
-                    const int e = __umulhi((uint32_t)(u * 16 + nr), S.inv_s);
+                    const int e = expert_of(S, u * 16 + nr);
                     sc[0] = P.k1[e]; sc[2] = P.k2[e];
                     if (S.gated) sc[1] = P.kg[e];
                 }
@@ -488,7 +495,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             const int j = r0 - my_static;                                      // shared rounds: their number
             for (int r = r0; r < r1; ++r) {
                 if (rank >= slots(r, n) || !mine) continue;
-                const int e = __umulhi((uint32_t)(unit_of(r, rank, unit_list) * 16 + nr), S.inv_s);
+                const int e = expert_of(S, unit_of(r, rank, unit_list) * 16 + nr);
                 const float *z = zs + (size_t)min(r, my_static) * 3 * 16 * T8 + tid;
                 const float up = z[0], pre = S.gated ? z[16 * T8] : up;
                 float h = 0.0f;
@@ -735,7 +742,8 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
 FfnShape shape_for(const d2d_layer_desc &D, int T)
 {
     FfnShape S = {};
-    S.T = T; S.d = D.d; S.d_ff = D.d_ff; S.E = D.n_experts; S.s = D.expert_size; S.inv_s = (uint32_t)((0x100000000ull + D.expert_size - 1) / D.expert_size); S.W = (D.n_experts + 31) / 32;
+    S.T = T; S.d = D.d; S.d_ff = D.d_ff; S.E = D.n_experts; S.s = D.expert_size; S.inv_s = (uint32_t)((0x100000000ull + D.expert_size - 1) / D.expert_size);      // (0 for s = 1: not used)
+    S.W = (D.n_experts + 31) / 32;
     S.act = D.act; S.gated = D.gated ? 1 : 0;
     S.planes = T <= d2d_decode_max_tokens(D) ? 3 : 1;
     return S;

@@ -667,7 +667,7 @@ def test_small_fp32_layer_runs_in_one_launch(api, T, act, gated, lists):
 
 # decode batches (cluster router + streaming expert kernel) at the edges of their tiles: token blocks of 8 / 16 / 32, the
 # last batch they take and the first they do not, experts of one unit (16 neurons), of two, and not of whole units (24: the
-# kept units are found from the mask), a width of 12 column blocks, output tiles of 1 / 2 / 4 / 8 per warp, fewer units than
+# kept units are found from the mask) and of one neuron, a width of 12 column blocks, output tiles of 1 / 2 / 4 / 8 per warp, fewer units than
 # CTAs, several scorers (E > 256), codes; a row of b1-less gated neurons
 DECODE_CASES = [(dict(d=1024, d_ff=4096, E=256), t, False) for t in (1, 7, 8, 9, 16, 17, 32, 33)] + [
     (dict(d=768, d_ff=3072, E=128), 1, False), (dict(d=768, d_ff=3072, E=128), 12, False), (dict(d=768, d_ff=768, E=24), 20, False),
@@ -675,7 +675,9 @@ DECODE_CASES = [(dict(d=1024, d_ff=4096, E=256), t, False) for t in (1, 7, 8, 9,
     (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 8, False),
     (dict(d=4096, d_ff=5504, E=344, d_h=256), 3, False), (dict(d=64, d_ff=48, E=3, d_h=16), 6, False),
     (dict(d=1024, d_ff=4096, E=256), 6, True), (dict(d=1024, d_ff=4096, E=128, act="relu"), 2, True),
-    (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 4, True)]
+    (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 4, True)] + [
+    (dict(d=256, d_ff=96, E=96), 1, False), (dict(d=256, d_ff=96, E=96), 5, False), (dict(d=256, d_ff=96, E=96), 16, False),
+    (dict(d=256, d_ff=96, E=96), 3, True), (dict(d=256, d_ff=96, E=96), 100, False)]
 
 
 @pytest.mark.parametrize("shape,T,fp8", DECODE_CASES)
