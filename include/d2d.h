@@ -228,6 +228,27 @@ D2D_API d2d_status d2d_layer_get_expert_path(const d2d_layer *layer, int32_t *pa
  * (for bf16 batches above the decode sizes; reporting and tests). */
 D2D_API d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, int64_t n_sel, int32_t *path);
 
+/* How the streaming decode kernels take a batch of T tokens of n_layers layers
+ * (1, or a group's 2..4) of the shape `desc`: the rule of the calls, evaluated
+ * on the host (reporting and tests; needs no layer and, as long as the GPU is
+ * one of 148 SMs, no GPU).  D2D_ERR_UNSUPPORTED: such a batch takes other
+ * kernels.  Shared memory bounds how many tokens they take, 32 at most: one
+ * layer of bf16 weights 32 with d = 512 or 640, 16 with d = 768, 1024 or 2048,
+ * 8 with d = 4096. */
+typedef struct {
+    int32_t router;        /* 1: the decode router takes it too: d2d_layer_fwd and d2d_group_fwd run in two launches */
+    int32_t token_block;   /* 8, 16 or 32: tokens the kernel is built for                     */
+    int32_t cluster_size;  /* CTAs per cluster                                                */
+    int32_t clusters;      /* clusters per layer                                              */
+    int32_t rounds;        /* rounds of one 16-neuron unit per CTA, of the cluster with most  */
+    int32_t static_rounds; /* of these, rounds that start before the selection is known       */
+    int32_t stages;        /* 32 KB stages of the ring the weights stream through             */
+    int32_t list_entries;  /* largest list of kept units a cluster can get ...                */
+    int32_t list_capacity; /* ... and what it has room for                                    */
+} d2d_decode_plan;
+D2D_API d2d_status d2d_decode_plan_for(const d2d_layer_desc *desc, int32_t n_layers, int32_t T, int32_t fp8_experts,
+                                       d2d_decode_plan *plan);
+
 /* Clears the layer-owned device counters (the "last CTA" tickets, the tile and
  * sub-chunk counters of the expert kernels).  They reset themselves when a
  * call completes; a call that ended with D2D_ERR_TIMEOUT in the status word

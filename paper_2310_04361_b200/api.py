@@ -28,7 +28,7 @@ D2D_F32, D2D_BF16 = 0, 1
 ACTS = {"relu": 0, "gelu_erf": 1, "gelu_tanh": 2, "silu": 3}
 PATHS = {"auto": 0, "dense": 1, "gather": 2, "fused": 3}
 EXPORTS = ["d2d_status_str", "d2d_launch_count", "d2d_layer_create", "d2d_layer_create_fp8", "d2d_layer_get_fp8", "d2d_layer_destroy", "d2d_workspace_bytes",
-           "d2d_layer_set_expert_path", "d2d_layer_set_fused_rho_max", "d2d_layer_get_fused", "d2d_layer_expert_path_for", "d2d_layer_get_expert_path", "d2d_layer_reset_counters", "d2d_expert_up_gather_fwd", "d2d_expert_down_masked_fwd", "d2d_test_inject_fault",
+           "d2d_layer_set_expert_path", "d2d_layer_set_fused_rho_max", "d2d_layer_get_fused", "d2d_layer_expert_path_for", "d2d_decode_plan_for", "d2d_layer_get_expert_path", "d2d_layer_reset_counters", "d2d_expert_up_gather_fwd", "d2d_expert_down_masked_fwd", "d2d_test_inject_fault",
            "d2d_select_workspace_bytes", "d2d_router_fwd", "d2d_select_dynk", "d2d_select_dynk_static", "d2d_select_topk",
            "d2d_routing_from_mask", "d2d_moe_ffn_fwd", "d2d_expert_up_fwd", "d2d_expert_down_fwd", "d2d_layer_fwd", "d2d_layer_fwd_host_workspace_bytes",
            "d2d_layer_fwd_host", "d2d_group_create", "d2d_group_destroy", "d2d_group_workspace_bytes", "d2d_group_fwd"]
@@ -47,6 +47,11 @@ class RoutingStruct(ctypes.Structure):
     _fields_ = [("mask", c_void_p), ("k", c_void_p), ("counts", c_void_p), ("offsets", c_void_p),
                 ("perm", c_void_p), ("tok_off", c_void_p), ("tok_exp", c_void_p), ("n_sel", c_void_p),
                 ("status", c_void_p), ("perm_capacity", c_int64)]
+
+
+class DecodePlan(ctypes.Structure):
+    _fields_ = [(n, c_int32) for n in ("router", "token_block", "cluster_size", "clusters", "rounds", "static_rounds", "stages",
+                                       "list_entries", "list_capacity")]
 
 
 _lib.d2d_launch_count.restype = ctypes.c_uint64
@@ -74,6 +79,7 @@ _lib.d2d_layer_set_expert_path.argtypes = [c_void_p, c_int, c_int32, ctypes.c_do
 _lib.d2d_layer_set_fused_rho_max.argtypes = [c_void_p, ctypes.c_double]
 _lib.d2d_layer_get_fused.argtypes = [c_void_p, POINTER(c_int32), POINTER(ctypes.c_double)]
 _lib.d2d_layer_expert_path_for.argtypes = [c_void_p, c_int32, ctypes.c_int64, POINTER(c_int32)]
+_lib.d2d_decode_plan_for.argtypes = [POINTER(LayerDesc), c_int32, c_int32, c_int32, POINTER(DecodePlan)]
 _lib.d2d_layer_get_expert_path.argtypes = [c_void_p, POINTER(c_int32), POINTER(c_int32), POINTER(ctypes.c_double)]
 _lib.d2d_layer_reset_counters.argtypes = [c_void_p, c_void_p]
 _lib.d2d_test_inject_fault.argtypes = [c_int32]
@@ -430,6 +436,16 @@ class LayerGroup:
         if rc != D2D_OK:
             raise D2DError(rc, "d2d_group_fwd")
         return y, routings
+
+
+def decode_plan(desc: LayerDesc, T: int, n_layers: int = 1, fp8_experts: bool = False) -> DecodePlan | None:
+    """How the streaming decode kernels take T tokens of n_layers layers of this shape; None if other kernels do."""
+    plan = DecodePlan()
+    rc = _lib.d2d_decode_plan_for(ctypes.byref(desc), n_layers, T, int(fp8_experts), ctypes.byref(plan))
+    if rc == 2:
+        return None
+    _check(rc, "d2d_decode_plan_for")
+    return plan
 
 
 def select_dynk(R, tau: float, routing: Routing | None = None, dual: bool = False, stream=None,

@@ -598,6 +598,19 @@ d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, int64_t 
     return D2D_OK;
 }
 
+d2d_status d2d_decode_plan_for(const d2d_layer_desc *desc, int32_t n_layers, int32_t T, int32_t fp8_experts, d2d_decode_plan *plan)
+{
+    if (!desc || !plan || n_layers < 1 || n_layers > D2D_MAX_GROUP || T < 1) return D2D_ERR_INVALID_ARG;
+    if (desc->d <= 0 || desc->d_ff <= 0 || desc->n_experts <= 0 || desc->expert_size <= 0 || desc->d_h <= 0 ||
+        (int64_t)desc->n_experts * desc->expert_size != desc->d_ff)
+        return D2D_ERR_INVALID_ARG;
+    d2d_decode_plan p = {};
+    if (!d2d_decode_ffn_plan(*desc, n_layers, T, fp8_experts != 0, &p)) return D2D_ERR_UNSUPPORTED;
+    p.router = d2d_decode_router_supports(*desc, T) ? 1 : 0;
+    *plan = p;
+    return D2D_OK;
+}
+
 d2d_status d2d_layer_get_fused(const d2d_layer *layer, int32_t *group, double *rho_max)
 {
     if (!layer) return D2D_ERR_INVALID_ARG;

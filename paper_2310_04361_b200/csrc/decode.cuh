@@ -50,6 +50,7 @@ size_t d2d_decode_scratch_bytes(const d2d_layer_desc &D, int T);
 d2d_status d2d_decode_layers(const d2d_layer *const *layers, int n, const void *x, int T, float tau, const d2d_routing *routing, float *R,
                              void *const *scratch, void *y, cudaStream_t st);
 bool d2d_decode_ffn_supports(const d2d_layer_desc &D, int n_layers, int T, bool fp8);
+bool d2d_decode_ffn_plan(const d2d_layer_desc &D, int n_layers, int T, bool fp8, d2d_decode_plan *out);
 // after_router: launched right behind d2d_decode_router on `st` (weights and x are then read before it has finished)
 d2d_status d2d_decode_ffn(const d2d_layer_desc &D, int n_layers, const d2d_decode_ffn_args &a, const void *x, int T, bool after_router,
                           cudaStream_t st);

@@ -33,7 +33,7 @@ constexpr int NCW = 16, NC = NCW * 32, NT = NC + 32;      // consumer warps / th
 constexpr int SUB_BYTES = 16 * 128;                       // a block: 16 rows x 128 bytes, 128-byte swizzle
 constexpr int STAGE_BLOCKS = 16, STAGE_BYTES = STAGE_BLOCKS * SUB_BYTES;
 constexpr int MAX_STAGES = 6;
-constexpr int MAX_UNITS = 4096, MAX_LIST = 128;
+constexpr int MAX_UNITS = 4096, MAX_LIST = 128;          // units of a layer; entries of a cluster's list (see plan)
 constexpr int H_ROW = 48;                                 // bytes between tokens' rows of 16 hidden values: free of bank conflicts
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -714,6 +714,9 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
         const int clusters = (cl == 4 ? sms * 33 / 37 : sms) / n_layers / cl;
         if (clusters < 1 || tiles_per_warp<WT>(S.d, cl, S.T) == 0) continue;
         const int rounds = d2d_cdiv(d2d_cdiv(U, cl), clusters);
+        // A cluster's list of kept units holds up to cl entries a round.  One layer never needs more than 128; several large
+        // ones, which share the clusters, can (four of d_ff = 17408 in clusters of four: 34 rounds).
+        if (rounds * cl > MAX_LIST) continue;
         if (best == 0 || rounds < best) {
             best = rounds;
             S.cl = cl;
@@ -826,6 +829,23 @@ d2d_status d2d_decode_ffn_maps(d2d_layer *L)
     L->dec_maps = 0;
     if (L->desc.dtype != D2D_BF16) return D2D_OK;
     return L->q_w1 ? make_maps<uint8_t>(L, L->q_w1, L->q_wg, L->q_w2t) : make_maps<__nv_bfloat16>(L, L->w1, L->w_gate, L->w2t);
+}
+
+// The cut of a batch as d2d_decode_ffn takes it, for d2d_decode_plan_for
+bool d2d_decode_ffn_plan(const d2d_layer_desc &D, int n_layers, int T, bool fp8, d2d_decode_plan *out)
+{
+    if (!d2d_decode_ffn_supports(D, n_layers, T, fp8)) return false;
+    FfnShape S = shape_for(D, T);
+    if (!(fp8 ? plan<uint8_t>(S, n_layers) : plan<__nv_bfloat16>(S, n_layers))) return false;
+    out->token_block = 8 * nt8_for(T);
+    out->cluster_size = S.cl;
+    out->clusters = S.clusters;
+    out->rounds = d2d_cdiv(d2d_cdiv(S.d_ff / 16, S.cl), S.clusters);
+    out->static_rounds = S.n_static;
+    out->stages = S.stages;
+    out->list_entries = out->rounds * S.cl;
+    out->list_capacity = MAX_LIST;
+    return true;
 }
 
 // Whole 16-neuron units, rows of whole 128-byte blocks, a batch whose rows fit shared memory beside three stages.
