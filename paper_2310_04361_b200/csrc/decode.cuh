@@ -3,6 +3,7 @@
 #pragma once
 
 #include "d2d_common.cuh"
+#include "tc_common.cuh"
 
 // Outputs and weights of one layer's router; a group of layers runs as one grid (blockIdx.y = layer).
 struct d2d_decode_router_layer {
@@ -93,27 +94,10 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Bounded wait for a barrier that other CTAs of the cluster complete (see mbar_wait_warp: whole warps, about a second)
+// Wait for a barrier that other CTAs of the cluster complete (whole warps, about a second at most)
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, int32_t *status)
 {
-    unsigned long long t0 = 0;
-    for (uint32_t it = 0; it < (1u << 22); ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-        if (done) return true;
-        if ((it & 31u) == 31u) {
-            unsigned long long now;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > 1000000000ull) break;
-        }
-    }
-    if (status) atomicMax(status, (int32_t)D2D_ERR_TIMEOUT);
-    return false;
+    return d2d_tc::mbar_wait_warp<true>(bar, parity, status);
 }
 
 }  // namespace d2d_decode

@@ -214,6 +214,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // (every thread has passed the dependency wait here: the host never combines n_sel with late_wait)
     const bool run = ep.n_sel == nullptr || (long long)__ldcg(ep.n_sel) > ep.n_sel_max;
 
+    // Waits for barriers that threads of the pair's other CTA arrive at: the ring of work items (its slots are written and read
+    // across the pair) and the accumulators handed back.  The operand and accumulator-full barriers are completed by the copy
+    // engine and the tensor core.
+    auto peer_wait = [&](uint64_t *bar, uint32_t parity) { return mbar_wait<64, 32, PAIR>(smem_u32(bar), parity, ep.status); };
+    auto peer_wait_warp = [&](uint64_t *bar, uint32_t parity) { return mbar_wait_warp<PAIR>(smem_u32(bar), parity, ep.status); };
+
     if (!run) {
         // nothing to do
     } else if (warp == 0) {
@@ -238,13 +244,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     const uint32_t sl = local & 1u, use = local >> 1;
                     if (rank != 0) {
                         // the leader draws for the pair
-                        ok = mbar_wait(smem_u32(&sched_full[sl]), use & 1u, ep.status);
+                        ok = peer_wait(&sched_full[sl], use & 1u);
                         if (!ok) break;
                         item = sched_item[sl];
                         mbar_arrive_cluster(map_to_cta(smem_u32(&sched_empty[sl]), 0));
                         if (item < 0) break;
                     } else {
-                        ok = mbar_wait(smem_u32(&sched_empty[sl]), (use & 1u) ^ 1u, ep.status);
+                        ok = peer_wait(&sched_empty[sl], (use & 1u) ^ 1u);
                         if (!ok) break;
                         // A worker's first item is its own index (no round trip to the counter before the first loads); the
                         // counter hands out the items from n_workers on.  Every worker draws exactly one value past the end,
@@ -334,7 +340,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 int item = worker + (int)local * n_workers;
                 if (dyn) {
                     const uint32_t sl = local & 1u, su = local >> 1;
-                    ok = mbar_wait_warp(smem_u32(&sched_full[sl]), su & 1u, ep.status);
+                    ok = peer_wait_warp(&sched_full[sl], su & 1u);
                     if (!ok) break;
                     item = sched_item[sl];
                     __syncwarp();                              // every lane has read the slot before it is handed back
@@ -348,7 +354,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 const bool one = !GATED && k_splits == 1;
                 const int kb0 = one ? 0 : (int)((long long)sp * nkb / k_splits), kb1 = one ? nkb : (int)((long long)(sp + 1) * nkb / k_splits);
                 const uint32_t buf = local & 1u, use = local >> 1;
-                ok = mbar_wait_warp(smem_u32(&bar_acc_empty[buf]), (use & 1u) ^ 1u, ep.status);   // epilogue drained this buffer
+                ok = peer_wait_warp(&bar_acc_empty[buf], (use & 1u) ^ 1u);   // epilogue drained this buffer
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem_base + buf * BUF_COLS;
@@ -417,7 +423,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 int item = worker + (int)local * n_workers;
                 bool go = true;
                 if (dyn) {
-                    go = mbar_wait(smem_u32(&sched_full[buf]), use & 1u, ep.status);
+                    go = peer_wait(&sched_full[buf], use & 1u);
                     if (go) {
                         item = sched_item[buf];
                         if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&sched_empty[buf]), 0));

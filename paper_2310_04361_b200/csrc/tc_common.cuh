@@ -21,58 +21,62 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// Bounded wait for the phase with the given parity; false (and status set) when the limit runs out.  SPIN polls run
-// back to back, later ones are SLEEP nanoseconds apart.
-template <int SPIN = 64, int SLEEP = 32>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t *status)
+// Whether the phase with the given parity has completed.  CLUSTER: for a barrier that threads of ANOTHER CTA of the cluster
+// arrive at after they wrote or read what the waiter goes on with; their release and this acquire have to reach that far (the
+// form without a scope orders this CTA's own threads only).
+template <bool CLUSTER = false> __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
 {
-    for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
-        uint32_t done;
+    uint32_t done;
+    if (CLUSTER)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    else
         asm volatile(
             "{\n\t.reg .pred p;\n\t"
             "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
             "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
+            : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0;
+}
+
+// Bounded wait for the phase with the given parity; false (and status set) when the limit runs out.  SPIN polls run
+// back to back, later ones are SLEEP nanoseconds apart.
+template <int SPIN = 64, int SLEEP = 32, bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t *status)
+{
+    for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
+        if (mbar_test<CLUSTER>(bar, parity)) return true;
         if (it > (uint32_t)SPIN) __nanosleep(SLEEP);
     }
     if (status) atomicMax(status, (int32_t)D2D_ERR_TIMEOUT);
     return false;
 }
 
-// One non-blocking test of the phase with the given parity.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
-{
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
 // Bounded wait for whole warps: try_wait may suspend the warp in hardware until the phase completes or a time
 // limit passes, so thirty-two waiting lanes cost no issue slots.  Nothing in the loop depends on the lane (same
 // barrier, same parity, the timer is read by one warp instruction), so the lanes stay in step and take the same
 // decision; a vote at the end would make that explicit but measured 1.8 % slower on the ViT-shaped layer.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int32_t *status)
+template <bool CLUSTER = false> __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int32_t *status)
 {
     // how long one try may suspend is up to the hardware, so the bound is in time: about a second by the global timer
     unsigned long long t0 = 0;
     for (uint32_t it = 0; it < WAIT_LIMIT; ++it) {
         uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
+        if (CLUSTER)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
         if ((it & 31u) == 31u) {                               // rarely reached: a try normally ends with the phase complete
             unsigned long long now;
