@@ -41,6 +41,7 @@ struct ws_layout {
     size_t u_off, r_off, sel_off, ffn_off, total;
 };
 
+// What a call with exactly T tokens needs
 ws_layout layout_for(const d2d_layer *L, int T)
 {
     ws_layout w;
@@ -152,6 +153,8 @@ d2d_status d2d_decode_layers(const d2d_layer *const *layers, int n, const void *
     const d2d_status rc = d2d_decode_router(D, n, ra, x, T, tau, 1, T * D.d, st);
     return rc != D2D_OK ? rc : d2d_decode_ffn(D, n, fa, x, T, true, st);
 }
+
+size_t d2d_layer_ws_bytes(const d2d_layer *L, int T) { return layout_for(L, T).total; }
 
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 {
@@ -638,7 +641,7 @@ d2d_status d2d_layer_reset_counters(d2d_layer *layer, void *stream)
 size_t d2d_workspace_bytes(const d2d_layer *layer, int32_t max_tokens)
 {
     if (!layer || max_tokens < 0) return 0;
-    return layout_for(layer, max_tokens).total;
+    return d2d_largest_up_to(max_tokens, [&](int T) { return layout_for(layer, T).total; });
 }
 
 size_t d2d_select_workspace_bytes(int32_t T, int32_t E)
@@ -901,7 +904,7 @@ static host_call_layout host_layout(const d2d_layer *L, int T)
     h.perm_off = take(Tn * E * 4);
     h.scalars_off = take((2 + d2d_layer::kHostChunks) * 4);     // n_sel, then one status word per chunk
     h.ws_off = off;
-    off += layout_for(L, (int)Tn).total;
+    off += d2d_workspace_bytes(L, (int)Tn);                     // the batch and every chunk of it
     h.total = off;
     return h;
 }

@@ -98,6 +98,23 @@ int d2d_decode_max_tokens(const d2d_layer_desc &D);
 static inline size_t d2d_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 static inline int d2d_cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// Largest size(T) over the batches of 1 .. max_tokens tokens, for a size that grows with T except where another form of the call
+// begins: anywhere up to 64 tokens (the decode and single-CTA forms), and behind a multiple of 128 as long as the down
+// projection is split along K, which needs fewer 128-row tiles than half the SMs.
+template <typename F> static inline size_t d2d_largest_up_to(int max_tokens, F size)
+{
+    size_t most = size(max_tokens);
+    for (int T = 1; T <= 64 && T < max_tokens; ++T) {
+        const size_t n = size(T);
+        if (n > most) most = n;
+    }
+    for (int T = 128; T <= 128 * 128 && T < max_tokens; T += 128) {
+        const size_t n = size(T);
+        if (n > most) most = n;
+    }
+    return most;
+}
+
 // ---- launch wrappers implemented in the kernel files -------------------------------------
 
 d2d_status d2d_launch_router(const d2d_layer *L, const void *x, int T, float *R, float *u_ws, cudaStream_t st);
@@ -116,6 +133,7 @@ d2d_status d2d_launch_moe_ffn(const d2d_layer *L, const void *x, int T, const d2
                               void *ws, size_t ws_bytes, cudaStream_t st, int *up_counter = nullptr, int small_fused = 0,
                               const int32_t *n_sel = nullptr);
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T);
+size_t d2d_layer_ws_bytes(const d2d_layer *L, int T);      // workspace of a d2d_layer_fwd call with exactly T tokens
 
 // layer_token_fused.cu: the whole layer of a small float32 problem in one launch (router, rule, experts, lists).
 // ticket: a zeroed layer-owned word (left at zero).  The status word must be zero (or hold an earlier error) at launch.

@@ -76,7 +76,7 @@ group_layout layout_for(const d2d_group *g, int T)
     w.partial_off = off;
     if (g->merged && d2d_gemm_tc_splits((int)Tn, D.d, D.d_ff, g->n) > 1) off += d2d_align_up(n * Tn * D.d * 4, 256);
     w.seq_off = off;
-    off += d2d_workspace_bytes(g->layers[0], (int)Tn);
+    off += d2d_layer_ws_bytes(g->layers[0], (int)Tn);
     w.total = off;
     return w;
 }
@@ -163,7 +163,7 @@ d2d_status d2d_group_destroy(d2d_group *g)
 size_t d2d_group_workspace_bytes(const d2d_group *g, int32_t max_tokens)
 {
     if (!g || max_tokens < 0) return 0;
-    return layout_for(g, max_tokens).total;
+    return d2d_largest_up_to(max_tokens, [&](int T) { return layout_for(g, T).total; });
 }
 
 d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau, void *y, d2d_routing *routing,

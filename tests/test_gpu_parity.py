@@ -782,3 +782,32 @@ def test_layer_fwd_host_two_to_four_chunks(api, T):
     # a chunk may sum K in another order than the whole batch, which moves bf16 roundings
     assert _rel_err(yh.float().numpy(), y.float().cpu().numpy()) <= TOL_Y["bf16"]
     layer.close()
+
+
+# BERT-shaped (the down projection of up to 768 tokens is split along K), a layer that is narrow inside (the decode kernels'
+# accumulators outweigh the hidden activations of larger batches), a Llama-shaped one (decode up to 8 tokens)
+@pytest.mark.parametrize("shape", [dict(d=768, d_ff=3072, E=128), dict(d=1024, d_ff=64, E=4), dict(d=4096, d_ff=1024, E=32, gated=True, act="silu", d_h=256)])
+def test_a_workspace_serves_every_smaller_batch(api, shape):
+    """d2d_workspace_bytes(max_tokens) is enough for any call with up to max_tokens tokens, also of groups and host calls."""
+    cfg = wl.LayerConfig("edge", "bf16", **{**dict(d_h=128, act="gelu_erf", token_sigma=0.5, b1_shift=None), **shape}, T=64, seed=43)
+    layers = [api.Layer.from_config(cfg, wl.make_weights(cfg)) for _ in range(2)]
+    group = api.LayerGroup(layers)
+    sizes = {"layer": layers[0].workspace_bytes, "group": lambda T: int(api._lib.d2d_group_workspace_bytes(group.handle, T)),
+             "host": lambda T: int(api._lib.d2d_layer_fwd_host_workspace_bytes(layers[0].handle, T))}
+    for what, size in sizes.items():
+        at = [size(T) for T in range(1, 1500)]
+        assert all(a <= b for a, b in zip(at, at[1:])), what
+    # and the calls agree: a buffer sized for 769 tokens, batches on both sides of every change of form
+    x = torch.randn((769, cfg.d), device="cuda").bfloat16()
+    ws, gws = (torch.empty((size(769),), dtype=torch.uint8, device="cuda") for size in (sizes["layer"], sizes["group"]))
+    for T in (1, 2, 3, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 128, 129, 512, 513, 768, 769):
+        r = [layers[0].new_routing(T), layers[1].new_routing(T)]
+        y = torch.empty((2, T, cfg.d), dtype=torch.bfloat16, device="cuda")
+        rc = api._lib.d2d_layer_fwd(layers[0].handle, api._ptr(x), T, 0.5, api._ptr(y), None, api.ctypes.byref(r[0].struct), api._ptr(ws), ws.numel(), api._stream())
+        assert rc == 0, T
+        arr = (api.RoutingStruct * 2)(r[0].struct, r[1].struct)
+        rc = api._lib.d2d_group_fwd(group.handle, api._ptr(x), T, 0.5, api._ptr(y), arr, api._ptr(gws), gws.numel(), api._stream())
+        assert rc == 0, T
+        torch.cuda.synchronize()
+        assert r[0].status == 0 and r[1].status == 0
+    group.close()
