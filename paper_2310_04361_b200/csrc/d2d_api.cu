@@ -96,6 +96,11 @@ static bool use_small_ffn(const d2d_layer *L, int T)
 bool d2d_use_decode_ffn(const d2d_layer *L, int n_layers, int T)
 {
     if (T > d2d_decode_max_tokens(L->desc) && L->expert_path != D2D_PATH_AUTO) return false;
+    return d2d_can_decode_ffn(L, n_layers, T);
+}
+
+bool d2d_can_decode_ffn(const d2d_layer *L, int n_layers, int T)
+{
     return L->dec_maps && d2d_decode_ffn_supports(L->desc, n_layers, T, L->q_w1 != nullptr);
 }
 

@@ -58,6 +58,7 @@ d2d_status d2d_decode_ffn(const d2d_layer_desc &D, int n_layers, const d2d_decod
 
 // d2d_api.cu: the kernels' arguments for one layer, and whether a batch of T tokens takes the streaming expert kernel
 bool d2d_use_decode_ffn(const d2d_layer *L, int n_layers, int T);
+bool d2d_can_decode_ffn(const d2d_layer *L, int n_layers, int T);      // ... or would, whatever path the layer is set to
 d2d_decode_router_layer d2d_decode_router_args_for(const d2d_layer *L, const d2d_routing *r, float *R, float *zero);
 d2d_decode_ffn_layer d2d_decode_ffn_args_for(const d2d_layer *L, const d2d_routing *r, float *y32, unsigned int *ticket, void *y);
 

@@ -35,12 +35,14 @@ bool routing_full(const d2d_routing *r)
 }
 
 // Batches the cluster router and the streaming expert kernel take: every layer by the rule of d2d_layer_fwd, bf16 weights
-// in all of them or codes in all of them.
-bool decode_kernels(const d2d_group *g, int T)
+// in all of them or codes in all of them.  any_path: as if no layer had a path forced (the workspace does not depend on a
+// setting that may change between two calls).
+bool decode_kernels(const d2d_group *g, int T, bool any_path = false)
 {
     if (!d2d_decode_router_supports(g->desc, T)) return false;
     for (int l = 0; l < g->n; ++l)
-        if (!d2d_use_decode_ffn(g->layers[l], g->n, T) || (g->layers[l]->q_w1 != nullptr) != (g->layers[0]->q_w1 != nullptr)) return false;
+        if (!(any_path ? d2d_can_decode_ffn(g->layers[l], g->n, T) : d2d_use_decode_ffn(g->layers[l], g->n, T)) ||
+            (g->layers[l]->q_w1 != nullptr) != (g->layers[0]->q_w1 != nullptr)) return false;
     return true;
 }
 
@@ -65,7 +67,7 @@ group_layout layout_for(const d2d_group *g, int T)
     group_layout w;
     size_t off = 0;
     w.sel_off = off; w.sel_each = d2d_align_up(d2d_select_ws_bytes((int)Tn, D.n_experts), 256); off += n * w.sel_each;
-    const bool decode = (int)Tn <= 8 || decode_kernels(g, (int)Tn);
+    const bool decode = (int)Tn <= 8 || decode_kernels(g, (int)Tn, true);
     w.r_off = off; w.r_each = decode ? d2d_align_up(Tn * D.n_experts * 4, 256) : 0; off += n * w.r_each;
     w.u_off = off; w.u_each = decode ? d2d_align_up(Tn * D.d_h * 4, 256) : 0; off += n * w.u_each;
     w.y32_off = off; w.y32_each = decode ? d2d_decode_scratch_bytes(D, (int)Tn) : 0; off += n * w.y32_each;

@@ -811,3 +811,21 @@ def test_a_workspace_serves_every_smaller_batch(api, shape):
         torch.cuda.synchronize()
         assert r[0].status == 0 and r[1].status == 0
     group.close()
+
+
+def test_group_workspace_does_not_depend_on_a_forced_path(api):
+    """The binding looks a size up once; forcing a path and giving it free again must not change what a batch needs."""
+    cfg = wl.with_tokens(wl.CONFIGS["gpt2_attn"], 16)
+    layers = [api.Layer.from_config(cfg, wl.make_weights(cfg)) for _ in range(2)]
+    group = api.LayerGroup(layers)
+    x = api.to_device(wl.make_tokens(cfg), cfg.dtype)
+    ys = []
+    for path in ("dense", "auto"):
+        for layer in layers:
+            layer.set_expert_path(path)
+        y, rs = group.group_fwd(x, 0.0)                       # every expert: no decision at the threshold to differ in
+        torch.cuda.synchronize()
+        assert all(r.status == 0 for r in rs)
+        ys.append(y.float().cpu().numpy())
+    assert _rel_err(ys[0], ys[1]) <= TOL_Y["bf16"]
+    group.close()
