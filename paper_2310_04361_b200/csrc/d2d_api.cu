@@ -770,6 +770,45 @@ d2d_status d2d_expert_down_fwd(const d2d_layer *layer, const void *H, int32_t T,
     return d2d_gemm_tc(dn, (cudaStream_t)stream);
 }
 
+// The forms of a layer call, in the order in which they are tried.
+enum layer_form {
+    FORM_DECODE,             // decode batches: cluster router with selection and lists, streaming experts
+    FORM_FUSED_ROUTER,       // router and mask in one kernel, tensor-core experts, lists beside them
+    FORM_FUSED_ROUTER_LISTS, // the same router, then the lists, then experts that walk them
+    FORM_F32_SMALL,          // float32 layers that fit one SM's shared memory: one launch
+    FORM_TOKEN_FUSED,        // other small float32 problems: one launch
+    FORM_SMALL_ROUTER,       // decode batches the streaming kernels do not take: router that selects as well
+    FORM_MASKED,             // hidden layer, then scores and selection; tensor-core experts, lists beside them
+    FORM_PLAIN,              // scores, selection, experts, one after the other
+};
+
+static layer_form form_for(const d2d_layer *L, int T, bool lists)
+{
+    const d2d_layer_desc &D = L->desc;
+    const bool masked = use_dense_masked(L, T) && !use_small_ffn(L, T);
+    if (d2d_decode_router_supports(D, T) && d2d_use_decode_ffn(L, 1, T)) return FORM_DECODE;
+    if (d2d_router_fused_supports(D, T)) return masked ? FORM_FUSED_ROUTER : FORM_FUSED_ROUTER_LISTS;
+    if (d2d_layer_f32_small_supports(D, T, lists)) return FORM_F32_SMALL;
+    if (T > 8 && d2d_layer_token_fused_supports(D, T, lists)) return FORM_TOKEN_FUSED;
+    if (lists && d2d_small_router_supports(D, T)) return FORM_SMALL_ROUTER;
+    if (masked && !d2d_small_select_supports(T, D.n_experts)) return FORM_MASKED;
+    return FORM_PLAIN;
+}
+
+// Whether the form's expert kernels walk the per-expert lists (the others read the mask, and build the lists if they are wanted)
+static bool needs_lists(layer_form f) { return f == FORM_FUSED_ROUTER_LISTS || f == FORM_SMALL_ROUTER || f == FORM_PLAIN; }
+
+// The per-expert lists on the layer's side stream, behind what is queued on `st`
+static d2d_status fork_lists(const d2d_layer *L, int T, d2d_routing *r, void *ws, cudaStream_t st)
+{
+    if (cudaEventRecord(L->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(L->side_stream, L->ev_fork, 0) != cudaSuccess) return D2D_ERR_CUDA;
+    return d2d_launch_select(nullptr, T, L->desc.n_experts, 0.0f, 0, r, ws, L->side_stream, 1, L->tickets + 48);
+}
+static d2d_status join_lists(const d2d_layer *L, cudaStream_t st)
+{
+    return cudaEventRecord(L->ev_join, L->side_stream) == cudaSuccess && cudaStreamWaitEvent(st, L->ev_join, 0) == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+}
+
 d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float tau, void *y,
                          float *R_out, d2d_routing *routing, void *ws, size_t ws_bytes, void *stream)
 {
@@ -782,89 +821,65 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     if (!x || !y || !aligned16(x) || !aligned16(y) || (R_out && !aligned16(R_out))) return D2D_ERR_INVALID_ARG;
     const ws_layout w = layout_for(layer, T);
     if (!ws || !aligned16(ws) || ws_bytes < w.total) return D2D_ERR_WORKSPACE;
+    const layer_form form = form_for(layer, T, lists);
+    if (!lists && needs_lists(form)) return D2D_ERR_INVALID_ARG;
     char *base = (char *)ws;
     float *R = R_out ? R_out : (float *)(base + w.r_off);
+    void *ffn_ws = base + w.ffn_off;
+    const size_t ffn_bytes = w.total - w.ffn_off;
+    // the fused routers and router_scores also add up k: the number of selected pairs, which decides between the two up projections
+    int32_t *ksum = (int32_t *)(layer->tickets + 40);
     d2d_status rc;
-    if (d2d_decode_router_supports(layer->desc, T) && d2d_use_decode_ffn(layer, 1, T)) {
-        void *scratch = base + w.ffn_off;
-        return d2d_decode_layers(&layer, 1, x, T, tau, routing, R_out, &scratch, y, st);
-    }
-    if (d2d_router_fused_supports(layer->desc, T)) {
-        // router and dynamic-k mask in one kernel; the selection step then only builds the per-expert metadata
-        const bool dense = use_dense_masked(layer, T) && !use_small_ffn(layer, T);
-        if (!dense && cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
-        // tile counter of the up projection: layer-owned, zero at creation and reset by the kernel that used it, so no
-        // memset node sits in front of the router (the up projection may begin while the router is still running)
-        int *up_counter = dense ? (int *)(layer->tickets + 32) : nullptr;
-        // the scores themselves are written only when the caller asked for them: mask and k come out of the same kernel
-        // the router also adds up k: the number of selected pairs, which decides between the two up projections
-        int32_t *ksum = (int32_t *)(layer->tickets + 40);
-        rc = d2d_router_fused(layer, x, T, tau, 1, R_out, routing->mask, routing->k, routing->status, st, dense ? ksum : nullptr);
-        if (rc != D2D_OK) return rc;
-        if (dense) {
-            // The tensor-core expert kernels read only the mask: the per-expert lists (when the caller wants them) are
-            // built on the side stream while they run (the small metadata CTAs fit beside the persistent CTAs), join at the end.
-            if (lists) {
-                if (cudaEventRecord(layer->ev_fork, st) != cudaSuccess ||
-                    cudaStreamWaitEvent(layer->side_stream, layer->ev_fork, 0) != cudaSuccess)
-                    return D2D_ERR_CUDA;
-                rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1, layer->tickets + 48);
-                if (rc != D2D_OK) return rc;
-            }
-            rc = d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, up_counter, 0, ksum + 4);
-            if (lists && (cudaEventRecord(layer->ev_join, layer->side_stream) != cudaSuccess ||
-                          cudaStreamWaitEvent(st, layer->ev_join, 0) != cudaSuccess))
-                return D2D_ERR_CUDA;
-            return rc;
-        }
-        if (!lists) return D2D_ERR_INVALID_ARG;               // the expert kernels of this shape walk the per-expert lists
-        rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, st, 1);
-    } else if (d2d_layer_f32_small_supports(layer->desc, T, lists)) {
-        // float32 layers that fit one SM's shared memory: router, rule, experts and lists in one launch
-        return d2d_layer_f32_small(layer, x, T, tau, y, R_out, routing, lists, layer->tickets + 52, st);
-    } else if (T > 8 && d2d_layer_token_fused_supports(layer->desc, T, lists)) {
-        // small float32 problems: router, rule, experts and lists in one launch
+    switch (form) {
+    case FORM_DECODE: return d2d_decode_layers(&layer, 1, x, T, tau, routing, R_out, &ffn_ws, y, st);
+    case FORM_F32_SMALL: return d2d_layer_f32_small(layer, x, T, tau, y, R_out, routing, lists, layer->tickets + 52, st);
+    case FORM_TOKEN_FUSED:
         if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
         return d2d_layer_token_fused(layer, x, T, tau, y, R_out, routing, lists, layer->tickets + 52, st);
-    } else if (lists && d2d_small_router_supports(layer->desc, T)) {
-        // decode batches: the router kernel's last CTA selects as well (one launch for router + selection)
+    case FORM_FUSED_ROUTER:
+        // The scores are written only when the caller asked for them: mask and k come out of the same kernel.  The tensor-core
+        // expert kernels read only the mask: the per-expert lists (when the caller wants them) are built on the side stream while
+        // they run (the small metadata CTAs fit beside the persistent CTAs), join at the end.
+        rc = d2d_router_fused(layer, x, T, tau, 1, R_out, routing->mask, routing->k, routing->status, st, ksum);
+        if (rc == D2D_OK && lists) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
+        if (rc != D2D_OK) return rc;
+        // tile counter of the up projection: layer-owned, zero at creation and reset by the kernel that used it, so no memset node
+        // sits in front of the router (the up projection may begin while the router is still running)
+        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, (int *)(layer->tickets + 32), 0, ksum + 4);
+        return lists && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
+    case FORM_FUSED_ROUTER_LISTS:
+        if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
+        rc = d2d_router_fused(layer, x, T, tau, 1, R_out, routing->mask, routing->k, routing->status, st, nullptr);
+        if (rc == D2D_OK) rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, st, 1);
+        break;
+    case FORM_SMALL_ROUTER: {
+        // the router kernel's last CTA selects as well (one launch for router + selection)
         const bool small = use_small_ffn(layer, T);
         float *y32 = (float *)(base + w.ffn_off + 256);
-        rc = d2d_small_router(layer, x, T, R, base + w.u_off, st, routing, tau, 1, small ? y32 : nullptr,
-                              small ? T * layer->desc.d : 0);
+        rc = d2d_small_router(layer, x, T, R, base + w.u_off, st, routing, tau, 1, small ? y32 : nullptr, small ? T * layer->desc.d : 0);
         if (rc != D2D_OK) return rc;
-        return d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, nullptr, small ? 1 : 0);
-    } else if (use_dense_masked(layer, T) && !use_small_ffn(layer, T) && !d2d_small_select_supports(T, E)) {
-        // router shapes the fused kernel does not take, tensor-core expert step: the hidden layer by a GEMM, then scores,
-        // mask, k and the number of selected pairs by one kernel (two where the scores do not fit it); the per-expert lists
-        // (when wanted) are built on the side stream while the experts, which read only the mask, run
-        int32_t *ksum = (int32_t *)(layer->tickets + 40);
+        return d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, nullptr, small ? 1 : 0);
+    }
+    case FORM_MASKED:
+        // router shapes the fused kernel does not take: the hidden layer by a GEMM, then scores, mask, k and the number of selected
+        // pairs by one kernel (two where the scores do not fit it); lists as above
         if (d2d_router_scores_supports(layer->desc, T)) {
             rc = d2d_router_scores(layer, x, base + w.u_off + 256, T, tau, R_out, routing->mask, routing->k, routing->status, st, ksum);
         } else {
             rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
             if (rc == D2D_OK) rc = d2d_launch_dynk_mask(R, T, E, tau, routing, ksum, st);
         }
+        if (rc == D2D_OK && lists) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
         if (rc != D2D_OK) return rc;
-        if (lists) {
-            if (cudaEventRecord(layer->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(layer->side_stream, layer->ev_fork, 0) != cudaSuccess)
-                return D2D_ERR_CUDA;
-            rc = d2d_launch_select(nullptr, T, E, tau, 0, routing, base + w.sel_off, layer->side_stream, 1, layer->tickets + 48);
-            if (rc != D2D_OK) return rc;
-        }
-        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st, nullptr, 0, ksum + 4);
-        if (lists && (cudaEventRecord(layer->ev_join, layer->side_stream) != cudaSuccess || cudaStreamWaitEvent(st, layer->ev_join, 0) != cudaSuccess))
-            return D2D_ERR_CUDA;
-        return rc;
-    } else if (!lists) {
-        return D2D_ERR_INVALID_ARG;                           // every other path builds (and its expert kernels use) the lists
-    } else {
+        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, nullptr, 0, ksum + 4);
+        return lists && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
+    case FORM_PLAIN:
         rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
-        if (rc != D2D_OK) return rc;
-        rc = d2d_launch_select(R, T, E, tau, 0, routing, base + w.sel_off, st);
+        if (rc == D2D_OK) rc = d2d_launch_select(R, T, E, tau, 0, routing, base + w.sel_off, st);
+        break;
     }
     if (rc != D2D_OK) return rc;
-    return d2d_launch_moe_ffn(layer, x, T, routing, y, base + w.ffn_off, w.total - w.ffn_off, st);
+    return d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st);
 }
 
 // Ends a host call: its n status words come back with everything else queued on `st` (a blocking copy after the
@@ -878,16 +893,8 @@ static d2d_status finish_host_call(const d2d_layer *layer, const int32_t *status
     return (d2d_status)worst;
 }
 
-// Whether d2d_layer_fwd takes a batch without the per-expert lists (the order of its branches)
-static bool lists_optional(const d2d_layer *L, int T)
-{
-    const d2d_layer_desc &D = L->desc;
-    const bool masked = use_dense_masked(L, T) && !use_small_ffn(L, T);
-    if (d2d_decode_router_supports(D, T) && d2d_use_decode_ffn(L, 1, T)) return true;
-    if (d2d_router_fused_supports(D, T)) return masked;
-    return d2d_layer_f32_small_supports(D, T, false) || (T > 8 && d2d_layer_token_fused_supports(D, T, false)) ||
-           (masked && !d2d_small_select_supports(T, D.n_experts));
-}
+// Whether a batch can do without the per-expert lists
+static bool lists_optional(const d2d_layer *L, int T) { return !needs_lists(form_for(L, T, false)); }
 
 // Carves routing buffers + x/y staging + the layer workspace out of one device buffer.
 struct host_call_layout {

@@ -829,3 +829,40 @@ def test_group_workspace_does_not_depend_on_a_forced_path(api):
         ys.append(y.float().cpu().numpy())
     assert _rel_err(ys[0], ys[1]) <= TOL_Y["bf16"]
     group.close()
+
+
+# one shape per form of a layer call, batches on both sides of every change of form; the batches that need the lists
+FORM_T = (1, 4, 5, 8, 9, 16, 17, 32, 33, 64, 65, 256, 257, 300)
+FORM_SHAPES = [("bf16", dict(d=256, d_ff=512, E=32, d_h=128), ()), ("bf16", dict(d=256, d_ff=512, E=32, d_h=72), FORM_T[:10]),
+               ("bf16", dict(d=256, d_ff=520, E=65, d_h=128), FORM_T[:2]), ("f32", dict(d=64, d_ff=256, E=16, d_h=32), ()),
+               ("f32", dict(d=256, d_ff=1024, E=32, d_h=64), FORM_T[:4]), ("f32", dict(d=256, d_ff=4096, E=32, d_h=64), FORM_T)]
+
+
+@pytest.mark.parametrize("dtype,shape,need", FORM_SHAPES)
+def test_calls_without_lists_agree_with_host_calls(api, dtype, shape, need):
+    """A batch whose form reads only the mask may leave the lists out, any other is refused; a host call, which leaves them
+    out wherever it may, takes both."""
+    cfg = wl.LayerConfig("form", dtype, **shape, T=300, act="gelu_erf", token_sigma=0.5, b1_shift=-0.3, seed=47)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    xd, tol = api.to_device(x, cfg.dtype), TOL_Y["f32" if dtype == "f32" else "bf16"]
+    refused = []
+    for T in FORM_T:
+        y, r = layer.layer_fwd(xd[:T], 0.0)
+        torch.cuda.synchronize()
+        assert r.status == 0
+        y = y.float().cpu().numpy()
+        try:
+            y2, r2 = layer.layer_fwd(xd[:T], 0.0, routing=layer.new_routing(T, lists=False))
+        except api.D2DError as e:
+            assert e.code == 1
+            refused.append(T)
+        else:
+            torch.cuda.synchronize()
+            assert r2.status == 0 and _rel_err(y2.float().cpu().numpy(), y) <= tol
+        xh = xd[:T].cpu().pin_memory()
+        yh = _poison(torch.empty_like(xh)).pin_memory()
+        layer.layer_fwd_host(xh, 0.0, yh, layer.host_workspace(T))
+        assert _rel_err(yh.float().numpy(), y) <= tol
+    assert tuple(refused) == need
+    layer.close()
