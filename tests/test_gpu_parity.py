@@ -665,10 +665,11 @@ def test_small_fp32_layer_runs_in_one_launch(api, T, act, gated, lists):
     layer.close()
 
 
-# decode batches (cluster router + streaming expert kernel) at the edges of their tiles: token blocks of 8 / 16 / 32, the
-# last batch they take and the first they do not, experts of one unit (16 neurons), of two, and not of whole units (24: the
-# kept units are found from the mask) and of one neuron, a width of 12 column blocks, output tiles of 1 / 2 / 4 / 8 per warp, fewer units than
-# CTAs, several scorers (E > 256), codes; a row of b1-less gated neurons
+# decode batches (cluster router + streaming expert kernel) at the edges of their tiles: every instance of the expert kernel
+# (token blocks of 8 / 16 / 32, output tiles of 1 / 2 / 4 / 8 per warp, bf16 weights and codes: test_decode_plan.py goes through
+# them), the last batch a width takes and the first it does not, experts of one unit (16 neurons), of two, not of whole units
+# (24: the kept units are found from the mask) and of one neuron, a width of 12 column blocks, fewer units than CTAs, several
+# scorers (E > 256), a row of b1-less gated neurons
 DECODE_CASES = [(dict(d=1024, d_ff=4096, E=256), t, False) for t in (1, 7, 8, 9, 16, 17, 32, 33)] + [
     (dict(d=768, d_ff=3072, E=128), 1, False), (dict(d=768, d_ff=3072, E=128), 12, False), (dict(d=768, d_ff=768, E=24), 20, False),
     (dict(d=2048, d_ff=1600, E=100), 5, False), (dict(d=2048, d_ff=1600, E=100), 16, False), (dict(d=2048, d_ff=1600, E=100), 1, False),
@@ -677,7 +678,12 @@ DECODE_CASES = [(dict(d=1024, d_ff=4096, E=256), t, False) for t in (1, 7, 8, 9,
     (dict(d=1024, d_ff=4096, E=256), 6, True), (dict(d=1024, d_ff=4096, E=128, act="relu"), 2, True),
     (dict(d=4096, d_ff=5504, E=172, gated=True, act="silu", b1_shift=None, d_h=256), 4, True)] + [
     (dict(d=256, d_ff=96, E=96), 1, False), (dict(d=256, d_ff=96, E=96), 5, False), (dict(d=256, d_ff=96, E=96), 16, False),
-    (dict(d=256, d_ff=96, E=96), 3, True), (dict(d=256, d_ff=96, E=96), 100, False)]
+    (dict(d=256, d_ff=96, E=96), 3, True), (dict(d=256, d_ff=96, E=96), 100, False)] + [
+    (dict(d=512, d_ff=2048, E=128), 17, False), (dict(d=512, d_ff=2048, E=128), 32, False), (dict(d=640, d_ff=2560, E=160), 20, False),
+    (dict(d=640, d_ff=2560, E=160), 33, False), (dict(d=896, d_ff=1792, E=28), 32, False), (dict(d=768, d_ff=768, E=32), 16, False),
+    (dict(d=704, d_ff=1408, E=88), 12, False), (dict(d=1024, d_ff=2048, E=128), 12, True), (dict(d=512, d_ff=1024, E=64), 24, True),
+    (dict(d=2048, d_ff=1600, E=100), 5, True), (dict(d=2048, d_ff=1600, E=100), 12, True), (dict(d=768, d_ff=1536, E=96), 20, True),
+    (dict(d=640, d_ff=1280, E=80), 10, True), (dict(d=1152, d_ff=2304, E=144), 3, True)]
 
 
 @pytest.mark.parametrize("shape,T,fp8", DECODE_CASES)
@@ -691,13 +697,20 @@ def test_decode_batches_at_the_edges_of_their_tiles(api, shape, T, fp8):
             w[name] = w[name] if w[name] is None else oracle.quantize_experts_e4m3(w[name], cfg.E)[2]
         w["w2"] = np.ascontiguousarray(oracle.quantize_experts_e4m3(np.ascontiguousarray(w["w2"].T), cfg.E)[2].T)
     act, xd = oracle.ACT_BY_NAME[cfg.act], api.to_device(x, cfg.dtype)
+    plan = api.decode_plan(layer.desc, T, fp8_experts=fp8)
+    streamed = plan is not None and plan.router == 1
     for tau in (0.9, 0.3, 0.0):
         R = _poison(torch.empty((T, cfg.E), dtype=torch.float32, device="cuda"))
         y = _poison(torch.empty((T, cfg.d), dtype=torch.bfloat16, device="cuda"))
         _poison(layer.workspace(T))
-        y, r = layer.layer_fwd(xd, tau, y=y, R_out=R, routing=layer.new_routing(T, dual=True))
+        r = layer.new_routing(T, dual=True)
+        launches = api.launch_count()
+        y, r = layer.layer_fwd(xd, tau, y=y, R_out=R, routing=r)
+        launches = api.launch_count() - launches
         torch.cuda.synchronize()
         assert r.status == 0
+        # two launches: the kernels this test is about, where the plan says that they take the batch
+        assert (launches == 2) == streamed, (launches, streamed)
         assert _rel_err(R.cpu().numpy(), oracle.router(x, w["w_r1"], w["b_r1"], w["w_r2"], w["b_r2"])) <= TOL_R["bf16"]
         G = oracle.unpack_mask(r.mask_u32(), cfg.E)
         assert np.array_equal(G, oracle.select(R.cpu().numpy(), tau)[0])
