@@ -5,14 +5,15 @@ One step = one pass of the whole hot path (router_fwd -> select_dynk -> moe_ffn_
 C-ABI call d2d_layer_fwd) over one batch of synthetic tokens.  Default workload: the largest
 single-GPU configuration, the Llama-style gated layer (d=4096, d_ff=11008, 344 experts x 32
 neurons, 8192 tokens) at tau = 0.4; the other configurations are timed in the same run and
-reported in `per_config` of the same JSON line.
+reported in `per_config` of the full record.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload llama] [--tau 0.4]
                     [--tokens T] [--bernoulli p] [--path auto|dense|gather|fused] [--experts-per-group g] [--fp8-experts]
-                    [--sweep] [--no-per-config] [--no-cpu-baseline] [--no-graph] [--group N]
+                    [--sweep] [--no-per-config] [--no-cpu-baseline] [--no-graph] [--group N] [--details FILE]
     python bench.py --impl reference ...      # times the CPU oracle on the host cores
 
-Prints ONE JSON line on stdout (rank 0).  Multi-GPU: launched by torch.distributed.run, one
+Prints ONE short JSON line on stdout (rank 0): the headline.  The full record (every configuration, the comparators,
+stages, histograms) goes to stderr as one JSON line, or to FILE with --details FILE.  Multi-GPU: launched by torch.distributed.run, one
 process per GPU, each rank runs the same layer on its own batch (tokens are independent: no
 data-path collective), value = all ranks' tokens / max-over-ranks time ("weak" scaling).
 """
@@ -82,6 +83,7 @@ def parse_args():
     p.add_argument("--group", type=int, default=0,
                    help="also time N layers of the workload's shape on the shared input as one d2d_group_fwd call "
                         "(the Q, K, V projections of an attention layer) against N separate d2d_layer_fwd calls")
+    p.add_argument("--details", default=None, metavar="FILE", help="write the full record there instead of to stderr")
     args = p.parse_args()
     if args.tau is None:
         args.tau = 0.4
@@ -258,6 +260,46 @@ def run_reference(args):
     }
     print(json.dumps(line), flush=True)
     return 0
+
+
+# ------------------------------------------------------------------------------------------ output
+
+# What the line on stdout holds of the full record, and of its parts
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "ms_median", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "run", "e2e", "gpu_launches", "clocks", "roofline", "cpu_baseline", "dense_ffn")
+HEADLINE_PARTS = {
+    "run": ("l2", "parallelism"),
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_median"),
+    "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "executed_frac", "traffic", "path_taken"),
+    "cpu_baseline": ("value", "unit", "cores", "kind"),
+    "dense_ffn": ("step_interleaved_ms", "torch_eager_ms", "library_layer_tau0_ms"),
+}
+
+
+def headline(record):
+    """The record cut down to one line that a reader of the last kilobytes of a log gets whole (a record with every
+    configuration is 24 KB).  Floats of the nested parts keep six digits."""
+    def short(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v
+
+    line = {}
+    for key in HEADLINE:
+        v = record[key]
+        if isinstance(v, dict) and key in HEADLINE_PARTS:
+            v = {k: short(v[k]) for k in HEADLINE_PARTS[key] if k in v}
+        line[key] = v
+    return line
+
+
+def emit(record, details):
+    """Headline on stdout, the full record to the file or to stderr."""
+    if details:
+        with open(details, "w") as f:
+            json.dump(record, f)
+            f.write("\n")
+    else:
+        print(json.dumps(record), file=sys.stderr, flush=True)
+    print(json.dumps(headline(record)), flush=True)
 
 
 # ------------------------------------------------------------------------------------------ GPU arm
@@ -687,7 +729,7 @@ def run_ours(args):
             "config": config_dict(cfg, args.tau, args.bernoulli),
             "run": {"tokens_per_gpu": T, "rho": rho, "pruned_flop_fraction": 1 - rho, "k": khist,
                     "step": "d2d_moe_ffn_fwd on the override mask" if args.bernoulli is not None else "d2d_layer_fwd",
-                    "l2": f"flushed between steps by writing a {L2_FLUSH_BYTES >> 20} MiB buffer (outside the events)",
+                    "l2": f"flushed between steps ({L2_FLUSH_BYTES >> 20} MiB written outside the events)",
                     "launch": "eager" if args.no_graph else "CUDA graph replay of the library's launch sequence",
                     "parallelism": f"token-sharded replicas x{world}, no collective"},
             "e2e": e2e, "gpu_launches": launches_per_step * args.steps,
@@ -702,7 +744,7 @@ def run_ours(args):
             line["tau_sweep"] = sweep
         if group_res is not None:
             line["group"] = group_res
-        print(json.dumps(line), flush=True)
+        emit(line, args.details)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
