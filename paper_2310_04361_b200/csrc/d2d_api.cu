@@ -898,7 +898,7 @@ static bool lists_optional(const d2d_layer *L, int T) { return !needs_lists(form
 
 // Carves routing buffers + x/y staging + the layer workspace out of one device buffer.
 struct host_call_layout {
-    size_t x_off, y_off, mask_off, k_off, counts_off, offsets_off, perm_off, scalars_off, ws_off, total;
+    size_t x_off, y_off, mask_off, k_off, counts_off, offsets_off, perm_off, scalars_off, ws_off;      // the layer's workspace is last
 };
 
 static host_call_layout host_layout(const d2d_layer *L, int T)
@@ -916,15 +916,13 @@ static host_call_layout host_layout(const d2d_layer *L, int T)
     h.perm_off = take(Tn * E * 4);
     h.scalars_off = take((2 + d2d_layer::kHostChunks) * 4);     // n_sel, then one status word per chunk
     h.ws_off = off;
-    off += d2d_workspace_bytes(L, (int)Tn);                     // the batch and every chunk of it
-    h.total = off;
     return h;
 }
 
 size_t d2d_layer_fwd_host_workspace_bytes(const d2d_layer *layer, int32_t max_tokens)
 {
     if (!layer || max_tokens < 0) return 0;
-    return host_layout(layer, max_tokens).total;
+    return host_layout(layer, max_tokens).ws_off + d2d_workspace_bytes(layer, max_tokens > 0 ? max_tokens : 1);      // chunks are smaller batches
 }
 
 d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_t T, float tau, void *y_host,
@@ -934,7 +932,6 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     if (T == 0) return D2D_OK;
     if (!x_host || !y_host || !ws || !aligned16(ws)) return D2D_ERR_INVALID_ARG;
     const host_call_layout h = host_layout(layer, T);
-    if (ws_bytes < h.total) return D2D_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     char *base = (char *)ws;
     const size_t tok_bytes = (size_t)layer->desc.d * layer->elem;
@@ -980,11 +977,17 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
             for (int c = 1; c <= d2d_layer::kHostChunks; ++c) bounds[c] = c * chunk < T && c < n ? c * chunk : T;
         }
     }
+    size_t layer_bytes = layout_for(layer, T).total;
+    for (int c = 0; n_chunks > 1 && c < n_chunks; ++c) {
+        const size_t n = layout_for(layer, bounds[c + 1] - bounds[c]).total;
+        if (n > layer_bytes) layer_bytes = n;
+    }
+    if (ws_bytes < h.ws_off + layer_bytes) return D2D_ERR_WORKSPACE;
     if (n_chunks == 1) {
         D2D_CUDA_TRY(cudaMemcpyAsync(base + h.x_off, x_host, row_bytes, cudaMemcpyHostToDevice, st));
         if (lists_optional(layer, T)) r.counts = r.offsets = r.perm = r.n_sel = nullptr;      // nobody sees them
         d2d_status rc = d2d_layer_fwd(layer, base + h.x_off, T, tau, base + h.y_off, nullptr, &r,
-                                      base + h.ws_off, h.total - h.ws_off, st);
+                                      base + h.ws_off, layer_bytes, st);
         if (rc != D2D_OK) return rc;
         D2D_CUDA_TRY(cudaMemcpyAsync(y_host, base + h.y_off, row_bytes, cudaMemcpyDeviceToHost, st));
         return finish_host_call(layer, r.status, 1, st);
@@ -1015,7 +1018,7 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
         r.n_sel = lists ? n_sel : nullptr;
         D2D_CUDA_TRY(cudaStreamWaitEvent(st, layer->ev_in[c], 0));
         rc = d2d_layer_fwd(layer, base + h.x_off + (size_t)t0 * tok_bytes, tc, tau, base + h.y_off + (size_t)t0 * tok_bytes,
-                           nullptr, &r, base + h.ws_off, h.total - h.ws_off, st);
+                           nullptr, &r, base + h.ws_off, layer_bytes, st);
         if (rc != D2D_OK) break;
         D2D_CUDA_TRY(cudaEventRecord(layer->ev_done[c], st));
         D2D_CUDA_TRY(cudaStreamWaitEvent(layer->copy_out, layer->ev_done[c], 0));
