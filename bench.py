@@ -37,10 +37,10 @@ L2_FLUSH_BYTES = 256 << 20
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from ncu captures of that
 # kernel on that workload (absent: no capture of that combination); keyed by (workload, tokens, kernel).
 # The full-size figures are one-pass captures of those two counters alone: the masked dense up projection reads
-# 610.4 MB and writes 174.9 MB; the gathered one (tau = 0.4) reads 2911.9 MB and writes 107.8 MB (token rows and
+# 513.6 MB and writes 167.5 MB; the gathered one (tau = 0.4) reads 2911.9 MB and writes 107.8 MB (token rows and
 # weight rows together exceed what L2 keeps, so rows are fetched again for many of the groups that use them).
 NCU_TRAFFIC_BYTES = {
-    ("llama", 8192, "dense_up"): 610_425_088 + 174_942_464,
+    ("llama", 8192, "dense_up"): 513_562_368 + 167_494_144,
     ("llama", 8192, "gather_up"): 2_911_860_736 + 107_819_520,
 }
 
@@ -592,7 +592,7 @@ def run_ours(args):
             welem = 1 if args.fp8_experts else elem           # 8-bit expert weights: one byte per weight
             touched = n_used * (cfg.n_mat * cfg.s * cfg.d * welem + cfg.s * elem) + 2 * T * cfg.d * elem + cfg.d * elem
             achieved = touched / (t_ffn * 1e-3) / 1e9
-            roofline = {"bound": "hbm", "kernel": "moe_ffn_fwd (small_ffn_kernel)" if launches_per_step <= 2 else "moe_ffn_fwd", "achieved": achieved,
+            roofline = {"bound": "hbm", "kernel": "moe_ffn_fwd (decode_ffn_kernel)" if launches_per_step <= 2 else "moe_ffn_fwd", "achieved": achieved,
                         "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"], "traffic": None,
                         "peak_source": f"{peaks['source']} HBM copy", "algorithmic_bytes_per_launch": touched,
                         "experts_touched": n_used, "kernel_ms": t_ffn}

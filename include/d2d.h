@@ -36,7 +36,7 @@
  *   D2D_DECODE_MAX_TOKENS=n  0..8: bf16 batches of up to n tokens keep float32
  *                            hidden activations and take decode kernels also where
  *                            a path is forced or the shape is one the streaming
- *                            decode kernels (up to 32 tokens) do not take.  Default:
+ *                            decode kernels (d2d_decode_plan_for) do not take.  Default:
  *                            4 tokens, 2 for layers with more than 256 KB of weights
  *                            per expert.
  *   D2D_HOST_CHUNKS=n        1..4: number of pipelined chunks d2d_layer_fwd_host
@@ -379,7 +379,7 @@ D2D_API d2d_status d2d_test_inject_fault(int32_t kind);
  * (counts, offsets, perm, n_sel and the dual) may be NULL as a set, in which
  * case they are not built -- allowed where the expert kernels read only the
  * mask (bf16 batches of more than 64 tokens; from 5 tokens with d_h = 128 and
- * E <= 256; those of up to 32 tokens that the streaming decode kernels take;
+ * E <= 256; those that the streaming decode kernels take, d2d_decode_plan_for;
  * small float32 problems), D2D_ERR_INVALID_ARG elsewhere.  Work is enqueued on `stream`; the per-expert
  * metadata may be built on a stream the layer owns, joined back into `stream`
  * before the call's last operation, so everything the call writes is ordered
@@ -425,8 +425,8 @@ D2D_API d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host
  * bf16, not gated, d_h = 128, E a multiple of 32 and at most 256, d_ff a
  * multiple of 64: the group owns stacked copies of the weights and the routers
  * run as one grid, the up projections as one GEMM and the down projections as
- * one batched GEMM; batches the decode kernels take (bf16: up to 32 tokens,
- * fp32: up to 8, of most shapes) are served in two launches for all layers.  Other shapes run the
+ * one batched GEMM; batches the decode kernels take (bf16: see
+ * d2d_decode_plan_for; fp32: up to 8 tokens) are served in two launches for all layers.  Other shapes run the
  * layers one after the other.  Device status: timeouts of the merged GEMMs
  * are reported in routing[0].status.  Like a layer, a group (and its layers)
  * serves one call at a time. */

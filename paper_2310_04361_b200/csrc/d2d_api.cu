@@ -64,8 +64,8 @@ ws_layout layout_for(const d2d_layer *L, int T)
 // Up to this many tokens a bf16 layer takes CUDA-core arithmetic (the streaming decode kernels then carry float32 hidden
 // activations as three bf16 terms, so that results are as precise as those of small_batch_ffn.cu), above it tensor-core
 // arithmetic with bf16 hidden activations.  Measured with small_batch_ffn.cu, which still serves the shapes the streaming
-// kernels do not take (us per layer call, decode kernels / tensor-core path): GPT-2-medium-shaped FFN (64 KB of weights per expert) T = 3: 31 / 39, T = 4: 33 / 39, T = 5:
-// 41 / 40, T = 8: 43 / 39; Llama-shaped layer (786 KB per expert) T = 1: 84 / 129, T = 2: 108 / 133, T = 3: 221 / 133,
+// kernels do not take, before those existed (us per layer call, small_batch_ffn.cu / tensor-core path): GPT-2-medium-shaped FFN
+// (64 KB of weights per expert) T = 3: 31 / 39, T = 4: 33 / 39, T = 5: 41 / 40, T = 8: 43 / 39; Llama-shaped layer (786 KB per expert) T = 1: 84 / 129, T = 2: 108 / 133, T = 3: 221 / 133,
 // T = 4: 229 / 127.  So 4 tokens for small experts, 2 for large ones; D2D_DECODE_MAX_TOKENS overrides both.
 int d2d_decode_max_tokens(const d2d_layer_desc &D)
 {
@@ -175,20 +175,25 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
     return need;
 }
 
-// Density up to which the gathered pair beats the masked dense pair for this shape and batch size: the default
-// crossover of the automatic choice.  Measured on B200: the gathered kernel is bound by the rate at which token rows
-// can be copied into the A stages (about the same time per 128 x 64 tile of gathered rows whatever the MMA width), so
-// with full-width groups a gathered row costs about 1.2 x a dense one, and the kernel has a fixed part (the scan of the
-// mask, a ragged tile per group visit) worth about five tiles per CTA.  Against a dense up projection of
-// T / 128 x Nd tiles (Nd = 256-column tiles across d_ff) on S SMs that fixed part is T0 = 5 * 128 * 1.2 * S / Nd
-// tokens' worth of dense time, so the pair wins while the fraction of kept (token, group) pairs
+// Density up to which the automatic choice takes the gathered pair for this shape and batch size.  The gathered kernel is bound
+// by the rate at which token rows can be copied into the A stages (about the same time per 128 x 64 tile of gathered rows
+// whatever the MMA width), so with full-width groups a gathered row costs about 1.2 x a dense one, and the kernel has a fixed
+// part (the scan of the mask, a ragged tile per group visit) worth about five tiles per CTA.  Against a dense up projection of
+// T / 128 x Nd tiles (Nd = 256-column tiles across d_ff) on S SMs that fixed part is T0 = 5 * 128 * 1.2 * S / Nd tokens' worth
+// of dense time, so the pair is taken while the fraction of kept (token, group) pairs
 //     u = 1 - (1 - rho)^g  <  U - T0 / T,
-// U = 0.85 for 256 MMA columns (less for narrower groups).  Checked against measured crossovers: Llama-shaped
-// layer u = 0.70 at 8192 tokens, 0.55 at 4096; paper's latency shape 0.7 at 50432 tokens (357 against 374 us at rho = 0.4, 387 against 381 us at 0.5); ViT-shaped 0.5 at
-// 25216; never for the BERT-shaped layer at 4096 tokens.
+// U = 0.85 for 256 MMA columns (less for narrower groups).  U was fitted to a dense pair without CTA pairs and TMA stores; the
+// present one is faster, so the rule takes the gathered pair in a band of densities where the dense one would be level or
+// ahead.  Layer or expert step with each forced and with the choice, one interleaved loop under sustained load (us, dense /
+// gathered / automatic; the rule's limit):
+//     Llama-shaped, 8192 tokens   rho 0.35  1669 / 1972 / 1729   0.22  1689 / 1696 / 1717   0.12  1640 / 1346 / 1361   (0.25)
+//                   4096 tokens   rho 0.22   859 /  894 /  903   0.12   892 /  782 /  793   0.07   879 /  667 /  680   (0.17)
+//                   2048 tokens   rho 0.12   434 /  489 /  468   0.07   422 /  439 /  456   0.02   420 /  337 /  346   (0.05)
+//     paper's shape, 50432        rho 0.4    366 /  390 /  413   0.3    366 /  357 /  378   0.2    363 /  319 /  337   (0.42)
+// (the last includes 10 to 45 us for the kernels of the forms that are not taken, which are launched and return).
 int d2d_tc_sm_count();      // gemm_tc.cu
 
-static const double kAutoMinUpFlop = 2e11;      // smallest up projection for which the automatic choice is made
+static const double kAutoMinUpFlop = 2e11;      // smallest up projection for which the automatic choice is made, see launch_tc_experts
 
 static double default_gather_rho_max(const d2d_layer_desc &D, int g, int T)
 {
@@ -202,11 +207,11 @@ static double default_gather_rho_max(const d2d_layer_desc &D, int g, int T)
     return 1.0 - pow(1.0 - u_max, 1.0 / g);
 }
 
-// Density up to which the fused gathered kernel beats both pairs.  Its merge moves 4 d bytes of vector reductions per
+// Density up to which the automatic choice takes the fused gathered kernel.  Its merge moves 4 d bytes of vector reductions per
 // kept (token, group) pair through each SM's path to L2, next to the token and weight rows coming in, and its float32
-// accumulator is written once and read once more than the other paths' output: measured on B200 (d = 768, 128-neuron
-// groups, 50432 tokens: 141 / 151 / 174 / 244 us at 1 / 2 / 5 / 10 % of the pairs kept, gathered pair 217 / 225 / 231 /
-// 248 us) it wins while at most about 8 % of the (token, group) pairs are kept.
+// accumulator is written once and read once more than the other paths' output.  It is taken while at most 8 % of the (token,
+// group) pairs are kept.  Measured (d = 768, 128-neuron groups, 50432 tokens, us, fused / gathered pair at 1 / 2 / 5 / 8 / 10 /
+// 15 % of the pairs): 140 / 220, 150 / 226, 175 / 235, 220 / 249, 256 / 263, 335 / 294.
 static double default_fused_rho_max(int g)
 {
     if (g <= 0) return 0.0;
@@ -235,9 +240,11 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     int path = L->expert_path;
     if (L->gather_group <= 0) path = D2D_PATH_DENSE;
     // The automatic choice costs a few launches that return at once and the overlap of the router with the masked dense
-    // kernel's main loops (measured on the ViT-shaped layer, 1.2e11 FLOP: 241 us against 224 us at every density, while
-    // the gathered paths win there only below rho = 0.03): it is made only for problems whose up projection takes long
-    // enough (2e11 FLOP, about 150 us of tensor-core time) that this is noise.
+    // kernel's main loops (ViT-shaped layer, 1.2e11 FLOP: 241 us against 224 us at every density when the line was drawn), so it
+    // is made only for problems whose up projection takes long enough (2e11 FLOP, about 150 us of tensor-core time) that this is
+    // little.  What the line gives away: on the ViT-shaped layer the gathered pair wins below rho = 0.03 (205 against 219 us at
+    // 0.023), and on the paper's shape at 12608 tokens (6e10 FLOP, expert step) the fused kernel wins up to rho = 0.17 (58 / 73 / 87
+    // against 110 us at 0.01 / 0.05 / 0.1).
     const double up_flop = 2.0 * (double)T * D.d * D.d_ff * (D.gated ? 2.0 : 1.0);
     if (path == D2D_PATH_AUTO && (up_flop < kAutoMinUpFlop || !n_sel)) path = D2D_PATH_DENSE;
     const double rho_max = L->gather_rho_max >= 0.0 ? L->gather_rho_max : default_gather_rho_max(D, L->gather_group, T);

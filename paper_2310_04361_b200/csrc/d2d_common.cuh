@@ -91,8 +91,8 @@ extern unsigned long long d2d_launch_counter;
 
 bool d2d_tc_pdl_enabled();      // gemm_tc.cu: false when D2D_GEMM_PDL=0 asks for fully serialised launches
 
-// Largest batch served by the decode kernels (cp.async CUDA-core kernels, two launches per layer call); larger bf16
-// batches take the tensor-core path.  4 by default, D2D_DECODE_MAX_TOKENS=n (0 .. 8) overrides it for tuning.
+// Up to this many tokens bf16 layers keep float32 hidden activations (2 or 4 by expert size; D2D_DECODE_MAX_TOKENS=n, 0 .. 8,
+// overrides it for tuning).  The streaming decode kernels take larger batches too, with bf16 hidden activations.
 int d2d_decode_max_tokens(const d2d_layer_desc &D);
 
 static inline size_t d2d_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

@@ -31,7 +31,9 @@ struct EpiParams {
     int mask_words;
     int expert_size;
     int32_t *status;
-    uint32_t inv_expert_size;        // ceil(2^32 / expert_size): column / expert_size = umulhi(column, inv) for columns < 2^16
+    // ceil(2^32 / expert_size), for sizes that are multiples of 8: column / expert_size = umulhi(column, inv) for columns that are,
+    // too, up to columns x size = 2^35 (such a column is at least 8 below the next expert; 2^16 columns of any size)
+    uint32_t inv_expert_size;
     int *tile_counter;               // device counter (zero at launch) for dynamic tile scheduling, NULL = static round-robin
     int late_wait;                   // 1: only the epilogue waits for the previous kernel of the stream (see below)
     int gate_cat;                    // 1 (gated): tm_b covers up and gate rows interleaved in blocks of BN, one load brings both
@@ -712,7 +714,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
 // single CTAs 0.457 / 0.40 / 0.345 at bn = 256 / 192 / 128, pairs 0.42 / 0.345 / 0.29.  Wider tiles win ties.
 // Pairs: not for one row tile, nor for K below 2048, where their coarser tiles and set-up cost more than the fill saves
 // (BERT-shaped layer with pairs in both projections / in the down projection / none: 55.6 / 51.7 / 52.4 us; ViT-shaped
-// 252 / 248.5 / 249; Llama-shaped down projection 506-533 us with pairs, 550 without).
+// 252 / 248.5 / 249; Llama-shaped down projection 505-533 us with pairs under sustained load, 550 without).
 struct tile_choice { int bn; bool pair; };
 tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok, bool gated)
 {

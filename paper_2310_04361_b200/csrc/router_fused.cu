@@ -390,8 +390,9 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
 // 48 KB each) are in flight at once; a fourth k-block takes the first one's place.  The scores fill up to 384 TMEM columns, too
 // many for registers, so the epilogue reads them twice: once for the row maxima, once for the mask words.
 // Bound by latency (one CTA per SM at most, one tile each): loads, 4 k-blocks of MMAs, two passes over TMEM.  Measured at
-// d = 4096, d_h = 256, E = 344, 8192 tokens, from the router's start to the up projection: 92 us against 124 us for a GEMM
-// that wrote R and a kernel that read it twice (11 MB each way); the whole layer 1668 -> 1626 us, at 128 tokens 121 -> 114.
+// d = 4096, d_h = 256, E = 344, against a GEMM that wrote R and a kernel that read it twice (11 MB each way): hidden layer and
+// scores 38 us against 57 us at 8192 tokens (launches on their own, cold L2); the whole layer 110.7 -> 104.6 us at 128 tokens,
+// at 8192 in three runs of each side 1688 to 1716 -> 1629 to 1692.
 constexpr int S_MAX_KB = 4, S_STAGES = 3, S_STAGE_BYTES = 384 * 128, S_WORDS = 3;      // a part owns mask words p, p + 4, p + 8
 __global__ void __launch_bounds__(NTHREADS, 1)
 router_scores_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_constant__ CUtensorMap tm_w2,

@@ -1,6 +1,6 @@
 // Inline-PTX building blocks shared by the tensor-core kernels (tcgen05.mma with TMEM accumulators, TMA tile
-// loads, mbarrier pipelines) and the activation math of their epilogues.  Everything here is a per-CTA operation;
-// no load is shared between CTAs.
+// loads, mbarrier pipelines) and the activation math of their epilogues.  Every load brings a CTA its own data: no
+// load is shared between CTAs.
 #pragma once
 
 #include <cuda.h>
