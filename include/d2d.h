@@ -236,7 +236,7 @@ D2D_API d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, 
  * layer of bf16 weights 32 with d = 512 or 640, 16 with d = 768, 1024 or 2048,
  * 8 with d = 4096. */
 typedef struct {
-    int32_t router;        /* 1: the decode router takes it too: d2d_layer_fwd and d2d_group_fwd run in two launches */
+    int32_t router;        /* 1: the decode router takes it too: d2d_layer_fwd and d2d_group_fwd (no path forced) are two launches */
     int32_t token_block;   /* 8, 16 or 32: tokens the kernel is built for                     */
     int32_t cluster_size;  /* CTAs per cluster                                                */
     int32_t clusters;      /* clusters per layer                                              */
@@ -428,8 +428,9 @@ D2D_API d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host
  * one batched GEMM; batches the decode kernels take (bf16: see
  * d2d_decode_plan_for; fp32: up to 8 tokens) are served in two launches for all layers.  Other shapes run the
  * layers one after the other.  Device status: timeouts of the merged GEMMs
- * are reported in routing[0].status.  Like a layer, a group (and its layers)
- * serves one call at a time. */
+ * are reported in routing[0].status; after one, reset the counters of every
+ * layer and create the group anew (it has a tile counter of its own).  Like a
+ * layer, a group (and its layers) serves one call at a time. */
 typedef struct d2d_group d2d_group;
 D2D_API d2d_status d2d_group_create(d2d_layer *const *layers, int32_t n_layers, void *stream, d2d_group **out);
 D2D_API d2d_status d2d_group_destroy(d2d_group *group);
