@@ -879,3 +879,32 @@ def test_calls_without_lists_agree_with_host_calls(api, dtype, shape, need):
         assert _rel_err(yh.float().numpy(), y) <= tol
     assert tuple(refused) == need
     layer.close()
+
+
+def test_group_whose_lists_do_not_fit_runs_its_layers(api):
+    """Four layers share the clusters; at this d_ff a cluster's list of kept units has no room for all of its units, so the
+    group must take another form (each layer alone still takes the streaming kernels), with the same results."""
+    n, T, d, d_ff, E = 4, 20, 640, 65536, 512
+    g = torch.Generator(device="cuda").manual_seed(53)
+
+    def normal(*shape, std):
+        return (torch.randn(shape, generator=g, device="cuda") * std).bfloat16()
+
+    layers = [api.Layer(d, d_ff, E, 128, "bf16", "relu", False, {
+        "w_r1": normal(128, d, std=d ** -0.5), "w_r2": normal(E, 128, std=128 ** -0.5), "w1": normal(d_ff, d, std=0.02),
+        "w2": normal(d, d_ff, std=0.02), "b2": normal(d, std=0.02)}) for _ in range(n)]
+    desc = layers[0].desc
+    assert api.decode_plan(desc, T, n) is None and api.decode_plan(desc, T, 1).router == 1
+    group = api.LayerGroup(layers)
+    x = torch.randn((T, d), generator=g, device="cuda").bfloat16()
+    _poison(group.workspace(T))
+    y, rs = group.group_fwd(x, 0.4)
+    for layer, yl, r in zip(layers, y, rs):
+        y1, r1 = layer.layer_fwd(x, 0.4)
+        torch.cuda.synchronize()
+        assert r.status == 0 and r1.status == 0
+        assert torch.equal(r.mask, r1.mask) and torch.equal(r.counts, r1.counts) and torch.equal(r.perm, r1.perm)
+        assert _rel_err(yl.float().cpu().numpy(), y1.float().cpu().numpy()) <= 2e-2      # sums in another order, rounded to bf16
+    group.close()
+    for layer in layers:
+        layer.close()
