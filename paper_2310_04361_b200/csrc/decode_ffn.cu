@@ -48,11 +48,23 @@ template <typename WT> __host__ __device__ constexpr int seg_cols() { return NCW
 __host__ __device__ constexpr int x_pitch(int d) { return (d * 2 + 127) / 128 * 128 + 16; }
 
 // One stage: 16 rows from `row` on, the 128-byte column blocks from `block` on (3-D map: column in block, row, block)
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int row, int block, uint32_t bar)
+// `policy`: weights that do not stay in L2 from one call to the next anyway leave it first, so that what both decode kernels
+// keep coming back to (their instructions above all) stays: with 270 MB of weights passing through L2 in a call, every piece of
+// code that an SM ran for the first time in a launch came from a busy memory, 1 to 2 us a time (Llama-shaped layer, 7 tokens:
+// 68.5 -> 65.5 us, 8-bit weights at 1 token: 55.7 -> 53).  Layers whose weights L2 holds lose by it (d = 1024, 13 tokens, 16 MB:
+// 15.4 -> 15.7 us, three layers of 8 MB: 17.3 -> 17.9).
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int row, int block, uint32_t bar, uint64_t policy)
 {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(block), "r"(bar) : "memory");
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst), "l"(map), "r"(0), "r"(row), "r"(block), "r"(bar), "l"(policy) : "memory");
+}
+__device__ __forceinline__ uint64_t weight_policy(bool pass)
+{
+    uint64_t p;
+    if (pass) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+    return p;
 }
 __device__ __forceinline__ void red_add4(float *p, float4 v)
 {
@@ -134,6 +146,7 @@ struct FfnShape {
     int planes;              // 3: hidden values kept to float32 precision and exact activations; 1: bf16 and the fast ones
     int cl, clusters;        // CTAs per cluster, clusters per layer
     int n_static, stages;    // rounds fixed by the cluster's index; stages of the ring
+    int pass;                // the weights only pass through L2
     int up_blocks;           // blocks one request of the up matrices brings
     int nb, sps;             // blocks of a unit's rows of W2T one CTA reads (its d / cl columns); units per stage of those
 };
@@ -211,6 +224,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         uint32_t it = 0, phase = 1;                                            // stages requested; parity of "free" at `slot`
         int slot = -1;
         bool ok = true;
+        const uint64_t policy = weight_policy(S.pass);
         // waits for the next stage, announces `blocks` blocks for it and returns its address
         auto next_stage = [&](int blocks) -> uint32_t {
             if (++slot == S.stages) slot = 0;
@@ -227,7 +241,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             for (int q = 0; q < nq && ok; ++q)
                 for (int m = 0; m < n_mat && ok; ++m) {
                     const uint32_t dst = next_stage(S.up_blocks);
-                    if (ok && lane == 0) tma_load_3d(dst, m ? &P.tm_wg : &P.tm_w1, u * 16, q * STAGE_BLOCKS, full_bar());
+                    if (ok && lane == 0) tma_load_3d(dst, m ? &P.tm_wg : &P.tm_w1, u * 16, q * STAGE_BLOCKS, full_bar(), policy);
                     __syncwarp();
                 }
         };
@@ -243,7 +257,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                     const uint32_t dst = next_stage((k1 - k0) * (PARTS > 1 ? STAGE_BLOCKS : S.nb));
                     if (ok && lane == 0)
                         for (int k = k0; k < k1; ++k)
-                            tma_load_3d(dst + (k - k0) * S.nb * SUB_BYTES, &P.tm_w2t, unit_of(r, k, unit_list_p) * 16, rank * S.nb + part * STAGE_BLOCKS, full_bar());
+                            tma_load_3d(dst + (k - k0) * S.nb * SUB_BYTES, &P.tm_w2t, unit_of(r, k, unit_list_p) * 16, rank * S.nb + part * STAGE_BLOCKS, full_bar(), policy);
                     __syncwarp();
                 }
             return -1;
@@ -731,6 +745,7 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
     if (best == 0) return false;
     const int blocks = S.d / sub_cols<WT>();
     S.up_blocks = blocks < STAGE_BLOCKS ? blocks : STAGE_BLOCKS;
+    S.pass = (double)n_layers * (S.gated ? 3.0 : 2.0) * S.d_ff * S.d * sizeof(WT) > 64e6;       // half of L2
     S.nb = blocks / S.cl;
     S.sps = S.nb >= STAGE_BLOCKS ? 1 : STAGE_BLOCKS / S.nb < S.cl ? STAGE_BLOCKS / S.nb : S.cl;
     // Rounds a cluster starts on before the selection is known: what the ring holds beside the up stages, which are used up
