@@ -183,7 +183,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     const int xp = x_pitch(d);
     unsigned char *ring = smem;
     unsigned char *xs = ring + (size_t)S.stages * STAGE_BYTES;
-    float *red = reinterpret_cast<float *>(xs + (size_t)T8 * xp);              // [n_mat][16 warps][16][T8]
+    float *red = reinterpret_cast<float *>(xs + (size_t)T * xp);               // [n_mat][16 warps][16][T8]
     float *zs = red + (size_t)n_mat * NCW * 16 * T8;                           // [n_static + 1][3][16 * T8] up, gate, scale of a round
     unsigned char *hs = reinterpret_cast<unsigned char *>(zs + (size_t)(S.n_static + 1) * 3 * 16 * T8);     // [n_static + 2][CL][planes][T8] rows
     uint32_t *smask = reinterpret_cast<uint32_t *>(hs + (size_t)(S.n_static + 2) * CL * S.planes * T8 * H_ROW);     // [T][W], then the union [W]
@@ -394,7 +394,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                             }
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                const unsigned char *xr = xs + min(g, T - 1) * xp + (k0 + h * (SUB / 2)) * 2 + c * 32;
+                                const int xo = (k0 + h * (SUB / 2)) * 2 + c * 32;
                                 uint32_t wa[2][8];
                                 widen16(a[h][0], wa[0]);
                                 widen16(a[h][1], wa[1]);
@@ -402,7 +402,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                                 for (int t = 0; t < NT8; ++t)
 #pragma unroll
                                     for (int p = 0; p < 2; ++p) {
-                                        const uint4 xb = *reinterpret_cast<const uint4 *>(xr + t * 8 * xp + p * 16);
+                                        const uint4 xb = *reinterpret_cast<const uint4 *>(xs + min(t * 8 + g, T - 1) * xp + xo + p * 16);
                                         mma16816(s[m][t * CH], wa[0][4 * p], wa[1][4 * p], wa[0][4 * p + 1], wa[1][4 * p + 1], xb.x, xb.y);
                                         mma16816(s[m][t * CH + CH - 1], wa[0][4 * p + 2], wa[1][4 * p + 2], wa[0][4 * p + 3], wa[1][4 * p + 3], xb.z, xb.w);
                                     }
@@ -702,10 +702,11 @@ constexpr size_t kSmemLimit = 218 * 1024;
 
 int nt8_for(int T) { return T <= 8 ? 1 : T <= 16 ? 2 : 4; }
 
-template <typename WT> size_t fixed_smem(const FfnShape &S)
+// Shared memory beside the ring, with `rows` rows of x
+template <typename WT> size_t fixed_smem(const FfnShape &S, size_t rows)
 {
     const size_t t8 = 8 * (size_t)nt8_for(S.T);
-    return 1024 + t8 * x_pitch(S.d) + (size_t)(S.gated ? 2 : 1) * NCW * 16 * t8 * 4 + (size_t)(S.n_static + 1) * 3 * 16 * t8 * 4 +
+    return 1024 + rows * x_pitch(S.d) + (size_t)(S.gated ? 2 : 1) * NCW * 16 * t8 * 4 + (size_t)(S.n_static + 1) * 3 * 16 * t8 * 4 +
            (size_t)(S.n_static + 2) * S.cl * S.planes * t8 * H_ROW + (size_t)(S.T + 1) * S.W * 4;
 }
 
@@ -754,12 +755,17 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
     const int per_up = d2d_cdiv(S.d, seg_cols<WT>()) * (S.gated ? 2 : 1), per_down = d2d_cdiv(S.d, seg_cols<WT>());
     const int most = nt8_for(S.T) > 2 ? 2 : 4;
     S.n_static = most;                                       // (the largest, while the ring is sized)
-    const size_t f = fixed_smem<WT>(S);
-    S.stages = f >= kSmemLimit ? 0 : (int)((kSmemLimit - f) / STAGE_BYTES);
+    // A batch is taken if its whole token block fits beside three stages; the ring then also gets the room of the rows it lacks.
+    const auto stages_with = [&](size_t rows) {
+        const size_t f = fixed_smem<WT>(S, rows);
+        return f >= kSmemLimit ? 0 : (int)((kSmemLimit - f) / STAGE_BYTES);
+    };
+    if (stages_with(8 * (size_t)nt8_for(S.T)) < 3) return false;
+    S.stages = stages_with((size_t)S.T);
     if (S.stages > MAX_STAGES) S.stages = MAX_STAGES;
     const int fit = (S.stages + per_up) / (per_up + per_down);
     S.n_static = S.planes == 3 ? 0 : fit < 1 ? 1 : fit < most ? fit : most;
-    return S.stages >= 3;
+    return true;
 }
 
 FfnShape shape_for(const d2d_layer_desc &D, int T)
@@ -786,7 +792,7 @@ d2d_status launch(const FfnShape &S, int n_layers, const d2d_decode_ffn_args &a,
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S.clusters * S.cl, n_layers, 1);
     cfg.blockDim = dim3(NT, 1, 1);
-    cfg.dynamicSmemBytes = fixed_smem<WT>(S) + (size_t)S.stages * STAGE_BYTES;
+    cfg.dynamicSmemBytes = fixed_smem<WT>(S, (size_t)S.T) + (size_t)S.stages * STAGE_BYTES;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
