@@ -34,7 +34,7 @@ namespace {
 
 using namespace d2d_decode;
 
-constexpr int NCW = 16, NC = NCW * 32, NT = NC + 32;      // consumer warps / threads, all threads
+constexpr int NCW = 16, NC = NCW * 32, NT = NC + 64;      // consumer warps / threads, all threads (a producer warp, a signalling one)
 constexpr int SUB_BYTES = 16 * 128;                       // a block: 16 rows x 128 bytes, 128-byte swizzle
 constexpr int STAGE_BLOCKS = 16, STAGE_BYTES = STAGE_BLOCKS * SUB_BYTES;
 constexpr int MAX_STAGES = 6;
@@ -76,13 +76,20 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster4(uint32_t addr, uint4 v)
+// 16 bytes into the shared memory of another CTA of the cluster; counted by that CTA's barrier
+__device__ __forceinline__ void st_async4(uint32_t addr, uint4 v, uint32_t bar)
 {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive_cluster(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// ... announcing `bytes` bytes of asynchronous stores (which order themselves, and may have been counted before: relaxed)
+__device__ __forceinline__ void arrive_cluster(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -170,11 +177,12 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     const d2d_decode_ffn_layer &P = args.l[blockIdx.y];
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);       // swizzle atoms are 1024 bytes
-    __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], h_full[3], h_empty[2];
+    __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], h_full[3], h_empty[2], h_read[2], bar_go;
     __shared__ int unit_list[MAX_LIST], unit_list_p[MAX_LIST], n_units;
     __shared__ uint32_t keep_bits[MAX_UNITS / 32];
     __shared__ int keep_pre[MAX_UNITS / 32];
     __shared__ unsigned int my_ticket;
+    __shared__ volatile int rounds_s;                          // all rounds of this cluster, for the signalling warp
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c = lane & 3;
     const int warp = __shfl_sync(FULL, tid >> 5, 0);           // warp-uniform for the compiler: see mma16816
     const int d = S.d, T = S.T, U = S.d_ff / 16, CL = S.cl, NCL = S.clusters;
@@ -194,7 +202,11 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             d2d_tc::mbar_init(smem_addr(&bar_empty[i]), NCW);
         }
         for (int i = 0; i < 3; ++i) d2d_tc::mbar_init(smem_addr(&h_full[i]), CL);
-        for (int i = 0; i < 2; ++i) d2d_tc::mbar_init(smem_addr(&h_empty[i]), NCW * CL);
+        for (int i = 0; i < 2; ++i) {
+            d2d_tc::mbar_init(smem_addr(&h_empty[i]), CL);
+            d2d_tc::mbar_init(smem_addr(&h_read[i]), NCW);
+        }
+        d2d_tc::mbar_init(smem_addr(&bar_go), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
@@ -279,7 +291,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             load_list(unit_list_p, lane, 32);
             __syncwarp();
         } else {
-            asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");           // the consumers have built unit_list
+            asm volatile("bar.sync 2, %0;" ::"n"(NC + 32) : "memory");           // the consumers have built unit_list
             n = n_units;
             for (int i = lane; i < MAX_LIST; i += 32) unit_list_p[i] = unit_list[i];
             __syncwarp();
@@ -300,6 +312,18 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         if (!ok)
             for (uint32_t k = it > (uint32_t)S.stages ? it - S.stages : 0; k + 1 < it; ++k)
                 d2d_tc::mbar_wait_warp(smem_addr(&bar_full[k % S.stages]), (k / S.stages) & 1u, P.status);
+        cluster_arrive();
+    } else if (warp == NCW + 1) {
+        // ------------------------------------------------------------------ tells the cluster that a round's hidden values have been
+        // read.  A release at cluster scope takes 0.6 us: a consumer warp would hold up all others with it.
+        bool ok = CL > 1 && d2d_tc::mbar_wait_warp(smem_addr(&bar_go), 0, P.status);
+        __syncwarp();
+        const int nj = ok ? rounds_s - my_static : 0;
+        for (int j = 0; ok && j + 2 < nj; ++j) {
+            ok = d2d_tc::mbar_wait_warp(smem_addr(&h_read[j & 1]), (j >> 1) & 1u, P.status);
+            __syncwarp();
+            if (ok && lane < CL) arrive_cluster(cluster_addr(smem_addr(&h_empty[j & 1]), lane));
+        }
         cluster_arrive();
     } else {
         // ------------------------------------------------------------------ consumers
@@ -499,7 +523,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             } else if (tid == 0) {
                 n_units = 0;
             }
-            asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
+            asm volatile("bar.sync 2, %0;" ::"n"(NC + 32) : "memory");
             n = n_units;
         };
 
@@ -508,8 +532,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         auto buffer = [&](int r) { return hs + (size_t)(r < my_static ? r : S.n_static + ((r - my_static) & 1)) * CL * S.planes * T8 * H_ROW; };
 
         // ---- hidden values of rounds [r0, r1): activation and selection on this CTA's sums into its own buffers, from there to
-        // the other CTAs of the cluster, a warp per receiver (16-byte stores and one arrival; 4-byte asynchronous stores by
-        // the threads that have the values took 2.6 us)
+        // the other CTAs of the cluster, a warp per receiver (16-byte asynchronous stores; 4-byte ones by the threads that have
+        // the values took 2.6 us, plain stores and an arrival that releases them 1.4)
         auto finish = [&](int r0, int r1) {
             const int j = r0 - my_static;                                      // shared rounds: their number
             for (int r = r0; r < r1; ++r) {
@@ -536,19 +560,23 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             consumer_bar();
             if (CL > 1 && warp < CL) {
                 if (j >= 2 && ok) ok = mbar_wait_cluster(smem_addr(&h_empty[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
+                const uint32_t full = smem_addr(&h_full[j < 0 ? 2 : j & 1]);
                 if (warp != rank) {
+                    uint32_t bytes = 0;
                     for (int r = r0; r < r1; ++r) {
                         if (rank >= slots(r, n)) break;
+                        bytes += 32u * (uint32_t)(NT8 == 1 ? T8 * S.planes : T);
                         const unsigned char *own = buffer(r) + (size_t)rank * S.planes * T8 * H_ROW;
                         const uint32_t to = cluster_addr(smem_addr(own), warp);
                         for (int i = lane; i < 2 * T8 * S.planes; i += 32) {
                             const int off = (i >> 1) * H_ROW + (i & 1) * 16;
-                            if (NT8 == 1 || (i >> 1) < T) st_cluster4(to + off, *reinterpret_cast<const uint4 *>(own + off));
+                            if (NT8 == 1 || (i >> 1) < T) st_async4(to + off, *reinterpret_cast<const uint4 *>(own + off), cluster_addr(full, warp));
                         }
                     }
+                    if (lane == 0) arrive_cluster(cluster_addr(smem_addr(&h_full[j < 0 ? 2 : j & 1]), warp), bytes);
+                } else if (lane == 0) {
+                    d2d_tc::mbar_arrive(full);
                 }
-                __syncwarp();
-                if (lane == 0) arrive_cluster(cluster_addr(smem_addr(&h_full[j < 0 ? 2 : j & 1]), warp));
             }
         };
         // (A CTA's own slot of a shared round's buffer is written again two rounds later, behind the barriers of that round's up
@@ -609,10 +637,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                     stage_done();
                 }
             }
-            // the buffer's next use is the shared round after the next: every CTA of the cluster hears from every warp that has
-            // read it
-            if (CL > 1 && j >= 0 && r + 2 < R && lane == 0)
-                for (int q = 0; q < CL; ++q) arrive_cluster(cluster_addr(smem_addr(&h_empty[j & 1]), q));
+            // the buffer's next use is the shared round after the next
+            if (CL > 1 && j >= 0 && r + 2 < R && lane == 0) d2d_tc::mbar_arrive(smem_addr(&h_read[j & 1]));
         };
 
         // Order of work: the up projections of the static rounds; then, with the selection there, hidden values one round
@@ -625,6 +651,10 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 mask_ready();
                 ready = true;
                 R = rounds_for(n);
+                if (tid == 0) {
+                    rounds_s = R;
+                    d2d_tc::mbar_arrive(smem_addr(&bar_go));
+                }
             }
             if (ready && rd == R) break;
             if (!ready || (rf == ru && up_next(ru, rd, R))) {
@@ -791,7 +821,7 @@ d2d_status launch(const FfnShape &S, int n_layers, const d2d_decode_ffn_args &a,
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S.clusters * S.cl, n_layers, 1);
-    cfg.blockDim = dim3(NT, 1, 1);
+    cfg.blockDim = dim3(S.cl > 1 ? NT : NT - 32, 1, 1);        // clusters of one have nobody to signal to
     cfg.dynamicSmemBytes = fixed_smem<WT>(S, (size_t)S.T) + (size_t)S.stages * STAGE_BYTES;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
