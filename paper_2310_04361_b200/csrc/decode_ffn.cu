@@ -600,7 +600,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 for (int part = 0; part < PARTS; ++part) {
                     stage_wait();
                     unsigned char *stage = ring + (size_t)slot * STAGE_BYTES;
-#pragma unroll(PARTS == 1 ? 4 : 1)
+#pragma unroll(NT8 == 1 || PARTS > 1 ? 1 : 4)
                     for (int k = k0; k < k1; ++k) {
                         uint32_t hb[3][NT8][2];
 #pragma unroll
@@ -758,7 +758,9 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
     const int U = S.d_ff / 16, sms = d2d_tc_sm_count();
     int best = 0;
     // Fewest rounds first (the rounds stream the weights), then the larger cluster (fewer sums to merge).  Clusters of four
-    // reach 132 of 148 SMs, smaller ones all of them.  One or two rows of sums are cheaper to merge than hidden values to
+    // reach 132 of 148 SMs, smaller ones all of them.  The smallest batches, which keep a fraction of the experts, do not run all
+    // rounds: there the larger cluster wins unless it would make a quarter more of them (Llama-shaped layer, clusters of two / four:
+    // 45.6 / 43.6 us at 1 token, 43.9 / 42.0 with 8-bit weights; 60.5 / 62.6 at 7 tokens, 55.2 / 61.0 at 4 with 8-bit weights).  One or two rows of sums are cheaper to merge than hidden values to
     // exchange (1.2 us).
     for (int cl = S.T * S.d <= 2048 && tiles_per_warp<WT>(S.d, 1, S.T) ? 1 : 4; cl >= 1; cl /= 2) {
         const int clusters = (cl == 4 ? sms * 33 / 37 : sms) / n_layers / cl;
@@ -767,7 +769,7 @@ template <typename WT> bool plan(FfnShape &S, int n_layers)
         // A cluster's list of kept units holds up to cl entries a round.  One layer never needs more than 128; several large
         // ones, which share the clusters, can (four of d_ff = 17408 in clusters of four: 34 rounds).
         if (rounds * cl > MAX_LIST) continue;
-        if (best == 0 || rounds < best) {
+        if (best == 0 || (S.planes == 3 ? rounds * 5 < best * 4 : rounds < best)) {
             best = rounds;
             S.cl = cl;
             S.clusters = d2d_cdiv(d2d_cdiv(U, cl), rounds);
