@@ -704,10 +704,10 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         // ---- the CTA that is last to add to these columns finishes them: + b2, bf16
         consumer_bar();
         if (tid == 0) {
-            __threadfence();                                                   // orders the whole CTA's additions (the barrier before it)
-            my_ticket = atomicAdd(P.ticket + rank, 1u);
+            // releases the whole CTA's additions (the barrier before it) and acquires everybody's: one round trip, where two fences
+            // around the addition made three
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(my_ticket) : "l"(P.ticket + rank) : "memory");
             if (my_ticket == (unsigned)NCL - 1) P.ticket[rank] = 0u;
-            __threadfence();
         }
         consumer_bar();
         const int per_row = my_ticket == (unsigned)NCL - 1 ? DC / 4 : 0;
