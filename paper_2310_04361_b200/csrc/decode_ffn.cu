@@ -118,22 +118,27 @@ template <bool TRANS> __device__ __forceinline__ void ldmatrix4(uint32_t (&o)[4]
     else
         asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]) : "r"(addr) : "memory");
 }
-// Two columns of two rows of codes -> two bf16x2 words, lower half = first row
-__device__ __forceinline__ void load_pairs(const unsigned char *r0, const unsigned char *r1, uint32_t &o0, uint32_t &o1)
+// Column j of four of two rows of codes (four adjacent columns each) as a bf16 pair, lower half = first row
+template <int J> __device__ __forceinline__ uint32_t pair_of(uint32_t r0, uint32_t r1)
 {
-    const uint32_t a = *reinterpret_cast<const uint16_t *>(r0), b = *reinterpret_cast<const uint16_t *>(r1);
-    o0 = e4m3_to_bf16x2(__byte_perm(a, b, 0x4404));
-    o1 = e4m3_to_bf16x2(__byte_perm(a, b, 0x5414));
+    return e4m3_to_bf16x2(__byte_perm(r0, r1, ((4 + J) << 12) | (J << 4)));
 }
-// Sixteen codes -> eight bf16x2 words
+// Sixteen codes -> eight float16 pairs, in order
 __device__ __forceinline__ void widen16(const uint4 &r, uint32_t (&o)[8])
 {
     const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        o[2 * i] = e4m3_to_bf16x2(__byte_perm(w[i], 0, 0x1404));
-        o[2 * i + 1] = e4m3_to_bf16x2(__byte_perm(w[i], 0, 0x3424));
+        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tcvt.rn.f16x2.e4m3x2 %0, lo;\n\tcvt.rn.f16x2.e4m3x2 %1, hi;\n\t}"
+            : "=r"(o[2 * i]), "=r"(o[2 * i + 1]) : "r"(w[i]));
     }
+}
+// mma16816 on float16 operands
+__device__ __forceinline__ void mma16816_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
 __device__ __forceinline__ float act_accurate(int act, float z)
@@ -174,6 +179,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     constexpr bool Q8 = sizeof(WT) == 1;
     constexpr int SUB = sub_cols<WT>(), SEG = seg_cols<WT>();
     constexpr int TPS = SUB / 16, PARTS = TPW > TPS ? TPW / TPS : 1, TPP = TPW > TPS ? TPS : TPW;      // tiles per warp: of a full stage; stages per unit; per stage
+    constexpr int ACC = Q8 && TPW == 1 ? 2 : TPW;              // codes: tiles come in pairs (32 columns)
     const d2d_decode_ffn_layer &P = args.l[blockIdx.y];
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);       // swizzle atoms are 1024 bytes
@@ -183,6 +189,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     __shared__ int keep_pre[MAX_UNITS / 32];
     __shared__ unsigned int my_ticket;
     __shared__ volatile int rounds_s;                          // all rounds of this cluster, for the signalling warp
+    __shared__ uint32_t x_max[Q8 ? T8 * 16 : 1];               // codes: largest magnitude of the pieces of the token rows ...
+    __shared__ float x_inv[T8];                                // ... and what takes the scaling of a row back
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c = lane & 3;
     const int warp = __shfl_sync(FULL, tid >> 5, 0);           // warp-uniform for the compiler: see mma16816
     const int d = S.d, T = S.T, U = S.d_ff / 16, CL = S.cl, NCL = S.clusters;
@@ -329,13 +337,53 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         // ------------------------------------------------------------------ consumers
         // x does not depend on the router (the kernel behind which this one may start early waits for its own
         // predecessor before it lets this one start)
-        for (int i = tid, t = 0; t < T; ) {
-            if (i >= d / 8) { i -= d / 8; ++t; continue; }
-            cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
-            i += NC;
+        if (!Q8) {
+            for (int i = tid, t = 0; t < T; ) {
+                if (i >= d / 8) { i -= d / 8; ++t; continue; }
+                cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
+                i += NC;
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        } else {
+            // as float16, scaled so that the largest value of the piece lies in [2^14, 2^15): WPT warps a token, a piece of the row each
+            const int wpt = T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1, part = warp % wpt, np = d / 8;
+            const int i0 = np * part / wpt, i1 = np * (part + 1) / wpt;
+            uint32_t m = 0u;
+            for (int t = warp / wpt; t < T; t += NCW / wpt) {
+                const uint4 *row = reinterpret_cast<const uint4 *>(x + (size_t)t * d);
+                m = 0u;
+                for (int i = i0 + lane; i < i1; i += 32) {
+                    const uint4 v = row[i];
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) m = max(m, max(w[q] & 0x7fffu, (w[q] >> 16) & 0x7fffu));
+                    *reinterpret_cast<uint4 *>(xs + (size_t)t * xp + i * 16) = v;
+                }
+                m = __reduce_max_sync(FULL, m);
+                if (lane == 0) x_max[t * 16 + part] = m;
+            }
+            consumer_bar();
+            for (int t = warp / wpt; t < T; t += NCW / wpt) {
+                m = 0u;
+                for (int q = 0; q < wpt; ++q) m = max(m, x_max[t * 16 + q]);
+                const int sh = min(120, 141 - (int)(m >> 7));
+                const float f = __uint_as_float((uint32_t)(127 + sh) << 23);
+                if (lane == 0 && part == 0) x_inv[t] = __uint_as_float((uint32_t)(127 - sh) << 23);
+                for (int i = i0 + lane; i < i1; i += 32) {
+                    uint4 *at = reinterpret_cast<uint4 *>(xs + (size_t)t * xp + i * 16);
+                    const uint4 v = *at;
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                    uint32_t o[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float lo = __uint_as_float(w[q] << 16) * f, hi = __uint_as_float(w[q] & 0xffff0000u) * f;
+                        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(o[q]) : "f"(hi), "f"(lo));
+                    }
+                    *at = make_uint4(o[0], o[1], o[2], o[3]);
+                }
+            }
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
         consumer_bar();
 
         int slot = 0, n = 0;
@@ -427,8 +475,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
 #pragma unroll
                                     for (int p = 0; p < 2; ++p) {
                                         const uint4 xb = *reinterpret_cast<const uint4 *>(xs + min(t * 8 + g, T - 1) * xp + xo + p * 16);
-                                        mma16816(s[m][t * CH], wa[0][4 * p], wa[1][4 * p], wa[0][4 * p + 1], wa[1][4 * p + 1], xb.x, xb.y);
-                                        mma16816(s[m][t * CH + CH - 1], wa[0][4 * p + 2], wa[1][4 * p + 2], wa[0][4 * p + 3], wa[1][4 * p + 3], xb.z, xb.w);
+                                        mma16816_f16(s[m][t * CH], wa[0][4 * p], wa[1][4 * p], wa[0][4 * p + 1], wa[1][4 * p + 1], xb.x, xb.y);
+                                        mma16816_f16(s[m][t * CH + CH - 1], wa[0][4 * p + 2], wa[1][4 * p + 2], wa[0][4 * p + 3], wa[1][4 * p + 3], xb.z, xb.w);
                                     }
                             }
                         }
@@ -462,7 +510,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                     float v = 0.0f;
 #pragma unroll
                     for (int w = 0; w < NCW; ++w) v += p[w * 16 * T8];
-                    if (Q8) v = ldexpf(v, sc[m]);
+                    if (Q8) v = ldexpf(v * x_inv[tok], sc[m]);
                     z[m * 16 * T8] = m == 0 ? v + bias : v;
                 }
                 if (Q8) z[2 * 16 * T8] = ldexpf(1.0f, sc[2]);
@@ -582,11 +630,11 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         // (A CTA's own slot of a shared round's buffer is written again two rounds later, behind the barriers of that round's up
         // projection, which every warp reaches after it has read the buffer.)
 
-        // ---- down projection of round r onto this CTA's columns.  A tile's 16 columns: bf16 weights g and g + 8 of lane (g, c),
-        // codes 2 g and 2 g + 1.
-        float acc[TPW][NT8][4];
+        // ---- down projection of round r onto this CTA's columns.  A tile's 16 columns: bf16 weights g and g + 8 of lane (g, c);
+        // codes 4 g and 4 g + 1 of a 32-column pair of tiles, 4 g + 2 and 4 g + 3 in its second tile.
+        float acc[ACC][NT8][4];
 #pragma unroll
-        for (int i = 0; i < TPW; ++i)
+        for (int i = 0; i < ACC; ++i)
 #pragma unroll
             for (int t = 0; t < NT8; ++t) acc[i][t][0] = acc[i][t][1] = acc[i][t][2] = acc[i][t][3] = 0.0f;
         const int DC = d / CL;
@@ -612,25 +660,40 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                                 hb[p][t][0] = *reinterpret_cast<const uint32_t *>(hr);
                                 hb[p][t][1] = *reinterpret_cast<const uint32_t *>(hr + 16);
                             }
+                        auto products = [&](float (&o)[NT8][4], const uint32_t (&a)[4]) {
 #pragma unroll
-                        for (int i = 0; i < TPP; ++i) {
-                            const int tile = warp + NCW * i;
-                            if (PARTS == 1 && tile * 16 >= DC) break;
-                            unsigned char *st = stage + ((k - k0) * S.nb + tile * 16 / SUB) * SUB_BYTES;
-                            const int col = tile * 16 % SUB * (int)sizeof(WT);
-                            uint32_t a[4];
-                            if (!Q8) {
-                                // matrices: neurons 0-7 and 8-15 (lane / 16), columns 0-7 and 8-15 (lane / 8 % 2)
-                                ldmatrix4<true>(a, smem_addr(st) + swz((lane & 7) + lhalf * 8, col + ((lane >> 3) & 1) * 16));
-                            } else {
-                                load_pairs(st + swz(2 * c, col + g * 2), st + swz(2 * c + 1, col + g * 2), a[0], a[1]);
-                                load_pairs(st + swz(2 * c + 8, col + g * 2), st + swz(2 * c + 9, col + g * 2), a[2], a[3]);
-                            }
-#pragma unroll
-                            for (int t = 0; t < NT8; ++t) mma16816(acc[part * TPP + i][t], a[0], a[1], a[2], a[3], hb[0][t][0], hb[0][t][1]);
+                            for (int t = 0; t < NT8; ++t) mma16816(o[t], a[0], a[1], a[2], a[3], hb[0][t][0], hb[0][t][1]);
                             if (NT8 == 1 && S.planes == 3) {
-                                mma16816(acc[part * TPP + i][0], a[0], a[1], a[2], a[3], hb[1][0][0], hb[1][0][1]);
-                                mma16816(acc[part * TPP + i][0], a[0], a[1], a[2], a[3], hb[2][0][0], hb[2][0][1]);
+                                mma16816(o[0], a[0], a[1], a[2], a[3], hb[1][0][0], hb[1][0][1]);
+                                mma16816(o[0], a[0], a[1], a[2], a[3], hb[2][0][0], hb[2][0][1]);
+                            }
+                        };
+                        const unsigned char *piece = stage + (k - k0) * S.nb * SUB_BYTES;
+                        if (!Q8) {
+#pragma unroll
+                            for (int i = 0; i < TPP; ++i) {
+                                const int tile = warp + NCW * i;
+                                if (PARTS == 1 && tile * 16 >= DC) break;
+                                // matrices: neurons 0-7 and 8-15 (lane / 16), columns 0-7 and 8-15 (lane / 8 % 2)
+                                uint32_t a[4];
+                                ldmatrix4<true>(a, smem_addr(piece + tile * 16 / SUB * SUB_BYTES) +
+                                                       swz((lane & 7) + lhalf * 8, tile * 16 % SUB * 2 + ((lane >> 3) & 1) * 16));
+                                products(acc[part * TPP + i], a);
+                            }
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < (TPP + 1) / 2; ++i) {
+                                const int pair = warp + NCW * i;
+                                if (PARTS == 1 && pair * 32 >= DC) break;
+                                const unsigned char *st = piece + pair * 32 / SUB * SUB_BYTES;
+                                uint32_t r[4];                    // neurons 2c, 2c + 1, 2c + 8, 2c + 9: four columns each
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    r[q] = *reinterpret_cast<const uint32_t *>(st + swz(2 * c + (q & 1) + (q >> 1) * 8, pair * 32 % SUB + g * 4));
+                                const uint32_t a0[4] = {pair_of<0>(r[0], r[1]), pair_of<1>(r[0], r[1]), pair_of<0>(r[2], r[3]), pair_of<1>(r[2], r[3])};
+                                const uint32_t a1[4] = {pair_of<2>(r[0], r[1]), pair_of<3>(r[0], r[1]), pair_of<2>(r[2], r[3]), pair_of<3>(r[2], r[3])};
+                                products(acc[part * TPP + 2 * i], a0);
+                                products(acc[part * TPP + 2 * i + 1], a1);
                             }
                         }
                     }
@@ -670,34 +733,39 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             }
         }
         cluster_arrive();                                                      // this CTA sends nothing to the others any more
-        // ---- this CTA's sums.  Codes: two lanes put their column pairs together; bf16: four lanes (g of a group of four) exchange
-        // their four values each, so that every lane has four adjacent columns of one token: 16 bytes per reduction.
+        // ---- this CTA's sums.  Codes: a lane has four adjacent columns of two tokens; bf16: four lanes (g of a group of four)
+        // exchange their four values each, so that every lane has four adjacent columns of one token: 16 bytes per reduction.
         if (R > 0) {
+            if (Q8) {
 #pragma unroll
-            for (int i = 0; i < TPW; ++i) {
-                const int tile = (i % TPP) * NCW + warp, col0 = (i / TPP) * STAGE_BLOCKS * SUB + tile * 16;
+                for (int i = 0; i < ACC / 2; ++i) {
+                    constexpr int PAIRS = (TPP + 1) / 2;                       // of a stage
+                    const int col = (i / PAIRS) * STAGE_BLOCKS * SUB + ((i % PAIRS) * NCW + warp) * 32 + g * 4;
 #pragma unroll
-                for (int t = 0; t < NT8; ++t) {
-                    const float(&v)[4] = acc[i][t];
-                    const bool o1 = g & 1, o2 = g & 2;
-                    float4 o;
-                    int tk, col;
-                    if (Q8) {
-                        const float p0 = __shfl_xor_sync(FULL, o1 ? v[0] : v[1], 4), p1 = __shfl_xor_sync(FULL, o1 ? v[2] : v[3], 4);
-                        o = o1 ? make_float4(p0, p1, v[1], v[3]) : make_float4(v[0], v[2], p0, p1);
-                        tk = 2 * c + (o1 ? 1 : 0);
-                        col = (g & ~1) * 2;
-                    } else {
+                    for (int t = 0; t < NT8; ++t) {
+                        const float(&v)[4] = acc[2 * i][t], (&w)[4] = acc[2 * i + 1][t];
+                        const int tk = t * 8 + 2 * c;
+                        float *o = P.y32 + (size_t)tk * d + rank * DC + col;
+                        if (tk < T && col < DC) red_add4(o, make_float4(v[0], v[2], w[0], w[2]));
+                        if (tk + 1 < T && col < DC) red_add4(o + d, make_float4(v[1], v[3], w[1], w[3]));
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < TPW; ++i) {
+                    const int tile = (i % TPP) * NCW + warp, col0 = (i / TPP) * STAGE_BLOCKS * SUB + tile * 16;
+#pragma unroll
+                    for (int t = 0; t < NT8; ++t) {
+                        const float(&v)[4] = acc[i][t];
+                        const bool o1 = g & 1, o2 = g & 2;
                         // 4 x 4 transpose over the lanes: value j of all four goes to lane j of the group
                         const float x0 = __shfl_xor_sync(FULL, o1 ? v[0] : v[1], 4), x1 = __shfl_xor_sync(FULL, o1 ? v[2] : v[3], 4);
                         const float a0 = o1 ? x0 : v[0], a1 = o1 ? v[1] : x0, b0 = o1 ? x1 : v[2], b1 = o1 ? v[3] : x1;   // (a0, a1): value o1, (b0, b1): value 2 + o1 of the lane pair
                         const float y0 = __shfl_xor_sync(FULL, o2 ? a0 : b0, 8), y1 = __shfl_xor_sync(FULL, o2 ? a1 : b1, 8);
-                        o = o2 ? make_float4(y0, y1, b0, b1) : make_float4(a0, a1, y0, y1);
-                        tk = 2 * c + (o1 ? 1 : 0);
-                        col = (o2 ? 8 : 0) + (g & 4);
+                        const float4 o = o2 ? make_float4(y0, y1, b0, b1) : make_float4(a0, a1, y0, y1);
+                        const int tk = t * 8 + 2 * c + (o1 ? 1 : 0), col = (o2 ? 8 : 0) + (g & 4);
+                        if (tk < T && col0 + col < DC) red_add4(P.y32 + (size_t)tk * d + rank * DC + col0 + col, o);
                     }
-                    tk += t * 8;
-                    if (tk < T && col0 + col < DC) red_add4(P.y32 + (size_t)tk * d + rank * DC + col0 + col, o);
                 }
             }
         }
