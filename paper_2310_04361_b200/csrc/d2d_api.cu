@@ -182,15 +182,15 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 // T / 128 x Nd tiles (Nd = 256-column tiles across d_ff) on S SMs that fixed part is T0 = 5 * 128 * 1.2 * S / Nd tokens' worth
 // of dense time, so the pair is taken while the fraction of kept (token, group) pairs
 //     u = 1 - (1 - rho)^g  <  U - T0 / T,
-// U = 0.85 for 256 MMA columns (less for narrower groups).  U was fitted to a dense pair without CTA pairs and TMA stores; the
-// present one is faster, so the rule takes the gathered pair in a band of densities where the dense one would be level or
-// ahead.  Layer or expert step with each forced and with the choice, one interleaved loop under sustained load (us, dense /
-// gathered / automatic; the rule's limit):
-//     Llama-shaped, 8192 tokens   rho 0.35  1669 / 1972 / 1729   0.22  1689 / 1696 / 1717   0.12  1640 / 1346 / 1361   (0.25)
-//                   4096 tokens   rho 0.22   859 /  894 /  903   0.12   892 /  782 /  793   0.07   879 /  667 /  680   (0.17)
-//                   2048 tokens   rho 0.12   434 /  489 /  468   0.07   422 /  439 /  456   0.02   420 /  337 /  346   (0.05)
-//     paper's shape, 50432        rho 0.4    366 /  390 /  413   0.3    366 /  357 /  378   0.2    363 /  319 /  337   (0.42)
-// (the last includes 10 to 45 us for the kernels of the forms that are not taken, which are launched and return).
+// U = 0.85 for 256 MMA columns (less for narrower groups).
+// Gated layers run in pairs of CTAs: U = 0.73 and three tiles.  Llama-shaped layer, up projections back to back (us, gathered /
+// masked dense): 8192 tokens, u 0.62 and 0.24: 883 / 951 and 386 / 943; 2560 tokens: 310 / 300 and 192 / 300, that is 85 + 0.159 u T
+// against 0.1165 T; the kernels of the form that is not taken and the zero fill cost the choice another 40.
+// Plain layers: U was fitted to a dense pair without CTA pairs and TMA stores; the present one is faster, so the rule takes the
+// gathered pair in a band of densities where the dense one would be level or ahead.  Paper's shape, 50432 tokens, expert step with
+// each forced and with the choice, one interleaved loop under sustained load (us, dense / gathered / automatic; the rule's limit):
+//     rho 0.4    366 /  390 /  413   0.3    366 /  357 /  378   0.2    363 /  319 /  337   (0.42)
+// (the last includes 14 to 24 us for the kernels of the forms that are not taken, which are launched and return).
 int d2d_tc_sm_count();      // gemm_tc.cu
 
 static const double kAutoMinUpFlop = 2e11;      // smallest up projection for which the automatic choice is made, see launch_tc_experts
@@ -199,9 +199,9 @@ static double default_gather_rho_max(const d2d_layer_desc &D, int g, int T)
 {
     if (g <= 0 || T <= 0) return -1.0;
     const int n_mma = g * D.expert_size * (D.gated ? 2 : 1);
-    double U = n_mma >= 256 ? 0.85 : n_mma >= 192 ? 0.64 : n_mma >= 128 ? 0.43 : 0.25;
+    double U = n_mma >= 256 ? (D.gated ? 0.73 : 0.85) : n_mma >= 192 ? 0.64 : n_mma >= 128 ? 0.43 : 0.25;
     const double nd = ceil((double)D.d_ff * (D.gated ? 2.0 : 1.0) / 256.0);
-    const double T0 = 5.0 * 128.0 * 1.2 * (double)d2d_tc_sm_count() / nd;
+    const double T0 = (D.gated ? 3.0 : 5.0) * 128.0 * 1.2 * (double)d2d_tc_sm_count() / nd;
     const double u_max = U - T0 / (double)T;
     if (u_max <= 0.0) return 0.0;
     return 1.0 - pow(1.0 - u_max, 1.0 / g);

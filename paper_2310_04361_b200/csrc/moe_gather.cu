@@ -27,6 +27,11 @@
 //               gathers (cp.async.bulk.tensor tile::gather4: no fence, but about 80 cycles per 512-byte gather).
 //               The stage period stays at about half a microsecond per 128 x 64 tile of gathered rows.
 //   warps 6-13  epilogue: tcgen05.ld, bias, activation, selection bits, 32-byte stores to the token's row of H
+// Gated layers: a cluster of two CTAs shares tiles of 256 rows (tcgen05.mma.cta_group::2).  Each gathers its own 128 rows and
+// stages half of the weight rows (the leader W1's, its peer W_gate's), so that a k-block brings 32 KB into an SM instead of 48 and
+// the ring holds six instead of four; the leader's scheduler and MMA warps work for both.  Llama-shaped layer, up projection
+// back to back at 8192 tokens: 984 -> 883 us at u = 0.62 (0.62 -> 0.55 us a k-block: the gathered rows remain the bound), 436 -> 386
+// at 0.24; at 2560 tokens 350 -> 310 and 227 -> 192.
 // Every wait is bounded (status D2D_ERR_TIMEOUT), all roles meet at the final barrier, TMEM is freed.
 #include "moe_gather.cuh"
 #include "tc_common.cuh"
@@ -89,12 +94,14 @@ __host__ __device__ constexpr int pow2_cols(int v) { return v <= 32 ? 32 : v <= 
 // The MMA warp's work for one tile: nkb k-blocks from the stage ring into the accumulator at `acc`.  The A tiles were
 // written by cp.async (generic proxy) and their arrival is observed through the stage's barrier; the proxy fence that
 // makes them visible to the tensor core's (async-proxy) reads is executed here, between that observation and the MMAs.
+// PAIR: the leader's warp, for both CTAs; the peer's A tiles are announced to this CTA's barrier (see forward_tile).
+template <bool PAIR = false>
 __device__ __forceinline__ bool mma_tile(uint8_t *smem, uint64_t *bar_full, uint64_t *bar_empty, uint64_t *acc_full, uint32_t acc,
                                          uint32_t idesc, int nkb, int stages, int stage_bytes, uint32_t &it, int32_t *status)
 {
     for (int kb = 0; kb < nkb; ++kb, ++it) {
         const uint32_t s = it % (uint32_t)stages, round = it / (uint32_t)stages;
-        if (!mbar_wait_warp(smem_u32(&bar_full[s]), round & 1u, status)) return false;
+        if (!mbar_wait_warp<PAIR>(smem_u32(&bar_full[s]), round & 1u, status)) return false;
         fence_async_smem();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
@@ -103,23 +110,49 @@ __device__ __forceinline__ bool mma_tile(uint8_t *smem, uint64_t *bar_full, uint
 #pragma unroll
             for (int k = 0; k < BK / UMMA_K; ++k) {
                 const uint64_t koff = (uint64_t)((k * UMMA_K * 2) >> 4);
-                umma_bf16(acc, da + koff, db + koff, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                if (PAIR) umma_bf16_pair(acc, da + koff, db + koff, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+                else umma_bf16(acc, da + koff, db + koff, idesc, (kb > 0 || k > 0) ? 1u : 0u);
             }
-            umma_commit(smem_u32(&bar_empty[s]));
+            if (PAIR) umma_commit_pair(smem_u32(&bar_empty[s]));
+            else umma_commit(smem_u32(&bar_empty[s]));
         }
         __syncwarp();
     }
-    if (elect_one()) umma_commit(smem_u32(acc_full));
+    if (elect_one()) {
+        if (PAIR) umma_commit_pair(smem_u32(acc_full));
+        else umma_commit(smem_u32(acc_full));
+    }
     __syncwarp();
+    return true;
+}
+
+// Pairs, the peer's side: A stages that have landed here are announced to the leader, whose instructions make this SM's tensor
+// core read them.  The rows stay in this SM and the proxy fence has ordered them, so the arrival itself is relaxed: as a release at
+// cluster scope it waited for the gather's copies in flight and took longer than a k-block (Llama-shaped layer 1985 us instead of
+// 1600).
+__device__ __forceinline__ bool forward_tile(uint64_t *bar_full, int nkb, int stages, uint32_t &it, int32_t *status)
+{
+    for (int kb = 0; kb < nkb; ++kb, ++it) {
+        const uint32_t s = it % (uint32_t)stages, round = it / (uint32_t)stages;
+        if (!mbar_wait_warp(smem_u32(&bar_full[s]), round & 1u, status)) return false;
+        fence_async_smem();
+        if (elect_one())
+            asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_to_cta(smem_u32(&bar_full[s]), 0)) : "memory");
+        __syncwarp();
+    }
     return true;
 }
 
 // The scheduler warp's whole job (see the file header): draws sub-chunks of groups from the device counters, compacts
 // the tokens that keep the group into the FIFO, emits tiles through the descriptor ring, ends the stream with a
 // sentinel, and lets the CTA that finishes last reset the counters.
+// PAIR: the leader's, for both CTAs: tiles of up to 256 rows, the first 128 the leader's; FIFO and descriptors go to both.
+template <bool PAIR = false>
 __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *fifo, uint64_t *tile_full, uint64_t *tile_empty,
                                               TileDesc *tdesc, uint32_t *live, int lane)
 {
+    constexpr int TM = PAIR ? 2 * BM : BM;
+    const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     const int Ng = p.n_groups, SUB = p.sub, n_sub = (p.T + SUB - 1) / SUB;        // SUB is a multiple of 256
     // Groups the CTAs work in at the same time.  The host's value keeps that many groups' weight rows in L2.  When
     // few tokens keep a group, a visit of a CTA to a group should still yield several full tiles (its last tile is
@@ -129,7 +162,7 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
     if (p.n_sel) {
         const float rho = fminf((float)__ldcg(p.n_sel) / ((float)p.T * (float)(Ng * p.g)), 1.0f);
         const float u = fmaxf(1.0f - __expf((float)p.g * log1pf(-fminf(rho, 0.999f))), 1e-6f);
-        const float need = p.visit_tiles * (float)BM * (float)gridDim.x / (u * (float)p.T);
+        const float need = p.visit_tiles * (float)TM * (float)n_workers / (u * (float)p.T);
         const int w = need >= (float)Ng ? Ng : (int)need;
         Wn = w > Wn ? w : Wn;
     }
@@ -139,12 +172,19 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
     bool ok = true;
     auto emit = [&](uint32_t start, int n_rows, int group) -> bool {
         const uint32_t sl = tile_seq % TR, use = tile_seq / TR;
-        if (!mbar_wait_warp(smem_u32(&tile_empty[sl]), (use & 1u) ^ 1u, p.status)) return false;
+        if (!mbar_wait_warp<PAIR>(smem_u32(&tile_empty[sl]), (use & 1u) ^ 1u, p.status)) return false;
         __syncwarp();                                     // the FIFO entries written by all lanes are ordered before the arrival
         if (lane == 0) {
             tdesc[sl].start = (int)start;
             tdesc[sl].n_rows = n_rows;
             tdesc[sl].group = group;
+            if (PAIR) {
+                const uint32_t to = map_to_cta(smem_u32(&tdesc[sl]), 1);
+                st_cluster_u32(to, start);
+                st_cluster_u32(to + 4, (uint32_t)n_rows);
+                st_cluster_u32(to + 8, (uint32_t)group);
+                mbar_arrive_cluster(map_to_cta(smem_u32(&tile_full[sl]), 1));
+            }
             mbar_arrive(smem_u32(&tile_full[sl]));
         }
         ++tile_seq;
@@ -155,7 +195,7 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
     // rows stay in L2 while the token rows stream by.  Before it picks its next group a CTA takes a snapshot of all
     // counters (one round trip for the whole warp) and skips the groups that are used up: a counter only grows, so
     // "used up" is final and the walk over the order below never has to go back.
-    int j = 0, G = (int)blockIdx.x % Wn;                  // position in the order: lane (blockIdx.x + j) % Wn, group G
+    int j = 0, G = worker % Wn;                  // position in the order: lane (blockIdx.x + j) % Wn, group G
     while (ok) {
         for (int base = 0; base < Ng; base += 32) {
             const int gi = base + lane;
@@ -168,7 +208,7 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
             G += Wn;
             if (G >= Ng) {
                 ++j;
-                G = ((int)blockIdx.x + j) % Wn;
+                G = (worker + j) % Wn;
             }
         }
         __syncwarp();                                     // everyone has read the snapshot before it is rewritten
@@ -199,12 +239,16 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
                 for (int q = 0; q < 8; ++q) {
                     const bool keep = bits[q] != 0u;
                     const uint32_t bk = __ballot_sync(0xffffffffu, keep);
-                    if (keep) fifo[(head + __popc(bk & lower)) % FIFO_CAP] = (uint32_t)(t0 + q * 32 + lane);
+                    if (keep) {
+                        uint32_t *at = fifo + (head + __popc(bk & lower)) % FIFO_CAP;
+                        *at = (uint32_t)(t0 + q * 32 + lane);
+                        if (PAIR) st_cluster_u32(map_to_cta(smem_u32(at), 1), (uint32_t)(t0 + q * 32 + lane));
+                    }
                     head += __popc(bk);
                 }
-                while (head - emitted >= (uint32_t)BM && ok) {
-                    ok = emit(emitted % FIFO_CAP, BM, G);
-                    emitted += BM;
+                while (head - emitted >= (uint32_t)TM && ok) {
+                    ok = emit(emitted % FIFO_CAP, TM, G);
+                    emitted += TM;
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q) bits[q] = bits_next[q];
@@ -222,14 +266,14 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
     if (lane == 0) {
         __threadfence();
         const int done = atomicAdd(p.ctr + Ng, 1);
-        if (done == (int)gridDim.x - 1) {
+        if (done == n_workers - 1) {
             for (int i = 0; i <= Ng; ++i) p.ctr[i] = 0;
             __threadfence();
         }
     }
 }
 
-template <int ACT, bool GATED>
+template <int ACT, bool GATED, bool PAIR>
 __global__ void __launch_bounds__(NTHREADS, 1)
 moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_wg, const GatherParams p)
 {
@@ -246,30 +290,37 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
     const int n_mma = GATED ? 2 * p.gs : p.gs;              // columns of one MMA = accumulator columns of a tile
     const uint32_t buf_cols = (uint32_t)pow2_cols(n_mma);
     const uint32_t tmem_cols = 2u * buf_cols < 32u ? 32u : 2u * buf_cols;
+    const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;      // 0: the CTA that schedules and issues the MMAs
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
             // the W1 request (with its byte count) + one arrival per gather thread, triggered when its copies have landed
-            mbar_init(smem_u32(&bar_full[s]), 1 + N_GATHER_WARPS * 32);
+            // (pairs: the leader's also counts the peer's announcement, whose own barrier counts its gather threads only)
+            mbar_init(smem_u32(&bar_full[s]), PAIR ? N_GATHER_WARPS * 32 + (rank == 0 ? 2 : 0) : 1 + N_GATHER_WARPS * 32);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&bar_acc_full[b]), 1);
-            mbar_init(smem_u32(&bar_acc_empty[b]), N_EPI_WARPS);
+            mbar_init(smem_u32(&bar_acc_empty[b]), PAIR ? 2 * N_EPI_WARPS : N_EPI_WARPS);
         }
         for (int t = 0; t < TR; ++t) {
             mbar_init(smem_u32(&tile_full[t]), 1);
-            mbar_init(smem_u32(&tile_empty[t]), N_GATHER_WARPS + 1 + N_EPI_WARPS);
+            mbar_init(smem_u32(&tile_empty[t]), (PAIR ? 2 : 1) * (N_GATHER_WARPS + 1 + N_EPI_WARPS));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == WARP_MMA) {
+    if (warp == WARP_MMA && PAIR) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)), "r"(tmem_cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else if (warp == WARP_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)), "r"(tmem_cols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (PAIR) cluster_sync_all();          // the peer's barriers are initialised before anything signals them
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
     // everything above overlaps the tail of the previous kernel of the stream; the mask (and x) may be its output
@@ -279,26 +330,47 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
     const long long n_sel_now = p.n_sel ? (long long)__ldcg(p.n_sel) : 0;
     const bool run = p.n_sel == nullptr || (n_sel_now > p.n_sel_min && n_sel_now <= p.n_sel_max);      // (-1, LLONG_MAX]: always
 
-    if (run && warp == WARP_SCHED) {
-        run_scheduler(p, fifo, tile_full, tile_empty, tdesc, live, lane);
-    } else if (run && warp == WARP_MMA) {
-        // ------------------------------------------------------------------ MMA issuer (whole warp walks, one lane issues)
-        const uint32_t idesc = instr_desc_bf16(BM, n_mma);
+    // a tile's descriptor has been read: back to the scheduler (the leader's)
+    auto tile_release = [&](uint32_t sl) {
+        if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&tile_empty[sl]), 0));
+        else mbar_arrive(smem_u32(&tile_empty[sl]));
+    };
+    if (run && PAIR && rank != 0 && warp == WARP_SCHED) {
+        // the leader's scheduler works for both CTAs
+    } else if (run && PAIR && rank != 0 && warp == WARP_MMA) {
+        // ------------------------------------------------------------------ the peer's: announce the A stages to the leader
         uint32_t it = 0;
         bool ok = true;
         for (uint32_t ti = 0; ok; ++ti) {
             const uint32_t sl = ti % TR;
-            ok = mbar_wait_warp(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
+            ok = mbar_wait_warp<PAIR>(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
             if (!ok) break;
             const int n_rows = tdesc[sl].n_rows;
             __syncwarp();
             if (n_rows < 0) break;
-            if (elect_one()) mbar_arrive(smem_u32(&tile_empty[sl]));
+            if (elect_one()) tile_release(sl);
+            ok = forward_tile(bar_full, nkb, p.stages, it, p.status);
+        }
+    } else if (run && warp == WARP_SCHED) {
+        run_scheduler<PAIR>(p, fifo, tile_full, tile_empty, tdesc, live, lane);
+    } else if (run && warp == WARP_MMA) {
+        // ------------------------------------------------------------------ MMA issuer (whole warp walks, one lane issues)
+        const uint32_t idesc = instr_desc_bf16(PAIR ? 2 * BM : BM, n_mma);
+        uint32_t it = 0;
+        bool ok = true;
+        for (uint32_t ti = 0; ok; ++ti) {
+            const uint32_t sl = ti % TR;
+            ok = mbar_wait_warp<PAIR>(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
+            if (!ok) break;
+            const int n_rows = tdesc[sl].n_rows;
+            __syncwarp();
+            if (n_rows < 0) break;
+            if (elect_one()) tile_release(sl);
             const uint32_t buf = ti & 1u, use = ti >> 1;
-            ok = mbar_wait_warp(smem_u32(&bar_acc_empty[buf]), (use & 1u) ^ 1u, p.status);
+            ok = mbar_wait_warp<PAIR>(smem_u32(&bar_acc_empty[buf]), (use & 1u) ^ 1u, p.status);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            ok = mma_tile(smem, bar_full, bar_empty, &bar_acc_full[buf], tmem_base + buf * buf_cols, idesc, nkb, p.stages, p.stage_bytes, it,
+            ok = mma_tile<PAIR>(smem, bar_full, bar_empty, &bar_acc_full[buf], tmem_base + buf * buf_cols, idesc, nkb, p.stages, p.stage_bytes, it,
                           p.status);
         }
     } else if (run && warp >= WARP_GATHER0 && warp < WARP_EPI0) {
@@ -310,28 +382,34 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
         bool ok = true;
         for (uint32_t ti = 0; ok; ++ti) {
             const uint32_t sl = ti % TR;
-            ok = mbar_wait_warp(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
+            ok = mbar_wait_warp<PAIR>(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
             if (!ok) break;
             const int start = tdesc[sl].start, n_rows = tdesc[sl].n_rows, G = tdesc[sl].group;
             if (n_rows < 0) break;
             const __nv_bfloat16 *src[PASSES];
 #pragma unroll
             for (int j = 0; j < PASSES; ++j) {
-                int r = rbase + ROWS_PER_PASS * j;
+                const int r = rank * BM + rbase + ROWS_PER_PASS * j;
                 // rows past the end of a ragged tile are zero-filled (no memory traffic) and never stored
                 src[j] = r < n_rows ? p.x + (size_t)fifo[(uint32_t)(start + r) % FIFO_CAP] * p.d + chunk * 8 : nullptr;
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tile_empty[sl]));
+            if (lane == 0) tile_release(sl);
             for (int kb = 0; kb < nkb; ++kb, ++it) {
                 const uint32_t s = it % (uint32_t)p.stages, round = it / (uint32_t)p.stages;
                 ok = mbar_wait_warp(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, p.status);
                 if (!ok) break;
                 const uint32_t stage = smem_u32(smem + (size_t)s * p.stage_bytes), full = smem_u32(&bar_full[s]);
                 if (gw == 0 && elect_one()) {
-                    mbar_expect_tx(full, (uint32_t)(p.stage_bytes - A_BYTES));
-                    tma_load_2d(stage + A_BYTES, &tm_w1, kb * BK, G * p.gs, full);
-                    if (GATED) tma_load_2d(stage + A_BYTES + p.gs * 128, &tm_wg, kb * BK, G * p.gs, full);
+                    if (PAIR) {
+                        // the leader stages the up rows, its peer the gate rows; both are credited to the leader's barrier
+                        if (rank == 0) mbar_expect_tx(full, 2u * (uint32_t)(p.stage_bytes - A_BYTES));
+                        tma_load_2d_pair(stage + A_BYTES, rank == 0 ? &tm_w1 : &tm_wg, kb * BK, G * p.gs, map_to_cta(full, 0));
+                    } else {
+                        mbar_expect_tx(full, (uint32_t)(p.stage_bytes - A_BYTES));
+                        tma_load_2d(stage + A_BYTES, &tm_w1, kb * BK, G * p.gs, full);
+                        if (GATED) tma_load_2d(stage + A_BYTES + p.gs * 128, &tm_wg, kb * BK, G * p.gs, full);
+                    }
                 }
                 const bool in_k = kb * BK + chunk * 8 < p.d;                       // zero fill past K
 #pragma unroll
@@ -353,15 +431,15 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
         bool ok = true;
         for (uint32_t ti = 0; ok; ++ti) {
             const uint32_t sl = ti % TR;
-            ok = mbar_wait_warp(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
+            ok = mbar_wait_warp<PAIR>(smem_u32(&tile_full[sl]), (ti / TR) & 1u, p.status);
             if (!ok) break;
             const int start = tdesc[sl].start, n_rows = tdesc[sl].n_rows, G = tdesc[sl].group;
             if (n_rows < 0) break;
-            const int r = quad * 32 + lane;
+            const int r = rank * BM + quad * 32 + lane;
             const bool valid = r < n_rows;
             const uint32_t tok = valid ? fifo[(uint32_t)(start + r) % FIFO_CAP] : 0u;
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&tile_empty[sl]));
+            if (lane == 0) tile_release(sl);
             // which experts of the group this token keeps (the load is covered by the wait for the accumulator)
             const int e0 = G * p.g;
             const uint32_t bits = valid ? __ldg(p.mask + (size_t)tok * p.W + (e0 >> 5)) >> (e0 & 31) : 0u;
@@ -428,13 +506,19 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bar_acc_empty[buf]));
+            if (lane == 0) {
+                if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&bar_acc_empty[buf]), 0));
+                else mbar_arrive(smem_u32(&bar_acc_empty[buf]));
+            }
         }
     }
 
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == WARP_MMA)
+    if (PAIR) cluster_sync_all();          // neither CTA releases shared memory or TMEM while the other may still use it
+    if (warp == WARP_MMA && PAIR)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
+    else if (warp == WARP_MMA)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(tmem_cols) : "memory");
 }
 
@@ -1044,11 +1128,11 @@ bool ensure_attr(const void *kern, bool (&done)[64])
     return true;
 }
 
-template <int ACT, bool GATED>
+template <int ACT, bool GATED, bool PAIR = false>
 d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
 {
     const int gs = a.g * a.s;
-    const int b_rows = GATED ? 2 * gs : gs;
+    const int b_rows = GATED && !PAIR ? 2 * gs : gs;        // staged by one CTA
     GatherParams p = {};
     p.x = (const __nv_bfloat16 *)a.x; p.mask = a.mask; p.b1 = (const __nv_bfloat16 *)a.b1; p.H = (__nv_bfloat16 *)a.H;
     p.status = a.status; p.ctr = a.ctr; p.n_sel = a.n_sel; p.n_sel_min = a.n_sel_min; p.n_sel_max = a.n_sel_max;
@@ -1059,11 +1143,11 @@ d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
     int stages = (192 * 1024) / p.stage_bytes;
     p.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
     // about 48 MB of weight rows in flight: the rest of L2 holds the token rows and the outputs
-    const long long group_bytes = (long long)b_rows * a.d * 2;
+    const long long group_bytes = (long long)gs * (GATED ? 2 : 1) * a.d * 2;
     long long window = (48ll << 20) / (group_bytes > 0 ? group_bytes : 1);
     p.window = (int)(window < 4 ? 4 : window > p.n_groups ? p.n_groups : window);
     if (p.window > p.n_groups) p.window = p.n_groups;
-    p.visit_tiles = 8.0f;
+    p.visit_tiles = PAIR ? 4.0f : 8.0f;
     // tokens per draw: about eight draws per CTA (the CTAs then finish together), 256 .. 1024
     const long long want = (long long)a.T * p.n_groups / (8ll * d2d_tc_sm_count());
     p.sub = want >= 1024 ? 1024 : want >= 512 ? 512 : 256;
@@ -1076,32 +1160,34 @@ d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
     } else {
         twg = tw1;
     }
-    auto kern = moe_gather_up_kernel<ACT, GATED>;
+    auto kern = moe_gather_up_kernel<ACT, GATED, PAIR>;
     static bool attr_set[64] = {};
     if (!ensure_attr((const void *)kern, attr_set)) return D2D_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(d2d_tc_sm_count(), 1, 1);
+    cfg.gridDim = dim3(PAIR ? d2d_tc_sm_count() & ~1 : d2d_tc_sm_count(), 1, 1);
     cfg.blockDim = dim3(NTHREADS, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = PAIR ? 2 : 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 2 : 1;
     const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, tw1, twg, p);
     D2D_LAUNCHED(1);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
-template <bool GATED>
+template <bool GATED, bool PAIR = false>
 d2d_status launch_act(const d2d_gather_args &a, cudaStream_t st)
 {
     switch (a.act) {
-    case D2D_ACT_RELU: return launch<D2D_ACT_RELU, GATED>(a, st);
-    case D2D_ACT_GELU_ERF: return launch<D2D_ACT_GELU_ERF, GATED>(a, st);
-    case D2D_ACT_GELU_TANH: return launch<D2D_ACT_GELU_TANH, GATED>(a, st);
-    case D2D_ACT_SILU: return launch<D2D_ACT_SILU, GATED>(a, st);
+    case D2D_ACT_RELU: return launch<D2D_ACT_RELU, GATED, PAIR>(a, st);
+    case D2D_ACT_GELU_ERF: return launch<D2D_ACT_GELU_ERF, GATED, PAIR>(a, st);
+    case D2D_ACT_GELU_TANH: return launch<D2D_ACT_GELU_TANH, GATED, PAIR>(a, st);
+    case D2D_ACT_SILU: return launch<D2D_ACT_SILU, GATED, PAIR>(a, st);
     }
     return D2D_ERR_INVALID_ARG;
 }
@@ -1129,7 +1215,7 @@ d2d_status d2d_moe_gather_up(const d2d_gather_args &a, cudaStream_t st)
 {
     if (a.T <= 0) return D2D_OK;
     if (a.g < 1 || a.g > 32 || a.n_experts > 2048) return D2D_ERR_UNSUPPORTED;
-    return a.w_gate ? launch_act<true>(a, st) : launch_act<false>(a, st);
+    return a.w_gate ? launch_act<true, true>(a, st) : launch_act<false>(a, st);
 }
 
 bool d2d_moe_down_masked_supports(const d2d_layer_desc &D)

@@ -61,6 +61,34 @@ def _structured_mask(cfg, T, p, seed):
     return G
 
 
+# gated layers: pairs of CTAs share tiles of 256 rows, the first 128 the leader's.  Rows kept per group around both limits, none and
+# all of them, groups of 32 to 128 neurons, a width that is not a multiple of a k-block and fewer k-blocks than stages
+@pytest.mark.parametrize("d,g", [(256, 4), (208, 1), (992, 2)])
+def test_gathered_pairs_at_the_edges_of_their_tiles(api, d, g):
+    T, s, counts = 700, 32, (0, 1, 127, 128, 129, 255, 256, 257, 511, 512, 513, 700)
+    E = len(counts) * g + (-len(counts) * g) % 32
+    cfg = wl.LayerConfig("pair", "bf16", d=d, d_ff=E * s, E=E, d_h=64, act="silu", T=T, gated=True, token_sigma=0.5, seed=23)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    layer.set_expert_path("gather", group=g)
+    xd, rng = api.to_device(x, cfg.dtype), np.random.default_rng(d)
+    G = np.zeros((T, E), np.uint8)
+    for i, n in enumerate(counts):
+        G[rng.permutation(T)[:n], i * g + rng.integers(0, g, n)] = 1
+    r = _routing(api, G, E)
+    want = layer.expert_up_fwd(xd, r).view(torch.int16).cpu().numpy().reshape(T, E, s)
+    for _ in range(2):                               # the second call starts on the counters the first one left
+        H = torch.full((T, cfg.d_ff), float("nan"), dtype=torch.bfloat16, device="cuda")
+        got = layer.expert_up_gather_fwd(xd, r, H).view(torch.int16).cpu().numpy().reshape(T, E, s)
+        assert np.array_equal(got[G.astype(bool)], want[G.astype(bool)])      # the same products in the same order
+        untouched = ~np.repeat(G.reshape(T, E // g, g).any(2), g, axis=1)
+        assert (got[untouched] == got[untouched][0, 0]).all()
+    y = layer.moe_ffn_fwd(xd, r)
+    y_ref = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[cfg.act], G)
+    assert r.status == 0 and _rel_err(y.float().cpu().numpy(), y_ref) <= TOL_Y
+    layer.close()
+
+
 # (workload, tokens, experts per group or 0 = default, densities)
 GATHER_CASES = [
     ("bert", 700, 0, (0.0, 0.03, 0.3, 1.0)),        # s = 24, default g = 4 (96 columns), ragged 256-token sub-chunk
