@@ -218,6 +218,24 @@ static double default_fused_rho_max(int g)
     return 1.0 - pow(1.0 - 0.08, 1.0 / g);
 }
 
+// The form of the expert step as far as it is known before the launch: the one that is set, or the dense pair where the shape or the
+// size leaves no choice.
+// The automatic choice costs a few launches that return at once and the overlap of the router with the masked dense
+// kernel's main loops (ViT-shaped layer, 1.2e11 FLOP: 241 us against 224 us at every density when the line was drawn), so it
+// is made only for problems whose up projection takes long enough (2e11 FLOP, about 150 us of tensor-core time) that this is
+// little.  What the line gives away: on the ViT-shaped layer the gathered pair wins below rho = 0.03 (205 against 219 us at
+// 0.023), and on the paper's shape at 12608 tokens (6e10 FLOP, expert step) the fused kernel wins up to rho = 0.17 (58 / 73 / 87
+// against 110 us at 0.01 / 0.05 / 0.1).
+static int path_before_launch(const d2d_layer *L, int T, bool counted)
+{
+    const d2d_layer_desc &D = L->desc;
+    int path = L->expert_path;
+    if (L->gather_group <= 0) path = D2D_PATH_DENSE;
+    const double up_flop = 2.0 * (double)T * D.d * D.d_ff * (D.gated ? 2.0 : 1.0);
+    if (path == D2D_PATH_AUTO && (up_flop < kAutoMinUpFlop || !counted)) path = D2D_PATH_DENSE;
+    return path;
+}
+
 // Expert step of bf16 batches above the decode sizes, on the tensor cores.
 //   up projection    two kernels that compute the same H = G * A(x W1^T + b1):
 //     masked dense   one GEMM over all of d_ff, the selection applied as a mask in the epilogue; its time does not
@@ -234,19 +252,10 @@ static double default_fused_rho_max(int g)
 // on this stream is the router, which writes only the mask (and R, k), so that a forced masked dense up projection
 // may overlap it with its main loops and draw its tiles dynamically.
 static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *y,
-                                    void *ws, cudaStream_t st, int *up_counter, const int32_t *n_sel)
+                                    void *ws, cudaStream_t st, int *up_counter, const int32_t *n_sel, bool lists)
 {
     const d2d_layer_desc &D = L->desc;
-    int path = L->expert_path;
-    if (L->gather_group <= 0) path = D2D_PATH_DENSE;
-    // The automatic choice costs a few launches that return at once and the overlap of the router with the masked dense
-    // kernel's main loops (ViT-shaped layer, 1.2e11 FLOP: 241 us against 224 us at every density when the line was drawn), so it
-    // is made only for problems whose up projection takes long enough (2e11 FLOP, about 150 us of tensor-core time) that this is
-    // little.  What the line gives away: on the ViT-shaped layer the gathered pair wins below rho = 0.03 (205 against 219 us at
-    // 0.023), and on the paper's shape at 12608 tokens (6e10 FLOP, expert step) the fused kernel wins up to rho = 0.17 (58 / 73 / 87
-    // against 110 us at 0.01 / 0.05 / 0.1).
-    const double up_flop = 2.0 * (double)T * D.d * D.d_ff * (D.gated ? 2.0 : 1.0);
-    if (path == D2D_PATH_AUTO && (up_flop < kAutoMinUpFlop || !n_sel)) path = D2D_PATH_DENSE;
+    const int path = path_before_launch(L, T, n_sel != nullptr);
     const double rho_max = L->gather_rho_max >= 0.0 ? L->gather_rho_max : default_gather_rho_max(D, L->gather_group, T);
     long long n_sel_max = (long long)(rho_max * (double)T * (double)D.n_experts);
     d2d_status rc;
@@ -323,11 +332,12 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     dn.k_splits = k_splits;
     dn.partial = partial;
     dn.partial_zero = path == D2D_PATH_DENSE;
+    if (lists) dn.lists = d2d_list_job_for(r, 1, T, D.n_experts, false);
     return d2d_gemm_tc(dn, st);
 }
 
 d2d_status d2d_launch_moe_ffn(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *y,
-                              void *ws, size_t ws_bytes, cudaStream_t st, int *up_counter, int small_fused, const int32_t *n_sel)
+                              void *ws, size_t ws_bytes, cudaStream_t st, int *up_counter, int small_fused, const int32_t *n_sel, bool lists)
 {
     if (ws_bytes < d2d_moe_ffn_ws_bytes(L, T)) return D2D_ERR_WORKSPACE;
     if (d2d_use_decode_ffn(L, 1, T)) {
@@ -338,7 +348,7 @@ d2d_status d2d_launch_moe_ffn(const d2d_layer *L, const void *x, int T, const d2
         return d2d_decode_ffn(L->desc, 1, a, x, T, false, st);
     }
     if (use_small_ffn(L, T)) return has_lists(r) ? d2d_small_ffn(L, x, T, r, y, ws, st, small_fused) : D2D_ERR_INVALID_ARG;
-    if (use_dense_masked(L, T)) return launch_tc_experts(L, x, T, r, y, ws, st, up_counter, n_sel ? n_sel : r->n_sel);
+    if (use_dense_masked(L, T)) return launch_tc_experts(L, x, T, r, y, ws, st, up_counter, n_sel ? n_sel : r->n_sel, lists);
     return d2d_launch_moe_ffn_token(L, x, T, r, y, st);
 }
 
@@ -816,6 +826,13 @@ static d2d_status join_lists(const d2d_layer *L, cudaStream_t st)
     return cudaEventRecord(L->ev_join, L->side_stream) == cudaSuccess && cudaStreamWaitEvent(st, L->ev_join, 0) == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
+// Whether the down projection builds the lists on the side: the dense pair, few tokens, no token-major dual
+static bool lists_ride(const d2d_layer *L, int T, const d2d_routing *r)
+{
+    const d2d_layer_desc &D = L->desc;
+    return !r->tok_off && path_before_launch(L, T, true) == D2D_PATH_DENSE && d2d_lists_ride(T, D.n_experts, d2d_gemm_tc_splits(T, D.d, D.d_ff));
+}
+
 d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float tau, void *y,
                          float *R_out, d2d_routing *routing, void *ws, size_t ws_bytes, void *stream)
 {
@@ -824,6 +841,7 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     cudaStream_t st = (cudaStream_t)stream;
     const int E = layer->desc.n_experts;
     const bool lists = has_lists(routing);
+    bool fork = false, ride = false;                         // lists beside the experts: on the side stream, or by the down projection
     if (T == 0) return lists ? d2d_launch_select(nullptr, 0, E, tau, 0, routing, ws, st) : D2D_OK;
     if (!x || !y || !aligned16(x) || !aligned16(y) || (R_out && !aligned16(R_out))) return D2D_ERR_INVALID_ARG;
     const ws_layout w = layout_for(layer, T);
@@ -848,12 +866,14 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
         // expert kernels read only the mask: the per-expert lists (when the caller wants them) are built on the side stream while
         // they run (the small metadata CTAs fit beside the persistent CTAs), join at the end.
         rc = d2d_router_fused(layer, x, T, tau, 1, R_out, routing->mask, routing->k, routing->status, st, ksum);
-        if (rc == D2D_OK && lists) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
+        ride = lists && lists_ride(layer, T, routing);
+        fork = lists && !ride;
+        if (rc == D2D_OK && fork) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
         if (rc != D2D_OK) return rc;
         // tile counter of the up projection: layer-owned, zero at creation and reset by the kernel that used it, so no memset node
         // sits in front of the router (the up projection may begin while the router is still running)
-        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, (int *)(layer->tickets + 32), 0, ksum + 4);
-        return lists && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
+        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, (int *)(layer->tickets + 32), 0, ksum + 4, ride);
+        return fork && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
     case FORM_FUSED_ROUTER_LISTS:
         if (cudaMemsetAsync(routing->status, 0, sizeof(int32_t), st) != cudaSuccess) return D2D_ERR_CUDA;
         rc = d2d_router_fused(layer, x, T, tau, 1, R_out, routing->mask, routing->k, routing->status, st, nullptr);
@@ -876,10 +896,12 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
             rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
             if (rc == D2D_OK) rc = d2d_launch_dynk_mask(R, T, E, tau, routing, ksum, st);
         }
-        if (rc == D2D_OK && lists) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
+        ride = lists && lists_ride(layer, T, routing);
+        fork = lists && !ride;
+        if (rc == D2D_OK && fork) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
         if (rc != D2D_OK) return rc;
-        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, nullptr, 0, ksum + 4);
-        return lists && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
+        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, nullptr, 0, ksum + 4, ride);
+        return fork && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
     case FORM_PLAIN:
         rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);
         if (rc == D2D_OK) rc = d2d_launch_select(R, T, E, tau, 0, routing, base + w.sel_off, st);

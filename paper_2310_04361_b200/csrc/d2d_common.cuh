@@ -128,10 +128,11 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
                              void *ws, cudaStream_t st, int mask_ready = 0, unsigned int *zero_ticket = nullptr);
 
 // up_counter: see launch_tc_experts (NULL unless the fused router was launched just before on `st`)
+// lists: r's lists are to be built on the side (only where d2d_api.cu's lists_ride says so)
 // n_sel: device word that holds the number of selected pairs when the expert kernels start (NULL: r->n_sel)
 d2d_status d2d_launch_moe_ffn(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *y,
                               void *ws, size_t ws_bytes, cudaStream_t st, int *up_counter = nullptr, int small_fused = 0,
-                              const int32_t *n_sel = nullptr);
+                              const int32_t *n_sel = nullptr, bool lists = false);
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T);
 size_t d2d_layer_ws_bytes(const d2d_layer *L, int T);      // workspace of a d2d_layer_fwd call with exactly T tokens
 

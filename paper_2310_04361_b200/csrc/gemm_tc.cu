@@ -46,6 +46,30 @@ struct EpiParams {
     int test_skip_load;              // test aid: CTA 0 never requests the A tile of its first k-block (see d2d_gemm_args)
 };
 
+// Lists a down projection builds before its first tile.  Launches without any do without the parameter: 80 bytes in two of a
+// layer's launches cost it 1 us.
+struct NoLists {};
+template <int N> struct ListsOf { typedef d2d_list_jobs<N> type; };
+template <> struct ListsOf<0> { typedef NoLists type; };
+__device__ __forceinline__ void build_lists(const NoLists &, int, int, int, uint8_t *) {}
+// by the epilogue warps, one mask word of one layer per CTA; scratch in the output buffers, which nothing uses yet
+template <int N> __device__ __forceinline__ void build_lists(const d2d_list_jobs<N> &j, int T, int ew, int lane, uint8_t *scratch)
+{
+    for (int i = (int)blockIdx.x; i < j.n * j.W; i += (int)gridDim.x) {
+        const auto sync = [] { asm volatile("bar.sync 1, 512;" ::: "memory"); };
+        const int l = N == 1 ? 0 : i / j.W;
+        d2d_lists::lists_of_word<16, 2>(j.l[l], i - l * j.W, T, j.E, j.W, ew, lane, reinterpret_cast<uint16_t *>(scratch),
+                                        reinterpret_cast<int *>(scratch + 2048), sync);
+        sync();
+    }
+}
+inline void set_lists(NoLists &, const d2d_gemm_args &) {}
+template <int N> void set_lists(d2d_list_jobs<N> &j, const d2d_gemm_args &g)
+{
+    j.n = g.lists.n; j.T = g.lists.T; j.E = g.lists.E; j.W = g.lists.W;
+    for (int l = 0; l < N; ++l) j.l[l] = g.lists.l[l];
+}
+
 // Tile index -> (row tile, column tile).  Plain order is row-major: CTAs that run together share a few rows of A and
 // sweep all of B, so B is streamed from HBM once per wave when A and B together exceed L2.  With bands, the tiles of
 // `band` consecutive row tiles are walked column by column: the band's rows of A stay in L2 while B is streamed once
@@ -131,10 +155,11 @@ __host__ __device__ constexpr int pow2_at_least(int v) { return v <= 32 ? 32 : v
 // A k-block then brings 16 + BN / 16 KB into an SM instead of 16 + BN / 8: the fill from L2 (about 117 GB/s per SM), not
 // the tensor pipe, bounds the single-CTA main loop.  Two accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the
 // next.  GATED: two B tiles (up, gate) share the A tile; the epilogue forms A(gate) * (up + bias).
-template <int BN, int STAGES, int EPI, int ACT, bool GATED, bool PAIR>
+template <int BN, int STAGES, int EPI, int ACT, bool GATED, bool PAIR, int LISTS>
 __global__ void __launch_bounds__(NTHREADS_V2) __maxnreg__(GATED ? 96 : 80)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-               const __grid_constant__ CUtensorMap tm_b2, const __grid_constant__ CUtensorMap tm_out, EpiParams ep, int M, int N, int K, int k_splits)
+               const __grid_constant__ CUtensorMap tm_b2, const __grid_constant__ CUtensorMap tm_out, EpiParams ep, int M, int N, int K, int k_splits,
+               const typename ListsOf<LISTS>::type lists)
 {
     constexpr int TM = PAIR ? 2 * BM : BM;                // rows of the tile a CTA (pair) computes
     // rows of B this CTA stages (of each matrix; a gated pair: the leader the up rows, its peer the gate rows, all BN of them)
@@ -416,6 +441,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
         uint32_t out_n = 0;                                 // output buffers used so far
         for (int i = (int)blockIdx.x * (N_EPI_WARPS * 32) + (int)threadIdx.x - 64; i < ep.zero_n; i += (int)gridDim.x * (N_EPI_WARPS * 32))
             ep.zero[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        build_lists(lists, M, ew, lane, out_s);
         for (uint32_t local = 0;; ++local) {
             const uint32_t buf = local & 1u, use = local >> 1;
             // ONE thread takes the item from the ring, works out its coordinates (integer divisions), waits for the accumulator
@@ -647,9 +673,13 @@ template <typename K> bool ensure_smem_attr(K kern, size_t smem, bool (&done)[64
     return true;
 }
 
-template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false>
+template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false, int LISTS = 0>
 d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
 {
+    if constexpr ((EPI == D2D_EPI_BIAS_BF16 || EPI == D2D_EPI_PARTIAL_F32) && LISTS == 0) {
+        if (g.lists.n == 1) return launch<BN, EPI, ACT, GATED, PAIR, 1>(g, st);
+        if (g.lists.n > 1) return launch<BN, EPI, ACT, GATED, PAIR, D2D_MAX_GROUP>(g, st);
+    }
     constexpr int B_ROWS = PAIR && !GATED ? BN / 2 : BN, TM = PAIR ? 2 * BM : BM;
     constexpr int STAGE_BYTES = BM * BK * 2 + (GATED && !PAIR ? 2 : 1) * B_ROWS * BK * 2;
     constexpr int STAGES = STAGE_BUDGET / STAGE_BYTES > 8 ? 8 : STAGE_BUDGET / STAGE_BYTES;
@@ -677,7 +707,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
         const cuuint32_t box[3] = {64, 32, 1};
         if (!d2d_tc_encode_map(&to, false, 3, g.out, dims, strides, box)) return D2D_ERR_CUDA;
     }
-    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED, PAIR>;
+    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED, PAIR, LISTS>;
     static bool attr_set[64] = {};
     if (!ensure_smem_attr(kern, SMEM, attr_set)) return D2D_ERR_CUDA;
     const int es = g.expert_size > 0 ? g.expert_size : 1;
@@ -686,6 +716,8 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
                  g.tile_counter, (g.pdl_late_wait && !g.n_sel && d2d_tc_pdl_enabled()) ? 1 : 0, gate_cat ? 1 : 0,
                  band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max, (float4 *)g.zero, g.zero ? (int)(g.zero_floats / 4) : 0,
                  (g.test_skip_load && !g.tile_counter && !g.pdl_late_wait && !g.n_sel) ? 1 : 0};
+    typename ListsOf<LISTS>::type lists = {};
+    set_lists(lists, g);
     const int k_splits = g.k_splits > 1 ? g.k_splits : 1;
     const int tiles = d2d_cdiv(g.N, BN) * d2d_cdiv(g.M, TM) * k_splits * batch;
     const int workers = PAIR ? d2d_tc_sm_count() / 2 : d2d_tc_sm_count();
@@ -703,7 +735,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = d2d_tc_pdl_enabled() ? 2 : 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits, lists);
     D2D_LAUNCHED(1);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }

@@ -5,6 +5,7 @@
 #include <cuda.h>
 
 #include "d2d_common.cuh"
+#include "lists.cuh"
 
 enum d2d_gemm_epilogue {
     D2D_EPI_RELU_BF16 = 0,   // out bf16 = relu(acc + bias)                 router layer 1
@@ -61,6 +62,9 @@ struct d2d_gemm_args {
     // work).  Cannot be combined with pdl_late_wait.
     const int32_t *n_sel;
     long long n_sel_max;
+    // Per-expert lists to build on the side (D2D_EPI_BIAS_BF16, d2d_lists_ride): by the epilogue warps, which wait for the first
+    // accumulator anyway; the masks must be there when the previous kernel of the stream has completed.  n = 0: none.
+    d2d_list_job lists;
     // Test aid for the failure-handling test (host-made fault, nothing traps or spins without bound): CTA 0 leaves out
     // the load of the A tile of its first k-block, so the barrier of that stage never completes; the bounded waits of
     // the MMA warp, the epilogue and the producer run out, D2D_ERR_TIMEOUT is recorded, every role reaches the final
@@ -70,6 +74,17 @@ struct d2d_gemm_args {
 
 // Number of K slices d2d_gemm_tc would use for a [M,N,K] down projection (1 = no split) and the float32 scratch it needs.
 int d2d_gemm_tc_splits(int M, int N, int K, int batch = 1);
+
+// Whether the lists of a batch can be left to the GEMM of its down projection: as many tokens as a CTA's epilogue warps take in one
+// go (512) or, before a main loop that is not split, in two.  On a stream of their own they cost the layer a launch, two events
+// and two waits between streams, and its call the programmatic launch behind it.  GPT-2-medium-shaped FFN, back to back: 30.8 ->
+// 26.8 us at 64 tokens, 34.7 -> 33.0 at 333, 43.2 -> 39.9 at 1000 (not split); split along K and in two goes they hold the
+// partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection that have no tile they held
+// up the down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
+static inline bool d2d_lists_ride(int T, int E, int k_splits)
+{
+    return T <= (k_splits > 1 ? 512 : 1024) && (long long)T * ((E + 31) / 32) <= 16384;
+}
 
 // Enqueues C = epilogue(A B^T).  Requires K % 8 == 0 and 16-byte aligned base pointers.
 d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st);

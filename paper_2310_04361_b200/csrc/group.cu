@@ -214,11 +214,17 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         const d2d_router_weights rw = {g->w_r1, g->b_r1, g->w_r2, g->b_r2};
         d2d_status rc = d2d_router_fused_group(g->layers, n, rw, x, T, tau, routing, mask_cat, n * W, st);
         if (rc != D2D_OK) return rc;
-        // per-expert metadata of every layer on the side stream, beside the GEMMs (which read only the merged mask)
-        if (cudaEventRecord(g->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(g->side_stream, g->ev_fork, 0) != cudaSuccess)
-            return D2D_ERR_CUDA;
-        rc = d2d_launch_lists(routing, n, T, E, base + w.sel_off, w.sel_each, g->side_stream);
-        if (rc != D2D_OK) return rc;
+        // per-expert metadata of every layer: by the down projection, or on the side stream beside the GEMMs (which read only the
+        // merged mask)
+        const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff, n);
+        bool ride = d2d_lists_ride(T, E, k_splits);
+        for (int l = 0; l < n; ++l) ride = ride && !routing[l].tok_off;
+        if (!ride) {
+            if (cudaEventRecord(g->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(g->side_stream, g->ev_fork, 0) != cudaSuccess)
+                return D2D_ERR_CUDA;
+            rc = d2d_launch_lists(routing, n, T, E, base + w.sel_off, w.sel_each, g->side_stream);
+            if (rc != D2D_OK) return rc;
+        }
         void *H = base + w.h_off;
         d2d_gemm_args up = {};
         up.tile_counter = g->up_counter;
@@ -226,7 +232,6 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         up.a = x; up.b = g->w1; up.bias = g->b1; up.out = H;
         up.M = T; up.N = n * D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
         up.mask = mask_cat; up.mask_words = n * W; up.expert_size = D.expert_size; up.status = routing[0].status;
-        const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff, n);
         float *partial = k_splits > 1 ? (float *)(base + w.partial_off) : nullptr;
         up.zero = partial; up.zero_floats = (long long)n * T * D.d;
         rc = d2d_gemm_tc(up, st);
@@ -237,8 +242,9 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         dn.k_splits = k_splits;
         dn.partial = partial;
         dn.partial_zero = 1;
+        if (ride) dn.lists = d2d_list_job_for(routing, n, T, E, false);
         rc = d2d_gemm_tc(dn, st);
-        if (cudaEventRecord(g->ev_join, g->side_stream) != cudaSuccess || cudaStreamWaitEvent(st, g->ev_join, 0) != cudaSuccess)
+        if (!ride && (cudaEventRecord(g->ev_join, g->side_stream) != cudaSuccess || cudaStreamWaitEvent(st, g->ev_join, 0) != cudaSuccess))
             return D2D_ERR_CUDA;
         return rc;
     }

@@ -13,6 +13,7 @@
 //                   lower lanes: tokens come out in ascending order
 //   dual kernels    exclusive scan of k -> tok_off; one warp per token writes tok_exp
 #include "d2d_common.cuh"
+#include "lists.cuh"
 
 namespace {
 
@@ -143,18 +144,6 @@ k_from_mask_kernel(const uint32_t *__restrict__ mask, int T, int W, int32_t *__r
 
 // ---------------------------------------------------------------------------- bucketing
 
-// Lane j returns the bitmap, over this warp's 32 tokens, of bit j of `word`.
-__device__ __forceinline__ uint32_t transpose_bits(uint32_t word, int lane)
-{
-    uint32_t col = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const uint32_t b = __ballot_sync(FULL, (word >> j) & 1u);
-        if (lane == j) col = b;
-    }
-    return col;
-}
-
 // Exclusive scan of one int per thread over a 256-thread CTA; returns the exclusive prefix and
 // leaves the CTA total in *total_out (shared).
 __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, int *total_out)
@@ -186,95 +175,18 @@ __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, i
 }
 
 // Lists of a batch small enough for every CTA to look at all of the mask: one CTA per mask word (32 experts) and layer, no
-// order between CTAs, so counts, offsets and lists take one launch and no scratch.  A CTA adds up the pairs of the words
-// before its own (what its first list starts at), counts its 32 experts per warp (a warp has a contiguous range of 32-token
-// groups), scans, and writes.  k != NULL: k and the status word are wanted too.  Bound by latency; as small as
-// bucket_count_scan_kernel, for the same reason.  What it saves is the host's time (two launches, a memset and, for a mask that
-// is given, two more): see d2d_launch_select for the line.
-struct ListsIO {
-    const uint32_t *mask;
-    int32_t *k, *counts, *offsets, *perm, *n_sel, *status;
-    long long capacity;
-};
-struct ListsGroup { ListsIO l[D2D_MAX_GROUP]; };
+// order between CTAs, so counts, offsets and lists take one launch and no scratch (lists.cuh).  k != NULL: k and the status word
+// are wanted too.  Bound by latency; as small as bucket_count_scan_kernel, for the same reason.  What it saves is the host's time
+// (two launches, a memset and, for a mask that is given, two more): see d2d_launch_select for the line.
 constexpr int LISTS_GROUPS = 4, LISTS_MAX_T = LISTS_GROUPS * TOKB;      // 32-token groups of a warp, held in registers
 
 __global__ void __launch_bounds__(TOKB, 6)
-lists_kernel(const __grid_constant__ ListsGroup g, int T, int E, int W)
+lists_kernel(const __grid_constant__ d2d_list_job g)
 {
-    constexpr int NWARP = TOKB / 32;
-    __shared__ uint16_t cnt[NWARP][32];
-    __shared__ int sums[NWARP];
-    const ListsIO &io = g.l[blockIdx.y];
-    const uint32_t *__restrict__ mask = io.mask;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x;
-    int before = 0;
-    for (int t = threadIdx.x; t < T; t += TOKB) {
-        const uint32_t *row = mask + (size_t)t * W;
-        int n = 0;
-        for (int i = 0; i < w; ++i) n += __popc(__ldg(row + i));
-        before += n;
-        if (io.k && w == W - 1) io.k[t] = n + __popc(__ldg(row + w));
-    }
-    before = __reduce_add_sync(FULL, before);
-    const int per = (T + TOKB - 1) / TOKB * 32;                 // tokens of a warp
-    const int t0 = warp * per, e = w * 32 + lane;
-    uint32_t col[LISTS_GROUPS];                                 // per group of 32 tokens: which of them keep expert e
-#pragma unroll
-    for (int i = 0; i < LISTS_GROUPS; ++i) {
-        const int t = t0 + i * 32 + lane;
-        col[i] = i * 32 < per && t < T ? __ldg(mask + (size_t)t * W + w) : 0u;
-    }
-    int mine = 0;
-#pragma unroll
-    for (int i = 0; i < LISTS_GROUPS; ++i) {
-        col[i] = transpose_bits(col[i], lane);
-        if (e >= E) col[i] = 0u;
-        mine += __popc(col[i]);
-    }
-    cnt[warp][lane] = (uint16_t)mine;
-    if (lane == 0) sums[warp] = before;
-    __syncthreads();
-    int total = 0, earlier = 0;
-    before = 0;
-#pragma unroll
-    for (int i = 0; i < NWARP; ++i) {
-        const int c = cnt[i][lane];
-        if (i < warp) earlier += c;
-        total += c;
-        before += sums[i];
-    }
-    int inc = total;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(FULL, inc, o);
-        if (lane >= o) inc += v;
-    }
-    const int first = before + inc - total;
-    if (warp == 0 && e < E) {
-        io.counts[e] = total;
-        io.offsets[e] = first;
-        if (e == E - 1) {
-            const int all = first + total;
-            io.offsets[E] = all;
-            *io.n_sel = all;
-            const int over = (long long)all > io.capacity ? (int)D2D_ERR_CAPACITY : 0;
-            if (io.k) *io.status = over;
-            else if (over) atomicMax(io.status, over);
-        }
-    }
-    int pos = first + earlier;
-#pragma unroll
-    for (int i = 0; i < LISTS_GROUPS; ++i) {
-        if (i * 32 >= per) break;
-#pragma unroll 4
-        for (int j = 0; j < 32; ++j) {
-            const uint32_t b = __shfl_sync(FULL, col[i], j);
-            const int at = __shfl_sync(FULL, pos, j) + __popc(b & ((1u << lane) - 1u));
-            if (((b >> lane) & 1u) && at < io.capacity) io.perm[at] = t0 + i * 32 + lane;
-        }
-        pos += __popc(col[i]);
-    }
+    __shared__ uint16_t cnt[TOKB];
+    __shared__ int sums[TOKB / 32];
+    d2d_lists::lists_of_word<TOKB / 32, LISTS_GROUPS>(g.l[blockIdx.y], blockIdx.x, g.T, g.E, g.W, threadIdx.x >> 5, threadIdx.x & 31, cnt, sums,
+                                                      [] { __syncthreads(); });
 }
 
 // Per-expert token counts of each 256-token block (8 warps x 32 tokens; a warp turns its
@@ -303,7 +215,7 @@ bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     {
         const int w = blockIdx.y;                // one 32-expert mask word per CTA
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        sh.cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
+        sh.cnt[warp][lane] = (uint16_t)__popc(d2d_lists::transpose_bits(word, lane));
         __syncthreads();
         if (warp == 0) {
             int total = 0;
@@ -401,7 +313,7 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
         // start of this CTA's run inside expert e's list (lane = expert); issued early to hide the latency
         const long long cta_base = e < E ? (long long)__ldg(offsets + e) + __ldg(blockbase + (size_t)blockIdx.x * E + e) : 0;
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
+        cnt[warp][lane] = (uint16_t)__popc(d2d_lists::transpose_bits(word, lane));
         __syncthreads();
         int before = 0;
         for (int i = 0; i < warp; ++i) before += cnt[i][lane];
@@ -501,13 +413,19 @@ static bool lists_in_one_launch(int T, int E, bool alone)
     return T <= (alone ? LISTS_MAX_T : LISTS_MAX_T / 2) && (long long)T * ((E + 31) / 32) <= 16384;
 }
 
-static void launch_lists(const d2d_routing *r, int n, int T, int E, bool with_k, cudaStream_t st)
+d2d_list_job d2d_list_job_for(const d2d_routing *r, int n, int T, int E, bool with_k)
 {
-    ListsGroup g = {};
+    d2d_list_job g = {};
+    g.n = n; g.T = T; g.E = E; g.W = (E + 31) / 32;
     for (int l = 0; l < n; ++l)
         g.l[l] = {r[l].mask, with_k ? r[l].k : nullptr, r[l].counts, r[l].offsets, r[l].perm, r[l].n_sel, r[l].status,
                   (long long)r[l].perm_capacity};
-    lists_kernel<<<dim3((E + 31) / 32, n), TOKB, 0, st>>>(g, T, E, (E + 31) / 32);
+    return g;
+}
+
+static void launch_lists(const d2d_routing *r, int n, int T, int E, bool with_k, cudaStream_t st)
+{
+    lists_kernel<<<dim3((E + 31) / 32, n), TOKB, 0, st>>>(d2d_list_job_for(r, n, T, E, with_k));
     D2D_LAUNCHED(1);
 }
 
