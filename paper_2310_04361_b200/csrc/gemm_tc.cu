@@ -46,8 +46,8 @@ struct EpiParams {
     int test_skip_load;              // test aid: CTA 0 never requests the A tile of its first k-block (see d2d_gemm_args)
 };
 
-// Lists a down projection builds before its first tile.  Launches without any do without the parameter: 80 bytes in two of a
-// layer's launches cost it 1 us.
+// Lists a down projection builds before its first tile.  Launches without any do without the code: carrying it cost a short layer
+// call 1 us, whether it ran or not.
 struct NoLists {};
 template <int N> struct ListsOf { typedef d2d_list_jobs<N> type; };
 template <> struct ListsOf<0> { typedef NoLists type; };
@@ -58,7 +58,7 @@ template <int N> __device__ __forceinline__ void build_lists(const d2d_list_jobs
     for (int i = (int)blockIdx.x; i < j.n * j.W; i += (int)gridDim.x) {
         const auto sync = [] { asm volatile("bar.sync 1, 512;" ::: "memory"); };
         const int l = N == 1 ? 0 : i / j.W;
-        d2d_lists::lists_of_word<16, 2>(j.l[l], i - l * j.W, T, j.E, j.W, ew, lane, reinterpret_cast<uint16_t *>(scratch),
+        d2d_lists::lists_of_word<16>(j.l[l], i - l * j.W, T, j.E, j.W, ew, lane, reinterpret_cast<uint16_t *>(scratch),
                                         reinterpret_cast<int *>(scratch + 2048), sync);
         sync();
     }

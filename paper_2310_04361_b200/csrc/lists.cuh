@@ -20,62 +20,55 @@ d2d_list_job d2d_list_job_for(const d2d_routing *r, int n, int T, int E, bool wi
 #ifdef __CUDACC__
 namespace d2d_lists {
 
-// Lane j returns the bitmap, over this warp's 32 tokens, of bit j of `word`.
-__device__ __forceinline__ uint32_t transpose_bits(uint32_t word, int lane)
-{
-    uint32_t col = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-        const uint32_t b = __ballot_sync(0xffffffffu, (word >> j) & 1u);
-        if (lane == j) col = b;
-    }
-    return col;
-}
-
 // Mask word w of one layer (32 experts) by NWARP warps that meet at `sync`: adds up the pairs of the words before its own (what
 // its first list starts at), counts its experts per warp (a warp has a contiguous range of 32-token groups), scans, and writes.
-// At most GROUPS * 32 * NWARP tokens.  cnt: [NWARP * 32], sums: [NWARP], shared.
-template <int NWARP, int GROUPS, typename Sync>
+// At most 65535 tokens a warp.  cnt: [NWARP * 32], sums: [NWARP], shared.  A warp sees a group's holders of an expert as one ballot.
+// Loops are kept short: this runs once per launch, and code that an SM runs for the first time is slow (with the groups' words
+// in registers and the loops over them unrolled eight times, a layer call of 64 tokens took 4 us longer).
+template <int NWARP, typename Sync>
 __device__ __forceinline__ void lists_of_word(const d2d_list_io &io, int w, int T, int E, int W, int warp, int lane, uint16_t *cnt, int *sums, Sync sync)
 {
     constexpr int N = NWARP * 32;
     const uint32_t *__restrict__ mask = io.mask;
     const int per = (T + N - 1) / N * 32;                 // tokens of a warp
-    const int t0 = warp * per, e = w * 32 + lane;
-    uint32_t col[GROUPS];                                 // per group of 32 tokens: which of them keep expert e
-#pragma unroll
-    for (int i = 0; i < GROUPS; ++i) {
-        const int t = t0 + i * 32 + lane;
-        col[i] = i * 32 < per && t < T ? __ldg(mask + (size_t)t * W + w) : 0u;
-    }
+    const int t0 = warp * per, t1 = min(T, t0 + per), e = w * 32 + lane;
+    const uint32_t valid = E - w * 32 >= 32 ? 0xffffffffu : (1u << (E - w * 32)) - 1u, lower = (1u << lane) - 1u;
+    auto word_of = [&](int t) { return t < t1 ? __ldg(mask + (size_t)t * W + w) & valid : 0u; };
+    uint32_t word = word_of(t0 + lane);
     int before = 0;
+#pragma unroll 1
     for (int t = warp * 32 + lane; t < T; t += N) {
         const uint32_t *row = mask + (size_t)t * W;
         int n = 0;
-        for (int i0 = 0; i0 < w; i0 += 8) {                     // eight loads in flight: one after the other they were most of the time
-            uint32_t v[8];
+#pragma unroll 1
+        for (int i0 = 0; i0 < w; i0 += 4) {
+            uint32_t v[4];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = i0 + i < w ? __ldg(row + i0 + i) : 0u;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) n += __popc(v[i]);
+            for (int i = 0; i < 4; ++i) v[i] = i0 + i < w ? __ldg(row + i0 + i) : 0u;
+            n += __popc(v[0]) + __popc(v[1]) + __popc(v[2]) + __popc(v[3]);
         }
         before += n;
         if (io.k && w == W - 1) io.k[t] = n + __popc(__ldg(row + w));
     }
     before = __reduce_add_sync(0xffffffffu, before);
     int mine = 0;
-#pragma unroll
-    for (int i = 0; i < GROUPS; ++i) {
-        col[i] = transpose_bits(col[i], lane);
-        if (e >= E) col[i] = 0u;
-        mine += __popc(col[i]);
+#pragma unroll 1
+    for (int t = t0; t < t1; t += 32) {
+        const uint32_t now = word;
+        word = word_of(t + 32 + lane);
+#pragma unroll 4
+        for (int j = 0; j < 32; ++j) {
+            const uint32_t b = __ballot_sync(0xffffffffu, (now >> j) & 1u);
+            if (lane == j) mine += __popc(b);
+        }
     }
     cnt[warp * 32 + lane] = (uint16_t)mine;
     if (lane == 0) sums[warp] = before;
     sync();
+    word = word_of(t0 + lane);
     int total = 0, earlier = 0;
     before = 0;
-#pragma unroll
+#pragma unroll 4
     for (int i = 0; i < NWARP; ++i) {
         const int c = cnt[i * 32 + lane];
         if (i < warp) earlier += c;
@@ -102,16 +95,17 @@ __device__ __forceinline__ void lists_of_word(const d2d_list_io &io, int w, int 
         }
     }
     int pos = first + earlier;
-#pragma unroll
-    for (int i = 0; i < GROUPS; ++i) {
-        if (i * 32 >= per) break;
+#pragma unroll 1
+    for (int t = t0; t < t1; t += 32) {
+        const uint32_t now = word;
+        word = word_of(t + 32 + lane);
 #pragma unroll 4
         for (int j = 0; j < 32; ++j) {
-            const uint32_t b = __shfl_sync(0xffffffffu, col[i], j);
-            const int at = __shfl_sync(0xffffffffu, pos, j) + __popc(b & ((1u << lane) - 1u));
-            if (((b >> lane) & 1u) && at < io.capacity) io.perm[at] = t0 + i * 32 + lane;
+            const uint32_t b = __ballot_sync(0xffffffffu, (now >> j) & 1u);
+            const int at = __shfl_sync(0xffffffffu, pos, j) + __popc(b & lower);
+            if (((now >> j) & 1u) && at < io.capacity) io.perm[at] = t + lane;
+            if (lane == j) pos += __popc(b);
         }
-        pos += __popc(col[i]);
     }
 }
 

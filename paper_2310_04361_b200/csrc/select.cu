@@ -144,6 +144,18 @@ k_from_mask_kernel(const uint32_t *__restrict__ mask, int T, int W, int32_t *__r
 
 // ---------------------------------------------------------------------------- bucketing
 
+// Lane j returns the bitmap, over this warp's 32 tokens, of bit j of `word`.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t word, int lane)
+{
+    uint32_t col = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t b = __ballot_sync(FULL, (word >> j) & 1u);
+        if (lane == j) col = b;
+    }
+    return col;
+}
+
 // Exclusive scan of one int per thread over a 256-thread CTA; returns the exclusive prefix and
 // leaves the CTA total in *total_out (shared).
 __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, int *total_out)
@@ -178,14 +190,14 @@ __device__ __forceinline__ int block_exscan_256(int v, int *warp_sums /*[8]*/, i
 // order between CTAs, so counts, offsets and lists take one launch and no scratch (lists.cuh).  k != NULL: k and the status word
 // are wanted too.  Bound by latency; as small as bucket_count_scan_kernel, for the same reason.  What it saves is the host's time
 // (two launches, a memset and, for a mask that is given, two more): see d2d_launch_select for the line.
-constexpr int LISTS_GROUPS = 4, LISTS_MAX_T = LISTS_GROUPS * TOKB;      // 32-token groups of a warp, held in registers
+constexpr int LISTS_MAX_T = 4 * TOKB;
 
 __global__ void __launch_bounds__(TOKB, 6)
 lists_kernel(const __grid_constant__ d2d_list_job g)
 {
     __shared__ uint16_t cnt[TOKB];
     __shared__ int sums[TOKB / 32];
-    d2d_lists::lists_of_word<TOKB / 32, LISTS_GROUPS>(g.l[blockIdx.y], blockIdx.x, g.T, g.E, g.W, threadIdx.x >> 5, threadIdx.x & 31, cnt, sums,
+    d2d_lists::lists_of_word<TOKB / 32>(g.l[blockIdx.y], blockIdx.x, g.T, g.E, g.W, threadIdx.x >> 5, threadIdx.x & 31, cnt, sums,
                                                       [] { __syncthreads(); });
 }
 
@@ -215,7 +227,7 @@ bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     {
         const int w = blockIdx.y;                // one 32-expert mask word per CTA
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        sh.cnt[warp][lane] = (uint16_t)__popc(d2d_lists::transpose_bits(word, lane));
+        sh.cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
         __syncthreads();
         if (warp == 0) {
             int total = 0;
@@ -313,7 +325,7 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
         // start of this CTA's run inside expert e's list (lane = expert); issued early to hide the latency
         const long long cta_base = e < E ? (long long)__ldg(offsets + e) + __ldg(blockbase + (size_t)blockIdx.x * E + e) : 0;
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
-        cnt[warp][lane] = (uint16_t)__popc(d2d_lists::transpose_bits(word, lane));
+        cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
         __syncthreads();
         int before = 0;
         for (int i = 0; i < warp; ++i) before += cnt[i][lane];
