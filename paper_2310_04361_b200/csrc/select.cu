@@ -131,10 +131,14 @@ topk_mask_kernel(const float *__restrict__ R, int T, int E, int W, int kk,
     }
 }
 
-// k from a caller-supplied mask (override protocol of Sec. 4.4).
+// k from a caller-supplied mask (override protocol of Sec. 4.4); also clears what the kernels behind it add to (a memset each took
+// as long as this kernel).
 __global__ void __launch_bounds__(256)
-k_from_mask_kernel(const uint32_t *__restrict__ mask, int T, int W, int32_t *__restrict__ k)
+k_from_mask_kernel(const uint32_t *__restrict__ mask, int T, int W, int32_t *__restrict__ k, unsigned int *ticket, int32_t *status)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x == 0) { *ticket = 0u; *status = 0; }
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T) return;
     int kt = 0;
@@ -224,6 +228,8 @@ bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     __shared__ unsigned int my_ticket;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = blockIdx.x * TOKB + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     {
         const int w = blockIdx.y;                // one 32-expert mask word per CTA
         const uint32_t word = (t < T) ? __ldg(mask + (size_t)t * W + w) : 0u;
@@ -239,10 +245,9 @@ bucket_count_scan_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        __threadfence();                         // the whole CTA's counts (the barrier before it)
-        my_ticket = atomicAdd(ticket, 1u);
+        // releases the whole CTA's counts (the barrier before it); the last one acquires everybody's
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(my_ticket) : "l"(ticket) : "memory");
         if (my_ticket == (unsigned int)(nblk * W - 1)) *ticket = 0u;      // ready for the next call
-        __threadfence();                         // the last one: every other CTA's block counts are visible now
     }
     __syncthreads();
     if (my_ticket != (unsigned int)(nblk * W - 1)) return;
@@ -318,6 +323,8 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     __shared__ uint16_t cnt[TOKB / 32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t = blockIdx.x * TOKB + threadIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t lower = (1u << lane) - 1u;
     {
         const int w = blockIdx.y;                // one 32-expert mask word per CTA
@@ -481,7 +488,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
     // a mask that is given, lists in one launch: that kernel writes k and the status word as well
     const bool one = T > 0 && lists_in_one_launch(T, E, !mask_ready), given = !R && !mask_ready;
     const bool small = topk == 0 && d2d_small_select_supports(T, E);
-    if (!mask_ready && !(given && one && !small)) D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
+    if (!mask_ready && !(given && T > 0 && !small)) D2D_CUDA_TRY(cudaMemsetAsync(out->status, 0, sizeof(int32_t), st));
     if (T == 0) {
         D2D_CUDA_TRY(cudaMemsetAsync(out->counts, 0, sizeof(int32_t) * (size_t)E, st));
         D2D_CUDA_TRY(cudaMemsetAsync(out->offsets, 0, sizeof(int32_t) * (size_t)(E + 1), st));
@@ -490,6 +497,10 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         return D2D_OK;
     }
     if (small) return d2d_small_select(R, T, E, tau, out, st, mask_ready);
+    const int nblk = d2d_cdiv(T, TOKB);
+    // the ticket must start at zero (the kernel leaves it there): a word the caller keeps, or cleared on every call
+    unsigned int *ticket = zero_ticket ? zero_ticket : (unsigned int *)ws;
+    int32_t *blockcounts = (int32_t *)((char *)ws + 256);
     const int warps_per_cta = 8;
     const int grid_tok = d2d_cdiv(T, warps_per_cta);
     if (R) {
@@ -498,7 +509,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         else
             dynk_mask_kernel<<<grid_tok, 256, 0, st>>>(R, T, E, W, tau, out->mask, out->k, out->status, nullptr);
     } else if (given && !one) {
-        k_from_mask_kernel<<<d2d_cdiv(T, 256), 256, 0, st>>>(out->mask, T, W, out->k);
+        k_from_mask_kernel<<<nblk, 256, 0, st>>>(out->mask, T, W, out->k, ticket, out->status);
     }
     if (one) {
         D2D_LAUNCHED(R ? 1 : 0);
@@ -506,16 +517,20 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         launch_dual(out, T, W, st);
         return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
     }
-    const int nblk = d2d_cdiv(T, TOKB);
-    // the ticket must start at zero (the kernel leaves it there): a word the caller keeps, or cleared on every call
-    unsigned int *ticket = zero_ticket ? zero_ticket : (unsigned int *)ws;
-    int32_t *blockcounts = (int32_t *)((char *)ws + 256);
-    if (!zero_ticket) D2D_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st));
-    bucket_count_scan_kernel<<<dim3(nblk, W), TOKB, 0, st>>>(out->mask, T, E, W, nblk, blockcounts, ticket, out->counts,
-                                                    out->offsets, out->n_sel, out->status,
-                                                    (long long)out->perm_capacity);
-    bucket_fill_kernel<<<dim3(nblk, W), TOKB, 0, st>>>(out->mask, T, E, W, blockcounts, out->offsets, out->perm,
-                                              (long long)out->perm_capacity);
+    if (!zero_ticket && !given) D2D_CUDA_TRY(cudaMemsetAsync(ticket, 0, sizeof(unsigned int), st));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblk, W, 1);
+    cfg.blockDim = dim3(TOKB, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, bucket_count_scan_kernel, (const uint32_t *)out->mask, T, E, W, nblk, blockcounts, ticket, out->counts,
+                                    out->offsets, out->n_sel, out->status, (long long)out->perm_capacity));
+    D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, bucket_fill_kernel, (const uint32_t *)out->mask, T, E, W, (const int32_t *)blockcounts,
+                                    (const int32_t *)out->offsets, out->perm, (long long)out->perm_capacity));
     D2D_LAUNCHED(mask_ready ? 2 : 3);
     launch_dual(out, T, W, st);
     return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
