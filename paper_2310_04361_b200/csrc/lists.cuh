@@ -25,15 +25,17 @@ namespace d2d_lists {
 // At most 65535 tokens a warp.  cnt: [NWARP * 32], sums: [NWARP], shared.  A warp sees a group's holders of an expert as one ballot.
 // Loops are kept short: this runs once per launch, and code that an SM runs for the first time is slow (with the groups' words
 // in registers and the loops over them unrolled eight times, a layer call of 64 tokens took 4 us longer).
-template <int NWARP, typename Sync>
+// FRESH: the mask was written by this very launch (other CTAs of it), so it is read from L2.
+template <int NWARP, bool FRESH = false, typename Sync>
 __device__ __forceinline__ void lists_of_word(const d2d_list_io &io, int w, int T, int E, int W, int warp, int lane, uint16_t *cnt, int *sums, Sync sync)
 {
     constexpr int N = NWARP * 32;
-    const uint32_t *__restrict__ mask = io.mask;
+    const uint32_t *mask = io.mask;
+    auto load = [](const uint32_t *p) { return FRESH ? __ldcg(p) : __ldg(p); };
     const int per = (T + N - 1) / N * 32;                 // tokens of a warp
     const int t0 = warp * per, t1 = min(T, t0 + per), e = w * 32 + lane;
     const uint32_t valid = E - w * 32 >= 32 ? 0xffffffffu : (1u << (E - w * 32)) - 1u, lower = (1u << lane) - 1u;
-    auto word_of = [&](int t) { return t < t1 ? __ldg(mask + (size_t)t * W + w) & valid : 0u; };
+    auto word_of = [&](int t) { return t < t1 ? load(mask + (size_t)t * W + w) & valid : 0u; };
     uint32_t word = word_of(t0 + lane);
     int before = 0;
 #pragma unroll 1
@@ -44,11 +46,11 @@ __device__ __forceinline__ void lists_of_word(const d2d_list_io &io, int w, int 
         for (int i0 = 0; i0 < w; i0 += 4) {
             uint32_t v[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = i0 + i < w ? __ldg(row + i0 + i) : 0u;
+            for (int i = 0; i < 4; ++i) v[i] = i0 + i < w ? load(row + i0 + i) : 0u;
             n += __popc(v[0]) + __popc(v[1]) + __popc(v[2]) + __popc(v[3]);
         }
         before += n;
-        if (io.k && w == W - 1) io.k[t] = n + __popc(__ldg(row + w));
+        if (io.k && w == W - 1) io.k[t] = n + __popc(load(row + w));
     }
     before = __reduce_add_sync(0xffffffffu, before);
     int mine = 0;
