@@ -526,7 +526,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = !mask_ready && d2d_tc_pdl_enabled() ? 1 : 0;      // (on a side stream they would only sit on the experts' SMs earlier)
     D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, bucket_count_scan_kernel, (const uint32_t *)out->mask, T, E, W, nblk, blockcounts, ticket, out->counts,
                                     out->offsets, out->n_sel, out->status, (long long)out->perm_capacity));
     D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, bucket_fill_kernel, (const uint32_t *)out->mask, T, E, W, (const int32_t *)blockcounts,
