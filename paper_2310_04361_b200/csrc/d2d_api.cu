@@ -808,12 +808,20 @@ static layer_form form_for(const d2d_layer *L, int T, bool lists)
     if (d2d_layer_f32_small_supports(D, T, lists)) return FORM_F32_SMALL;
     if (T > 8 && d2d_layer_token_fused_supports(D, T, lists)) return FORM_TOKEN_FUSED;
     if (lists && d2d_small_router_supports(D, T)) return FORM_SMALL_ROUTER;
-    if (masked && !d2d_small_select_supports(T, D.n_experts)) return FORM_MASKED;
+    // (From 33 tokens on also where one CTA could select: it would take a kernel more and a pass over the batch.  Llama-shaped layer:
+    // 105 -> 94 us at 40 tokens, 108 -> 97 at 64.  Up to 32 tokens the cluster router is the faster start: 87 and 93 at 20.)
+    if (masked && (!d2d_small_select_supports(T, D.n_experts) || (d2d_router_scores_supports(D, T) && !d2d_decode_router_supports(D, T))))
+        return FORM_MASKED;
     return FORM_PLAIN;
 }
 
 // Whether the form's expert kernels walk the per-expert lists (the others read the mask, and build the lists if they are wanted)
-static bool needs_lists(layer_form f) { return f == FORM_FUSED_ROUTER_LISTS || f == FORM_SMALL_ROUTER || f == FORM_PLAIN; }
+// or have always been called with them (up to 64 tokens of a router in two kernels)
+static bool needs_lists(const d2d_layer *L, int T, layer_form f)
+{
+    return f == FORM_FUSED_ROUTER_LISTS || f == FORM_SMALL_ROUTER || f == FORM_PLAIN ||
+           (f == FORM_MASKED && d2d_small_select_supports(T, L->desc.n_experts));
+}
 
 // The per-expert lists on the layer's side stream, behind what is queued on `st`
 static d2d_status fork_lists(const d2d_layer *L, int T, d2d_routing *r, void *ws, cudaStream_t st)
@@ -830,7 +838,8 @@ static d2d_status join_lists(const d2d_layer *L, cudaStream_t st)
 static bool lists_ride(const d2d_layer *L, int T, const d2d_routing *r)
 {
     const d2d_layer_desc &D = L->desc;
-    return !r->tok_off && path_before_launch(L, T, true) == D2D_PATH_DENSE && d2d_lists_ride(T, D.n_experts, d2d_gemm_tc_splits(T, D.d, D.d_ff));
+    return !r->tok_off && path_before_launch(L, T, true) == D2D_PATH_DENSE &&
+           d2d_lists_ride(T, D.n_experts, d2d_gemm_tc_splits(T, D.d, D.d_ff), 2.0 * T * D.d * D.d_ff);
 }
 
 d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float tau, void *y,
@@ -847,7 +856,7 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
     const ws_layout w = layout_for(layer, T);
     if (!ws || !aligned16(ws) || ws_bytes < w.total) return D2D_ERR_WORKSPACE;
     const layer_form form = form_for(layer, T, lists);
-    if (!lists && needs_lists(form)) return D2D_ERR_INVALID_ARG;
+    if (!lists && needs_lists(layer, T, form)) return D2D_ERR_INVALID_ARG;
     char *base = (char *)ws;
     float *R = R_out ? R_out : (float *)(base + w.r_off);
     void *ffn_ws = base + w.ffn_off;
@@ -923,7 +932,7 @@ static d2d_status finish_host_call(const d2d_layer *layer, const int32_t *status
 }
 
 // Whether a batch can do without the per-expert lists
-static bool lists_optional(const d2d_layer *L, int T) { return !needs_lists(form_for(L, T, false)); }
+static bool lists_optional(const d2d_layer *L, int T) { return !needs_lists(L, T, form_for(L, T, false)); }
 
 // Carves routing buffers + x/y staging + the layer workspace out of one device buffer.
 struct host_call_layout {

@@ -81,9 +81,11 @@ int d2d_gemm_tc_splits(int M, int N, int K, int batch = 1);
 // 26.8 us at 64 tokens, 34.7 -> 33.0 at 333, 43.2 -> 39.9 at 1000 (not split); split along K and in two goes they hold the
 // partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection that have no tile they held
 // up the down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
-static inline bool d2d_lists_ride(int T, int E, int k_splits)
+// Above 1e10 FLOP of down projection the call is not short any more and the side stream is the better place (Llama-shaped
+// layer: 100.4 -> 95.1 at 100 tokens, but 130.9 -> 133.9 at 200).
+static inline bool d2d_lists_ride(int T, int E, int k_splits, double down_flop)
 {
-    return T <= (k_splits > 1 ? 512 : 1024) && (long long)T * ((E + 31) / 32) <= 16384;
+    return T <= (k_splits > 1 ? 512 : 1024) && (long long)T * ((E + 31) / 32) <= 16384 && down_flop <= 1e10;
 }
 
 // Enqueues C = epilogue(A B^T).  Requires K % 8 == 0 and 16-byte aligned base pointers.

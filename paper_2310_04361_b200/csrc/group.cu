@@ -217,7 +217,7 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         // per-expert metadata of every layer: by the down projection, or on the side stream beside the GEMMs (which read only the
         // merged mask)
         const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff, n);
-        bool ride = d2d_lists_ride(T, E, k_splits);
+        bool ride = d2d_lists_ride(T, E, k_splits, 2.0 * n * T * D.d * D.d_ff);
         for (int l = 0; l < n; ++l) ride = ride && !routing[l].tok_off;
         if (!ride) {
             if (cudaEventRecord(g->ev_fork, st) != cudaSuccess || cudaStreamWaitEvent(g->side_stream, g->ev_fork, 0) != cudaSuccess)

@@ -100,3 +100,34 @@ def test_layer_with_8bit_experts_matches_the_oracle_on_the_dequantised_weights(a
         y_full = oracle.moe_ffn(x, w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], act, G)
         assert _rel_err(y_ref, y_full) > 1e-3
     layer.close()
+
+
+# The decode kernel multiplies 8-bit codes with token rows scaled into float16.  Rows at both ends of bfloat16's exponents, of zeros,
+# with one value 2^27 times the others (which must still count: against their own sum they are all there is where the outlier's
+# weights are zero), and a row with an infinity beside them.  Errors per token: bf16 rounding of the hidden values and of y, 2^-9 each,
+# averaged over many terms: 1e-2 in the 2-norm bounds them.
+@pytest.mark.parametrize("T", [1, 2, 6])
+def test_8bit_expert_step_on_rows_of_any_scale(api, T):
+    cfg = wl.LayerConfig("scale", "bf16", d=256, d_ff=512, E=32, d_h=64, act="relu", T=T, b1_shift=None, has_b2=False, seed=61)
+    w = wl.make_weights(cfg)
+    w["w1"][:, 7] = 0.0
+    _, wq = _quantised(cfg, w)
+    layer = api.Layer.from_config(cfg, w, fp8_experts=True)
+    rng = np.random.default_rng(T)
+    base = wl.round_to_bf16(rng.standard_normal((7, cfg.d)).astype(np.float32))
+    rows = base * np.float32(2.0) ** np.array([0, 90, -100, 0, 0, 0, 0], np.float32)[:, None]
+    rows[3] = 0.0
+    rows[4, 7] = 2.0 ** 27
+    rows[5, 3] = np.inf
+    for start in range(0, 7, T):
+        x = rows[[(start + i) % 7 for i in range(T)]]
+        r = api.routing_from_mask(torch.full((T, 1), -1, dtype=torch.int32, device="cuda"), cfg.E)
+        y = layer.moe_ffn_fwd(api.to_device(x, cfg.dtype), r).float().cpu().numpy().astype(np.float64)
+        for t in range(T):
+            if np.isinf(x[t]).any():
+                assert not np.isfinite(y[t]).all()
+                continue
+            h = np.maximum(x[t].astype(np.float64) @ wq["w1"].astype(np.float64).T, 0.0)
+            ref = h @ wq["w2"].astype(np.float64).T
+            assert np.linalg.norm(y[t] - ref) <= 1e-2 * np.linalg.norm(ref), (start, t)
+    layer.close()

@@ -780,6 +780,46 @@ def test_lists_from_a_given_mask(api, T, E):
         assert np.array_equal(r.k.cpu().numpy(), G.sum(1))
 
 
+# lists built by the down projection: one and two goes of 512 tokens, split and unsplit contractions, on both sides of every limit,
+# ragged last words; a router in two kernels from 33 tokens on; a group
+@pytest.mark.parametrize("shape,Ts", [(dict(d=256, d_ff=33 * 16, E=33), (33, 65, 512, 513)), (dict(d=1024, d_ff=4096, E=256), (400, 1000, 1024, 1025)),
+                                      (dict(d=768, d_ff=3072, E=192), (200, 700)), (dict(d=512, d_ff=300 * 16, E=300, d_h=256), (33, 40, 64, 128, 600))])
+def test_lists_built_beside_the_experts(api, shape, Ts):
+    cfg = wl.LayerConfig("ride", "bf16", **{**dict(d_h=128, act="gelu_erf", token_sigma=0.5, b1_shift=-0.3), **shape}, T=max(Ts), seed=59)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    xd = api.to_device(x, cfg.dtype)
+    for T in Ts:
+        for tau in (0.4, 0.0):
+            r = layer.new_routing(T)
+            _poison(r.perm), _poison(r.counts), _poison(r.offsets)
+            y, _ = layer.layer_fwd(xd[:T], tau, routing=r)
+            torch.cuda.synchronize()
+            G = oracle.unpack_mask(r.mask_u32(), cfg.E)
+            assert r.status == 0
+            _check_routing(r, G, dual=False)
+        small = layer.new_routing(T, perm_capacity=int(G.sum()) - 1)
+        layer.layer_fwd(xd[:T], 0.0, routing=small)
+        torch.cuda.synchronize()
+        assert small.status == 7                               # D2D_ERR_CAPACITY
+    layer.close()
+
+
+@pytest.mark.parametrize("T", [33, 149, 297, 1000])
+def test_fp32_layer_lists_without_the_dual(api, T):
+    """The last CTA's lists of a one-launch float32 layer: from the words that this launch wrote, twice with other decisions."""
+    cfg = wl.with_tokens(wl.CONFIGS["tiny"], T)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    r = layer.new_routing(T)
+    for tau in (0.7, 0.2, 0.0):
+        layer.layer_fwd(api.to_device(x, cfg.dtype), tau, routing=r)
+        torch.cuda.synchronize()
+        assert r.status == 0
+        _check_routing(r, oracle.unpack_mask(r.mask_u32(), cfg.E), dual=False)
+    layer.close()
+
+
 @pytest.mark.parametrize("T", [1023, 1024, 2559, 2560, 3583, 3585])
 def test_layer_fwd_host_two_to_four_chunks(api, T):
     cfg, w, x, layer = _setup(api, "bert", T)
