@@ -20,7 +20,8 @@ using d2d_tc::tma_load_2d; using d2d_tc::smem_desc_sw128; using d2d_tc::instr_de
 using d2d_tc::umma_commit; using d2d_tc::tmem_ld16_issue; using d2d_tc::tmem_ld_wait;
 
 constexpr int BM = 128, BK = 64, UMMA_K = 16;
-constexpr int STAGES = 5;          // 5 x 32 KB of operands in flight: the first GEMM's main loop is bound by load latency
+// 5 x 32 KB of operands in flight: the first GEMM's main loop is bound by load latency; 3 where two CTAs share an SM
+__host__ __device__ constexpr int stages_for(bool two) { return two ? 3 : 5; }
 constexpr int NTHREADS = 64 + 512;       // TMA warp, MMA warp, 16 epilogue warps
 
 // every barrier wait of this kernel: 4096 back-to-back polls, then one poll every 128 ns
@@ -106,8 +107,10 @@ __device__ __forceinline__ void store_scores16(float *__restrict__ R, int row, i
 // blockIdx.y picks the router.  Their weights are stacked (W_r1 [n*DH, d], b_r1 [n*DH], W_r2 [n*E, DH], b_r2 [n*E]);
 // every router writes its own outputs and, when mask_cat is given, its mask words once more into a merged mask
 // [T, cat_words] at word offset l * ceil(E/32) (the selection mask of the merged up projection).
-template <int DH>
-__global__ void __launch_bounds__(NTHREADS, 1)
+// TWO: two CTAs per SM, for batches of more row tiles than SMs (see launch_for): three stages, u in the ring's last one, the scores in
+// the columns of u's accumulator (both are used up by then), scores read from TMEM twice instead of kept in registers.
+template <int DH, bool TWO>
+__global__ void __launch_bounds__(NTHREADS, TWO ? 2 : 1)
 router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w1,
                     const __grid_constant__ CUtensorMap tm_w2, const __nv_bfloat16 *__restrict__ b_r1_all,
                     const __nv_bfloat16 *__restrict__ b_r2_all, int T, int d, int E, int EN /* E rounded up to 16 */,
@@ -122,6 +125,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     // conditions are collected in a word of the layer and published once (no memset in front of the kernel)
     int32_t *const ksum = io.ksum[layer];
     int32_t *__restrict__ status = ksum ? ksum + 2 : io.l[layer].status;
+    constexpr int STAGES = stages_for(TWO);
     constexpr int KB2 = DH / BK;                          // k-blocks of the second GEMM
     constexpr int A_BYTES = BM * BK * 2, B1_BYTES = DH * BK * 2;
     constexpr int STAGE_BYTES = A_BYTES + B1_BYTES;
@@ -130,9 +134,11 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *u_s = smem + (size_t)STAGES * STAGE_BYTES;
+    uint8_t *u_s = smem + (size_t)(TWO ? STAGES - 1 : STAGES) * STAGE_BYTES;
     uint8_t *w2_s = smem;                                  // aliases the first stages (see above)
-    static_assert((size_t)KB2 * W2_KB_BYTES <= (size_t)STAGES * STAGE_BYTES, "W_r2 must fit in the operand ring");
+    static_assert((size_t)KB2 * W2_KB_BYTES <= (size_t)(TWO ? STAGES - 1 : STAGES) * STAGE_BYTES, "W_r2 must fit in the operand ring");
+    static_assert(!TWO || U_BYTES <= STAGE_BYTES, "u must fit in a stage");
+    constexpr uint32_t TMEM_COLS = TWO ? 256 : 512;
     constexpr int W2_STAGES = (KB2 * W2_KB_BYTES + STAGE_BYTES - 1) / STAGE_BYTES;      // stages W_r2 overwrites
     __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES], bar_w2, bar_acc1, bar_u_ready, bar_acc2;
     __shared__ uint32_t tmem_base_holder;
@@ -160,7 +166,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
-                     "r"(512u)
+                     "r"(TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -168,7 +174,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
-    const uint32_t tmem_r = tmem_base + 256;
+    const uint32_t tmem_r = TWO ? tmem_base : tmem_base + 256;
     // the set-up above may overlap the tail of the previous kernel of the stream
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the expert up projection that follows on the stream may start its operand loads and MMAs on the SMs this
@@ -283,7 +289,20 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int W = (E + 31) / 32;
-            float v[2][32];
+            float v[TWO ? 1 : 2][TWO ? 16 : 32];
+            // 16 scores of this thread's row, from column c0 on
+            auto scores16 = [&](int c0, float *o) {
+                uint32_t acc[16];
+                tmem_ld16(tmem_r + lane_base + (uint32_t)c0, acc);
+#pragma unroll
+                for (int j = 0; j < 16; j += 4) {
+                    const float4 b = *reinterpret_cast<const float4 *>(b2_s + c0 + j);
+                    o[j] = fabsf(__uint_as_float(acc[j]) + b.x);
+                    o[j + 1] = fabsf(__uint_as_float(acc[j + 1]) + b.y);
+                    o[j + 2] = fabsf(__uint_as_float(acc[j + 2]) + b.z);
+                    o[j + 3] = fabsf(__uint_as_float(acc[j + 3]) + b.w);
+                }
+            };
             // Scores are non-negative, so their bit patterns order like the values, with infinities and NaNs on top: ONE integer
             // maximum per element yields the row maximum and whether a score is not finite.
             uint32_t mb = 0u;
@@ -296,29 +315,21 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             const int c0 = w * 32 + h * 16;
+                            float *const o = TWO ? v[0] : &v[TWO ? 0 : q][TWO ? 0 : h * 16];
                             if (c0 < EN) {
-                                uint32_t acc[16];
-                                tmem_ld16(tmem_r + lane_base + (uint32_t)c0, acc);
-#pragma unroll
-                                for (int j = 0; j < 16; j += 4) {
-                                    const float4 b = *reinterpret_cast<const float4 *>(b2_s + c0 + j);
-                                    v[q][h * 16 + j] = fabsf(__uint_as_float(acc[j]) + b.x);
-                                    v[q][h * 16 + j + 1] = fabsf(__uint_as_float(acc[j + 1]) + b.y);
-                                    v[q][h * 16 + j + 2] = fabsf(__uint_as_float(acc[j + 2]) + b.z);
-                                    v[q][h * 16 + j + 3] = fabsf(__uint_as_float(acc[j + 3]) + b.w);
-                                }
+                                scores16(c0, o);
                                 if (whole) {
 #pragma unroll
-                                    for (int j = 0; j < 16; ++j) mb = max(mb, __float_as_uint(v[q][h * 16 + j]));
+                                    for (int j = 0; j < 16; ++j) mb = max(mb, __float_as_uint(o[j]));
                                 } else {
 #pragma unroll
                                     for (int j = 0; j < 16; ++j)
-                                        if (c0 + j < E) mb = max(mb, __float_as_uint(v[q][h * 16 + j]));
+                                        if (c0 + j < E) mb = max(mb, __float_as_uint(o[j]));
                                 }
-                                if (R && row < T) store_scores16(R, row, E, c0, &v[q][h * 16]);
+                                if (R && row < T) store_scores16(R, row, E, c0, o);
                             } else {
 #pragma unroll
-                                for (int j = 0; j < 16; ++j) v[q][h * 16 + j] = 0.0f;
+                                for (int j = 0; j < 16; ++j) o[j] = 0.0f;
                             }
                         }
                     }
@@ -341,8 +352,18 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
                         const int w = part + 4 * q;
                         if (w < W) {
                             uint32_t word = 0u;
+                            if constexpr (TWO) {
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) word |= !(v[q][j] < thr) ? 1u << j : 0u;
+                                for (int h = 0; h < 2; ++h) {
+                                    if (w * 32 + h * 16 >= EN) continue;
+                                    scores16(w * 32 + h * 16, v[0]);
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j) word |= !(v[0][j] < thr) ? 1u << (h * 16 + j) : 0u;
+                                }
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 32; ++j) word |= !(v[q][j] < thr) ? 1u << j : 0u;
+                            }
                             if (w * 32 + 32 > E) word &= (1u << (E - w * 32)) - 1u;
                             if (row < T) {
                                 mask[(size_t)row * W + w] = word;
@@ -380,7 +401,7 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 1) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
 }
 
@@ -576,21 +597,30 @@ d2d_status launch_kernel(K kern, bool (&done)[64], dim3 grid, size_t smem, cudaS
     return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
-template <int DH>
-d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T, float tau, int do_mask,
+template <int DH, bool TWO>
+d2d_status launch_for(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T, float tau, int do_mask,
                   const RouterGroupIO &io, cudaStream_t st)
 {
     constexpr int STAGE_BYTES = BM * BK * 2 + DH * BK * 2;
     constexpr int KB2 = DH / BK;
-    constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + (size_t)KB2 * BM * 128 + 1024;
+    constexpr size_t SMEM = (size_t)stages_for(TWO) * STAGE_BYTES + (TWO ? 0 : (size_t)KB2 * BM * 128) + 1024;
     CUtensorMap tx, tw1, tw2;
     if (!d2d_tc_make_map(&tx, x, T, D.d, BM) || !d2d_tc_make_map(&tw1, w.w_r1, D.d_h * n_layers, D.d, DH) ||
         !d2d_tc_make_map(&tw2, w.w_r2, D.n_experts * n_layers, D.d_h, 256))
         return D2D_ERR_CUDA;
     static bool attr_set[64] = {};                         // the attribute is per device
-    return launch_kernel(router_fused_kernel<DH>, attr_set, dim3(d2d_cdiv(T, BM), n_layers, 1), SMEM, st, tx, tw1, tw2,
+    return launch_kernel(router_fused_kernel<DH, TWO>, attr_set, dim3(d2d_cdiv(T, BM), n_layers, 1), SMEM, st, tx, tw1, tw2,
                          (const __nv_bfloat16 *)w.b_r1, (const __nv_bfloat16 *)w.b_r2, T, D.d, D.n_experts,
                          (D.n_experts + 15) / 16 * 16, tau, do_mask, io);
+}
+
+template <int DH>
+d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T, float tau, int do_mask,
+                  const RouterGroupIO &io, cudaStream_t st)
+{
+    // More row tiles than SMs: two CTAs per SM
+    return d2d_cdiv(T, BM) * n_layers > d2d_tc_sm_count() ? launch_for<DH, true>(D, w, n_layers, x, T, tau, do_mask, io, st)
+                                                          : launch_for<DH, false>(D, w, n_layers, x, T, tau, do_mask, io, st);
 }
 
 }  // namespace

@@ -948,3 +948,35 @@ def test_group_whose_lists_do_not_fit_runs_its_layers(api):
     group.close()
     for layer in layers:
         layer.close()
+
+
+@pytest.mark.parametrize("T,d,E", [(148 * 128, 768, 192), (148 * 128 + 1, 768, 192), (25216, 128, 33), (2 * 148 * 128 + 5, 64, 256),
+                                   (19000, 200, 24), (50000, 1024, 100)])
+def test_router_of_batches_of_more_tiles_than_sms(api, T, d, E):
+    """Two CTAs share an SM there.  Rows do not depend on one another and both forms do the same arithmetic in the same
+    order, so scores and decisions equal those of the batch cut into pieces that the other form takes."""
+    g = torch.Generator(device="cuda:0").manual_seed(T + E)
+
+    def normal(*shape, std=1.0):
+        return (torch.randn(shape, generator=g, device="cuda:0") * std).to(torch.bfloat16)
+
+    cfg = wl.LayerConfig("wide batch", "bf16", d=d, d_ff=16 * E, E=E, d_h=128, act="relu", T=T)
+    layer = api.Layer.from_config(cfg, dict(w_r1=normal(128, d, std=d ** -0.5), b_r1=normal(128, std=0.1), w_r2=normal(E, 128, std=0.1),
+                                            b_r2=normal(E, std=0.1), w1=normal(16 * E, d, std=0.02), b1=None, w_gate=None,
+                                            w2=normal(d, 16 * E, std=0.02), b2=normal(d, std=0.02)), device="cuda:0")
+    x = normal(T, d)
+    x[T - 3, 1] = float("inf")                       # a row whose scores are not finite keeps every expert
+    R = torch.empty((T, E), dtype=torch.float32, device="cuda:0")
+    _, r = layer.layer_fwd(x, 0.4, R_out=R)
+    _, bare = layer.layer_fwd(x, 0.4)
+    torch.cuda.synchronize()
+    assert r.status == bare.status == 5                        # D2D_ERR_NONFINITE
+    assert torch.equal(r.mask, bare.mask) and torch.equal(r.k, bare.k)
+    for t0 in range(0, T, 9001):
+        t1 = min(T, t0 + 9001)
+        Rp = torch.empty((t1 - t0, E), dtype=torch.float32, device="cuda:0")
+        _, rp = layer.layer_fwd(x[t0:t1].contiguous(), 0.4, R_out=Rp)
+        torch.cuda.synchronize()
+        assert torch.equal(R[t0:t1].view(torch.int32), Rp.view(torch.int32))
+        assert torch.equal(r.mask[t0:t1], rp.mask) and torch.equal(r.k[t0:t1], rp.k)
+    layer.close()
