@@ -808,10 +808,9 @@ static layer_form form_for(const d2d_layer *L, int T, bool lists)
     if (d2d_layer_f32_small_supports(D, T, lists)) return FORM_F32_SMALL;
     if (T > 8 && d2d_layer_token_fused_supports(D, T, lists)) return FORM_TOKEN_FUSED;
     if (lists && d2d_small_router_supports(D, T)) return FORM_SMALL_ROUTER;
-    // (From 33 tokens on also where one CTA could select: it would take a kernel more and a pass over the batch.  Llama-shaped layer:
-    // 105 -> 94 us at 40 tokens, 108 -> 97 at 64.  Up to 32 tokens the cluster router is the faster start: 87 and 93 at 20.)
-    if (masked && (!d2d_small_select_supports(T, D.n_experts) || (d2d_router_scores_supports(D, T) && !d2d_decode_router_supports(D, T))))
-        return FORM_MASKED;
+    // (Also where one CTA could select, which would take a kernel more and a pass over the batch, and where the cluster router could
+    // score: behind the router in two kernels the up projection starts at once.)
+    if (masked && (!d2d_small_select_supports(T, D.n_experts) || d2d_router_scores_supports(D, T))) return FORM_MASKED;
     return FORM_PLAIN;
 }
 
@@ -909,7 +908,8 @@ d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t T, float
         fork = lists && !ride;
         if (rc == D2D_OK && fork) rc = fork_lists(layer, T, routing, base + w.sel_off, st);
         if (rc != D2D_OK) return rc;
-        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st, nullptr, 0, ksum + 4, ride);
+        rc = d2d_launch_moe_ffn(layer, x, T, routing, y, ffn_ws, ffn_bytes, st,
+                                d2d_router_scores_supports(layer->desc, T) ? (int *)(layer->tickets + 32) : nullptr, 0, ksum + 4, ride);
         return fork && join_lists(layer, st) != D2D_OK ? D2D_ERR_CUDA : rc;
     case FORM_PLAIN:
         rc = d2d_launch_router(layer, x, T, R, (float *)(base + w.u_off), st);

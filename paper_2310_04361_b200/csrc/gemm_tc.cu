@@ -236,7 +236,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // tiles of its first k-blocks BEFORE it waits for that kernel and only the A tiles after (static schedule only)
     const bool early_b = !PAIR && !dyn && !ep.late_wait && ep.n_sel == nullptr;
     if (warp >= 2 || (!ep.late_wait && !(early_b && warp == 0))) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (router's hidden layer: only threads that have waited let the next kernel start, see router_scores_kernel)
+    if (EPI != D2D_EPI_RELU_BF16 || !early_b || warp != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // density-adaptive dispatch: below the crossover the gathered kernel, launched next to this one, does the work
     // (every thread has passed the dependency wait here: the host never combines n_sel with late_wait)
     const bool run = ep.n_sel == nullptr || (long long)__ldcg(ep.n_sel) > ep.n_sel_max;

@@ -459,8 +459,10 @@ router_scores_kernel(const __grid_constant__ CUtensorMap tm_u, const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The up projection behind this kernel may start at once, beside the hidden layer: this kernel runs since every CTA of that one
+    // has waited for what came before, so x and the workspace are the layer's own; what depends on the mask waits for this kernel.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == 0) {
         if (lane == 0) {
@@ -618,7 +620,10 @@ template <int DH>
 d2d_status launch(const d2d_layer_desc &D, const d2d_router_weights &w, int n_layers, const void *x, int T, float tau, int do_mask,
                   const RouterGroupIO &io, cudaStream_t st)
 {
-    // More row tiles than SMs: two CTAs per SM
+    // More row tiles than SMs: two CTAs per SM, so that the last round is not a nearly empty one of its own and the up projection
+    // starts behind the first.  Bound by the latency of a CTA's chain (loads, two GEMMs, epilogues), which two CTAs overlap.  ViT-shaped
+    // layer, 25216 tokens (197 tiles on 148 SMs): 248.4 us with one CTA per SM, 245.0 with two.  Up to one tile per SM the
+    // five stages of the other form are in nobody's way and hide more of the latency.
     return d2d_cdiv(T, BM) * n_layers > d2d_tc_sm_count() ? launch_for<DH, true>(D, w, n_layers, x, T, tau, do_mask, io, st)
                                                           : launch_for<DH, false>(D, w, n_layers, x, T, tau, do_mask, io, st);
 }
