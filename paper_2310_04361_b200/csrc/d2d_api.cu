@@ -193,7 +193,12 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 // (the last includes 14 to 24 us for the kernels of the forms that are not taken, which are launched and return).
 int d2d_tc_sm_count();      // gemm_tc.cu
 
-static const double kAutoMinUpFlop = 2e11;      // smallest up projection for which the automatic choice is made, see launch_tc_experts
+// Smallest up projection for which the automatic choice is made, see path_before_launch.  Gated layers with the library's own limit on
+// the density: more, since smaller ones leave the gathered pair a few densities and lose the overlap with the router at the others
+// (Llama-shaped layer back to back, dense / with the choice, which takes the gathered pair where marked *: 1200 tokens 291 / 337 at
+// rho = 0.22, 293 / 331 at 0.03; 1500 tokens 334 / 396 at 0.22, 336 / 379 at 0.07, 323 / 287* at 0.03; above the line, 1800 tokens 406 /
+// 470, 397 / 369*, 397 / 328*; 2560 tokens 592 / 626 at 0.22, 553 / 508* at 0.12, 512 / 443* at 0.07).
+static double auto_min_up_flop(const d2d_layer *L) { return L->desc.gated && L->gather_rho_max < 0.0 ? 3.2e11 : 2e11; }
 
 static double default_gather_rho_max(const d2d_layer_desc &D, int g, int T)
 {
@@ -232,7 +237,7 @@ static int path_before_launch(const d2d_layer *L, int T, bool counted)
     int path = L->expert_path;
     if (L->gather_group <= 0) path = D2D_PATH_DENSE;
     const double up_flop = 2.0 * (double)T * D.d * D.d_ff * (D.gated ? 2.0 : 1.0);
-    if (path == D2D_PATH_AUTO && (up_flop < kAutoMinUpFlop || !counted)) path = D2D_PATH_DENSE;
+    if (path == D2D_PATH_AUTO && (up_flop < auto_min_up_flop(L) || !counted)) path = D2D_PATH_DENSE;
     return path;
 }
 
@@ -614,7 +619,7 @@ d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, int64_t 
         const double up_flop = 2.0 * (double)T * D.d * D.d_ff * (D.gated ? 2.0 : 1.0);
         const double pairs = (double)T * (double)D.n_experts;
         const double rho_max = layer->gather_rho_max >= 0.0 ? layer->gather_rho_max : default_gather_rho_max(D, layer->gather_group, T);
-        if (up_flop < kAutoMinUpFlop) p = D2D_PATH_DENSE;
+        if (up_flop < auto_min_up_flop(layer)) p = D2D_PATH_DENSE;
         else if (layer->fused_group > 0 && layer->fused_rho_max > 0.0 && n_sel <= (long long)(layer->fused_rho_max * pairs)) p = D2D_PATH_FUSED;
         else if (n_sel <= (long long)(rho_max * pairs) || (layer->fused_group > 0 && n_sel <= (long long)(layer->fused_rho_max * pairs))) p = D2D_PATH_GATHER;
         else p = D2D_PATH_DENSE;
