@@ -897,16 +897,26 @@ bool d2d_tc_pdl_enabled()
 
 bool d2d_gemm_tc_available() { return get_encode() != nullptr; }
 
-int d2d_gemm_tc_splits(int M, int N, int K, int batch)
+// Slices of K and tile width.  Split are only problems whose output tiles would occupy less than half of the SMs (a few hundred
+// tokens at most).  With tiles of 64 columns a slice is at least two k-blocks; tiles of 128 columns need more slices for the same
+// number of CTAs, hence more partial sums, and bring more weight bytes in flight (16 KB a stage instead of 8: the narrow ones reached
+// 3.1 TB/s on 90 MB of weights): they are taken where a slice is 40 k-blocks or more (14 us of main loop, against about 4 for the
+// sums).  Llama-shaped layer (d_ff = 11008), back to back: 74.7 -> 68.3 us at 40 tokens, 82.5 -> 76.4 at 128, and 113.5 -> 101.3 at 200,
+// where narrow tiles leave nothing to split.
+struct split_choice { int n, bn; };
+static split_choice pick_split(int M, int N, int K, int batch)
 {
-    // only problems whose 128 x 64 output tiles would occupy less than half of the SMs (a few hundred tokens at most)
-    if (N & 3) return 1;
-    const int tiles = d2d_cdiv(M, BM) * d2d_cdiv(N, 64) * (batch > 1 ? batch : 1);
-    const int nkb = d2d_cdiv(K, BK);
-    int splits = d2d_tc_sm_count() / (tiles > 0 ? tiles : 1);
-    if (splits > nkb / 2) splits = nkb / 2;          // at least two k-blocks per slice
-    return splits >= 2 ? splits : 1;
+    if (N & 3) return {1, 64};
+    const int nkb = d2d_cdiv(K, BK), sms = d2d_tc_sm_count();
+    const long rows = (long)d2d_cdiv(M, BM) * (batch > 1 ? batch : 1);
+    const int wide = (int)(sms / (rows * d2d_cdiv(N, 128)));
+    if (wide >= 2 && N % 128 == 0 && nkb / wide >= 40) return {wide, 128};
+    int splits = (int)(sms / (rows * d2d_cdiv(N, 64)));
+    if (splits > nkb / 2) splits = nkb / 2;
+    return {splits >= 2 ? splits : 1, 64};
 }
+
+int d2d_gemm_tc_splits(int M, int N, int K, int batch) { return M > 0 ? pick_split(M, N, K, batch).n : 1; }
 
 d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
 {
@@ -923,7 +933,8 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
             p.epilogue = D2D_EPI_PARTIAL_F32;
             p.bias = nullptr;
             p.out = g.partial;
-            const d2d_status rc = launch<64, D2D_EPI_PARTIAL_F32, 0, false>(p, st);
+            const d2d_status rc = pick_split(g.M, g.N, g.K, batch).bn == 128 ? launch<128, D2D_EPI_PARTIAL_F32, 0, false>(p, st)
+                                                                             : launch<64, D2D_EPI_PARTIAL_F32, 0, false>(p, st);
             if (rc != D2D_OK) return rc;
             const int blocks = d2d_cdiv(batch * g.M * g.N, 1024);
             cudaLaunchConfig_t cfg = {};

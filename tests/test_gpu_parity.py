@@ -1010,3 +1010,34 @@ def test_layers_in_a_row_without_synchronisation(api, T):
         assert float((a.float() - b.float()).norm() / a.float().norm()) <= 2.0 ** -6
     for layer in layers:
         layer.close()
+
+
+# down projections split along a long K, in slices of 128-column tiles: one to four row tiles of tokens around their edges, a ragged last
+# k-block, and a width that keeps the narrow tiles
+@pytest.mark.parametrize("d,d_ff,E,T", [(4096, 11008, 172, 65), (4096, 11008, 172, 129), (4096, 11008, 172, 256), (4096, 11008, 172, 257),
+                                        (1024, 5160, 129, 1100), (1032, 10304, 161, 200)])
+def test_down_projection_in_slices_of_k(api, d, d_ff, E, T):
+    g = torch.Generator(device="cuda").manual_seed(T)
+
+    def normal(*shape, std):
+        return (torch.randn(shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+
+    cfg = wl.LayerConfig("slices", "bf16", d=d, d_ff=d_ff, E=E, d_h=128, act="relu", T=T)
+    w = dict(w_r1=normal(128, d, std=d ** -0.5), b_r1=None, w_r2=normal(E, 128, std=0.1), b_r2=None, w1=normal(d_ff, d, std=d ** -0.5), b1=None,
+             w_gate=None, w2=normal(d, d_ff, std=0.02), b2=normal(d, std=0.02))
+    layer = api.Layer.from_config(cfg, w, device="cuda:0")
+    layer.set_expert_path("dense")
+    x = normal(T, d, std=1.0)
+    r = layer.new_routing(T)
+    _poison(r.perm), _poison(r.counts)
+    for rep in range(2):
+        y, _ = layer.layer_fwd(x, 0.3, routing=r)
+        torch.cuda.synchronize()
+        assert r.status == 0
+        G = torch.from_numpy(oracle.unpack_mask(r.mask_u32(), E).astype(np.float64)).cuda().repeat_interleave(cfg.s, 1)
+        h = (torch.relu(x.double() @ w["w1"].double().T) * G).to(torch.bfloat16).double()
+        ref = h @ w["w2"].double().T + w["b2"].double()
+        # y is rounded to bf16 (2^-9 of a value); h may be rounded the other way at ties of its float32 sum (2^-8 of some
+        # of d_ff values, far below that in the norm)
+        assert float((y.double() - ref).norm() / ref.norm()) <= 2.0 ** -8
+    layer.close()
