@@ -621,7 +621,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                             if (NT8 == 1 || (i >> 1) < T) st_async4(to + off, *reinterpret_cast<const uint4 *>(own + off), cluster_addr(full, warp));
                         }
                     }
-                    if (lane == 0) arrive_cluster(cluster_addr(smem_addr(&h_full[j < 0 ? 2 : j & 1]), warp), bytes);
+                    if (lane == 0) arrive_cluster(cluster_addr(full, warp), bytes);
                 } else if (lane == 0) {
                     d2d_tc::mbar_arrive(full);
                 }

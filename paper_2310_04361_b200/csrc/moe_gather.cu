@@ -29,9 +29,9 @@
 //   warps 6-13  epilogue: tcgen05.ld, bias, activation, selection bits, 32-byte stores to the token's row of H
 // Gated layers: a cluster of two CTAs shares tiles of 256 rows (tcgen05.mma.cta_group::2).  Each gathers its own 128 rows and
 // stages half of the weight rows (the leader W1's, its peer W_gate's), so that a k-block brings 32 KB into an SM instead of 48 and
-// the ring holds six instead of four; the leader's scheduler and MMA warps work for both.  Llama-shaped layer, up projection
-// back to back at 8192 tokens: 984 -> 883 us at u = 0.62 (0.62 -> 0.55 us a k-block: the gathered rows remain the bound), 436 -> 386
-// at 0.24; at 2560 tokens 350 -> 310 and 227 -> 192.
+// the ring holds six instead of four; the leader's scheduler and MMA warps work for both, the peer's MMA warp announces its rows to
+// the leader.  Llama-shaped layer, up projection back to back at 8192 tokens: 984 -> 883 us at u = 0.62 (0.62 -> 0.55 us a k-block:
+// the gathered rows remain the bound), 436 -> 386 at 0.24; at 2560 tokens 350 -> 310 and 227 -> 192.
 // Every wait is bounded (status D2D_ERR_TIMEOUT), all roles meet at the final barrier, TMEM is freed.
 #include "moe_gather.cuh"
 #include "tc_common.cuh"
@@ -46,6 +46,7 @@ constexpr int MAX_SUB = 1024;            // most tokens per scheduler draw (a mu
 constexpr int TR = 4;                    // tile descriptors in flight
 constexpr int FIFO_CAP = 2048;           // row entries; in use at any time: TR * 128 emitted + 127 pending + MAX_SUB new
 constexpr int MAX_STAGES = 8;
+constexpr uint32_t NOTE_BYTES = 16;      // of a stage of the pair's peer, copied to the leader to announce it (see forward_tile)
 #ifndef D2D_GATHER_WARPS
 #define D2D_GATHER_WARPS 4
 #endif
@@ -89,12 +90,20 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar)
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// `bytes` bytes of this CTA's shared memory to another CTA of the cluster, credited to a barrier there when they have arrived
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
 __host__ __device__ constexpr int pow2_cols(int v) { return v <= 32 ? 32 : v <= 64 ? 64 : v <= 128 ? 128 : 256; }
 
 // The MMA warp's work for one tile: nkb k-blocks from the stage ring into the accumulator at `acc`.  The A tiles were
 // written by cp.async (generic proxy) and their arrival is observed through the stage's barrier; the proxy fence that
 // makes them visible to the tensor core's (async-proxy) reads is executed here, between that observation and the MMAs.
-// PAIR: the leader's warp, for both CTAs; the peer's A tiles are announced to this CTA's barrier (see forward_tile).
+// PAIR: the leader's warp, for both CTAs; the peer's A tiles are announced to this CTA's barrier, which releases and acquires at
+// cluster scope (see forward_tile).
 template <bool PAIR = false>
 __device__ __forceinline__ bool mma_tile(uint8_t *smem, uint64_t *bar_full, uint64_t *bar_empty, uint64_t *acc_full, uint32_t acc,
                                          uint32_t idesc, int nkb, int stages, int stage_bytes, uint32_t &it, int32_t *status)
@@ -127,17 +136,23 @@ __device__ __forceinline__ bool mma_tile(uint8_t *smem, uint64_t *bar_full, uint
 }
 
 // Pairs, the peer's side: A stages that have landed here are announced to the leader, whose instructions make this SM's tensor
-// core read them.  The rows stay in this SM and the proxy fence has ordered them, so the arrival itself is relaxed: as a release at
-// cluster scope it waited for the gather's copies in flight and took longer than a k-block (Llama-shaped layer 1985 us instead of
-// 1600).
-__device__ __forceinline__ bool forward_tile(uint64_t *bar_full, int nkb, int stages, uint32_t &it, int32_t *status)
+// core read them.  What the leader goes on with are other threads' copies, so the announcement has to release them at cluster
+// scope (the leader's wait acquires there).  A warp that releases by itself (mbarrier.arrive.release.cluster) waits for it, longer
+// than a k-block takes.  So the copy engine does it: behind the proxy fence, 16 bytes of the stage are copied to a place of the
+// stage's own in the leader (`note`, which nobody reads), and the bytes are credited to the leader's barrier; that credit
+// (complete_tx) releases at cluster scope once the copy is done, and the warp goes on at once.  Llama-shaped layer, 8192 tokens,
+// tau = 0.4, back to back before the power limit sets in: 1608 us with two warps that release in turn, 1389 with four, 1339 this way
+// (1425 without pairs).  The copy has ended when the leader has consumed the stage.
+__device__ __forceinline__ bool forward_tile(uint8_t *smem, uint64_t *bar_full, uint4 *note, int nkb, int stages, int stage_bytes, uint32_t &it,
+                                             int32_t *status)
 {
     for (int kb = 0; kb < nkb; ++kb, ++it) {
         const uint32_t s = it % (uint32_t)stages, round = it / (uint32_t)stages;
         if (!mbar_wait_warp(smem_u32(&bar_full[s]), round & 1u, status)) return false;
         fence_async_smem();
         if (elect_one())
-            asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_to_cta(smem_u32(&bar_full[s]), 0)) : "memory");
+            bulk_copy_cluster(map_to_cta(smem_u32(&note[s]), 0), smem_u32(smem + (size_t)s * stage_bytes), NOTE_BYTES,
+                              map_to_cta(smem_u32(&bar_full[s]), 0));
         __syncwarp();
     }
     return true;
@@ -283,6 +298,7 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
     __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], bar_acc_full[2], bar_acc_empty[2], tile_full[TR], tile_empty[TR];
     __shared__ TileDesc tdesc[TR];
     __shared__ uint32_t tmem_base_holder;
+    __shared__ uint4 note[PAIR ? MAX_STAGES : 1];
     __shared__ uint32_t live[64];                             // scheduler: groups that still have sub-chunks (one bit each, E <= 2048)
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -295,8 +311,9 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
             // the W1 request (with its byte count) + one arrival per gather thread, triggered when its copies have landed
-            // (pairs: the leader's also counts the peer's announcement, whose own barrier counts its gather threads only)
-            mbar_init(smem_u32(&bar_full[s]), PAIR ? N_GATHER_WARPS * 32 + (rank == 0 ? 2 : 0) : 1 + N_GATHER_WARPS * 32);
+            // (pairs: the weight rows of both CTAs and the peer's announcement are bytes on the leader's barrier; the peer's own
+            // counts its gather threads only)
+            mbar_init(smem_u32(&bar_full[s]), (rank == 0 ? 1 : 0) + N_GATHER_WARPS * 32);
             mbar_init(smem_u32(&bar_empty[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -349,7 +366,7 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
             __syncwarp();
             if (n_rows < 0) break;
             if (elect_one()) tile_release(sl);
-            ok = forward_tile(bar_full, nkb, p.stages, it, p.status);
+            ok = forward_tile(smem, bar_full, note, nkb, p.stages, p.stage_bytes, it, p.status);
         }
     } else if (run && warp == WARP_SCHED) {
         run_scheduler<PAIR>(p, fifo, tile_full, tile_empty, tdesc, live, lane);
@@ -402,8 +419,9 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
                 const uint32_t stage = smem_u32(smem + (size_t)s * p.stage_bytes), full = smem_u32(&bar_full[s]);
                 if (gw == 0 && elect_one()) {
                     if (PAIR) {
-                        // the leader stages the up rows, its peer the gate rows; both are credited to the leader's barrier
-                        if (rank == 0) mbar_expect_tx(full, 2u * (uint32_t)(p.stage_bytes - A_BYTES));
+                        // the leader stages the up rows, its peer the gate rows; both are credited to the leader's barrier, as is
+                        // the peer's announcement of its own rows
+                        if (rank == 0) mbar_expect_tx(full, 2u * (uint32_t)(p.stage_bytes - A_BYTES) + NOTE_BYTES);
                         tma_load_2d_pair(stage + A_BYTES, rank == 0 ? &tm_w1 : &tm_wg, kb * BK, G * p.gs, map_to_cta(full, 0));
                     } else {
                         mbar_expect_tx(full, (uint32_t)(p.stage_bytes - A_BYTES));
