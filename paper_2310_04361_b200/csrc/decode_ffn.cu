@@ -133,6 +133,29 @@ __device__ __forceinline__ void widen16(const uint4 &r, uint32_t (&o)[8])
             : "=r"(o[2 * i]), "=r"(o[2 * i + 1]) : "r"(w[i]));
     }
 }
+__device__ __forceinline__ uint2 lds8(uint32_t addr)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint4 lds16(uint32_t addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+// Eight codes -> four bfloat16 pairs, in order (by way of float16: a code's value is exact in either)
+__device__ __forceinline__ void widen8(const uint2 &r, uint32_t (&o)[4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)((i < 2 ? r.x : r.y) >> (16 * (i & 1))), __NV_E4M3);
+        const float2 f = __half22float2(__half2(h));
+        const __nv_bfloat162 b = __floats2bfloat162_rn(f.x, f.y);
+        o[i] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+}
 // mma16816 on float16 operands
 __device__ __forceinline__ void mma16816_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -140,6 +163,62 @@ __device__ __forceinline__ void mma16816_f16(float (&d)[4], uint32_t a0, uint32_
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+
+// The up projection of a unit from codes and bfloat16 rows, for rows that float16 would not hold.  Rare, but what it does to the code
+// around it is paid by every call: a function of its own where accumulators leave registers for one, in line where they do not
+// (Llama-shaped layer, us, function / in line / float16 alone: 38.3 / 39.5 / 37.9 at 1 token, 55.4 / 57.1 / 54.9 at 2; with 8 tiles a
+// warp 68.0 / 61.9 / 60.8 at 6, 62.0 / 59.0 / 58.3 at 8).
+struct up_rows {
+    uint32_t bar_full, bar_empty, ring, xs;
+    int xp, T, d, nq, n_mat, stages, warp, slot;
+    uint32_t phase;
+    int32_t *status;                                          // NULL: a wait has run out before, there is nothing to wait for
+};
+template <int NT8, int CH> struct up_sums {
+    float v[2][NT8 * CH][4];
+    int slot;
+    uint32_t phase;
+    bool ok;
+};
+template <int NT8, int CH> __device__ __forceinline__ up_sums<NT8, CH> up_spread_rows(up_rows a)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    up_sums<NT8, CH> o;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int t = 0; t < NT8 * CH; ++t) o.v[m][t][0] = o.v[m][t][1] = o.v[m][t][2] = o.v[m][t][3] = 0.0f;
+    o.ok = a.status != nullptr;
+#pragma unroll 1
+    for (int q = 0; q < a.nq; ++q) {
+        const int k0 = q * seg_cols<uint8_t>() + a.warp * sub_cols<uint8_t>();
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+            if (m == 1 && a.n_mat == 1) break;
+            if (o.ok) o.ok = d2d_tc::mbar_wait_warp(a.bar_full + 8 * a.slot, a.phase, a.status);
+            const uint32_t st = a.ring + a.slot * STAGE_BYTES + a.warp * SUB_BYTES;
+#pragma unroll 1
+            for (int hp = 0; hp < 4 && k0 < a.d; ++hp) {      // half of the columns, 8-byte part of a 16-byte piece
+                const int h = hp >> 1, p = hp & 1;
+                uint32_t wa[2][4];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) widen8(lds8(st + swz(g + 8 * i, c * 16 + h * 64) + p * 8), wa[i]);
+#pragma unroll
+                for (int t = 0; t < NT8; ++t) {
+                    const uint4 xb = lds16(a.xs + min(t * 8 + g, a.T - 1) * a.xp + (k0 + h * 64) * 2 + c * 32 + p * 16);
+                    mma16816(o.v[m][t * CH], wa[0][0], wa[1][0], wa[0][1], wa[1][1], xb.x, xb.y);
+                    mma16816(o.v[m][t * CH + CH - 1], wa[0][2], wa[1][2], wa[0][3], wa[1][3], xb.z, xb.w);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) d2d_tc::mbar_arrive(a.bar_empty + 8 * a.slot);
+            if (++a.slot == a.stages) { a.slot = 0; a.phase ^= 1u; }
+        }
+    }
+    o.slot = a.slot; o.phase = a.phase;
+    return o;
+}
+template <int NT8, int CH> __device__ __noinline__ up_sums<NT8, CH> up_spread_rows_call(up_rows a) { return up_spread_rows<NT8, CH>(a); }
 
 __device__ __forceinline__ float act_accurate(int act, float z)
 {
@@ -190,7 +269,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     __shared__ unsigned int my_ticket;
     __shared__ volatile int rounds_s;                          // all rounds of this cluster, for the signalling warp
     __shared__ uint32_t x_max[Q8 ? T8 * 16 : 1];               // codes: largest magnitude of the pieces of the token rows ...
-    __shared__ float x_inv[T8];                                // ... and what takes the scaling of a row back
+    __shared__ float x_inv[T8];                                // ... what takes the scaling of a row back ...
+    __shared__ int x_spread;                                   // ... and whether some row does not fit float16
     const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, c = lane & 3;
     const int warp = __shfl_sync(FULL, tid >> 5, 0);           // warp-uniform for the compiler: see mma16816
     const int d = S.d, T = S.T, U = S.d_ff / 16, CL = S.cl, NCL = S.clusters;
@@ -337,7 +417,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         // ------------------------------------------------------------------ consumers
         // x does not depend on the router (the kernel behind which this one may start early waits for its own
         // predecessor before it lets this one start)
-        if (!Q8) {
+        auto load_x = [&]() {
             for (int i = tid, t = 0; t < T; ) {
                 if (i >= d / 8) { i -= d / 8; ++t; continue; }
                 cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
@@ -345,11 +425,19 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
+            consumer_bar();
+        };
+        if (!Q8) {
+            load_x();
         } else {
-            // as float16, scaled so that the largest value of the piece lies in [2^14, 2^15): WPT warps a token, a piece of the row each
+            // Codes widen to float16 in one instruction, to bfloat16 in four, so the rows become float16 where that loses nothing: scaled
+            // so that a row's largest value lies in [2^14, 2^15), float16 has all eight bits of a value down to 2^-17, that is of one whose
+            // exponent is at most 31 below the largest.  A batch with a non-zero value further below stays bfloat16.
+            // WPT warps a token, a piece of the row each.
             const int wpt = T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1, part = warp % wpt, np = d / 8;
             const int i0 = np * part / wpt, i1 = np * (part + 1) / wpt;
             uint32_t m = 0u;
+            if (tid == 0) x_spread = 0;
             for (int t = warp / wpt; t < T; t += NCW / wpt) {
                 const uint4 *row = reinterpret_cast<const uint4 *>(x + (size_t)t * d);
                 m = 0u;
@@ -364,11 +452,14 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 if (lane == 0) x_max[t * 16 + part] = m;
             }
             consumer_bar();
+            bool spread = false;
             for (int t = warp / wpt; t < T; t += NCW / wpt) {
                 m = 0u;
                 for (int q = 0; q < wpt; ++q) m = max(m, x_max[t * 16 + q]);
                 const int sh = min(120, 141 - (int)(m >> 7));
                 const float f = __uint_as_float((uint32_t)(127 + sh) << 23);
+                // the smallest magnitude that fits, less one: magnitudes less one are compared, so that zeros fit
+                const uint32_t least = (uint32_t)max(((int)(m >> 7) - 31) * 128 - 1, 0);
                 if (lane == 0 && part == 0) x_inv[t] = __uint_as_float((uint32_t)(127 - sh) << 23);
                 for (int i = i0 + lane; i < i1; i += 32) {
                     uint4 *at = reinterpret_cast<uint4 *>(xs + (size_t)t * xp + i * 16);
@@ -377,14 +468,20 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                     uint32_t o[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
+                        spread |= ((w[q] & 0x7fffu) - 1u < least) | (((w[q] >> 16) & 0x7fffu) - 1u < least);
                         const float lo = __uint_as_float(w[q] << 16) * f, hi = __uint_as_float(w[q] & 0xffff0000u) * f;
                         asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(o[q]) : "f"(hi), "f"(lo));
                     }
                     *at = make_uint4(o[0], o[1], o[2], o[3]);
                 }
             }
+            if (spread) x_spread = 1;
+            consumer_bar();
+            if (__builtin_expect(x_spread != 0, 0)) {
+                if (tid < T) x_inv[tid] = 1.0f;
+                load_x();
+            }
         }
-        consumer_bar();
 
         int slot = 0, n = 0;
         uint32_t phase = 0;
@@ -425,8 +522,21 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             for (int m = 0; m < 2; ++m)
 #pragma unroll
                 for (int t = 0; t < NT8 * CH; ++t) s[m][t][0] = s[m][t][1] = s[m][t][2] = s[m][t][3] = 0.0f;
+            const bool spread = Q8 && *(volatile int *)&x_spread != 0;        // (read here: a register less)
+            if (Q8 && __builtin_expect(spread, 0)) {
+                const up_rows a = {smem_addr(bar_full), smem_addr(bar_empty), smem_addr(ring), smem_addr(xs), xp, T, d,
+                                   nq, n_mat, S.stages, warp, slot, phase, ok ? P.status : nullptr};
+                const up_sums<NT8, CH> o = TPW * NT8 <= 4 ? up_spread_rows_call<NT8, CH>(a) : up_spread_rows<NT8, CH>(a);
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int t = 0; t < NT8 * CH; ++t)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) s[m][t][i] = o.v[m][t][i];
+                slot = o.slot; phase = o.phase; ok = ok && o.ok;
+            }
 #pragma unroll 1
-            for (int q = 0; q < nq; ++q) {
+            for (int q = spread ? nq : 0; q < nq; ++q) {
                 const int k0 = q * SEG + warp * SUB;
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {

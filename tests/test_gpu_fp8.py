@@ -131,3 +131,31 @@ def test_8bit_expert_step_on_rows_of_any_scale(api, T):
             ref = h @ wq["w2"].astype(np.float64).T
             assert np.linalg.norm(y[t] - ref) <= 1e-2 * np.linalg.norm(ref), (start, t)
     layer.close()
+
+
+# Rows whose values lie further apart than float16 reaches: one value 2^16 .. 2^120 times the others, whose weights are zero, so that
+# the others are all there is.  31 powers of two below the largest is where float16 begins to lose bits (the small values of a normal
+# distribution first); the rows before and behind it take different formats, and so does a batch with one such row.  Errors as above.
+@pytest.mark.parametrize("gated,T", [(False, 1), (True, 2), (False, 6), (True, 8), (False, 20)])
+def test_8bit_expert_step_on_rows_of_any_spread(api, gated, T):
+    cfg = wl.LayerConfig("spread", "bf16", d=384, d_ff=512, E=32, d_h=64, act="relu", gated=gated, T=T, b1_shift=None, has_b2=False, seed=62)
+    w = wl.make_weights(cfg)
+    w["w1"][:, 7] = 0.0
+    if gated:
+        w["w_gate"][:, 7] = 0.0
+    _, wq = _quantised(cfg, w)
+    layer = api.Layer.from_config(cfg, w, fp8_experts=True)
+    rng = np.random.default_rng(T)
+    r = api.routing_from_mask(torch.full((T, 1), -1, dtype=torch.int32, device="cuda"), cfg.E)
+    for e in (16, 24, 28, 30, 31, 32, 33, 40, 60, 120):
+        x = wl.round_to_bf16(rng.standard_normal((T, cfg.d)).astype(np.float32))
+        x[T // 2, 7] = 2.0 ** e
+        x[:, 11] = 0.0
+        y = layer.moe_ffn_fwd(api.to_device(x, cfg.dtype), r).float().cpu().numpy().astype(np.float64)
+        xs, w1 = x.astype(np.float64), wq["w1"].astype(np.float64)
+        h = xs @ w1.T
+        h = np.maximum(xs @ wq["w_gate"].astype(np.float64).T, 0.0) * h if gated else np.maximum(h, 0.0)
+        ref = h @ wq["w2"].astype(np.float64).T
+        for t in range(T):
+            assert np.linalg.norm(y[t] - ref[t]) <= 1e-2 * np.linalg.norm(ref[t]), (e, t)
+    layer.close()
