@@ -169,7 +169,7 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
     // hidden activations H [T, d_ff] bf16 of the dense-masked path
     if (L->desc.dtype == D2D_BF16 && T > d2d_decode_max_tokens(L->desc)) {
         size_t h = d2d_align_up((size_t)T * L->desc.d_ff * 2, 256);
-        if (d2d_gemm_tc_splits(T, L->desc.d, L->desc.d_ff) > 1) h += d2d_align_up((size_t)T * L->desc.d * 4, 256);   // split-K partial sums
+        h += d2d_align_up(d2d_gemm_tc_partial_floats(T, L->desc.d, L->desc.d_ff) * 4, 256);      // split-K partial sums
         if (h > need) need = h;
     }
     return need;
@@ -295,7 +295,7 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
         up.a = x; up.b = L->w1; up.b_gate = D.gated ? L->w_gate : nullptr; up.b_cat = L->w1g; up.b_cat_block = 128; up.bias = L->b1; up.out = ws;
         up.M = T; up.N = D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
         up.mask = r->mask; up.mask_words = (D.n_experts + 31) / 32; up.expert_size = D.expert_size; up.status = r->status;
-        if (forced && k_splits > 1) { up.zero = partial; up.zero_floats = (long long)T * D.d; }
+        if (forced && k_splits > 1) { up.zero = partial; up.zero_floats = (long long)d2d_gemm_tc_partial_floats(T, D.d, D.d_ff); }
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
     }

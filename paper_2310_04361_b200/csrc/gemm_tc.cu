@@ -43,6 +43,7 @@ struct EpiParams {
     long long n_sel_max;
     float4 *zero;                    // optional: cleared by the epilogue warps before their first tile (see d2d_gemm_args)
     int zero_n;                      // 16-byte pieces
+    int slices_per_sum;              // split-K: so many slices add to one float32 buffer (see pick_split)
     int test_skip_load;              // test aid: CTA 0 never requests the A tile of its first k-block (see d2d_gemm_args)
 };
 
@@ -463,7 +464,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                 if (go) {
                     int tile = (!GATED && k_splits == 1) ? item : item / k_splits;
                     int prob = 0, tr, tc;
+                    const int sum = EPI == D2D_EPI_PARTIAL_F32 ? (item - tile * k_splits) / ep.slices_per_sum : 0;
                     if (ep.batch > 1) { prob = tile / tiles_pp; tile -= prob * tiles_pp; }
+                    prob += sum * ep.batch;                    // the buffers' problems follow one another
                     tile_coords(tile, (M + TM - 1) / TM, n_tiles, ep.band_rows, tr, tc);
                     epi_m0[buf] = tr * TM + rank * BM; epi_n0[buf] = tc * BN; epi_prob[buf] = prob;
                     go = mbar_wait(smem_u32(&bar_acc_full[buf]), use & 1u, ep.status);
@@ -675,11 +678,11 @@ template <typename K> bool ensure_smem_attr(K kern, size_t smem, bool (&done)[64
 }
 
 template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false, int LISTS = 0>
-d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
+d2d_status launch(const d2d_gemm_args &g, cudaStream_t st, int slices_per_sum = 1)
 {
     if constexpr ((EPI == D2D_EPI_BIAS_BF16 || EPI == D2D_EPI_PARTIAL_F32) && LISTS == 0) {
-        if (g.lists.n == 1) return launch<BN, EPI, ACT, GATED, PAIR, 1>(g, st);
-        if (g.lists.n > 1) return launch<BN, EPI, ACT, GATED, PAIR, D2D_MAX_GROUP>(g, st);
+        if (g.lists.n == 1) return launch<BN, EPI, ACT, GATED, PAIR, 1>(g, st, slices_per_sum);
+        if (g.lists.n > 1) return launch<BN, EPI, ACT, GATED, PAIR, D2D_MAX_GROUP>(g, st, slices_per_sum);
     }
     constexpr int B_ROWS = PAIR && !GATED ? BN / 2 : BN, TM = PAIR ? 2 * BM : BM;
     constexpr int STAGE_BYTES = BM * BK * 2 + (GATED && !PAIR ? 2 : 1) * B_ROWS * BK * 2;
@@ -715,7 +718,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st)
     EpiParams ep{(const __nv_bfloat16 *)g.bias, g.out, g.mask, g.mask_words, es, g.status,
                  (uint32_t)((0x100000000ull + (unsigned long long)es - 1) / (unsigned long long)es),
                  g.tile_counter, (g.pdl_late_wait && !g.n_sel && d2d_tc_pdl_enabled()) ? 1 : 0, gate_cat ? 1 : 0,
-                 band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max, (float4 *)g.zero, g.zero ? (int)(g.zero_floats / 4) : 0,
+                 band_rows_for(g.M, g.N, g.K, TM, GATED), batch, g.n_sel, g.n_sel_max, (float4 *)g.zero, g.zero ? (int)(g.zero_floats / 4) : 0, slices_per_sum,
                  (g.test_skip_load && !g.tile_counter && !g.pdl_late_wait && !g.n_sel) ? 1 : 0};
     typename ListsOf<LISTS>::type lists = {};
     set_lists(lists, g);
@@ -810,16 +813,20 @@ d2d_status launch_up(const d2d_gemm_args &g, cudaStream_t st)
 
 }  // namespace
 
-// y = bf16(partial + bias) after a split-K GEMM; `batch` problems back to back ([batch, M, N] sums, [batch, N] bias)
+// y = bf16(sum of the buffers + bias) after a split-K GEMM; `batch` problems back to back ([sums, batch, M, N], [batch, N] bias)
 __global__ void __launch_bounds__(256)
 splitk_finalize_kernel(const float *__restrict__ partial, const __nv_bfloat16 *__restrict__ bias, __nv_bfloat16 *__restrict__ out,
-                       int M, int N, int batch)
+                       int M, int N, int batch, int sums)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t per = (size_t)M * N, total = per * batch;
     for (size_t i = ((size_t)blockIdx.x * 256 + threadIdx.x) * 4; i < total; i += (size_t)gridDim.x * 1024) {
-        const float4 v = __ldcg(reinterpret_cast<const float4 *>(partial + i));
+        float4 v = __ldcg(reinterpret_cast<const float4 *>(partial + i));
+        for (int s = 1; s < sums; ++s) {
+            const float4 w = __ldcg(reinterpret_cast<const float4 *>(partial + (size_t)s * total + i));
+            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+        }
         const int c = (int)(i / per) * N + (int)(i % N);
         const float o[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -903,20 +910,32 @@ bool d2d_gemm_tc_available() { return get_encode() != nullptr; }
 // 3.1 TB/s on 90 MB of weights): they are taken where a slice is 40 k-blocks or more (14 us of main loop, against about 4 for the
 // sums).  Llama-shaped layer (d_ff = 11008), back to back: 74.7 -> 68.3 us at 40 tokens, 82.5 -> 76.4 at 128, and 113.5 -> 101.3 at 200,
 // where narrow tiles leave nothing to split.
-struct split_choice { int n, bn; };
+// A slice adds its partial sums to a float32 buffer.  Wide tiles have a buffer for every two slices: the sum of two does not depend on
+// which comes first, and the buffers are added in order, so these batches (Llama-shaped layer, 9 to 256 tokens) give the same bits on
+// every call.  Narrow tiles, mostly in more slices, share one buffer and do not (a buffer a slice: 23.8 instead of 22.1 us for the
+// BERT-shaped layer of 128 tokens, 29.3 instead of 27.5 for the GPT-2-medium-shaped one of 200).
+struct split_choice { int n, bn, per_sum; };
 static split_choice pick_split(int M, int N, int K, int batch)
 {
-    if (N & 3) return {1, 64};
+    if (N & 3) return {1, 64, 1};
     const int nkb = d2d_cdiv(K, BK), sms = d2d_tc_sm_count();
     const long rows = (long)d2d_cdiv(M, BM) * (batch > 1 ? batch : 1);
     const int wide = (int)(sms / (rows * d2d_cdiv(N, 128)));
-    if (wide >= 2 && N % 128 == 0 && nkb / wide >= 40) return {wide, 128};
+    if (wide >= 2 && N % 128 == 0 && nkb / wide >= 40) return {wide, 128, 2};
     int splits = (int)(sms / (rows * d2d_cdiv(N, 64)));
     if (splits > nkb / 2) splits = nkb / 2;
-    return {splits >= 2 ? splits : 1, 64};
+    if (splits < 2) splits = 1;
+    return {splits, 64, splits};
 }
 
 int d2d_gemm_tc_splits(int M, int N, int K, int batch) { return M > 0 ? pick_split(M, N, K, batch).n : 1; }
+
+size_t d2d_gemm_tc_partial_floats(int M, int N, int K, int batch)
+{
+    if (M <= 0) return 0;
+    const split_choice c = pick_split(M, N, K, batch);
+    return c.n > 1 ? (size_t)d2d_cdiv(c.n, c.per_sum) * (batch > 1 ? batch : 1) * M * N : 0;
+}
 
 d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
 {
@@ -928,13 +947,16 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
     case D2D_EPI_BIAS_BF16:
         if (g.k_splits > 1 && g.partial) {
             const int batch = g.batch > 1 ? g.batch : 1;
-            if (!g.partial_zero && cudaMemsetAsync(g.partial, 0, (size_t)batch * g.M * g.N * sizeof(float), st) != cudaSuccess) return D2D_ERR_CUDA;
+            const split_choice c = pick_split(g.M, g.N, g.K, batch);
+            const int sums = d2d_cdiv(c.n, c.per_sum);
+            if (c.n != g.k_splits) return D2D_ERR_INVALID_ARG;
+            if (!g.partial_zero && cudaMemsetAsync(g.partial, 0, (size_t)sums * batch * g.M * g.N * sizeof(float), st) != cudaSuccess) return D2D_ERR_CUDA;
             d2d_gemm_args p = g;
             p.epilogue = D2D_EPI_PARTIAL_F32;
             p.bias = nullptr;
             p.out = g.partial;
-            const d2d_status rc = pick_split(g.M, g.N, g.K, batch).bn == 128 ? launch<128, D2D_EPI_PARTIAL_F32, 0, false>(p, st)
-                                                                             : launch<64, D2D_EPI_PARTIAL_F32, 0, false>(p, st);
+            const d2d_status rc = c.bn == 128 ? launch<128, D2D_EPI_PARTIAL_F32, 0, false>(p, st, c.per_sum)
+                                              : launch<64, D2D_EPI_PARTIAL_F32, 0, false>(p, st, c.per_sum);
             if (rc != D2D_OK) return rc;
             const int blocks = d2d_cdiv(batch * g.M * g.N, 1024);
             cudaLaunchConfig_t cfg = {};
@@ -947,7 +969,7 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
             cfg.attrs = attr;
             cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
             const cudaError_t err = cudaLaunchKernelEx(&cfg, splitk_finalize_kernel, (const float *)g.partial, (const __nv_bfloat16 *)g.bias,
-                                                       (__nv_bfloat16 *)g.out, g.M, g.N, batch);
+                                                       (__nv_bfloat16 *)g.out, g.M, g.N, batch, sums);
             D2D_LAUNCHED(1);
             return err == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
         }

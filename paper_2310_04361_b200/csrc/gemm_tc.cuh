@@ -33,8 +33,8 @@ struct d2d_gemm_args {
     int expert_size;         // s: column c belongs to expert c / s
     int32_t *status;         // device status word, receives D2D_ERR_TIMEOUT if a bounded wait runs out
     // Split-K (D2D_EPI_BIAS_BF16 only): with k_splits > 1 the K range is cut into slices that run as separate work
-    // items, partial sums meet in `partial` (float32 [M, N], cleared by the call), a small kernel adds the bias and
-    // converts.  For problems with so few output tiles that most SMs would idle (decode batches).
+    // items, partial sums meet in `partial` (float32, d2d_gemm_tc_partial_floats of them, cleared by the call), a small kernel adds
+    // the bias and converts.  k_splits is d2d_gemm_tc_splits' number.  For problems with so few output tiles that most SMs would idle (decode batches).
     int k_splits;
     float *partial;
     int partial_zero;        // 1: an earlier kernel of the stream has cleared `partial`
@@ -72,8 +72,9 @@ struct d2d_gemm_args {
     int test_skip_load;
 };
 
-// Number of K slices d2d_gemm_tc would use for a [M,N,K] down projection (1 = no split) and the float32 scratch it needs.
+// Number of K slices d2d_gemm_tc would use for a [M,N,K] down projection (1 = no split), and the float32 scratch it then needs.
 int d2d_gemm_tc_splits(int M, int N, int K, int batch = 1);
+size_t d2d_gemm_tc_partial_floats(int M, int N, int K, int batch = 1);
 
 // Whether the lists of a batch can be left to the GEMM of its down projection: as many tokens as a CTA's epilogue warps take in one
 // go (512) or, before a main loop that is not split, in two.  On a stream of their own they cost the layer a launch, two events

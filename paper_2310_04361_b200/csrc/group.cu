@@ -54,7 +54,7 @@ struct group_layout {
     size_t y32_off, y32_each;      // per-layer float32 output accumulators (decode path)
     size_t mask_off;               // merged mask [T, n*W]
     size_t h_off;                  // merged hidden activations [T, n*d_ff] bf16
-    size_t partial_off;            // split-K sums of the batched down projection [n, T, d] float32
+    size_t partial_off;            // split-K sums of the batched down projection
     size_t seq_off;                // workspace of the sequential fallback
     size_t total;
 };
@@ -76,7 +76,7 @@ group_layout layout_for(const d2d_group *g, int T)
     w.h_off = off;
     if (g->merged) off += d2d_align_up(Tn * n * D.d_ff * 2, 256);
     w.partial_off = off;
-    if (g->merged && d2d_gemm_tc_splits((int)Tn, D.d, D.d_ff, g->n) > 1) off += d2d_align_up(n * Tn * D.d * 4, 256);
+    if (g->merged) off += d2d_align_up(d2d_gemm_tc_partial_floats((int)Tn, D.d, D.d_ff, g->n) * 4, 256);
     w.seq_off = off;
     off += d2d_layer_ws_bytes(g->layers[0], (int)Tn);
     w.total = off;
@@ -233,7 +233,7 @@ d2d_status d2d_group_fwd(const d2d_group *g, const void *x, int32_t T, float tau
         up.M = T; up.N = n * D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
         up.mask = mask_cat; up.mask_words = n * W; up.expert_size = D.expert_size; up.status = routing[0].status;
         float *partial = k_splits > 1 ? (float *)(base + w.partial_off) : nullptr;
-        up.zero = partial; up.zero_floats = (long long)n * T * D.d;
+        up.zero = partial; up.zero_floats = (long long)d2d_gemm_tc_partial_floats(T, D.d, D.d_ff, n);
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
         d2d_gemm_args dn = {};

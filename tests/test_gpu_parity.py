@@ -1041,3 +1041,22 @@ def test_down_projection_in_slices_of_k(api, d, d_ff, E, T):
         # of d_ff values, far below that in the norm)
         assert float((y.double() - ref).norm() / ref.norm()) <= 2.0 ** -8
     layer.close()
+
+
+# Down projections split into slices of 128-column tiles give the same bits on every call, in whatever order the slices finish (four
+# slices, the same with a ragged row tile, two; in front of them either up projection).
+@pytest.mark.parametrize("T,path", [(40, "dense"), (128, "dense"), (200, "dense"), (100, "gather")])
+def test_wide_split_down_projections_repeat(api, T, path):
+    cfg = wl.with_tokens(wl.CONFIGS["llama"], T)
+    layer = api.Layer.from_config(cfg, wl.make_weights(cfg), device="cuda:0")
+    layer.set_expert_path(path)
+    x = api.to_device(wl.make_tokens(cfg), cfg.dtype)
+    ws = layer.workspace(T)
+    first = None
+    for rep in range(12):
+        _poison(ws)
+        y = layer.layer_fwd(x, 0.3)[0].clone()
+        first = y if first is None else first
+        assert torch.equal(y.view(torch.int16), first.view(torch.int16)), rep
+    assert bool(torch.isfinite(first.float()).all())
+    layer.close()
