@@ -195,7 +195,7 @@ D2D_API d2d_status d2d_layer_destroy(d2d_layer *layer);
  *                    kernels are enqueued and the pair not needed returns at once,
  *                    so there is no host synchronisation.  Batches whose up
  *                    projection is below 2e11 FLOP (about 150 us of tensor-core
- *                    time; 3.2e11 for gated layers with the library's rho_max)
+ *                    time; 2.4e11 for gated layers with the library's rho_max)
  *                    always take the dense form: the gathered kernels'
  *                    fixed costs leave them little to win there, and the dense
  *                    kernel then keeps its overlap with the router.

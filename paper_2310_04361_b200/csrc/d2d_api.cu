@@ -194,11 +194,15 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 int d2d_tc_sm_count();      // gemm_tc.cu
 
 // Smallest up projection for which the automatic choice is made, see path_before_launch.  Gated layers with the library's own limit on
-// the density: more, since smaller ones leave the gathered pair a few densities and lose the overlap with the router at the others
-// (Llama-shaped layer back to back, dense / with the choice, which takes the gathered pair where marked *: 1200 tokens 291 / 337 at
-// rho = 0.22, 293 / 331 at 0.03; 1500 tokens 334 / 396 at 0.22, 336 / 379 at 0.07, 323 / 287* at 0.03; above the line, 1800 tokens 406 /
-// 470, 397 / 369*, 397 / 328*; 2560 tokens 592 / 626 at 0.22, 553 / 508* at 0.12, 512 / 443* at 0.07).
-static double auto_min_up_flop(const d2d_layer *L) { return L->desc.gated && L->gather_rho_max < 0.0 ? 3.2e11 : 2e11; }
+// the density: from where that limit lets the gathered pair in at 3.5 % of the pairs (1330 tokens of the Llama-shaped layer);
+// below, the choice would only cost them the overlap with the router.  Above it the choice is what lets sparse batches take the gathered
+// pair, and costs dense ones that overlap and the launches.  Llama-shaped layer, interleaved (us, dense form / with the choice, * =
+// which took the gathered pair):
+//     1400 tokens  rho 0.22  338 / 372   0.07  333 / 366    0.03  318 / 291*
+//     1500         rho 0.22  339 / 377   0.07  335 / 366    0.03  319 / 292*
+//     1760         rho 0.22  385 / 440   0.07  361 / 347*   0.03  348 / 300*
+// The line was at 3.2e11 for a while, which kept the first column and gave away the last (370 instead of 297 at 1760 tokens).
+static double auto_min_up_flop(const d2d_layer *L) { return L->desc.gated && L->gather_rho_max < 0.0 ? 2.4e11 : 2e11; }
 
 static double default_gather_rho_max(const d2d_layer_desc &D, int g, int T)
 {

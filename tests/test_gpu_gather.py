@@ -337,3 +337,28 @@ def test_fused_gathered_step_equals_oracle(api, name, T, g, d, ps):
     with pytest.raises(api.D2DError):
         layer.set_expert_path("fused", group=64)
     layer.close()
+
+
+# Where the automatic choice of a gated layer begins: sparse batches take the gathered pair from there on, others and shorter ones the
+# dense pair, and the call does what expert_path_for says (equal bits with that form forced).
+@pytest.mark.parametrize("T,rho,want", [(1300, 0.04, "dense"), (1400, 0.03, "gather"), (1500, 0.2, "dense"), (1760, 0.06, "gather"), (1760, 0.2, "dense")])
+def test_automatic_choice_of_gated_layers(api, T, rho, want):
+    g = torch.Generator(device="cuda").manual_seed(T)
+
+    def normal(*shape, std):
+        return (torch.randn(shape, generator=g, device="cuda") * std).to(torch.bfloat16)
+
+    base = wl.with_tokens(wl.CONFIGS["llama"], T)
+    w = dict(w_r1=normal(base.d_h, base.d, std=base.d ** -0.5), b_r1=None, w_r2=normal(base.E, base.d_h, std=0.1), b_r2=None,
+             w1=normal(base.d_ff, base.d, std=0.02), b1=None, w_gate=normal(base.d_ff, base.d, std=0.02), w2=normal(base.d, base.d_ff, std=0.02), b2=None)
+    layer = api.Layer.from_config(base, w, device="cuda:0")
+    x = normal(T, base.d, std=1.0)
+    keep = torch.rand((T, 32 * ((base.E + 31) // 32)), generator=g, device="cuda") < rho
+    keep[:, base.E:] = False
+    words = (keep.view(T, -1, 32).long() << torch.arange(32, device="cuda")).sum(-1)
+    r = api.routing_from_mask(torch.where(words >= 1 << 31, words - (1 << 32), words).to(torch.int32), base.E)
+    assert layer.expert_path_for(T, r.n_sel) == want
+    y = layer.moe_ffn_fwd(x, r)
+    layer.set_expert_path(want)
+    assert torch.equal(y.view(torch.int16), layer.moe_ffn_fwd(x, r).view(torch.int16))
+    layer.close()
