@@ -42,9 +42,12 @@ using namespace d2d_tc;
 
 constexpr int BM = 128, BK = 64, UMMA_K = 16;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int MAX_SUB = 1024;            // most tokens per scheduler draw (a multiple of 256 chosen per launch, see launch())
+constexpr int PIECE = 256;               // tokens the scheduler looks at before it emits the tiles they fill
 constexpr int TR = 4;                    // tile descriptors in flight
-constexpr int FIFO_CAP = 2048;           // row entries; in use at any time: TR * 128 emitted + 127 pending + MAX_SUB new
+// Row entries.  In use at any time, with tiles of up to 2 * BM rows (pairs): those of TR tiles that are emitted and not yet read by
+// all, less than a tile's pending, a piece's new ones.
+constexpr int FIFO_CAP = 2048;
+static_assert(TR * 2 * BM + (2 * BM - 1) + PIECE <= FIFO_CAP, "row entries are overwritten only after they have been read");
 constexpr int MAX_STAGES = 8;
 constexpr uint32_t NOTE_BYTES = 16;      // of a stage of the pair's peer, copied to the leader to announce it (see forward_tile)
 #ifndef D2D_GATHER_WARPS
@@ -168,7 +171,7 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
 {
     constexpr int TM = PAIR ? 2 * BM : BM;
     const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-    const int Ng = p.n_groups, SUB = p.sub, n_sub = (p.T + SUB - 1) / SUB;        // SUB is a multiple of 256
+    const int Ng = p.n_groups, SUB = p.sub, n_sub = (p.T + SUB - 1) / SUB;        // SUB is a multiple of PIECE
     // Groups the CTAs work in at the same time.  The host's value keeps that many groups' weight rows in L2.  When
     // few tokens keep a group, a visit of a CTA to a group should still yield several full tiles (its last tile is
     // ragged and costs as much as a full one), so the CTAs spread over more groups: with gridDim.x / Wn CTAs per
@@ -248,8 +251,8 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
             const int t_end = min((c + 1) * SUB, p.T);
             uint32_t bits[8], bits_next[8];
             load_piece(c * SUB, bits);
-            for (int t0 = c * SUB; t0 < t_end && ok; t0 += 256) {
-                if (t0 + 256 < t_end) load_piece(t0 + 256, bits_next);
+            for (int t0 = c * SUB; t0 < t_end && ok; t0 += PIECE) {
+                if (t0 + PIECE < t_end) load_piece(t0 + PIECE, bits_next);
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const bool keep = bits[q] != 0u;
@@ -288,10 +291,11 @@ __device__ __forceinline__ void run_scheduler(const GatherParams &p, uint32_t *f
     }
 }
 
-template <int ACT, bool GATED, bool PAIR>
+template <int ACT, bool GATED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_constant__ CUtensorMap tm_wg, const GatherParams p)
 {
+    constexpr bool PAIR = GATED;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint32_t *fifo = reinterpret_cast<uint32_t *>(smem + (size_t)p.stages * p.stage_bytes);     // [FIFO_CAP] token indices
@@ -426,7 +430,6 @@ moe_gather_up_kernel(const __grid_constant__ CUtensorMap tm_w1, const __grid_con
                     } else {
                         mbar_expect_tx(full, (uint32_t)(p.stage_bytes - A_BYTES));
                         tma_load_2d(stage + A_BYTES, &tm_w1, kb * BK, G * p.gs, full);
-                        if (GATED) tma_load_2d(stage + A_BYTES + p.gs * 128, &tm_wg, kb * BK, G * p.gs, full);
                     }
                 }
                 const bool in_k = kb * BK + chunk * 8 < p.d;                       // zero fill past K
@@ -1146,18 +1149,18 @@ bool ensure_attr(const void *kern, bool (&done)[64])
     return true;
 }
 
-template <int ACT, bool GATED, bool PAIR = false>
+template <int ACT, bool GATED>
 d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
 {
+    constexpr bool PAIR = GATED;
     const int gs = a.g * a.s;
-    const int b_rows = GATED && !PAIR ? 2 * gs : gs;        // staged by one CTA
     GatherParams p = {};
     p.x = (const __nv_bfloat16 *)a.x; p.mask = a.mask; p.b1 = (const __nv_bfloat16 *)a.b1; p.H = (__nv_bfloat16 *)a.H;
     p.status = a.status; p.ctr = a.ctr; p.n_sel = a.n_sel; p.n_sel_min = a.n_sel_min; p.n_sel_max = a.n_sel_max;
     p.T = a.T; p.d = a.d; p.d_ff = a.d_ff; p.W = (a.n_experts + 31) / 32;
     p.g = a.g; p.s = a.s; p.gs = gs; p.n_groups = a.n_experts / a.g;
     p.inv_s = (uint32_t)((0x100000000ull + (unsigned long long)a.s - 1) / (unsigned long long)a.s);
-    p.stage_bytes = A_BYTES + b_rows * 128;
+    p.stage_bytes = A_BYTES + gs * 128;                      // (a pair's CTA stages the rows of one of the two matrices)
     int stages = (192 * 1024) / p.stage_bytes;
     p.stages = stages > MAX_STAGES ? MAX_STAGES : stages;
     // about 48 MB of weight rows in flight: the rest of L2 holds the token rows and the outputs
@@ -1168,7 +1171,7 @@ d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
     p.visit_tiles = PAIR ? 4.0f : 8.0f;
     // tokens per draw: about eight draws per CTA (the CTAs then finish together), 256 .. 1024
     const long long want = (long long)a.T * p.n_groups / (8ll * d2d_tc_sm_count());
-    p.sub = want >= 1024 ? 1024 : want >= 512 ? 512 : 256;
+    p.sub = want >= 4 * PIECE ? 4 * PIECE : want >= 2 * PIECE ? 2 * PIECE : PIECE;
     const size_t smem = (size_t)p.stages * p.stage_bytes + FIFO_CAP * 4 + 1024;      // at most 192 + 8 + 1 KB
     if (smem > 208 * 1024) return D2D_ERR_UNSUPPORTED;
     CUtensorMap tw1, twg;
@@ -1178,7 +1181,7 @@ d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
     } else {
         twg = tw1;
     }
-    auto kern = moe_gather_up_kernel<ACT, GATED, PAIR>;
+    auto kern = moe_gather_up_kernel<ACT, GATED>;
     static bool attr_set[64] = {};
     if (!ensure_attr((const void *)kern, attr_set)) return D2D_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
@@ -1198,14 +1201,14 @@ d2d_status launch(const d2d_gather_args &a, cudaStream_t st)
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
-template <bool GATED, bool PAIR = false>
+template <bool GATED>
 d2d_status launch_act(const d2d_gather_args &a, cudaStream_t st)
 {
     switch (a.act) {
-    case D2D_ACT_RELU: return launch<D2D_ACT_RELU, GATED, PAIR>(a, st);
-    case D2D_ACT_GELU_ERF: return launch<D2D_ACT_GELU_ERF, GATED, PAIR>(a, st);
-    case D2D_ACT_GELU_TANH: return launch<D2D_ACT_GELU_TANH, GATED, PAIR>(a, st);
-    case D2D_ACT_SILU: return launch<D2D_ACT_SILU, GATED, PAIR>(a, st);
+    case D2D_ACT_RELU: return launch<D2D_ACT_RELU, GATED>(a, st);
+    case D2D_ACT_GELU_ERF: return launch<D2D_ACT_GELU_ERF, GATED>(a, st);
+    case D2D_ACT_GELU_TANH: return launch<D2D_ACT_GELU_TANH, GATED>(a, st);
+    case D2D_ACT_SILU: return launch<D2D_ACT_SILU, GATED>(a, st);
     }
     return D2D_ERR_INVALID_ARG;
 }
@@ -1233,7 +1236,7 @@ d2d_status d2d_moe_gather_up(const d2d_gather_args &a, cudaStream_t st)
 {
     if (a.T <= 0) return D2D_OK;
     if (a.g < 1 || a.g > 32 || a.n_experts > 2048) return D2D_ERR_UNSUPPORTED;
-    return a.w_gate ? launch_act<true, true>(a, st) : launch_act<false>(a, st);
+    return a.w_gate ? launch_act<true>(a, st) : launch_act<false>(a, st);
 }
 
 bool d2d_moe_down_masked_supports(const d2d_layer_desc &D)
@@ -1381,7 +1384,7 @@ static d2d_status launch_ffn(const d2d_gather_args &a, float *y32, void *y, cons
     if (p.window > p.n_groups) p.window = p.n_groups;
     p.visit_tiles = 8.0f;
     const long long want = (long long)a.T * p.n_groups / (8ll * d2d_tc_sm_count());
-    p.sub = want >= 1024 ? 1024 : want >= 512 ? 512 : 256;
+    p.sub = want >= 4 * PIECE ? 4 * PIECE : want >= 2 * PIECE ? 2 * PIECE : PIECE;
     CUtensorMap tw1, tw2;
     if (!d2d_tc_make_map(&tw1, a.w1, a.d_ff, a.d, gs) || !d2d_tc_make_map(&tw2, w2, a.d, a.d_ff, 128)) return D2D_ERR_CUDA;
     auto kern = moe_gather_ffn_kernel<ACT>;
