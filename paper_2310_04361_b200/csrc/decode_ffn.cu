@@ -166,7 +166,7 @@ __device__ __forceinline__ void mma16816_f16(float (&d)[4], uint32_t a0, uint32_
 
 // The up projection of a unit from codes and bfloat16 rows, for rows that float16 would not hold.  Rare, but what it does to the code
 // around it is paid by every call: a function of its own where accumulators leave registers for one, in line where they do not
-// (Llama-shaped layer, us, function / in line / float16 alone: 38.3 / 39.5 / 37.9 at 1 token, 55.4 / 57.1 / 54.9 at 2; with 8 tiles a
+// (Llama-shaped layer, us, function / in line / no such rows: 38.3 / 39.5 / 37.9 at 1 token, 55.4 / 57.1 / 54.9 at 2; with 8 tiles a
 // warp 68.0 / 61.9 / 60.8 at 6, 62.0 / 59.0 / 58.3 at 8).
 struct up_rows {
     uint32_t bar_full, bar_empty, ring, xs;
@@ -417,7 +417,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         // ------------------------------------------------------------------ consumers
         // x does not depend on the router (the kernel behind which this one may start early waits for its own
         // predecessor before it lets this one start)
-        auto load_x = [&]() {
+        if (!Q8) {
             for (int i = tid, t = 0; t < T; ) {
                 if (i >= d / 8) { i -= d / 8; ++t; continue; }
                 cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
@@ -426,27 +426,29 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             consumer_bar();
-        };
-        if (!Q8) {
-            load_x();
         } else {
-            // Codes widen to float16 in one instruction, to bfloat16 in four, so the rows become float16 where that loses nothing: scaled
-            // so that a row's largest value lies in [2^14, 2^15), float16 has all eight bits of a value down to 2^-17, that is of one whose
-            // exponent is at most 31 below the largest.  A batch with a non-zero value further below stays bfloat16.
-            // WPT warps a token, a piece of the row each.
+            // Codes widen to float16 in one instruction, to bfloat16 in four, so beside codes the rows become float16 where that loses
+            // nothing: scaled so that a row's largest value lies in [2^14, 2^15), float16 has all eight bits of a value down to 2^-17,
+            // that is of one whose exponent is at most 31 below the largest.  A batch with a non-zero value further below stays
+            // bfloat16: its rows are fetched again.
+            // wpt warps a token, a piece of the row each; a lane looks at what it fetched itself
             const int wpt = T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1, part = warp % wpt, np = d / 8;
             const int i0 = np * part / wpt, i1 = np * (part + 1) / wpt;
-            uint32_t m = 0u;
+            auto fetch = [&]() {
+                for (int t = warp / wpt; t < T; t += NCW / wpt)
+                    for (int i = i0 + lane; i < i1; i += 32) cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            };
             if (tid == 0) x_spread = 0;
+            fetch();
             for (int t = warp / wpt; t < T; t += NCW / wpt) {
-                const uint4 *row = reinterpret_cast<const uint4 *>(x + (size_t)t * d);
-                m = 0u;
+                uint32_t m = 0u;
                 for (int i = i0 + lane; i < i1; i += 32) {
-                    const uint4 v = row[i];
+                    const uint4 v = *reinterpret_cast<const uint4 *>(xs + (size_t)t * xp + i * 16);
                     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                     for (int q = 0; q < 4; ++q) m = max(m, max(w[q] & 0x7fffu, (w[q] >> 16) & 0x7fffu));
-                    *reinterpret_cast<uint4 *>(xs + (size_t)t * xp + i * 16) = v;
                 }
                 m = __reduce_max_sync(FULL, m);
                 if (lane == 0) x_max[t * 16 + part] = m;
@@ -454,7 +456,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             consumer_bar();
             bool spread = false;
             for (int t = warp / wpt; t < T; t += NCW / wpt) {
-                m = 0u;
+                uint32_t m = 0u;
                 for (int q = 0; q < wpt; ++q) m = max(m, x_max[t * 16 + q]);
                 const int sh = min(120, 141 - (int)(m >> 7));
                 const float f = __uint_as_float((uint32_t)(127 + sh) << 23);
@@ -477,9 +479,10 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             }
             if (spread) x_spread = 1;
             consumer_bar();
-            if (__builtin_expect(x_spread != 0, 0)) {
+            if (__builtin_expect(*(volatile int *)&x_spread != 0, 0)) {
                 if (tid < T) x_inv[tid] = 1.0f;
-                load_x();
+                fetch();
+                consumer_bar();
             }
         }
 
