@@ -332,7 +332,7 @@ D2D_API d2d_status d2d_select_dynk_static(const float *R, int32_t T, int32_t E, 
  * where float32 sums meet in memory in the order in which they finish: bf16
  * batches that the decode kernels take, the fused gathered kernel, and small
  * batches whose down projection is cut along d_ff into several slices of
- * 64-column tiles (d = 1024: up to 512 tokens; slices of 128-column tiles,
+ * 64-column tiles (d = 1024: up to 384 tokens; slices of 128-column tiles,
  * which wide layers with a long d_ff have up to 256 tokens, are added in
  * order).  `routing` must describe these T tokens. */
 D2D_API d2d_status d2d_moe_ffn_fwd(const d2d_layer *layer, const void *x, int32_t T, const d2d_routing *routing,

@@ -18,13 +18,13 @@
 // The last CTA to add to its columns (a ticket per rank) adds b2 and writes y.
 //
 // Measured, whole layer calls back to back (small_batch_ffn.cu or the tensor-core path -> these two kernels): d = 1024,
-// 256 experts of 16: 18.1 -> 12.4 us at 1 token, 38 -> 15.4 us at 13; d = 4096, 344 gated experts of 32: 114 -> 67 us at 7
-// tokens, 64 -> 51 us at 1 with 8-bit weights; three d = 1024 layers of 128 experts on 8 shared tokens: 43 -> 17.7 us.
+// 256 experts of 16: 18.1 -> 12.4 us at 1 token, 38 -> 14.8 us at 13; d = 4096, 344 gated experts of 32: 114 -> 59.6 us at 7
+// tokens, 64 -> 44 us at 1 with 8-bit weights; three d = 1024 layers of 128 experts on 8 shared tokens: 43 -> 16.6 us.
 //
 // How many tokens fit is a matter of shared memory: the token rows, the partial sums and the hidden values grow with them, and
 // the ring beside them needs three stages.  One layer of bf16 weights: 32 tokens with d = 512 or 640, 16 with 768, 1024 or 2048, 8
-// with 4096.  Beyond that the tensor-core path takes over with a step in time (d = 1024: 15.7 us at 16 tokens, 26.7 at 17; d = 4096:
-// 69 us at 8 tokens, 88 at 9).
+// with 4096.  Beyond that the tensor-core path takes over with a step in time (d = 1024: 15.1 us at 16 tokens, 24.5 at 17; d = 4096:
+// 63 us at 8 tokens, 73 at 9).
 #include <cuda_fp8.h>
 
 #include "decode.cuh"

@@ -908,7 +908,7 @@ bool d2d_gemm_tc_available() { return get_encode() != nullptr; }
 // tokens at most).  With tiles of 64 columns a slice is at least two k-blocks; tiles of 128 columns need more slices for the same
 // number of CTAs, hence more partial sums, and bring more weight bytes in flight (16 KB a stage instead of 8: the narrow ones reached
 // 3.1 TB/s on 90 MB of weights): they are taken where a slice is 40 k-blocks or more (14 us of main loop, against about 4 for the
-// sums).  Llama-shaped layer (d_ff = 11008), back to back: 74.7 -> 68.3 us at 40 tokens, 82.5 -> 76.4 at 128, and 113.5 -> 101.3 at 200,
+// sums).  Llama-shaped layer (d_ff = 11008), back to back: 74.7 -> 69.4 us at 40 tokens, 82.5 -> 80.5 at 128, and 113.5 -> 102.5 at 200,
 // where narrow tiles leave nothing to split.
 // A slice adds its partial sums to a float32 buffer.  Wide tiles have a buffer for every two slices: the sum of two does not depend on
 // which comes first, and the buffers are added in order, so these batches (Llama-shaped layer, 9 to 256 tokens) give the same bits on

@@ -79,11 +79,11 @@ size_t d2d_gemm_tc_partial_floats(int M, int N, int K, int batch = 1);
 // Whether the lists of a batch can be left to the GEMM of its down projection: as many tokens as a CTA's epilogue warps take in one
 // go (512) or, before a main loop that is not split, in two.  On a stream of their own they cost the layer a launch, two events
 // and two waits between streams, and its call the programmatic launch behind it.  GPT-2-medium-shaped FFN, back to back: 30.8 ->
-// 26.8 us at 64 tokens, 34.7 -> 33.0 at 333, 43.2 -> 39.9 at 1000 (not split); split along K and in two goes they hold the
-// partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection that have no tile they held
-// up the down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
-// Above 1e10 FLOP of down projection the call is not short any more and the side stream is the better place (Llama-shaped
-// layer: 100.4 -> 95.1 at 100 tokens, but 130.9 -> 133.9 at 200).
+// 24.0 us at 64 tokens, 34.2 -> 30.5 at 333, 41.2 -> 39.2 at 1000 (not split); Llama-shaped layer 78.0 -> 72.8 at 100.  Split along K
+// and in two goes they held the partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection
+// that have no tile they held up the down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
+// The line of 1e10 FLOP of down projection and the limit of 512 tokens are older than the present loops: with those the lists would
+// ride a little further (Llama-shaped layer 101.9 -> 98.5 at 200 tokens; ViT-shaped, 700 tokens: level).
 static inline bool d2d_lists_ride(int T, int E, int k_splits, double down_flop)
 {
     return T <= (k_splits > 1 ? 512 : 1024) && (long long)T * ((E + 31) / 32) <= 16384 && down_flop <= 1e10;

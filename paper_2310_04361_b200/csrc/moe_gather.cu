@@ -145,7 +145,7 @@ __device__ __forceinline__ bool mma_tile(uint8_t *smem, uint64_t *bar_full, uint
 // stage's own in the leader (`note`, which nobody reads), and the bytes are credited to the leader's barrier; that credit
 // (complete_tx) releases at cluster scope once the copy is done, and the warp goes on at once.  Llama-shaped layer, 8192 tokens,
 // tau = 0.4, back to back before the power limit sets in: 1608 us with two warps that release in turn, 1389 with four, 1339 this way
-// (1425 without pairs).  The copy has ended when the leader has consumed the stage.
+// (1425 without pairs).  The copy has ended when the leader has consumed the stage, and long before a role that gave up a wait leaves.
 __device__ __forceinline__ bool forward_tile(uint8_t *smem, uint64_t *bar_full, uint4 *note, int nkb, int stages, int stage_bytes, uint32_t &it,
                                              int32_t *status)
 {
