@@ -229,6 +229,17 @@ D2D_API d2d_status d2d_layer_get_expert_path(const d2d_layer *layer, int32_t *pa
  * (for bf16 batches above the decode sizes; reporting and tests). */
 D2D_API d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, int64_t n_sel, int32_t *path);
 
+/* Plain bf16 layers of at most 32 experts of 64 or 128 neurons (d and d_ff
+ * multiples of 256, weights that stay in L2) have one more form under
+ * D2D_PATH_AUTO with default limits: the tokens are ordered by the experts they
+ * keep, so that a tile of 128 rows needs few of them, and both projections skip
+ * the rest.  Like the others it changes speed only.
+ * *n_sel_max: the largest number of selected pairs with which d2d_moe_ffn_fwd
+ * takes it at T tokens, in place of whatever d2d_layer_expert_path_for names;
+ * -1: never.  (d2d_layer_fwd has the same limit from 2e11 FLOP of up projection
+ * on and does without the form below.) */
+D2D_API d2d_status d2d_layer_get_sorted(const d2d_layer *layer, int32_t T, int64_t *n_sel_max);
+
 /* How the streaming decode kernels take a batch of T tokens of n_layers layers
  * (1, or a group's 2..4) of the shape `desc`: the rule of the calls, evaluated
  * on the host (reporting and tests; needs no layer and, as long as the GPU is

@@ -28,7 +28,7 @@ D2D_F32, D2D_BF16 = 0, 1
 ACTS = {"relu": 0, "gelu_erf": 1, "gelu_tanh": 2, "silu": 3}
 PATHS = {"auto": 0, "dense": 1, "gather": 2, "fused": 3}
 EXPORTS = ["d2d_status_str", "d2d_launch_count", "d2d_layer_create", "d2d_layer_create_fp8", "d2d_layer_get_fp8", "d2d_layer_destroy", "d2d_workspace_bytes",
-           "d2d_layer_set_expert_path", "d2d_layer_set_fused_rho_max", "d2d_layer_get_fused", "d2d_layer_expert_path_for", "d2d_decode_plan_for", "d2d_layer_get_expert_path", "d2d_layer_reset_counters", "d2d_expert_up_gather_fwd", "d2d_expert_down_masked_fwd", "d2d_test_inject_fault",
+           "d2d_layer_set_expert_path", "d2d_layer_set_fused_rho_max", "d2d_layer_get_fused", "d2d_layer_expert_path_for", "d2d_layer_get_sorted", "d2d_decode_plan_for", "d2d_layer_get_expert_path", "d2d_layer_reset_counters", "d2d_expert_up_gather_fwd", "d2d_expert_down_masked_fwd", "d2d_test_inject_fault",
            "d2d_select_workspace_bytes", "d2d_router_fwd", "d2d_select_dynk", "d2d_select_dynk_static", "d2d_select_topk",
            "d2d_routing_from_mask", "d2d_moe_ffn_fwd", "d2d_expert_up_fwd", "d2d_expert_down_fwd", "d2d_layer_fwd", "d2d_layer_fwd_host_workspace_bytes",
            "d2d_layer_fwd_host", "d2d_group_create", "d2d_group_destroy", "d2d_group_workspace_bytes", "d2d_group_fwd"]
@@ -78,6 +78,7 @@ _lib.d2d_expert_down_masked_fwd.argtypes = [c_void_p, c_void_p, c_int32, POINTER
 _lib.d2d_layer_set_expert_path.argtypes = [c_void_p, c_int, c_int32, ctypes.c_double]
 _lib.d2d_layer_set_fused_rho_max.argtypes = [c_void_p, ctypes.c_double]
 _lib.d2d_layer_get_fused.argtypes = [c_void_p, POINTER(c_int32), POINTER(ctypes.c_double)]
+_lib.d2d_layer_get_sorted.argtypes = [c_void_p, c_int32, POINTER(ctypes.c_int64)]
 _lib.d2d_layer_expert_path_for.argtypes = [c_void_p, c_int32, ctypes.c_int64, POINTER(c_int32)]
 _lib.d2d_decode_plan_for.argtypes = [POINTER(LayerDesc), c_int32, c_int32, c_int32, POINTER(DecodePlan)]
 _lib.d2d_layer_get_expert_path.argtypes = [c_void_p, POINTER(c_int32), POINTER(c_int32), POINTER(ctypes.c_double)]
@@ -291,6 +292,12 @@ class Layer:
         group, rho = c_int32(), ctypes.c_double()
         _check(_lib.d2d_layer_get_fused(self.handle, ctypes.byref(group), ctypes.byref(rho)), "d2d_layer_get_fused")
         return group.value, rho.value
+
+    def sorted_limit(self, T: int) -> int:
+        """Selected pairs up to which moe_ffn_fwd orders the T tokens by the experts they keep; -1: never (d2d_layer_get_sorted)."""
+        n = ctypes.c_int64()
+        _check(_lib.d2d_layer_get_sorted(self.handle, int(T), ctypes.byref(n)), "d2d_layer_get_sorted")
+        return n.value
 
     def get_expert_path(self):
         path, group, rho = c_int32(), c_int32(), ctypes.c_double()

@@ -10,6 +10,7 @@
 #include "decode.cuh"
 #include "gemm_tc.cuh"
 #include "moe_gather.cuh"
+#include "moe_sorted.cuh"
 
 bool d2d_token_path_supports(const d2d_layer_desc &D);
 d2d_status d2d_launch_moe_ffn_token(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *y,
@@ -161,6 +162,15 @@ d2d_status d2d_decode_layers(const d2d_layer *const *layers, int n, const void *
 
 size_t d2d_layer_ws_bytes(const d2d_layer *L, int T) { return layout_for(L, T).total; }
 
+// Whether a batch may take the sorted form (moe_sorted.cu), by shape and size: from 5.8e10 FLOP of up projection on (12288 tokens of the
+// paper's shape).  Shorter batches have little to win over the dense pair, and where that runs in the end the kernels of the other form
+// cost 10 us (expert step, us, dense pair / sorted form at p = 0.02, 0.05, 0.1, 0.2: 12608 tokens 105 / 60, 75, 84, 104; 8000 tokens 69 /
+// 52, 59, 66, 79; 5000 tokens 47 / 46, 48, 54, 61).
+static bool sorted_shape(const d2d_layer_desc &D, int T)
+{
+    return 2.0 * (double)T * D.d * D.d_ff >= 5.8e10 && d2d_sorted_supports(D, T) && d2d_gemm_tc_splits(T, D.d, D.d_ff) == 1;
+}
+
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
 {
     size_t need = 256;
@@ -170,6 +180,7 @@ size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)
     if (L->desc.dtype == D2D_BF16 && T > d2d_decode_max_tokens(L->desc)) {
         size_t h = d2d_align_up((size_t)T * L->desc.d_ff * 2, 256);
         h += d2d_align_up(d2d_gemm_tc_partial_floats(T, L->desc.d, L->desc.d_ff) * 4, 256);      // split-K partial sums
+        if (sorted_shape(L->desc, T)) h += d2d_sorted_layout_for(L->desc, T).total;
         if (h > need) need = h;
     }
     return need;
@@ -245,6 +256,63 @@ static int path_before_launch(const d2d_layer *L, int T, bool counted)
     return path;
 }
 
+// Largest number of selected pairs with which the automatic choice takes the sorted form, -1: never.  Tiles of 128 ordered tokens can
+// tell apart about as many patterns of kept experts as there are tiles: with an entropy of h(rho) bits per decision a tile fixes
+// log2(T / 128) / h of the E experts and has all of the others in its union, which leaves 1 - (1 - rho) log2(T / 128) / (E h) of
+// the work.  (Independent decisions are the worst case; correlated ones leave less.)  The form is level with the dense pair where 0.73
+// is left: expert step of the paper's shape, us, sorted / dense, a box each: 50432 tokens p = 0.1 175 / 342, 0.2 266 / 348, 0.3 341 /
+// 356, 0.4 396 / 370 (the limit: 0.32); 25000 tokens 0.1 130 / 183, 0.2 172 / 178, 0.3 189 / 178 (0.28); 12608 tokens 0.1 84 / 106, 0.2
+// 104 / 106, 0.3 119 / 106 (0.23); and the choice itself costs 10 where the dense pair runs in the end.
+// in_layer_call: behind a router, which overlaps a dense up projection that is not chosen: only batches that had a choice anyway.
+static double default_fused_rho_max(int g);
+static long long sorted_n_sel_max(const d2d_layer *L, int T, bool in_layer_call)
+{
+    const d2d_layer_desc &D = L->desc;
+    if (L->expert_path != D2D_PATH_AUTO || L->gather_rho_max >= 0.0 || !sorted_shape(D, T)) return -1;
+    if (L->fused_group > 0 && L->fused_rho_max != default_fused_rho_max(L->fused_group)) return -1;
+    if (in_layer_call && 2.0 * (double)T * D.d * D.d_ff < auto_min_up_flop(L)) return -1;
+    const double patterns = log2((double)T / 128.0) / D.n_experts;
+    double lo = 0.0, hi = 0.5;
+    for (int i = 0; i < 14; ++i) {
+        const double rho = 0.5 * (lo + hi), h = -rho * log2(rho) - (1.0 - rho) * log2(1.0 - rho);
+        (1.0 - (1.0 - rho) * fmin(patterns / h, 1.0) <= 0.73 ? lo : hi) = rho;
+    }
+    return (long long)(lo * (double)T * (double)D.n_experts);
+}
+
+// The masked dense pair's arguments
+static d2d_gemm_args dense_up_args(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *H)
+{
+    const d2d_layer_desc &D = L->desc;
+    d2d_gemm_args up = {};
+    up.a = x; up.b = L->w1; up.b_gate = D.gated ? L->w_gate : nullptr; up.b_cat = L->w1g; up.b_cat_block = 128; up.bias = L->b1; up.out = H;
+    up.M = T; up.N = D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
+    up.mask = r->mask; up.mask_words = (D.n_experts + 31) / 32; up.expert_size = D.expert_size; up.status = r->status;
+    return up;
+}
+static d2d_gemm_args dense_down_args(const d2d_layer *L, const void *H, int T, void *y, int32_t *status)
+{
+    const d2d_layer_desc &D = L->desc;
+    d2d_gemm_args dn = {};
+    dn.a = H; dn.b = L->w2; dn.bias = L->b2; dn.out = y;
+    dn.M = T; dn.N = D.d; dn.K = D.d_ff; dn.epilogue = D2D_EPI_BIAS_BF16; dn.status = status;
+    return dn;
+}
+
+// The sorted form up to n_sel_max selected pairs, the masked dense pair above
+static d2d_status launch_sorted_or_dense(const d2d_layer *L, const void *x, int T, const d2d_routing *r, void *y, void *ws, cudaStream_t st,
+                                         const int32_t *n_sel, long long n_sel_max)
+{
+    char *const scratch = (char *)ws + d2d_align_up((size_t)T * L->desc.d_ff * 2, 256);
+    d2d_status rc = d2d_moe_sorted(L, x, T, r, y, ws, scratch, L->sorted_ctr, (int *)(L->tickets + 56), n_sel, n_sel_max, st);
+    if (rc != D2D_OK) return rc;
+    d2d_gemm_args up = dense_up_args(L, x, T, r, ws), dn = dense_down_args(L, ws, T, y, r->status);
+    up.n_sel = dn.n_sel = n_sel;
+    up.n_sel_max = dn.n_sel_max = n_sel_max;
+    rc = d2d_gemm_tc(up, st);
+    return rc != D2D_OK ? rc : d2d_gemm_tc(dn, st);
+}
+
 // Expert step of bf16 batches above the decode sizes, on the tensor cores.
 //   up projection    two kernels that compute the same H = G * A(x W1^T + b1):
 //     masked dense   one GEMM over all of d_ff, the selection applied as a mask in the epilogue; its time does not
@@ -264,6 +332,8 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
                                     void *ws, cudaStream_t st, int *up_counter, const int32_t *n_sel, bool lists)
 {
     const d2d_layer_desc &D = L->desc;
+    const long long n_sel_sorted = n_sel ? sorted_n_sel_max(L, T, n_sel != r->n_sel) : -1;
+    if (n_sel_sorted >= 0) return launch_sorted_or_dense(L, x, T, r, y, ws, st, n_sel, n_sel_sorted);
     const int path = path_before_launch(L, T, n_sel != nullptr);
     const double rho_max = L->gather_rho_max >= 0.0 ? L->gather_rho_max : default_gather_rho_max(D, L->gather_group, T);
     long long n_sel_max = (long long)(rho_max * (double)T * (double)D.n_experts);
@@ -291,14 +361,11 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff);
     float *partial = k_splits > 1 ? (float *)((char *)ws + d2d_align_up((size_t)T * D.d_ff * 2, 256)) : nullptr;
     if (path != D2D_PATH_GATHER) {
-        d2d_gemm_args up = {};
+        d2d_gemm_args up = dense_up_args(L, x, T, r, ws);
         const bool forced = path == D2D_PATH_DENSE;
         up.tile_counter = forced ? up_counter : nullptr;
         up.pdl_late_wait = forced && up_counter != nullptr;
         up.n_sel = forced ? nullptr : n_sel; up.n_sel_max = n_sel_max;
-        up.a = x; up.b = L->w1; up.b_gate = D.gated ? L->w_gate : nullptr; up.b_cat = L->w1g; up.b_cat_block = 128; up.bias = L->b1; up.out = ws;
-        up.M = T; up.N = D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
-        up.mask = r->mask; up.mask_words = (D.n_experts + 31) / 32; up.expert_size = D.expert_size; up.status = r->status;
         if (forced && k_splits > 1) { up.zero = partial; up.zero_floats = (long long)d2d_gemm_tc_partial_floats(T, D.d, D.d_ff); }
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
@@ -332,12 +399,10 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
         if (rc != D2D_OK || path == D2D_PATH_GATHER) return rc;
     }
     if (zero_fill && cudaStreamWaitEvent(st, L->ev_fill_join, 0) != cudaSuccess) return D2D_ERR_CUDA;
-    d2d_gemm_args dn = {};
-    dn.a = ws; dn.b = L->w2; dn.bias = L->b2; dn.out = y;
+    d2d_gemm_args dn = dense_down_args(L, ws, T, y, r->status);
     // after a zero fill this kernel serves the gathered range too: it only has to stay out of the fused kernel's range
     dn.n_sel = path == D2D_PATH_AUTO && (!zero_fill || n_sel_fused >= 0) ? n_sel : nullptr;
     dn.n_sel_max = zero_fill ? n_sel_fused : n_sel_max;
-    dn.M = T; dn.N = D.d; dn.K = D.d_ff; dn.epilogue = D2D_EPI_BIAS_BF16; dn.status = r->status;
     dn.k_splits = k_splits;
     dn.partial = partial;
     dn.partial_zero = path == D2D_PATH_DENSE;
@@ -442,7 +507,9 @@ d2d_status d2d_layer_create(const d2d_layer_desc *desc, const d2d_weights *w, vo
     L->expert_path = D2D_PATH_AUTO;
     L->fused_group = d2d_gather_ffn_group_for(D);
     L->fused_rho_max = default_fused_rho_max(L->fused_group);
-    L->gather_ctr_words = D.n_experts + 64;               // enough for any group size: E / g counters + the exit ticket
+    L->gather_ctr_words = (int)d2d_align_up(D.n_experts + 64, 64);      // enough for any group size: E / g counters + the exit ticket
+    const int sorted_at = L->gather_ctr_words;
+    if (d2d_sorted_supports(D, 1)) L->gather_ctr_words += D2D_SORTED_CTR_WORDS;
     const size_t ctr_off = total;
     total += d2d_align_up((size_t)L->gather_ctr_words * sizeof(int), 256);
     for (const piece &p : pieces)
@@ -461,6 +528,7 @@ d2d_status d2d_layer_create(const d2d_layer_desc *desc, const d2d_weights *w, vo
     L->slab_bytes = total;
     L->tickets = (unsigned int *)L->slab;
     L->gather_ctr = (int *)((char *)L->slab + ctr_off);
+    L->sorted_ctr = L->gather_ctr + sorted_at;
     size_t off = ctr_off + d2d_align_up((size_t)L->gather_ctr_words * sizeof(int), 256);
     d2d_status rc = cudaMemsetAsync(L->slab, 0, off, st) == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
     for (const piece &p : pieces) {
@@ -632,6 +700,13 @@ d2d_status d2d_layer_expert_path_for(const d2d_layer *layer, int32_t T, int64_t 
     return D2D_OK;
 }
 
+d2d_status d2d_layer_get_sorted(const d2d_layer *layer, int32_t T, int64_t *n_sel_max)
+{
+    if (!layer || !n_sel_max || T <= 0) return D2D_ERR_INVALID_ARG;
+    *n_sel_max = use_dense_masked(layer, T) ? sorted_n_sel_max(layer, T, false) : -1;
+    return D2D_OK;
+}
+
 d2d_status d2d_decode_plan_for(const d2d_layer_desc *desc, int32_t n_layers, int32_t T, int32_t fp8_experts, d2d_decode_plan *plan)
 {
     if (!desc || !plan || n_layers < 1 || n_layers > D2D_MAX_GROUP || T < 1) return D2D_ERR_INVALID_ARG;
@@ -740,12 +815,7 @@ d2d_status d2d_expert_up_fwd(const d2d_layer *layer, const void *x, int32_t T, c
     if (T == 0) return D2D_OK;
     if (!x || !H || !aligned16(x) || !aligned16(H) || !routing_ok(routing, false)) return D2D_ERR_INVALID_ARG;
     if (layer->desc.dtype != D2D_BF16 || layer->desc.d_ff % 8 || !d2d_gemm_tc_available()) return D2D_ERR_UNSUPPORTED;
-    const d2d_layer_desc &D = layer->desc;
-    d2d_gemm_args up = {};
-    up.a = x; up.b = layer->w1; up.b_gate = D.gated ? layer->w_gate : nullptr; up.b_cat = layer->w1g; up.b_cat_block = 128; up.bias = layer->b1; up.out = H;
-    up.M = T; up.N = D.d_ff; up.K = D.d; up.epilogue = D2D_EPI_UP_MASKED; up.act = D.act;
-    up.mask = routing->mask; up.mask_words = (D.n_experts + 31) / 32; up.expert_size = D.expert_size;
-    up.status = routing->status;
+    d2d_gemm_args up = dense_up_args(layer, x, T, routing, H);
     up.test_skip_load = __atomic_exchange_n(&g_test_fault, 0, __ATOMIC_RELAXED) == 1;
     return d2d_gemm_tc(up, (cudaStream_t)stream);
 }
@@ -789,11 +859,7 @@ d2d_status d2d_expert_down_fwd(const d2d_layer *layer, const void *H, int32_t T,
     if (T == 0) return D2D_OK;
     if (!H || !y || !aligned16(H) || !aligned16(y)) return D2D_ERR_INVALID_ARG;
     if (layer->desc.dtype != D2D_BF16 || layer->desc.d_ff % 8 || !d2d_gemm_tc_available()) return D2D_ERR_UNSUPPORTED;
-    const d2d_layer_desc &D = layer->desc;
-    d2d_gemm_args dn = {};
-    dn.a = H; dn.b = layer->w2; dn.bias = layer->b2; dn.out = y;
-    dn.M = T; dn.N = D.d; dn.K = D.d_ff; dn.epilogue = D2D_EPI_BIAS_BF16; dn.status = status;
-    return d2d_gemm_tc(dn, (cudaStream_t)stream);
+    return d2d_gemm_tc(dense_down_args(layer, H, T, y, status), (cudaStream_t)stream);
 }
 
 // The forms of a layer call, in the order in which they are tried.

@@ -44,7 +44,8 @@ struct d2d_layer {
     // that used them): word 0 decode router, word 16 decode experts, word 32 tile counter of the up projection, words
     // 40 / 41 / 42 sum of k, exit ticket and largest condition of the fused router, word 44 the number of selected pairs the fused router
     // publishes for the density-adaptive dispatch of the expert step, word 48 ticket of the lists built on the side stream, words
-    // 52 / 53 exit ticket and largest condition of the one-launch layer kernels of small float32 problems.  Like the side stream, they make concurrent
+    // 52 / 53 exit ticket and largest condition of the one-launch layer kernels of small float32 problems, words 56 / 57 tile counters of
+    // the projections of the sorted form.  Like the side stream, they make concurrent
     // d2d_layer_fwd calls on ONE layer object from several streams unsafe; use one layer object per stream for that.
     // A call that ended in D2D_ERR_TIMEOUT may leave them non-zero: d2d_layer_reset_counters clears them.
     unsigned int *tickets;
@@ -53,6 +54,7 @@ struct d2d_layer {
     // the density up to which the automatic choice takes the gathered path
     int *gather_ctr;
     int gather_ctr_words;
+    int *sorted_ctr;        // bucket counts of the sorted form (moe_sorted.cu), in the same words
     int gather_group;
     int expert_path;
     double gather_rho_max;

@@ -47,6 +47,32 @@ struct EpiParams {
     int test_skip_load;              // test aid: CTA 0 never requests the A tile of its first k-block (see d2d_gemm_args)
 };
 
+// Work lists of the kernels that run on tokens ordered by the experts they keep (see d2d_gemm_args::sorted).  Launches without any do
+// without the code.
+enum { SORTED_NONE = 0, SORTED_UP = 1, SORTED_DOWN = 2 };
+struct NoItems {};
+struct UpItems { const uint32_t *items; const int *n_items; };          // row tile << 8 | column tile
+struct DownItems { const uint2 *items; const int *order; int kpe; };    // (row tile, union of its masks); k-blocks of an expert
+template <int SORTED> struct ItemsOf { typedef NoItems type; };
+template <> struct ItemsOf<SORTED_UP> { typedef UpItems type; };
+template <> struct ItemsOf<SORTED_DOWN> { typedef DownItems type; };
+inline void set_items(NoItems &, const d2d_gemm_args &) {}
+inline void set_items(UpItems &s, const d2d_gemm_args &g) { s = {g.sorted.up_items, g.sorted.n_items}; }
+inline void set_items(DownItems &s, const d2d_gemm_args &g) { s = {g.sorted.down_items, g.sorted.order, g.expert_size / 64}; }
+
+// Number of items, and item `index`: row tile << 8 | column tile, and (down, cols of them per row tile) the union
+__device__ __forceinline__ int n_items(const UpItems &s, int) { return __ldcg(s.n_items); }
+__device__ __forceinline__ int n_items(const DownItems &, int tiles) { return tiles; }
+__device__ __forceinline__ uint2 item_at(const UpItems &s, int index, int) { return make_uint2(__ldcg(s.items + index), 0u); }
+__device__ __forceinline__ uint2 item_at(const DownItems &s, int index, int cols)
+{
+    const uint2 w = __ldcg(s.items + index / cols);
+    return make_uint2(w.x << 8 | (uint32_t)(index % cols), w.y);
+}
+// k-blocks of an item of the down projection
+__device__ __forceinline__ int kb_list(const DownItems &s, uint32_t uni) { return __popc(uni) * s.kpe; }
+template <typename Items> __device__ __forceinline__ int kb_list(const Items &, uint32_t) { return 0; }
+
 // Lists a down projection builds before its first tile.  Launches without any do without the code: carrying it cost a short layer
 // call 1 us, whether it ran or not.
 struct NoLists {};
@@ -156,12 +182,13 @@ __host__ __device__ constexpr int pow2_at_least(int v) { return v <= 32 ? 32 : v
 // A k-block then brings 16 + BN / 16 KB into an SM instead of 16 + BN / 8: the fill from L2 (about 117 GB/s per SM), not
 // the tensor pipe, bounds the single-CTA main loop.  Two accumulator buffers in TMEM let the epilogue of one tile overlap the MMAs of the
 // next.  GATED: two B tiles (up, gate) share the A tile; the epilogue forms A(gate) * (up + bias).
-template <int BN, int STAGES, int EPI, int ACT, bool GATED, bool PAIR, int LISTS>
+template <int BN, int STAGES, int EPI, int ACT, bool GATED, bool PAIR, int LISTS, int SORTED>
 __global__ void __launch_bounds__(NTHREADS_V2) __maxnreg__(GATED ? 96 : 80)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                const __grid_constant__ CUtensorMap tm_b2, const __grid_constant__ CUtensorMap tm_out, EpiParams ep, int M, int N, int K, int k_splits,
-               const typename ListsOf<LISTS>::type lists)
+               const typename ListsOf<LISTS>::type lists, const typename ItemsOf<SORTED>::type items)
 {
+    static_assert(SORTED == SORTED_NONE || (!GATED && !PAIR && LISTS == 0), "lists of work: plain layers, single CTAs");
     constexpr int TM = PAIR ? 2 * BM : BM;                // rows of the tile a CTA (pair) computes
     // rows of B this CTA stages (of each matrix; a gated pair: the leader the up rows, its peer the gate rows, all BN of them)
     constexpr int B_ROWS = PAIR && !GATED ? BN / 2 : BN;
@@ -184,6 +211,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // to the epilogue through a two-slot ring (a CTA that starts late, or gets slow tiles, simply draws fewer)
     __shared__ uint64_t sched_full[2], sched_empty[2];
     __shared__ volatile int sched_item[2];
+    __shared__ volatile uint32_t sched_uni[2];                       // down projection by list: experts of the tile
     uint8_t *out_s = smem + (size_t)STAGES * STAGE_BYTES;            // two output buffers behind the operand stages
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;      // warp-uniform: roles, columns
     const int nkb = (K + BK - 1) / BK;
@@ -232,7 +260,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     // and its writes are visible.  The next kernel of the stream may be scheduled onto SMs as this grid frees them.
     // With late_wait only the epilogue depends on that kernel (the selection mask written by the router): the
     // operand loads and the MMAs of the first tiles then overlap it, and only the epilogue warps wait.
-    const bool dyn = ep.tile_counter != nullptr;
+    const bool dyn = SORTED != SORTED_NONE || ep.tile_counter != nullptr;
     // early_b: the B operand (weights) does not depend on the previous kernel either, so the producer requests the B
     // tiles of its first k-blocks BEFORE it waits for that kernel and only the A tiles after (static schedule only)
     const bool early_b = !PAIR && !dyn && !ep.late_wait && ep.n_sel == nullptr;
@@ -241,7 +269,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
     if (EPI != D2D_EPI_RELU_BF16 || !early_b || warp != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // density-adaptive dispatch: below the crossover the gathered kernel, launched next to this one, does the work
     // (every thread has passed the dependency wait here: the host never combines n_sel with late_wait)
-    const bool run = ep.n_sel == nullptr || (long long)__ldcg(ep.n_sel) > ep.n_sel_max;
+    const bool run = ep.n_sel == nullptr || ((long long)__ldcg(ep.n_sel) > ep.n_sel_max) == (SORTED == SORTED_NONE);
 
     // Waits for barriers that threads of the pair's other CTA arrive at: the ring of work items (its slots are written and read
     // across the pair) and the accumulators handed back.  The operand and accumulator-full barriers are completed by the copy
@@ -251,6 +279,53 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
 
     if (!run) {
         // nothing to do
+    } else if (SORTED != SORTED_NONE && warp == 0) {
+        // ------------------------------------------------------------------ TMA producer, from a list of work
+        if constexpr (SORTED != SORTED_NONE) {
+            if (lane == 0) {
+                const int total = n_items(items, total_tiles);
+                // Items are drawn from the counter as in the dynamic schedule below, but two ahead: while one is worked on, the word
+                // of the next is on its way and the number of the one behind that is being drawn.
+                int index = worker, next = index < total ? n_workers + atomicAdd(ep.tile_counter, 1) : total;
+                uint2 word = index < total ? item_at(items, index, n_tiles) : make_uint2(0u, 0u);
+                uint32_t it = 0;
+                bool ok = true;
+                for (uint32_t local = 0; ok; ++local) {
+                    const uint32_t sl = local & 1u;
+                    ok = peer_wait(&sched_empty[sl], ((local >> 1) & 1u) ^ 1u);
+                    if (!ok) break;
+                    sched_item[sl] = index < total ? (int)word.x : -1;
+                    sched_uni[sl] = word.y;
+                    mbar_arrive(smem_u32(&sched_full[sl]));
+                    if (index >= total) break;
+                    const int m0 = (int)(word.x >> 8) * BM, n0 = (int)(word.x & 255u) * BN;
+                    uint32_t uni = word.y;
+                    index = next;
+                    word = index < total ? item_at(items, index, n_tiles) : make_uint2(0u, 0u);
+                    next = index < total ? n_workers + atomicAdd(ep.tile_counter, 1) : index;
+                    const auto block = [&](int kb) {
+                        const uint32_t s = it % STAGES, full = smem_u32(&bar_full[s]), dst = smem_u32(smem + (size_t)s * STAGE_BYTES);
+                        ok = mbar_wait(smem_u32(&bar_empty[s]), ((it / STAGES) & 1u) ^ 1u, ep.status);
+                        if (!ok) return;
+                        mbar_expect_tx(full, (uint32_t)STAGE_BYTES);
+                        tma_load_2d(dst, &tm_a, kb * BK, m0, full);
+                        tma_load_2d(dst + A_BYTES, &tm_b, kb * BK, n0, full);
+                        ++it;
+                    };
+                    if constexpr (SORTED == SORTED_UP) {
+                        for (int kb = 0; kb < nkb && ok; ++kb) block(kb);
+                    } else {
+                        // the k-blocks of the experts that some token of the tile keeps
+                        for (; uni && ok; uni &= uni - 1u) {
+                            const int kb0 = (__ffs(uni) - 1) * items.kpe;
+                            for (int k = 0; k < items.kpe && ok; ++k) block(kb0 + k);
+                        }
+                    }
+                }
+                // every worker that had an item draws one past the end, `total` values are drawn in all: the last leaves zero
+                if (index == n_workers + total - 1) *ep.tile_counter = 0;
+            }
+        }
     } else if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
         if (lane == 0) {
@@ -367,21 +442,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             bool have = false;
             for (;; ++local) {
                 int item = worker + (int)local * n_workers;
+                uint32_t uni = 0u;
                 if (dyn) {
                     const uint32_t sl = local & 1u, su = local >> 1;
                     ok = peer_wait_warp(&sched_full[sl], su & 1u);
                     if (!ok) break;
                     item = sched_item[sl];
+                    if (SORTED == SORTED_DOWN) uni = sched_uni[sl];
                     __syncwarp();                              // every lane has read the slot before it is handed back
                     if (elect_one()) mbar_arrive(smem_u32(&sched_empty[sl]));
                     if (item < 0) break;
                 }
-                if (item >= total_tiles) break;
+                if (SORTED == SORTED_NONE && item >= total_tiles) break;
                 const int sp = (!GATED && k_splits == 1) ? 0 : item % k_splits;
                 // no split is the common case: skip the divisions (measured: faster for the plain kernels, slower for the
                 // gated one, whose code layout is at its limit)
                 const bool one = !GATED && k_splits == 1;
-                const int kb0 = one ? 0 : (int)((long long)sp * nkb / k_splits), kb1 = one ? nkb : (int)((long long)(sp + 1) * nkb / k_splits);
+                const int kb0 = one ? 0 : (int)((long long)sp * nkb / k_splits),
+                          kb1 = SORTED == SORTED_DOWN ? kb_list(items, uni) : one ? nkb : (int)((long long)(sp + 1) * nkb / k_splits);
                 const uint32_t buf = local & 1u, use = local >> 1;
                 ok = peer_wait_warp(&bar_acc_empty[buf], (use & 1u) ^ 1u);   // epilogue drained this buffer
                 if (!ok) break;
@@ -456,12 +534,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     go = peer_wait(&sched_full[buf], use & 1u);
                     if (go) {
                         item = sched_item[buf];
+                        // (problem number: none here; whether the tile's tokens keep nothing)
+                        if (SORTED != SORTED_NONE) epi_prob[buf] = SORTED == SORTED_DOWN && sched_uni[buf] == 0u;
                         if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(&sched_empty[buf]), 0));
                         else mbar_arrive(smem_u32(&sched_empty[buf]));
                     }
                 }
-                go = go && item >= 0 && item < total_tiles;
-                if (go) {
+                go = go && item >= 0 && (SORTED != SORTED_NONE || item < total_tiles);
+                if (SORTED != SORTED_NONE) {
+                    if (go) {
+                        epi_m0[buf] = (item >> 8) * BM; epi_n0[buf] = (item & 255) * BN;
+                        go = mbar_wait(smem_u32(&bar_acc_full[buf]), use & 1u, ep.status);
+                    }
+                } else if (go) {
                     int tile = (!GATED && k_splits == 1) ? item : item / k_splits;
                     int prob = 0, tr, tc;
                     const int sum = EPI == D2D_EPI_PARTIAL_F32 ? (item - tile * k_splits) / ep.slices_per_sum : 0;
@@ -476,7 +561,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             asm volatile("bar.sync 1, %0;" ::"r"(N_EPI_WARPS * 32) : "memory");
             if (!epi_go[buf]) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int m0 = epi_m0[buf], n0 = epi_n0[buf], prob = epi_prob[buf];
+            const int m0 = epi_m0[buf], n0 = epi_n0[buf], prob = SORTED == SORTED_NONE ? epi_prob[buf] : 0;
+            const bool nothing = SORTED == SORTED_DOWN && epi_prob[buf] != 0;
+            // down projection by list: the tokens of the two rows whose 16-byte pieces this thread stores
+            int token[2] = {-1, -1};
+            if constexpr (SORTED == SORTED_DOWN) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int at = m0 + quad * 32 + 16 * i + 4 * part + (lane >> 3);
+                    if (at < M) token[i] = __ldcg(items.order + at);
+                }
+            }
             // this problem's bias entries and output matrix
             const __nv_bfloat16 *bias_g = ep.bias ? ep.bias + prob * N : nullptr;
             void *out_p = (char *)ep.out + (size_t)prob * M * N * ((EPI == D2D_EPI_ABS_F32 || EPI == D2D_EPI_PARTIAL_F32) ? 4 : 2);
@@ -504,7 +599,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
             // The common case gets a loop of its own with nothing else in it (the epilogue is sensitive to its
             // instruction-cache footprint): a full-width tile, vector-aligned rows and expert sizes that are multiples of 8.
             // Everything else (ragged last column tile, odd sizes) goes through the compact generic loop below.
-            const bool fast_tile = (N & 7) == 0 && n0 + BN <= N && (!mask_on || (ep.expert_size & 7) == 0);
+            // (lists of work come with whole column tiles only)
+            const bool fast_tile = SORTED != SORTED_NONE || (N & 7) == 0 && n0 + BN <= N && (!mask_on || (ep.expert_size & 7) == 0);
             uint32_t ra[16], rb[GATED ? 1 : 16], ga[GATED ? 16 : 1];
             if (fast_tile) {
                 // Non-gated: the next unit's accumulators are prefetched into a second register set.  Gated tiles need
@@ -529,6 +625,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                     if (!GATED && u + 1 < N_UNITS)                                // the next unit's load overlaps the math below
                         tmem_ld16_issue(tbase + (u + 1) * 64, (u & 1) ? ra : reinterpret_cast<uint32_t (&)[16]>(rb));
 
+                    if (SORTED == SORTED_DOWN && nothing) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) r[j] = 0u;
+                    }
                     float v[16];
                     epilogue_16<EPI, ACT, GATED>(r, g, v, bias_w);
                     if (EPI == D2D_EPI_UP_MASKED && u == 0 && mask_on) {
@@ -576,6 +676,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__
                         uint8_t *o = out_s + (out_n & 1u) * OUT_BUF_BYTES + (quad * 32 + lane) * 128;
                         *reinterpret_cast<uint4 *>(o + (((2 * part) ^ (lane & 7)) << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                         *reinterpret_cast<uint4 *>(o + (((2 * part + 1) ^ (lane & 7)) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        if constexpr (SORTED == SORTED_DOWN) {
+                            // rows go to their tokens: eight threads store 128 bytes of a row (the buffer is written again two units
+                            // on, behind the barrier of the next)
+                            asm volatile("bar.sync %0, 128;" ::"r"(2 + quad) : "memory");
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                const int rr = 16 * i + 4 * part + (lane >> 3), ch = lane & 7;
+                                const uint4 w = *reinterpret_cast<const uint4 *>(out_s + (out_n & 1u) * OUT_BUF_BYTES + (quad * 32 + rr) * 128 +
+                                                                                 ((ch ^ (rr & 7)) << 4));
+                                if (token[i] >= 0)
+                                    *reinterpret_cast<uint4 *>((__nv_bfloat16 *)out_p + (size_t)token[i] * N + n0 + u * 64 + ch * 8) = w;
+                            }
+                            ++out_n;
+                            continue;
+                        }
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         // the store before this one has read the other buffer: free for everybody behind the barrier
                         if (part == 0 && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -677,10 +792,10 @@ template <typename K> bool ensure_smem_attr(K kern, size_t smem, bool (&done)[64
     return true;
 }
 
-template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false, int LISTS = 0>
+template <int BN, int EPI, int ACT, bool GATED, bool PAIR = false, int LISTS = 0, int SORTED = SORTED_NONE>
 d2d_status launch(const d2d_gemm_args &g, cudaStream_t st, int slices_per_sum = 1)
 {
-    if constexpr ((EPI == D2D_EPI_BIAS_BF16 || EPI == D2D_EPI_PARTIAL_F32) && LISTS == 0) {
+    if constexpr ((EPI == D2D_EPI_BIAS_BF16 || EPI == D2D_EPI_PARTIAL_F32) && LISTS == 0 && SORTED == SORTED_NONE) {
         if (g.lists.n == 1) return launch<BN, EPI, ACT, GATED, PAIR, 1>(g, st, slices_per_sum);
         if (g.lists.n > 1) return launch<BN, EPI, ACT, GATED, PAIR, D2D_MAX_GROUP>(g, st, slices_per_sum);
     }
@@ -711,7 +826,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st, int slices_per_sum = 
         const cuuint32_t box[3] = {64, 32, 1};
         if (!d2d_tc_encode_map(&to, false, 3, g.out, dims, strides, box)) return D2D_ERR_CUDA;
     }
-    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED, PAIR, LISTS>;
+    auto kern = gemm_tc_kernel<BN, STAGES, EPI, ACT, GATED, PAIR, LISTS, SORTED>;
     static bool attr_set[64] = {};
     if (!ensure_smem_attr(kern, SMEM, attr_set)) return D2D_ERR_CUDA;
     const int es = g.expert_size > 0 ? g.expert_size : 1;
@@ -722,6 +837,8 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st, int slices_per_sum = 
                  (g.test_skip_load && !g.tile_counter && !g.pdl_late_wait && !g.n_sel) ? 1 : 0};
     typename ListsOf<LISTS>::type lists = {};
     set_lists(lists, g);
+    typename ItemsOf<SORTED>::type items = {};
+    set_items(items, g);
     const int k_splits = g.k_splits > 1 ? g.k_splits : 1;
     const int tiles = d2d_cdiv(g.N, BN) * d2d_cdiv(g.M, TM) * k_splits * batch;
     const int workers = PAIR ? d2d_tc_sm_count() / 2 : d2d_tc_sm_count();
@@ -739,7 +856,7 @@ d2d_status launch(const d2d_gemm_args &g, cudaStream_t st, int slices_per_sum = 
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = d2d_tc_pdl_enabled() ? 2 : 1;
-    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits, lists);
+    const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, ta, tb, tb2, to, ep, g.M, g.N, g.K, k_splits, lists, items);
     D2D_LAUNCHED(1);
     return err == cudaSuccess && cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
@@ -780,6 +897,9 @@ tile_choice pick_tile(int M, int N, int K, int batch, bool pairs_ok, bool gated)
 template <int EPI, int ACT, bool GATED>
 d2d_status launch_bn(const d2d_gemm_args &g, cudaStream_t st)
 {
+    if constexpr (EPI == D2D_EPI_UP_MASKED && !GATED) {
+        if (g.sorted.on) return launch<256, EPI, ACT, false, false, 0, SORTED_UP>(g, st);
+    }
     const bool pairs_ok = !g.test_skip_load && EPI != D2D_EPI_ABS_F32;
     if (GATED) {
         if (pairs_ok && g.M > BM) return launch<128, EPI, ACT, GATED, true>(g, st);
@@ -945,6 +1065,7 @@ d2d_status d2d_gemm_tc(const d2d_gemm_args &g, cudaStream_t st)
     case D2D_EPI_RELU_BF16: return launch_bn<D2D_EPI_RELU_BF16, 0, false>(g, st);
     case D2D_EPI_ABS_F32: return launch_bn<D2D_EPI_ABS_F32, 0, false>(g, st);
     case D2D_EPI_BIAS_BF16:
+        if (g.sorted.on) return launch<256, D2D_EPI_BIAS_BF16, 0, false, false, 0, SORTED_DOWN>(g, st);
         if (g.k_splits > 1 && g.partial) {
             const int batch = g.batch > 1 ? g.batch : 1;
             const split_choice c = pick_split(g.M, g.N, g.K, batch);

@@ -62,6 +62,10 @@ struct d2d_gemm_args {
     // work).  Cannot be combined with pdl_late_wait.
     const int32_t *n_sel;
     long long n_sel_max;
+    // Tokens ordered by the experts they keep (moe_sorted.cu): work from a list.  Up projection: up_items, *n_items of them; down
+    // projection: down_items, one per row tile, and the token of each row, to which its output goes.  The dispatch rule is the opposite
+    // then: the kernel works if *n_sel is at most n_sel_max.  Requires N % 256 == 0 and tile_counter.
+    struct { bool on; const uint32_t *up_items; const int *n_items; const uint2 *down_items; const int *order; } sorted;
     // Per-expert lists to build on the side (D2D_EPI_BIAS_BF16, d2d_lists_ride): by the epilogue warps, which wait for the first
     // accumulator anyway; the masks must be there when the previous kernel of the stream has completed.  n = 0: none.
     d2d_list_job lists;

@@ -1,0 +1,85 @@
+"""Expert step on tokens ordered by the experts they keep (layers of at most 32 experts): against the oracle on sampled tokens and,
+bit for bit, against the masked dense pair, at batches that begin and end tiles and buckets everywhere."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2310_04361_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+TOL_Y = 2e-2
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_2310_04361_b200 import api
+    return api
+
+
+def _keep(kind, T, E, rng):
+    if kind == "one mask":                                     # one bucket
+        return np.broadcast_to(np.arange(E) % 5 == 0, (T, E)).copy()
+    if kind == "nothing":                                      # no up projection at all
+        return np.zeros((T, E), bool)
+    if kind == "two kinds":                                    # a bucket that ends inside a tile, the other reaches the ragged end
+        k = np.zeros((T, E), bool)
+        k[: T // 2 + 7, 0] = True
+        k[T // 2 + 7:, E - 1] = True
+        return k[rng.permutation(T)]
+    p = float(kind)
+    k = rng.random((T, E)) < p
+    k[::97] = False                                            # tokens that keep nothing between others
+    k[5] = True                                                # and one that keeps everything
+    return k
+
+
+# (E, s, d, T): the paper's experts; experts of 64 neurons; a word full of experts; few; ragged last tiles, one of one row
+CASES = [(24, 128, 768, 12611, k) for k in ("0.02", "0.2", "one mask", "nothing", "two kinds")] + [
+    (32, 64, 1024, 14081, "0.05"), (8, 128, 1024, 27777, "0.1"), (32, 128, 512, 13953, "0.1")]
+
+
+@pytest.mark.parametrize("E,s,d,T,kind", CASES)
+def test_sorted_form(api, E, s, d, T, kind):
+    rng = np.random.default_rng(T + E)
+    cfg = dataclasses.replace(wl.CONFIGS["paper"], E=E, d_ff=E * s, d=d, T=T)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    G = _keep(kind, T, E, rng).astype(np.uint8)
+    r = api.routing_from_mask(torch.from_numpy(oracle.pack_mask(G).view(np.int32)).cuda(), E)
+    assert 0 <= r.n_sel <= layer.sorted_limit(T)               # the form is what runs
+    xd = api.to_device(x, cfg.dtype)
+    ys = []
+    for rep in range(2):                                       # the counters reset themselves; stale rows and cells would show
+        layer.workspace(T).fill_(0xff)                         # bf16 NaNs
+        y = torch.full((T, d), float("nan"), dtype=torch.bfloat16, device="cuda")
+        layer.moe_ffn_fwd(xd, r, y=y)
+        assert r.status == 0
+        ys.append(y)
+    layer.set_expert_path("dense")
+    assert layer.sorted_limit(T) == -1
+    yd = layer.moe_ffn_fwd(xd, r)
+    # the same products in the same order, plus exact zeros
+    for y in ys:
+        assert torch.equal(y.view(torch.int16), yd.view(torch.int16))
+    sample = np.unique(np.concatenate([[0, 5, 97, T - 2, T - 1], rng.integers(0, T, 120)]))
+    ref = oracle.moe_ffn(x[sample], w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[cfg.act], G[sample])
+    got = ys[0].float().cpu().numpy()[sample]
+    assert np.isfinite(got).all() and np.abs(got - ref).max() / np.abs(ref).max() <= TOL_Y
+    layer.close()
+
+
+def test_above_the_limit_the_dense_pair_runs(api):
+    cfg = wl.with_tokens(wl.CONFIGS["paper"], 12800)
+    layer = api.Layer.from_config(cfg, wl.make_weights(cfg))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((cfg.T, cfg.d), generator=g, device="cuda").to(torch.bfloat16)
+    words = ((torch.rand((cfg.T, 32), generator=g, device="cuda") < 0.5).long()[:, :24] << torch.arange(24, device="cuda")).sum(-1)
+    r = api.routing_from_mask(words.to(torch.int32)[:, None], cfg.E)
+    assert r.n_sel > layer.sorted_limit(cfg.T) > 0
+    y = layer.moe_ffn_fwd(x, r, y=torch.full_like(x, float("nan")))
+    layer.set_expert_path("dense")
+    assert torch.equal(y.view(torch.int16), layer.moe_ffn_fwd(x, r).view(torch.int16))
+    layer.close()
