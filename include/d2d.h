@@ -306,6 +306,10 @@ D2D_API d2d_status d2d_select_topk(const float *R, int32_t T, int32_t E, int32_t
  * must be zero); k, counts, offsets, perm, n_sel (and the dual) are written. */
 D2D_API d2d_status d2d_routing_from_mask(int32_t T, int32_t E, d2d_routing *out,
                                  void *ws, size_t ws_bytes, void *stream);
+/* The same with the decisions at `mask` (device, uint32 [T, ceil(E/32)]), which
+ * are copied to out->mask; entries of out->perm behind the lists become zero,
+ * so that none of the buffers (but tok_off / tok_exp) need be initialised. */
+D2D_API d2d_status d2d_routing_of_mask(const uint32_t *mask, int32_t T, int32_t E, d2d_routing *out, void *ws, size_t ws_bytes, void *stream);
 
 /* d2d_select_dynk for callers that may not allocate device memory.  (The paper
  * has no counterpart; this is a deployment convenience.)

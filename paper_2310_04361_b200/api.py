@@ -30,7 +30,7 @@ PATHS = {"auto": 0, "dense": 1, "gather": 2, "fused": 3}
 EXPORTS = ["d2d_status_str", "d2d_launch_count", "d2d_layer_create", "d2d_layer_create_fp8", "d2d_layer_get_fp8", "d2d_layer_destroy", "d2d_workspace_bytes",
            "d2d_layer_set_expert_path", "d2d_layer_set_fused_rho_max", "d2d_layer_get_fused", "d2d_layer_expert_path_for", "d2d_layer_get_sorted", "d2d_decode_plan_for", "d2d_layer_get_expert_path", "d2d_layer_reset_counters", "d2d_expert_up_gather_fwd", "d2d_expert_down_masked_fwd", "d2d_test_inject_fault",
            "d2d_select_workspace_bytes", "d2d_router_fwd", "d2d_select_dynk", "d2d_select_dynk_static", "d2d_select_topk",
-           "d2d_routing_from_mask", "d2d_moe_ffn_fwd", "d2d_expert_up_fwd", "d2d_expert_down_fwd", "d2d_layer_fwd", "d2d_layer_fwd_host_workspace_bytes",
+           "d2d_routing_from_mask", "d2d_routing_of_mask", "d2d_moe_ffn_fwd", "d2d_expert_up_fwd", "d2d_expert_down_fwd", "d2d_layer_fwd", "d2d_layer_fwd_host_workspace_bytes",
            "d2d_layer_fwd_host", "d2d_group_create", "d2d_group_destroy", "d2d_group_workspace_bytes", "d2d_group_fwd"]
 
 
@@ -70,6 +70,7 @@ _lib.d2d_router_fwd.argtypes = [c_void_p, c_void_p, c_int32, c_void_p, c_void_p,
 _lib.d2d_select_dynk.argtypes = [c_void_p, c_int32, c_int32, c_float, POINTER(RoutingStruct), c_void_p, c_size_t, c_void_p]
 _lib.d2d_select_dynk_static.argtypes = [c_void_p, c_int32, c_int32, c_float, POINTER(RoutingStruct), c_void_p]
 _lib.d2d_select_topk.argtypes = [c_void_p, c_int32, c_int32, c_int32, POINTER(RoutingStruct), c_void_p, c_size_t, c_void_p]
+_lib.d2d_routing_of_mask.argtypes = [c_void_p, c_int32, c_int32, POINTER(RoutingStruct), c_void_p, c_size_t, c_void_p]
 _lib.d2d_routing_from_mask.argtypes = [c_int32, c_int32, POINTER(RoutingStruct), c_void_p, c_size_t, c_void_p]
 _lib.d2d_moe_ffn_fwd.argtypes = [c_void_p, c_void_p, c_int32, POINTER(RoutingStruct), c_void_p, c_void_p, c_size_t, c_void_p]
 _lib.d2d_expert_up_fwd.argtypes = [c_void_p, c_void_p, c_int32, POINTER(RoutingStruct), c_void_p, c_void_p]
@@ -157,7 +158,7 @@ def _routing_plan(T: int, E: int, cap: int, dual: bool, lists: bool):
 class Routing:
     """Caller-owned device buffers for the routing of one batch (d2d_routing)."""
 
-    def __init__(self, T: int, E: int, device, dual: bool = False, perm_capacity: int | None = None, lists: bool = True):
+    def __init__(self, T: int, E: int, device, dual: bool = False, perm_capacity: int | None = None, lists: bool = True, _new=torch.zeros):
         """lists=False leaves out the per-expert lists (counts, offsets, perm, n_sel): d2d_layer_fwd then does not build them."""
         cap = T * E if perm_capacity is None else int(perm_capacity)
         key = (T, E, cap, dual, lists)
@@ -169,7 +170,7 @@ class Routing:
         self._shapes, words, off = plan
         self.T, self.E, self.W, self.lists = T, E, (E + 31) // 32, lists
         # One zeroed allocation for all buffers; the tensors over it are made when asked for
-        self._slab = torch.zeros((words,), dtype=torch.int32, device=device)
+        self._slab = _new((words,), dtype=torch.int32, device=device)
         base = self._slab.data_ptr()
         self.struct = RoutingStruct(*[None if o is None else base + o for o in off], cap if lists else 0)
 
@@ -489,11 +490,19 @@ def select_topk(R, kk: int, routing: Routing | None = None, dual: bool = False, 
 
 def routing_from_mask(mask_words, E: int, dual: bool = False, stream=None) -> Routing:
     """mask_words: device int32 tensor [T, ceil(E/32)] holding the uint32 mask words."""
-    T = mask_words.shape[0]
-    routing = Routing(T, E, mask_words.device, dual)
-    routing.mask.copy_(mask_words)
+    T, W = mask_words.shape[0], (E + 31) // 32
+    device = mask_words.device
+    # what the call reads as it is; anything else (which copy_ would convert or broadcast, or read on the tensor's own stream) is copied first
+    direct = (T > 0 and not dual and stream is None and mask_words.is_cuda and mask_words.dtype == torch.int32 and
+              mask_words.shape == (T, W) and mask_words.is_contiguous())
+    routing = Routing(T, E, device, dual, _new=torch.empty if direct else torch.zeros)
     nbytes = int(_lib.d2d_select_workspace_bytes(T, E))
-    ws = torch.empty((max(nbytes, 256),), dtype=torch.uint8, device=mask_words.device)
+    ws = torch.empty((max(nbytes, 256),), dtype=torch.uint8, device=device)
+    if direct:
+        _check(_lib.d2d_routing_of_mask(_ptr(mask_words), T, E, ctypes.byref(routing.struct), _ptr(ws), ws.numel(), _stream(stream)),
+               "d2d_routing_of_mask")
+        return routing
+    routing.mask.copy_(mask_words)
     _check(_lib.d2d_routing_from_mask(T, E, ctypes.byref(routing.struct), _ptr(ws), ws.numel(), _stream(stream)),
            "d2d_routing_from_mask")
     return routing

@@ -796,6 +796,14 @@ d2d_status d2d_routing_from_mask(int32_t T, int32_t E, d2d_routing *out, void *w
     return select_common(nullptr, T, E, 0.0f, 0, out, ws, ws_bytes, stream, true);
 }
 
+d2d_status d2d_routing_of_mask(const uint32_t *mask, int32_t T, int32_t E, d2d_routing *out, void *ws, size_t ws_bytes, void *stream)
+{
+    if (T < 0 || E <= 0 || !routing_ok(out, false) || (T > 0 && !mask)) return D2D_ERR_INVALID_ARG;
+    if (T > 0 && (!ws || ws_bytes < d2d_select_ws_bytes(T, E))) return D2D_ERR_WORKSPACE;
+    if (T == 0) return d2d_launch_select(nullptr, 0, E, 0.0f, 0, out, ws, (cudaStream_t)stream);
+    return d2d_launch_select_mask_of(mask, T, E, out, ws, (cudaStream_t)stream);
+}
+
 d2d_status d2d_moe_ffn_fwd(const d2d_layer *layer, const void *x, int32_t T, const d2d_routing *routing,
                            void *y, void *ws, size_t ws_bytes, void *stream)
 {

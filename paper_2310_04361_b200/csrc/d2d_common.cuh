@@ -128,6 +128,8 @@ d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d
 d2d_status d2d_launch_lists(const d2d_routing *r, int n, int T, int E, void *ws, size_t ws_each, cudaStream_t st);
 d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, const d2d_routing *out,
                              void *ws, cudaStream_t st, int mask_ready = 0, unsigned int *zero_ticket = nullptr);
+// Copies a mask into `out` and builds the rest from it, T > 0; entries of perm behind the lists become zero
+d2d_status d2d_launch_select_mask_of(const uint32_t *mask, int T, int E, const d2d_routing *out, void *ws, cudaStream_t st);
 
 // up_counter: see launch_tc_experts (NULL unless the fused router was launched just before on `st`)
 // lists: r's lists are to be built on the side (only where d2d_api.cu's lists_ride says so)

@@ -349,6 +349,114 @@ bucket_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W,
     }
 }
 
+// A mask that is given, in two kernels without a ticket.  The first has everything a 256-token block yields by itself: k, its tokens per
+// expert, and on request a copy of the mask and a cleared perm; the second's CTAs each add up the counts of all blocks before
+// they fill their part of the lists (as bucket_fill_kernel does), so no CTA scans for the others: a chain of latencies shorter by the
+// last CTA's scan, for reading the counts once per CTA (up to SUMS_MAX of them).  50432 tokens x 24 experts, from the first start to the
+// last end: 16 us where clearing perm, copying the mask, k, count with scan, and fill took 24.5; the call 16 us instead of 30 at 200 to
+// 12608 tokens, where that is the host's time.
+constexpr int SUMS_MAX = 16384;
+
+__global__ void __launch_bounds__(TOKB)
+mask_count_kernel(const uint32_t *__restrict__ mask, uint32_t *__restrict__ copy, int T, int E, int W, int32_t *__restrict__ k,
+                  int32_t *__restrict__ blockcounts, int32_t *__restrict__ perm, long long clear, int32_t *status)
+{
+    __shared__ uint16_t cnt[TOKB / 32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.y;
+    const int t = blockIdx.x * TOKB + threadIdx.x, e = w * 32 + lane;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t valid = E - w * 32 >= 32 ? FULL : (1u << (E - w * 32)) - 1u;
+    uint32_t word = t < T ? __ldg(mask + (size_t)t * W + w) : 0u;
+    if (copy && t < T) copy[(size_t)t * W + w] = word;
+    word &= valid;
+    if (w == 0 && t < T) {
+        int kt = __popc(word);
+        for (int i = 1; i < W; ++i) kt += __popc(__ldg(mask + (size_t)t * W + i) & (E - i * 32 >= 32 ? FULL : (1u << (E - i * 32)) - 1u));
+        k[t] = kt;
+    }
+    if (blockIdx.x == 0 && w == 0 && threadIdx.x == 0) *status = 0;
+    // this CTA's share of perm, in whole 16-byte pieces (perm is 16-byte aligned where it is cleared)
+    const long long per = (clear / ((long long)gridDim.x * gridDim.y) + 4) / 4 * 4, at = per * ((long long)w * gridDim.x + blockIdx.x);
+    const long long end = at + per < clear ? at + per : clear;
+    for (long long i = at + threadIdx.x * 4; i + 4 <= end; i += TOKB * 4) *reinterpret_cast<int4 *>(perm + i) = make_int4(0, 0, 0, 0);
+    if (at < end && threadIdx.x < (end & 3)) perm[(end & ~3ll) + threadIdx.x] = 0;
+    cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
+    __syncthreads();
+    if (warp == 0 && e < E) {
+        int total = 0;
+#pragma unroll
+        for (int i = 0; i < TOKB / 32; ++i) total += cnt[i][lane];
+        blockcounts[(size_t)blockIdx.x * E + e] = total;
+    }
+}
+
+__global__ void __launch_bounds__(TOKB)
+mask_fill_kernel(const uint32_t *__restrict__ mask, int T, int E, int W, int nblk, const int32_t *__restrict__ blockcounts,
+                 int32_t *__restrict__ counts, int32_t *__restrict__ offsets, int32_t *__restrict__ n_sel, int32_t *__restrict__ status,
+                 int32_t *__restrict__ perm, long long capacity)
+{
+    constexpr int NW = TOKB / 32;
+    __shared__ uint16_t cnt[NW][33];
+    __shared__ int earlier[NW][32], all[NW][32], front[NW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.y, b = blockIdx.x;
+    const int t = b * TOKB + threadIdx.x, e = w * 32 + lane;
+    const uint32_t lower = (1u << lane) - 1u, valid = E - w * 32 >= 32 ? FULL : (1u << (E - w * 32)) - 1u;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t word = t < T ? __ldg(mask + (size_t)t * W + w) & valid : 0u;
+    // this word's experts: tokens in the blocks before this one, and in all; and all pairs of the words before
+    int sum_b = 0, sum_all = 0, sum_f = 0;
+    if (e < E)
+#pragma unroll 8
+        for (int i = warp; i < nblk; i += NW) {
+            const int c = __ldcg(blockcounts + (size_t)i * E + e);
+            sum_all += c;
+            sum_b += i < b ? c : 0;
+        }
+    for (int i = warp; i < nblk; i += NW)
+        for (int j = lane; j < w * 32; j += 32) sum_f += __ldcg(blockcounts + (size_t)i * E + j);
+    sum_f = __reduce_add_sync(FULL, sum_f);
+    cnt[warp][lane] = (uint16_t)__popc(transpose_bits(word, lane));
+    earlier[warp][lane] = sum_b;
+    all[warp][lane] = sum_all;
+    if (lane == 0) front[warp] = sum_f;
+    __syncthreads();
+    int total = 0, before = 0, offset = 0;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        total += all[i][lane];
+        before += earlier[i][lane] + (i < warp ? cnt[i][lane] : 0);
+        offset += front[i];
+    }
+    int inc = total;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += n;
+    }
+    offset += inc - total;                                    // where expert e's list begins
+    if (b == 0 && warp == 0 && e < E) {
+        counts[e] = total;
+        offsets[e] = offset;
+        if (e == E - 1) {
+            offsets[E] = offset + total;
+            *n_sel = offset + total;
+            if ((long long)offset + total > capacity) atomicMax(status, (int32_t)D2D_ERR_CAPACITY);
+        }
+    }
+    const long long base = (long long)offset + before;
+#pragma unroll 4
+    for (int j = 0; j < 32; ++j) {
+        const uint32_t holders = __ballot_sync(FULL, (word >> j) & 1u);
+        const long long bj = __shfl_sync(FULL, base, j);
+        if ((word >> j) & 1u) {
+            const long long idx = bj + __popc(holders & lower);
+            if (idx < capacity) perm[idx] = t;
+        }
+    }
+}
+
 // Exclusive scan of one int per thread over a 1024-thread CTA (used by the token-major dual).
 __device__ __forceinline__ int block_exscan_1024(int v, int *warp_sums /*[32]*/, int *total_out)
 {
@@ -481,6 +589,39 @@ d2d_status d2d_launch_dynk_mask(const float *R, int T, int E, float tau, const d
     return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
 }
 
+// k, status and lists from a mask, by mask_count_kernel and mask_fill_kernel.  copy: the mask is to be copied to out->mask, perm cleared
+static bool mask_pair_fits(int T, int E) { return (long long)d2d_cdiv(T, TOKB) * E <= SUMS_MAX; }
+static d2d_status launch_mask_pair(const uint32_t *mask, int T, int E, const d2d_routing *out, bool copy, void *ws, cudaStream_t st)
+{
+    const int W = (E + 31) / 32, nblk = d2d_cdiv(T, TOKB);
+    int32_t *blockcounts = (int32_t *)((char *)ws + 256);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nblk, W, 1);
+    cfg.blockDim = dim3(TOKB, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
+    const long long capacity = (long long)out->perm_capacity;
+    D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, mask_count_kernel, mask, copy ? out->mask : (uint32_t *)nullptr, T, E, W, out->k, blockcounts, out->perm,
+                                    copy ? capacity : 0ll, out->status));
+    D2D_CUDA_TRY(cudaLaunchKernelEx(&cfg, mask_fill_kernel, mask, T, E, W, nblk, (const int32_t *)blockcounts, out->counts, out->offsets, out->n_sel,
+                                    out->status, out->perm, capacity));
+    D2D_LAUNCHED(2);
+    launch_dual(out, T, W, st);
+    return cudaGetLastError() == cudaSuccess ? D2D_OK : D2D_ERR_CUDA;
+}
+
+d2d_status d2d_launch_select_mask_of(const uint32_t *mask, int T, int E, const d2d_routing *out, void *ws, cudaStream_t st)
+{
+    if (T > 64 && mask_pair_fits(T, E) && (reinterpret_cast<uintptr_t>(out->perm) & 15) == 0) return launch_mask_pair(mask, T, E, out, true, ws, st);
+    D2D_CUDA_TRY(cudaMemcpyAsync(out->mask, mask, (size_t)T * ((E + 31) / 32) * 4, cudaMemcpyDeviceToDevice, st));
+    D2D_CUDA_TRY(cudaMemsetAsync(out->perm, 0, (size_t)out->perm_capacity * 4, st));
+    return d2d_launch_select(nullptr, T, E, 0.0f, 0, out, ws, st);
+}
+
 d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, const d2d_routing *out,
                              void *ws, cudaStream_t st, int mask_ready, unsigned int *zero_ticket)
 {
@@ -497,6 +638,7 @@ d2d_status d2d_launch_select(const float *R, int T, int E, float tau, int topk, 
         return D2D_OK;
     }
     if (small) return d2d_small_select(R, T, E, tau, out, st, mask_ready);
+    if (given && !one && mask_pair_fits(T, E)) return launch_mask_pair(out->mask, T, E, out, false, ws, st);
     const int nblk = d2d_cdiv(T, TOKB);
     // the ticket must start at zero (the kernel leaves it there): a word the caller keeps, or cleared on every call
     unsigned int *ticket = zero_ticket ? zero_ticket : (unsigned int *)ws;
