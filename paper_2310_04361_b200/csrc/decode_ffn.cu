@@ -133,6 +133,9 @@ __device__ __forceinline__ void widen16(const uint4 &r, uint32_t (&o)[8])
             : "=r"(o[2 * i]), "=r"(o[2 * i + 1]) : "r"(w[i]));
     }
 }
+// Place of columns 4 q .. 4 q + 3 (8 bytes) of a token row beside codes: every 32 columns, two 16-column pieces a and b, become
+// a[0..3] b[0..3] a[4..7] b[4..7] ..., so that a lane of a matrix instruction finds its four columns of both pieces in 16 bytes.
+__device__ __forceinline__ uint32_t x_place(int q) { return (uint32_t)((q & ~7) | ((q & 3) << 1) | ((q >> 2) & 1)) * 8u; }
 __device__ __forceinline__ uint2 lds8(uint32_t addr)
 {
     uint2 v;
@@ -434,19 +437,30 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             // wpt warps a token, a piece of the row each; a lane looks at what it fetched itself
             const int wpt = T <= 1 ? 16 : T <= 2 ? 8 : T <= 4 ? 4 : T <= 8 ? 2 : 1, part = warp % wpt, np = d / 8;
             const int i0 = np * part / wpt, i1 = np * (part + 1) / wpt;
-            auto fetch = [&]() {
+            auto fetch = [&](bool placed) {
                 for (int t = warp / wpt; t < T; t += NCW / wpt)
-                    for (int i = i0 + lane; i < i1; i += 32) cp_async16(smem_addr(xs + (size_t)t * xp + i * 16), x + (size_t)t * d + i * 8);
+                    for (int i = i0 + lane; i < i1; i += 32) {
+                        const __nv_bfloat16 *src = x + (size_t)t * d + i * 8;
+                        const uint32_t row = smem_addr(xs + (size_t)t * xp);
+                        if (placed) {
+                            cp_async8(row + x_place(2 * i), src);
+                            cp_async8(row + x_place(2 * i + 1), src + 4);
+                        } else {
+                            cp_async16(row + i * 16, src);
+                        }
+                    }
                 asm volatile("cp.async.commit_group;" ::: "memory");
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
             };
+            // a lane's own eight columns, as they lie after a placed fetch
+            auto own = [&](int t, int i, int h) { return reinterpret_cast<uint2 *>(xs + (size_t)t * xp + x_place(2 * i + h)); };
             if (tid == 0) x_spread = 0;
-            fetch();
+            fetch(true);
             for (int t = warp / wpt; t < T; t += NCW / wpt) {
                 uint32_t m = 0u;
                 for (int i = i0 + lane; i < i1; i += 32) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(xs + (size_t)t * xp + i * 16);
-                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                    const uint2 a = *own(t, i, 0), b = *own(t, i, 1);
+                    const uint32_t w[4] = {a.x, a.y, b.x, b.y};
 #pragma unroll
                     for (int q = 0; q < 4; ++q) m = max(m, max(w[q] & 0x7fffu, (w[q] >> 16) & 0x7fffu));
                 }
@@ -464,9 +478,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 const uint32_t least = (uint32_t)max(((int)(m >> 7) - 31) * 128 - 1, 0);
                 if (lane == 0 && part == 0) x_inv[t] = __uint_as_float((uint32_t)(127 - sh) << 23);
                 for (int i = i0 + lane; i < i1; i += 32) {
-                    uint4 *at = reinterpret_cast<uint4 *>(xs + (size_t)t * xp + i * 16);
-                    const uint4 v = *at;
-                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                    const uint2 a = *own(t, i, 0), b = *own(t, i, 1);
+                    const uint32_t w[4] = {a.x, a.y, b.x, b.y};
                     uint32_t o[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
@@ -474,14 +487,15 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                         const float lo = __uint_as_float(w[q] << 16) * f, hi = __uint_as_float(w[q] & 0xffff0000u) * f;
                         asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(o[q]) : "f"(hi), "f"(lo));
                     }
-                    *at = make_uint4(o[0], o[1], o[2], o[3]);
+                    *own(t, i, 0) = make_uint2(o[0], o[1]);
+                    *own(t, i, 1) = make_uint2(o[2], o[3]);
                 }
             }
             if (spread) x_spread = 1;
             consumer_bar();
             if (__builtin_expect(*(volatile int *)&x_spread != 0, 0)) {
                 if (tid < T) x_inv[tid] = 1.0f;
-                fetch();
+                fetch(false);
                 consumer_bar();
             }
         }
@@ -563,34 +577,24 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                                 }
                             }
                         } else {
-                            // lane = rows g, g + 8.  A row is eight 16-byte pieces; lane c takes pieces c and c + 4, odd rows in the other
-                            // order, so that eight lanes (two rows) do not meet in a bank
-                            const int flip = (g & 1) * 64;
-                            uint4 a[2][2];                        // [piece c / c + 4][row g / g + 8]
+                            // Two 16-code pieces of all rows at a time: lane (g, c) gets codes 4 c .. 4 c + 3 of rows g and g + 8 of each, that
+                            // is a matrix instruction's operand but for the order of its 16 columns, which the token rows share.  (Plain
+                            // 16-byte loads, half of them exchanged between registers so that they do not meet in a bank, and
+                            // addresses worked out load by load here and in the down projection kept the ALU pipe busy for 58 % of the
+                            // kernel, where the loops were bound by it: Llama-shaped layer, tau = 0.2, 41.8 -> 37.4 us at 1 token, 55.8 ->
+                            // 49.7 at 2, 60.0 -> 52.9 at 6.)
+                            const uint32_t sa = smem_addr(st) + lrow * 128 + ((lhalf ^ (lrow & 7)) << 4);
 #pragma unroll
-                            for (int h = 0; h < 2; ++h)
+                            for (int h = 0; h < 4; ++h) {
+                                uint32_t q[4], w[8];
+                                ldmatrix4<false>(q, sa ^ (uint32_t)(h * 32));
+                                widen16(make_uint4(q[0], q[1], q[2], q[3]), w);
 #pragma unroll
-                                for (int i = 0; i < 2; ++i) a[h][i] = *reinterpret_cast<const uint4 *>(st + swz(g + 8 * i, c * 16 + (h * 64 ^ flip)));
-#pragma unroll
-                            for (int i = 0; i < 2; ++i) {
-                                const uint4 p = a[0][i], o = a[1][i];
-                                a[0][i] = flip ? o : p;
-                                a[1][i] = flip ? p : o;
-                            }
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int xo = (k0 + h * (SUB / 2)) * 2 + c * 32;
-                                uint32_t wa[2][8];
-                                widen16(a[h][0], wa[0]);
-                                widen16(a[h][1], wa[1]);
-#pragma unroll
-                                for (int t = 0; t < NT8; ++t)
-#pragma unroll
-                                    for (int p = 0; p < 2; ++p) {
-                                        const uint4 xb = *reinterpret_cast<const uint4 *>(xs + min(t * 8 + g, T - 1) * xp + xo + p * 16);
-                                        mma16816_f16(s[m][t * CH], wa[0][4 * p], wa[1][4 * p], wa[0][4 * p + 1], wa[1][4 * p + 1], xb.x, xb.y);
-                                        mma16816_f16(s[m][t * CH + CH - 1], wa[0][4 * p + 2], wa[1][4 * p + 2], wa[0][4 * p + 3], wa[1][4 * p + 3], xb.z, xb.w);
-                                    }
+                                for (int t = 0; t < NT8; ++t) {
+                                    const uint4 xb = lds16(xs_addr + min(t * 8 + g, T - 1) * xp + (k0 + h * 32) * 2 + c * 16);
+                                    mma16816_f16(s[m][t * CH], w[0], w[2], w[1], w[3], xb.x, xb.y);
+                                    mma16816_f16(s[m][t * CH + CH - 1], w[4], w[6], w[5], w[7], xb.z, xb.w);
+                                }
                             }
                         }
                     }
@@ -751,6 +755,9 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
 #pragma unroll
             for (int t = 0; t < NT8; ++t) acc[i][t][0] = acc[i][t][1] = acc[i][t][2] = acc[i][t][3] = 0.0f;
         const int DC = d / CL;
+        // codes: where neurons 2 c and 2 c + 1 of the lane's four columns lie in a unit's rows
+        const uint32_t dn0 = (uint32_t)(warp / (SUB / 32) * SUB_BYTES) + swz(2 * c, warp % (SUB / 32) * 32 + g * 4),
+                       dn1 = (uint32_t)(warp / (SUB / 32) * SUB_BYTES) + swz(2 * c + 1, warp % (SUB / 32) * 32 + g * 4);
         auto down = [&](int r, int R) {
             const int j = r - my_static, nv = slots(r, n);
             if (ok && CL > 1) ok = mbar_wait_cluster(smem_addr(&h_full[j < 0 ? 2 : j & 1]), j < 0 ? 0u : (j >> 1) & 1u, P.status);
@@ -798,11 +805,10 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                             for (int i = 0; i < (TPP + 1) / 2; ++i) {
                                 const int pair = warp + NCW * i;
                                 if (PARTS == 1 && pair * 32 >= DC) break;
-                                const unsigned char *st = piece + pair * 32 / SUB * SUB_BYTES;
                                 uint32_t r[4];                    // neurons 2c, 2c + 1, 2c + 8, 2c + 9: four columns each
 #pragma unroll
                                 for (int q = 0; q < 4; ++q)
-                                    r[q] = *reinterpret_cast<const uint32_t *>(st + swz(2 * c + (q & 1) + (q >> 1) * 8, pair * 32 % SUB + g * 4));
+                                    r[q] = *reinterpret_cast<const uint32_t *>(piece + ((q & 1) ? dn1 : dn0) + (i * NCW * 32 / SUB * SUB_BYTES + (q >> 1) * 1024));
                                 const uint32_t a0[4] = {pair_of<0>(r[0], r[1]), pair_of<1>(r[0], r[1]), pair_of<0>(r[2], r[3]), pair_of<1>(r[2], r[3])};
                                 const uint32_t a1[4] = {pair_of<2>(r[0], r[1]), pair_of<3>(r[0], r[1]), pair_of<2>(r[2], r[3]), pair_of<3>(r[2], r[3])};
                                 products(acc[part * TPP + 2 * i], a0);
