@@ -34,7 +34,7 @@ namespace {
 
 using namespace d2d_decode;
 
-constexpr int NCW = 16, NC = NCW * 32, NT = NC + 64;      // consumer warps / threads, all threads (a producer warp, a signalling one)
+constexpr int NCW = 16, NC = NCW * 32, NT = NC + 64;      // consumer warps / threads, all threads (a producer warp, one that talks to the cluster)
 constexpr int SUB_BYTES = 16 * 128;                       // a block: 16 rows x 128 bytes, 128-byte swizzle
 constexpr int STAGE_BLOCKS = 16, STAGE_BYTES = STAGE_BLOCKS * SUB_BYTES;
 constexpr int MAX_STAGES = 6;
@@ -265,12 +265,12 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     const d2d_decode_ffn_layer &P = args.l[blockIdx.y];
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);       // swizzle atoms are 1024 bytes
-    __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], h_full[3], h_empty[2], h_read[2], bar_go;
+    __shared__ uint64_t bar_full[MAX_STAGES], bar_empty[MAX_STAGES], h_full[3], h_empty[2], h_read[2], h_done[2], bar_go;
     __shared__ int unit_list[MAX_LIST], unit_list_p[MAX_LIST], n_units;
     __shared__ uint32_t keep_bits[MAX_UNITS / 32];
     __shared__ int keep_pre[MAX_UNITS / 32];
     __shared__ unsigned int my_ticket;
-    __shared__ volatile int rounds_s;                          // all rounds of this cluster, for the signalling warp
+    __shared__ volatile int rounds_s, n_s;                     // all rounds of this cluster and the list's length, for the talking warp
     __shared__ uint32_t x_max[Q8 ? T8 * 16 : 1];               // codes: largest magnitude of the pieces of the token rows ...
     __shared__ float x_inv[T8];                                // ... what takes the scaling of a row back ...
     __shared__ int x_spread;                                   // ... and whether some row does not fit float16
@@ -296,6 +296,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
         for (int i = 0; i < 2; ++i) {
             d2d_tc::mbar_init(smem_addr(&h_empty[i]), CL);
             d2d_tc::mbar_init(smem_addr(&h_read[i]), NCW);
+            d2d_tc::mbar_init(smem_addr(&h_done[i]), NCW);
         }
         d2d_tc::mbar_init(smem_addr(&bar_go), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -321,6 +322,10 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             list[i] = __ldcg(P.units + 1 + j);
         }
     };
+
+    // Hidden values live in buffers [static round, or n_static + the parity of a shared round][slot]; the static rounds' are
+    // exchanged together, once.
+    auto buffer = [&](int r) { return hs + (size_t)(r < my_static ? r : S.n_static + ((r - my_static) & 1)) * CL * S.planes * T8 * H_ROW; };
 
     if (warp == NCW) {
         // ------------------------------------------------------------------ producer
@@ -404,16 +409,54 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             for (uint32_t k = it > (uint32_t)S.stages ? it - S.stages : 0; k + 1 < it; ++k)
                 d2d_tc::mbar_wait_warp(smem_addr(&bar_full[k % S.stages]), (k / S.stages) & 1u, P.status);
         cluster_arrive();
-    } else if (warp == NCW + 1) {
-        // ------------------------------------------------------------------ tells the cluster that a round's hidden values have been
-        // read.  A release at cluster scope takes 0.6 us: a consumer warp would hold up all others with it.
-        bool ok = CL > 1 && d2d_tc::mbar_wait_warp(smem_addr(&bar_go), 0, P.status);
+    } else if (warp > NCW) {
+        // ------------------------------------------------------------------ talks to the cluster: sends the hidden values, and tells
+        // the others that a round's have been read.  A release at cluster scope takes 0.6 us, sending as much: a consumer warp would
+        // hold up all others with it (Llama-shaped layer, tau = 0.2, us, with the sends by consumer warps / here: 37.7 / 35.4 at 1 token and
+        // 52.9 / 50.6 at 6, 8-bit weights; 59.4 / 56.6 at 7 tokens.  A warp for each other CTA: the same with clusters of two, and 43.7
+        // instead of 40.9 at 1 token, where they are of four.)
+        bool ok = d2d_tc::mbar_wait_warp(smem_addr(&bar_go), 0, P.status);
         __syncwarp();
-        const int nj = ok ? rounds_s - my_static : 0;
-        for (int j = 0; ok && j + 2 < nj; ++j) {
-            ok = d2d_tc::mbar_wait_warp(smem_addr(&h_read[j & 1]), (j >> 1) & 1u, P.status);
+        const uint32_t hs_addr = smem_addr(hs);
+        const int nj = ok ? rounds_s - my_static : 0, n = n_s, q0 = my_static > 0 ? 1 : 0;
+        for (int q = 0; ok && q < nj + q0; ++q) {
+            const int j = q - q0;                              // number of the shared round, or -1: the static ones
+            if (j >= 2) {                                      // the consumers have read the buffer's last contents: others may write it
+                ok = d2d_tc::mbar_wait_warp(smem_addr(&h_read[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
+                __syncwarp();
+                if (ok && lane < CL) arrive_cluster(cluster_addr(smem_addr(&h_empty[j & 1]), lane));
+            }
+            // two barriers in turn: the consumers are at most one round ahead, since a round's down projection waits for what is sent here
+            ok = ok && d2d_tc::mbar_wait_warp(smem_addr(&h_done[q & 1]), (q >> 1) & 1u, P.status);
             __syncwarp();
-            if (ok && lane < CL) arrive_cluster(cluster_addr(smem_addr(&h_empty[j & 1]), lane));
+            if (ok && j >= 2) ok = mbar_wait_cluster(smem_addr(&h_empty[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
+            __syncwarp();
+            const uint32_t full = smem_addr(&h_full[j < 0 ? 2 : j & 1]);
+            if (lane == 0) d2d_tc::mbar_arrive(full);
+            // 16-byte asynchronous stores, counted by the receiver's barrier (4-byte ones by the threads that have the values took 2.6
+            // us, plain stores and an arrival that releases them 1.4); a piece goes to all others at once
+            uint32_t to[3], bar[3], bytes = 0;
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+                to[p] = cluster_addr(hs_addr, (rank + 1 + p) % CL);
+                bar[p] = cluster_addr(full, (rank + 1 + p) % CL);
+            }
+            for (int r = j < 0 ? 0 : my_static + j; r < (j < 0 ? my_static : my_static + j + 1); ++r) {
+                if (rank >= slots(r, n)) break;
+                bytes += 32u * (uint32_t)(NT8 == 1 ? T8 * S.planes : T);
+                const uint32_t own = (uint32_t)(buffer(r) - hs) + (uint32_t)rank * S.planes * T8 * H_ROW;
+                for (int i = lane; i < 2 * T8 * S.planes; i += 32) {
+                    const uint32_t off = own + (i >> 1) * H_ROW + (i & 1) * 16;
+                    if (NT8 > 1 && (i >> 1) >= T) break;
+                    const uint4 v = lds16(hs_addr + off);
+#pragma unroll
+                    for (int p = 0; p < 3; ++p)
+                        if (p + 1 < CL) st_async4(to[p] + off, v, bar[p]);
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+                if (p + 1 < CL && lane == 0) arrive_cluster(bar[p], bytes);
         }
         cluster_arrive();
     } else {
@@ -692,13 +735,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             n = n_units;
         };
 
-        // Hidden values live in buffers [static round, or n_static + the parity of a shared round][slot]; the static rounds' are
-        // exchanged together, once.
-        auto buffer = [&](int r) { return hs + (size_t)(r < my_static ? r : S.n_static + ((r - my_static) & 1)) * CL * S.planes * T8 * H_ROW; };
-
-        // ---- hidden values of rounds [r0, r1): activation and selection on this CTA's sums into its own buffers, from there to
-        // the other CTAs of the cluster, a warp per receiver (16-byte asynchronous stores; 4-byte ones by the threads that have
-        // the values took 2.6 us, plain stores and an arrival that releases them 1.4)
+        // ---- hidden values of rounds [r0, r1): activation and selection on this CTA's sums into its own buffers
         auto finish = [&](int r0, int r1) {
             const int j = r0 - my_static;                                      // shared rounds: their number
             for (int r = r0; r < r1; ++r) {
@@ -722,26 +759,12 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                     o[0] = Q8 ? __float2bfloat16_rn(__bfloat162float(hb) * z[2 * 16 * T8]) : hb;
                 }
             }
-            consumer_bar();
-            if (CL > 1 && warp < CL) {
-                if (j >= 2 && ok) ok = mbar_wait_cluster(smem_addr(&h_empty[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
-                const uint32_t full = smem_addr(&h_full[j < 0 ? 2 : j & 1]);
-                if (warp != rank) {
-                    uint32_t bytes = 0;
-                    for (int r = r0; r < r1; ++r) {
-                        if (rank >= slots(r, n)) break;
-                        bytes += 32u * (uint32_t)(NT8 == 1 ? T8 * S.planes : T);
-                        const unsigned char *own = buffer(r) + (size_t)rank * S.planes * T8 * H_ROW;
-                        const uint32_t to = cluster_addr(smem_addr(own), warp);
-                        for (int i = lane; i < 2 * T8 * S.planes; i += 32) {
-                            const int off = (i >> 1) * H_ROW + (i & 1) * 16;
-                            if (NT8 == 1 || (i >> 1) < T) st_async4(to + off, *reinterpret_cast<const uint4 *>(own + off), cluster_addr(full, warp));
-                        }
-                    }
-                    if (lane == 0) arrive_cluster(cluster_addr(full, warp), bytes);
-                } else if (lane == 0) {
-                    d2d_tc::mbar_arrive(full);
-                }
+            if (CL > 1) {
+                const int q = j < 0 ? 0 : j + (my_static > 0 ? 1 : 0);
+                __syncwarp();
+                if (lane == 0) d2d_tc::mbar_arrive(smem_addr(&h_done[q & 1]));
+            } else {
+                consumer_bar();
             }
         };
         // (A CTA's own slot of a shared round's buffer is written again two rounds later, behind the barriers of that round's up
@@ -834,6 +857,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 ready = true;
                 R = rounds_for(n);
                 if (tid == 0) {
+                    n_s = n;
                     rounds_s = R;
                     d2d_tc::mbar_arrive(smem_addr(&bar_go));
                 }
@@ -1010,7 +1034,7 @@ d2d_status launch(const FfnShape &S, int n_layers, const d2d_decode_ffn_args &a,
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(S.clusters * S.cl, n_layers, 1);
-    cfg.blockDim = dim3(S.cl > 1 ? NT : NT - 32, 1, 1);        // clusters of one have nobody to signal to
+    cfg.blockDim = dim3(S.cl > 1 ? NT : NT - 32, 1, 1);        // clusters of one have nobody to talk to
     cfg.dynamicSmemBytes = fixed_smem<WT>(S, (size_t)S.T) + (size_t)S.stages * STAGE_BYTES;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
