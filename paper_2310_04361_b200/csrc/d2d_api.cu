@@ -1071,24 +1071,30 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     // chunk c+1 to the device (copy-in stream), the layer on chunk c (`stream`) and the copy of chunk c-1 back to the
     // host (copy-out stream) run at the same time; PCIe carries both directions at once.  The routing buffers and the
     // layer workspace are reused chunk after chunk, which is safe because the layer calls are serial on `stream`.
-    // The layer is the slowest of the three legs for the shapes where this matters, so the whole call takes about
-    // (copy-in of the first chunk) + (all layer calls) + (copy-out of the last chunk): the first and the last chunk
-    // are short, the ones in between long (a short chunk costs more per token, so there are few of them).
+    // Which leg is the slowest decides how: a token's FLOP take longer than its bytes over PCIe from 18000 hidden neurons times matrices
+    // on (1.4 PFLOP/s, 54 GB/s).
     int bounds[d2d_layer::kHostChunks + 1] = {0, T, T, T, T};
     int n_chunks = 1;
-    if (T >= 3584) {
-        // sizes 3T/16, 5T/16, 5T/16, 3T/16 in multiples of 128 tokens (measured on the Llama-shaped layer, 8192 tokens:
-        // 2.50 ms; T/8, 3T/8, 3T/8, T/8: 2.64; four equal chunks: 2.62; two equal chunks: 3.04)
-        const int a = d2d_cdiv(3 * (T / 16), 128) * 128, b = d2d_cdiv((T - 2 * a) / 2, 128) * 128;
-        bounds[1] = a; bounds[2] = a + b; bounds[3] = T - a > a + b ? T - a : a + b; bounds[4] = T;
-        n_chunks = 4;
-    } else if (T >= 1024 && row_bytes >= ((size_t)3 << 20)) {
-        // Equal chunks, as many as pay for their launches and partly filled rounds.  Measured with 1 / 2 / 3 / 4 (us), Llama-shaped
-        // layer at 1000 tokens: 535 / 483 / 554 / 626, 2000: 1007 / 747 / 731 / 781, 4000: 1932 / 1421 / 1361 / 1168;
-        // GPT-2-medium-shaped at 1000: 146 / 153 / 153 / 172, 2000: 227 / 190 / 197 / 218, 4000: 392 / 328 / 298 / 297.
-        n_chunks = T >= 2560 ? 3 : 2;
-        const int chunk = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
-        for (int c = 1; c < n_chunks; ++c) bounds[c] = c * chunk;
+    if (T >= 1024 && row_bytes >= ((size_t)3 << 20)) {
+        int first = 0, middle = 0;                           // sizes: first, middle, .., middle, the rest
+        if ((layer->desc.gated ? 3 : 2) * (int64_t)layer->desc.d_ff >= 18000) {
+            // The layer: the call takes about (copy-in of the first chunk) + (all layer calls) + (copy-out of the last), if a chunk is
+            // copied in while the layer works on the one before and out while it works on the next: sizes may grow and shrink by the
+            // ratio of the two times, 1.3.  Multiples of 256, the rows of a pair's tile.  Llama-shaped layer, us, sizes of before (3/16,
+            // 5/16, 5/16, 3/16 from 3584 tokens on, two or three equal ones below) / these: 8192 tokens 2288 / 2187, 6000 1734 / 1684, 4096
+            // 1209 / 1139, 3400 1082 / 958, 2500 944 / 773, 2000 710 / 678; two of 512 443 at 1024 tokens, three 482.
+            n_chunks = T >= 3328 ? 4 : T >= 1536 ? 3 : 2;
+            auto round256 = [](int v) { return v < 384 ? 256 : (v + 128) / 256 * 256; };
+            first = n_chunks == 2 ? d2d_cdiv(d2d_cdiv(T, 2), 128) * 128 : round256((n_chunks == 4 ? 7 : 10) * (T / 32));
+            middle = n_chunks == 2 ? first : round256((T - 2 * first) / (n_chunks - 2));
+        } else {
+            // The copies: equal chunks, as many as pay for their launches.  us with 2 / 3 / 4, GPT-2-medium-shaped layer: 2048 tokens 192 /
+            // 207 / 215, 3000 256 / 245 / 258, 4096 331 / 304 / 293, 6000 464 / 423 / 390 (sizes of before: 441); BERT-shaped: 3000 203 / 201
+            // / 216, 4096 256 / 236 / 247, 6000 364 / 328 / 307 (327).
+            n_chunks = row_bytes >= (size_t)7500000 ? 4 : T >= 2560 ? 3 : 2;
+            first = middle = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
+        }
+        for (int c = 1; c < n_chunks; ++c) bounds[c] = first + (c - 1) * middle < T ? first + (c - 1) * middle : T;
     }
     if (const char *e = getenv("D2D_HOST_CHUNKS")) {          // 1 .. 4 equal chunks, for tuning
         const int n = atoi(e);
