@@ -146,9 +146,6 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     __shared__ uint32_t pmax_s[4 * BM];                    // per column-part row maxima (bit patterns of non-negative floats)
     __shared__ int pk_s[4 * BM];
     __shared__ int warp_k[4], warp_bad[4];
-    for (int i = threadIdx.x; i < DH; i += NTHREADS) b1_s[i] = b_r1 ? __bfloat162float(b_r1[i]) : 0.0f;
-    for (int i = threadIdx.x; i < 256; i += NTHREADS) b2_s[i] = (b_r2 && i < E) ? __bfloat162float(b_r2[i]) : 0.0f;
-
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * BM;
     const int nkb = (d + BK - 1) / BK;
@@ -175,7 +172,13 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_holder;
     const uint32_t tmem_r = TWO ? tmem_base : tmem_base + 256;
-    // the set-up above may overlap the tail of the previous kernel of the stream
+    // The set-up above may overlap the tail of the previous kernel of the stream, and so may the weights' part of the first stages.
+    const int early = nkb < STAGES ? nkb : STAGES;
+    if (warp == 0 && lane == 0)
+        for (int kb = 0; kb < early; ++kb) {
+            mbar_expect_tx(smem_u32(&bar_full[kb]), (uint32_t)STAGE_BYTES);
+            tma_load_2d(smem_u32(smem + (size_t)kb * STAGE_BYTES) + A_BYTES, &tm_w1, kb * BK, layer * DH, smem_u32(&bar_full[kb]));
+        }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // the expert up projection that follows on the stream may start its operand loads and MMAs on the SMs this
     // grid leaves idle (T / 128 CTAs); its epilogue waits for this kernel to complete before it reads the mask
@@ -187,13 +190,15 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
             bool ok = true;
             for (int kb = 0; kb < nkb && ok; ++kb) {
                 const uint32_t s = kb % STAGES, round = kb / STAGES;
-                ok = mbar_wait(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, status);
-                if (!ok) break;
                 const uint32_t full = smem_u32(&bar_full[s]);
                 const uint32_t dst = smem_u32(smem + (size_t)s * STAGE_BYTES);
-                mbar_expect_tx(full, (uint32_t)STAGE_BYTES);
+                if (kb >= early) {
+                    ok = mbar_wait(smem_u32(&bar_empty[s]), (round & 1u) ^ 1u, status);
+                    if (!ok) break;
+                    mbar_expect_tx(full, (uint32_t)STAGE_BYTES);
+                    tma_load_2d(dst + A_BYTES, &tm_w1, kb * BK, layer * DH, full);
+                }
                 tma_load_2d(dst, &tm_x, kb * BK, m0, full);
-                tma_load_2d(dst + A_BYTES, &tm_w1, kb * BK, layer * DH, full);
             }
             // W_r2 goes into stages 0 .. W2_STAGES-1 once the MMAs of the last k-block that used each of them have retired
             for (int s = 0; s < W2_STAGES && ok; ++s) {
@@ -253,6 +258,10 @@ router_fused_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_const
         const int row = m0 + r_local;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         auto publish = [&](int k_warp, bool cond_warp) { publish_batch(ksum, io.l[layer].status, quad, lane, k_warp, cond_warp, warp_k, warp_bad); };
+        // biases, while the first GEMM runs (in front of the first barrier they held up its loads)
+        for (int i = (int)threadIdx.x - 64; i < DH; i += NTHREADS - 64) b1_s[i] = b_r1 ? __bfloat162float(b_r1[i]) : 0.0f;
+        for (int i = (int)threadIdx.x - 64; i < 256; i += NTHREADS - 64) b2_s[i] = (b_r2 && i < E) ? __bfloat162float(b_r2[i]) : 0.0f;
+        asm volatile("bar.sync 1, %0;" ::"n"(NTHREADS - 64) : "memory");
         int okw = 1;
         if (lane == 0) okw = mbar_wait(smem_u32(&bar_acc1), 0, status) ? 1 : 0;
         bool ok = __shfl_sync(0xffffffffu, okw, 0) != 0;
