@@ -360,6 +360,18 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
     // decode-sized batches: split K of the down projection over the SMs, partial sums in the float32 scratch behind H
     const int k_splits = d2d_gemm_tc_splits(T, D.d, D.d_ff);
     float *partial = k_splits > 1 ? (float *)((char *)ws + d2d_align_up((size_t)T * D.d_ff * 2, 256)) : nullptr;
+    // Wide layers: the cells the gathered kernel leaves alone are zero-filled, so that the TMA-fed dense down projection can follow
+    // whichever up projection ran; otherwise the down projection that applies the selection while it stages H follows the gathered
+    // kernel.  In front of both up projections: on the side stream beside the gathered kernel, behind the dense one, it saved nothing there
+    // (Llama-shaped layer, us, there / here: 3500 tokens at tau = 0.6 557 / 562, 6000 at 0.5 998 / 997, 8192 at 0.4 1657 / 1651), and where
+    // the dense form runs the events and waits between the streams held up the down projection (1536 tokens 384 / 372, 2048 479 / 463, 2560
+    // 591 / 574).
+    const bool zero_fill = path != D2D_PATH_DENSE && D.d >= 2048;
+    const long long hi = path == D2D_PATH_AUTO ? n_sel_max : LLONG_MAX;
+    if (zero_fill) {
+        rc = d2d_moe_zero_unkept(ws, r->mask, T, D.d_ff, D.n_experts, D.expert_size, L->gather_group, n_sel, n_sel_fused, hi, st);
+        if (rc != D2D_OK) return rc;
+    }
     if (path != D2D_PATH_GATHER) {
         d2d_gemm_args up = dense_up_args(L, x, T, r, ws);
         const bool forced = path == D2D_PATH_DENSE;
@@ -370,22 +382,7 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
         rc = d2d_gemm_tc(up, st);
         if (rc != D2D_OK) return rc;
     }
-    // Wide layers: the cells the gathered kernel leaves alone are zero-filled, so that the TMA-fed dense down projection
-    // can follow whichever up projection ran; otherwise the down projection that applies the selection while it stages
-    // H follows the gathered kernel.
-    const bool zero_fill = path != D2D_PATH_DENSE && D.d >= 2048;
     if (path != D2D_PATH_DENSE) {
-        const long long hi = path == D2D_PATH_AUTO ? n_sel_max : LLONG_MAX;
-        if (zero_fill) {
-            // on the layer's side stream: the fill and the gathered kernel write disjoint cells, and its small CTAs fit
-            // beside the persistent ones; joined before the down projection
-            if (cudaEventRecord(L->ev_fill_fork, st) != cudaSuccess || cudaStreamWaitEvent(L->side_stream, L->ev_fill_fork, 0) != cudaSuccess)
-                return D2D_ERR_CUDA;
-            rc = d2d_moe_zero_unkept(ws, r->mask, T, D.d_ff, D.n_experts, D.expert_size, L->gather_group, n_sel, n_sel_fused, hi,
-                                     L->side_stream);
-            if (rc != D2D_OK) return rc;
-            if (cudaEventRecord(L->ev_fill_join, L->side_stream) != cudaSuccess) return D2D_ERR_CUDA;
-        }
         d2d_gather_args ga = {};
         ga.x = x; ga.w1 = L->w1; ga.w_gate = D.gated ? L->w_gate : nullptr; ga.b1 = L->b1; ga.mask = r->mask; ga.H = ws;
         ga.T = T; ga.d = D.d; ga.d_ff = D.d_ff; ga.n_experts = D.n_experts; ga.s = D.expert_size; ga.g = L->gather_group;
@@ -398,7 +395,6 @@ static d2d_status launch_tc_experts(const d2d_layer *L, const void *x, int T, co
         rc = d2d_moe_down_masked(D, ws, r->mask, L->w2, L->b2, y, T, r->status, st, path == D2D_PATH_AUTO ? n_sel : nullptr, n_sel_fused, n_sel_max);
         if (rc != D2D_OK || path == D2D_PATH_GATHER) return rc;
     }
-    if (zero_fill && cudaStreamWaitEvent(st, L->ev_fill_join, 0) != cudaSuccess) return D2D_ERR_CUDA;
     d2d_gemm_args dn = dense_down_args(L, ws, T, y, r->status);
     // after a zero fill this kernel serves the gathered range too: it only has to stay out of the fused kernel's range
     dn.n_sel = path == D2D_PATH_AUTO && (!zero_fill || n_sel_fused >= 0) ? n_sel : nullptr;
@@ -551,9 +547,7 @@ d2d_status d2d_layer_create(const d2d_layer_desc *desc, const d2d_weights *w, vo
     if (rc == D2D_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = D2D_ERR_CUDA;
     if (rc == D2D_OK && (cudaStreamCreateWithFlags(&L->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
                          cudaEventCreateWithFlags(&L->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-                         cudaEventCreateWithFlags(&L->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-                         cudaEventCreateWithFlags(&L->ev_fill_fork, cudaEventDisableTiming) != cudaSuccess ||
-                         cudaEventCreateWithFlags(&L->ev_fill_join, cudaEventDisableTiming) != cudaSuccess))
+                         cudaEventCreateWithFlags(&L->ev_join, cudaEventDisableTiming) != cudaSuccess))
         rc = D2D_ERR_CUDA;
     if (rc == D2D_OK) {
         bool ok = cudaStreamCreateWithFlags(&L->copy_in, cudaStreamNonBlocking) == cudaSuccess &&
@@ -578,8 +572,6 @@ d2d_status d2d_layer_destroy(d2d_layer *layer)
 {
     if (!layer) return D2D_OK;
     if (layer->ev_join) cudaEventDestroy(layer->ev_join);
-    if (layer->ev_fill_fork) cudaEventDestroy(layer->ev_fill_fork);
-    if (layer->ev_fill_join) cudaEventDestroy(layer->ev_fill_join);
     if (layer->ev_fork) cudaEventDestroy(layer->ev_fork);
     if (layer->side_stream) cudaStreamDestroy(layer->side_stream);
     for (int c = 0; c < d2d_layer::kHostChunks; ++c) {

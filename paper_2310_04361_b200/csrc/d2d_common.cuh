@@ -28,7 +28,6 @@ struct d2d_layer {
     // expert GEMMs, which do not read it
     cudaStream_t side_stream;
     cudaEvent_t ev_fork, ev_join;
-    cudaEvent_t ev_fill_fork, ev_fill_join;      // zero fill of H beside the gathered up projection (side stream)
     // 8-bit expert weights (d2d_layer_create_fp8): e4m3 codes [d_ff, d] of W1, W_gate and the transposed W2, one scale
     // exponent per expert and matrix; NULL for ordinary layers.  w1, w_gate, w2, w2t, w1g then hold the dequantised values.
     void *q_slab;

@@ -1299,7 +1299,7 @@ d2d_status d2d_moe_down_masked(const d2d_layer_desc &D, const void *H, const uin
 // With them H is fully defined and the plain TMA-fed dense down projection can follow (10-20 % faster than the one
 // that applies the selection while it stages H); the price is (1 - u) T d_ff 2 bytes of stores at memory bandwidth,
 // which pays for wide layers (the down projection's time grows with d, the fill's does not).
-// One thread per 16-byte chunk: consecutive lanes write consecutive chunks of a token's row.
+// A warp per token and quarter of its row, a lane per 16-byte chunk.
 __global__ void __launch_bounds__(256)
 h_zero_unkept_kernel(__nv_bfloat16 *__restrict__ H, const uint32_t *__restrict__ mask, int T, int W, int d_ff, int g, uint32_t inv_gs,
                      const int32_t *n_sel, long long n_sel_min, long long n_sel_max)
@@ -1310,14 +1310,18 @@ h_zero_unkept_kernel(__nv_bfloat16 *__restrict__ H, const uint32_t *__restrict__
         const long long n = (long long)__ldcg(n_sel);
         if (!(n > n_sel_min && n <= n_sel_max)) return;
     }
-    const int chunks = d_ff >> 3;
+    const int chunks = d_ff >> 3, per = (chunks + 3) / 4, lane = threadIdx.x & 31;
     const uint32_t gm = g >= 32 ? 0xffffffffu : (1u << g) - 1u;
-    const long long total = (long long)T * chunks;
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long long)gridDim.x * 256) {
-        const int t = (int)(i / chunks), c = (int)(i - (long long)t * chunks);
-        const int e0 = (int)__umulhi((uint32_t)(c * 8), inv_gs) * g;              // first expert of the chunk's group
-        const uint32_t bits = (__ldg(mask + (size_t)t * W + (e0 >> 5)) >> (e0 & 31)) & gm;
-        if (bits == 0u) *reinterpret_cast<uint4 *>(H + (size_t)t * d_ff + (size_t)c * 8) = make_uint4(0u, 0u, 0u, 0u);
+    for (long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); i < 4ll * T; i += (long long)gridDim.x * 8) {
+        const long long t = i >> 2;
+        const int c0 = (int)(i & 3) * per, c1 = min(chunks, c0 + per);
+        const uint32_t *row = mask + t * W;
+        uint4 *h = reinterpret_cast<uint4 *>(H + t * d_ff);
+#pragma unroll 4
+        for (int c = c0 + lane; c < c1; c += 32) {
+            const int e0 = (int)__umulhi((uint32_t)(c * 8), inv_gs) * g;          // first expert of the chunk's group
+            if (((__ldg(row + (e0 >> 5)) >> (e0 & 31)) & gm) == 0u) h[c] = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
 }
 
@@ -1335,9 +1339,7 @@ d2d_status d2d_moe_zero_unkept(void *H, const uint32_t *mask, int T, int d_ff, i
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = d2d_tc_pdl_enabled() ? 1 : 0;
-    const long long total = (long long)T * (d_ff / 8);
-    const long long blocks = (total + 255) / 256;
-    const int cap = 16 * d2d_tc_sm_count();
+    const int blocks = d2d_cdiv(T, 2), cap = 8 * d2d_tc_sm_count();
     cfg.gridDim = dim3((unsigned)(blocks < cap ? blocks : cap), 1, 1);
     cfg.blockDim = dim3(256, 1, 1);
     const cudaError_t err = cudaLaunchKernelEx(&cfg, h_zero_unkept_kernel, (__nv_bfloat16 *)H, mask, T, (n_experts + 31) / 32, d_ff, g, inv_gs,
