@@ -81,16 +81,16 @@ int d2d_gemm_tc_splits(int M, int N, int K, int batch = 1);
 size_t d2d_gemm_tc_partial_floats(int M, int N, int K, int batch = 1);
 
 // Whether the lists of a batch can be left to the GEMM of its down projection: as many tokens as a CTA's epilogue warps take in one
-// go (512) or, before a main loop that is not split, in two.  On a stream of their own they cost the layer a launch, two events
-// and two waits between streams, and its call the programmatic launch behind it.  GPT-2-medium-shaped FFN, back to back: 30.8 ->
-// 24.0 us at 64 tokens, 34.2 -> 30.5 at 333, 41.2 -> 39.2 at 1000 (not split); Llama-shaped layer 78.0 -> 72.8 at 100.  Split along K
-// and in two goes they held the partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection
-// that have no tile they held up the down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
-// The line of 1e10 FLOP of down projection and the limit of 512 tokens are older than the present loops: with those the lists would
-// ride a little further (Llama-shaped layer 101.9 -> 98.5 at 200 tokens; ViT-shaped, 700 tokens: level).
+// go (512) or, before a main loop that is not split, in four.  On a stream of their own they cost the layer a launch, two events
+// and two waits between streams, and its call the programmatic launch behind it.  us, back to back, on a stream / here: GPT-2-medium-shaped
+// FFN 30.8 / 24.0 at 64 tokens, 34.2 / 30.5 at 333, 46.8 / 44.3 at 1100, 49.1 / 49.0 at 1500; its attention projection 38.6 / 33.0 at 1100,
+// 34.9 / 33.4 at 1500, 35.0 / 36.0 at 1792; BERT-shaped layer 39.1 / 37.2 at 1500, 39.5 / 39.7 at 1792, 47 / 60 at 4096; ViT-shaped 37.0 /
+// 33.6 at 1300; Llama-shaped 78.0 / 72.8 at 100, 77.1 / 73.6 at 120, 101.9 / 98.8 at 200.  Split along K and in two goes they held the
+// partial sums up (ViT-shaped layer, 700 tokens: 34.9 -> 38.2).  Built by CTAs of the up projection that have no tile they held up the
+// down projection (BERT-shaped layer, 1000 tokens: 32.1 here, 38.5 there).
 static inline bool d2d_lists_ride(int T, int E, int k_splits, double down_flop)
 {
-    return T <= (k_splits > 1 ? 512 : 1024) && (long long)T * ((E + 31) / 32) <= 16384 && down_flop <= 1e10;
+    return T <= (k_splits > 1 ? 512 : 1600) && (long long)T * ((E + 31) / 32) <= 16384 && down_flop <= 2e10;
 }
 
 // Enqueues C = epilogue(A B^T).  Requires K % 8 == 0 and 16-byte aligned base pointers.
