@@ -162,13 +162,13 @@ d2d_status d2d_decode_layers(const d2d_layer *const *layers, int n, const void *
 
 size_t d2d_layer_ws_bytes(const d2d_layer *L, int T) { return layout_for(L, T).total; }
 
-// Whether a batch may take the sorted form (moe_sorted.cu), by shape and size: from 5.8e10 FLOP of up projection on (12288 tokens of the
-// paper's shape).  Shorter batches have little to win over the dense pair, and where that runs in the end the kernels of the other form
-// cost 10 us (expert step, us, dense pair / sorted form at p = 0.02, 0.05, 0.1, 0.2: 12608 tokens 105 / 60, 75, 84, 104; 8000 tokens 69 /
-// 52, 59, 66, 79; 5000 tokens 47 / 46, 48, 54, 61).
+// Whether a batch may take the sorted form (moe_sorted.cu), by shape and size: from 1.1e11 FLOP of up projection on (23300 tokens of the
+// paper's shape).  Shorter batches win where few pairs are kept (expert step, us, dense pair / sorted form at p = 0.02, 0.05, 0.1, 0.2: 12608
+// tokens 105 / 60, 75, 84, 104; 8000 tokens 69 / 52, 59, 66, 79), but where the dense pair runs in the end the four kernels of the other
+// form cost it 10 to 20 us (14000 tokens, p = 0.3, routing and expert step 125 / 136; 30000, p = 0.45, 240 / 238).
 static bool sorted_shape(const d2d_layer_desc &D, int T)
 {
-    return 2.0 * (double)T * D.d * D.d_ff >= 5.8e10 && d2d_sorted_supports(D, T) && d2d_gemm_tc_splits(T, D.d, D.d_ff) == 1;
+    return 2.0 * (double)T * D.d * D.d_ff >= 1.1e11 && d2d_sorted_supports(D, T) && d2d_gemm_tc_splits(T, D.d, D.d_ff) == 1;
 }
 
 size_t d2d_moe_ffn_ws_bytes(const d2d_layer *L, int T)

@@ -37,8 +37,8 @@ def _keep(kind, T, E, rng):
 
 
 # (E, s, d, T): the paper's experts; experts of 64 neurons; a word full of experts; few; ragged last tiles, one of one row
-CASES = [(24, 128, 768, 12611, k) for k in ("0.02", "0.2", "one mask", "nothing", "two kinds")] + [
-    (32, 64, 1024, 14081, "0.05"), (8, 128, 1024, 27777, "0.1"), (32, 128, 512, 13953, "0.1")]
+CASES = [(24, 128, 768, 23555, k) for k in ("0.02", "0.2", "one mask", "nothing", "two kinds")] + [
+    (32, 64, 1024, 26369, "0.05"), (8, 128, 1024, 52481, "0.1"), (32, 128, 512, 26369, "0.1")]
 
 
 @pytest.mark.parametrize("E,s,d,T,kind", CASES)
@@ -72,7 +72,7 @@ def test_sorted_form(api, E, s, d, T, kind):
 
 
 def test_above_the_limit_the_dense_pair_runs(api):
-    cfg = wl.with_tokens(wl.CONFIGS["paper"], 12800)
+    cfg = wl.with_tokens(wl.CONFIGS["paper"], 24000)
     layer = api.Layer.from_config(cfg, wl.make_weights(cfg))
     g = torch.Generator(device="cuda").manual_seed(3)
     x = torch.randn((cfg.T, cfg.d), generator=g, device="cuda").to(torch.bfloat16)
