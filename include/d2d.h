@@ -418,9 +418,10 @@ D2D_API d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t 
  * ([T,d] of desc.dtype).  The call copies x to the device, runs the layer,
  * copies y back and synchronises `stream`; all device memory it needs comes
  * from `ws` (device, at least d2d_layer_fwd_host_workspace_bytes bytes).
- * Batches of 3584 tokens or more are cut into four chunks of 3/16, 5/16, 5/16
- * and 3/16 of the tokens, shorter ones of 3 MB or more into two or three (the call then takes about the copy-in of the first
- * chunk + the layer on all of them + the copy-out of the last) and pipelined over
+ * Batches of 1024 tokens and 3 MB or more are cut into two to four chunks
+ * (equal ones where the copies take longest, shorter ones at the ends where the
+ * layer does: the call then takes about the copy-in of the first chunk + the
+ * layer on all of them + the copy-out of the last) and pipelined over
  * two copy streams the layer owns (copy in / layer / copy out overlap; tokens
  * are independent, so the result is the same); this needs page-locked host
  * buffers to be effective.  Returns the data-dependent status as well
