@@ -438,7 +438,6 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
             if (ok && j >= 2) ok = mbar_wait_cluster(smem_addr(&h_empty[j & 1]), ((j >> 1) & 1u) ^ 1u, P.status);
             __syncwarp();
             const uint32_t full = smem_addr(&h_full[j < 0 ? 2 : j & 1]);
-            if (lane == 0) d2d_tc::mbar_arrive(full);
             // 16-byte asynchronous stores, counted by the receiver's barrier (4-byte ones by the threads that have the values took 2.6
             // us, plain stores and an arrival that releases them 1.4); a piece goes to all others at once
             uint32_t to[3], bar[3], bytes = 0;
@@ -463,6 +462,9 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
 #pragma unroll
             for (int p = 0; p < 3; ++p)
                 if (p + 1 < CL && lane == 0) arrive_cluster(bar[p], bytes);
+            // only now the CTA's own consumers: what they wait for here lets them write this slot again, two rounds on
+            __syncwarp();
+            if (lane == 0) d2d_tc::mbar_arrive(full);
         }
         cluster_arrive();
     } else {
@@ -778,8 +780,9 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 consumer_bar();
             }
         };
-        // (A CTA's own slot of a shared round's buffer is written again two rounds later, behind the barriers of that round's up
-        // projection, which every warp reaches after it has read the buffer.)
+        // (A CTA's own slot of a shared round's buffer is written again two rounds later.  The consumers have read it by then: the
+        // barriers of that round's up projection come behind their down projection.  So has the warp that sends it, which takes no
+        // part in those: that down projection waits for its arrival at h_full, and it arrives when it has read the slot.)
 
         // ---- down projection of round r onto this CTA's columns.  A tile's 16 columns: bf16 weights g and g + 8 of lane (g, c);
         // codes 4 g and 4 g + 1 of a 32-column pair of tiles, 4 g + 2 and 4 g + 3 in its second tile.

@@ -67,3 +67,24 @@ def test_arrivals_at_other_ctas_release(name):
     for op in re.findall(r"mbarrier\.arrive[\w.:]*", source(name)):
         if "shared::cluster" in op:
             assert ".release.cluster." in op or op == "mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64", op
+
+
+def test_a_sent_slot_is_read_before_its_owner_goes_on():
+    """The warp that sends a CTA's hidden values reads them from the CTA's own slot.  Two rounds later the consumers write that slot again,
+    behind a wait for the barrier that this warp arrives at: so the arrival has to come behind its last read, and behind all of its lanes'."""
+    text = source("decode_ffn.cu")
+    talk = text[text.index("} else if (warp > NCW) {"):]
+    talk = talk[:talk.index("cluster_arrive();")]
+    own = [m.start() for m in re.finditer(r"mbar_arrive\(full\)", talk)]
+    reads = [m.start() for m in re.finditer(r"lds16\(", talk)]
+    assert len(own) == 1 and reads and reads[-1] < own[0]
+    # the loop over the slot's pieces has ended, and its lanes have met
+    loop = talk.index("for (int r = ")
+    depth = 0
+    for end in range(talk.index("{", loop), len(talk)):
+        depth += {"{": 1, "}": -1}.get(talk[end], 0)
+        if depth == 0:
+            break
+    assert reads[-1] < end < own[0] and "__syncwarp();" in talk[end:own[0]]
+    # and every consumer of a shared round waits for that barrier before its down projection
+    assert re.search(r"auto down = .*?mbar_wait_cluster\(smem_addr\(&h_full\[j < 0 \? 2 : j & 1\]\)", text, re.S)
