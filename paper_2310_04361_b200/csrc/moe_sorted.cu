@@ -25,7 +25,7 @@ static_assert(N_BUCKETS == 1 << RANK_SHIFT && RANK_SHIFT == 6 + LOW_BITS, "bucke
 constexpr int THREADS = 512;                // = tokens of a CTA of the bucket kernel
 constexpr int TILE = 128;                   // rows of an output tile
 constexpr int BN = 256;                     // columns of an output tile of both projections
-constexpr int MAX_TILES = 2048;             // unions of the tiles, in shared memory of the CTA that lists the work
+constexpr int MAX_TILES = D2D_SORTED_MAX_TOKENS / TILE;       // unions of the tiles, in shared memory of the CTA that lists the work
 
 // Which bucket a mask belongs to.  Buckets with similar unions of experts should lie side by side: the upper six bits say which of six
 // blocks of adjacent experts have a kept one, in the order of a Gray code (neighbours differ in one block), the lower four are the
@@ -278,7 +278,7 @@ bool d2d_sorted_supports(const d2d_layer_desc &D, int T)
 {
     const bool size_ok = D.expert_size == 64 || D.expert_size == 128;
     return D.dtype == D2D_BF16 && !D.gated && D.n_experts <= 32 && size_ok && D.d % BN == 0 && D.d_ff % BN == 0 && D.d_ff / BN <= 256 &&
-           2.0 * D.d * D.d_ff < 48e6 && T > 0 && T <= MAX_TILES * TILE;
+           2.0 * D.d * D.d_ff < 48e6 && T > 0 && T <= D2D_SORTED_MAX_TOKENS;
 }
 
 d2d_sorted_layout d2d_sorted_layout_for(const d2d_layer_desc &D, int T)

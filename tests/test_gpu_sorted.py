@@ -83,3 +83,22 @@ def test_above_the_limit_the_dense_pair_runs(api):
     layer.set_expert_path("dense")
     assert torch.equal(y.view(torch.int16), layer.moe_ffn_fwd(x, r).view(torch.int16))
     layer.close()
+
+
+# the paper's shape, and one whose rows are wide beside its hidden layer (the copy of the rows outweighs the rest)
+@pytest.mark.parametrize("E,s,d", [(24, 128, 768), (8, 64, 2048)])
+def test_a_workspace_serves_every_smaller_batch_of_ordered_tokens(api, E, s, d):
+    """d2d_workspace_bytes(max_tokens) is enough for any batch of up to max_tokens tokens, also behind the largest that is ordered: the sizes
+    never fall.  Sizes only: nothing is allocated or run."""
+    cfg = dataclasses.replace(wl.CONFIGS["paper"], E=E, d_ff=E * s, d=d)
+    layer = api.Layer.from_config(cfg, wl.make_weights(cfg))
+    group = api.LayerGroup([layer])
+    edge = 2048 * 128
+    assert layer.sorted_limit(edge) >= 0 and layer.sorted_limit(edge + 1) == -1
+    batches = sorted({*range(1, 330001, 1009), *range(edge - 200, edge + 200), 16384, 16385, 23300, 23301, 330000, 500000})
+    for size in (layer.workspace_bytes, lambda T: int(api._lib.d2d_layer_fwd_host_workspace_bytes(layer.handle, T)),
+                 lambda T: int(api._lib.d2d_group_workspace_bytes(group.handle, T))):
+        at = [size(T) for T in batches]
+        assert all(a <= b for a, b in zip(at, at[1:]))
+    group.close()
+    layer.close()
