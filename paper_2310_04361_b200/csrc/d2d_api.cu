@@ -1038,6 +1038,37 @@ size_t d2d_layer_fwd_host_workspace_bytes(const d2d_layer *layer, int32_t max_to
     return host_layout(layer, max_tokens).ws_off + d2d_workspace_bytes(layer, max_tokens > 0 ? max_tokens : 1);      // chunks are smaller batches
 }
 
+// How a host call cuts T tokens: bounds[0 .. chunks], returns the number of chunks.  Which of the three legs (copy in, layer, copy out) is
+// the slowest decides: a bf16 token's FLOP take as long as its bytes over PCIe (54 GB/s) with 18000 hidden neurons times matrices at
+// 0.97 PFLOP/s, with 26000 at the sustained 1.4, which batches of a chunk's size do not reach.  At 18432 (d = 1536, plain) both cuts are
+// level (us, equal chunks / sizes by the layer: 1600 tokens 258 / 256, 3600 412 / 405); float32 layers take the equal ones, since each
+// chunk costs them most of a round of CTAs (d = 512, d_ff = 9216: 1600 tokens 7328 in two / 8091, 2000 8367 / 9519).
+static int cut_host_batch(const d2d_layer *L, int T, int *bounds)
+{
+    const size_t row_bytes = (size_t)T * L->desc.d * L->elem;
+    if (T < 1024 || row_bytes < ((size_t)3 << 20)) return 1;
+    int n_chunks = 2, first = 0, middle = 0;                 // sizes: first, middle, .., middle, the rest
+    if (L->desc.dtype == D2D_BF16 && (L->desc.gated ? 3 : 2) * (int64_t)L->desc.d_ff >= 18000) {
+        // The layer: the call takes about (copy-in of the first chunk) + (all layer calls) + (copy-out of the last), if a chunk is
+        // copied in while the layer works on the one before and out while it works on the next: sizes may grow and shrink by the
+        // ratio of the two times, 1.3.  Multiples of 256, the rows of a pair's tile.  Llama-shaped layer, us, sizes of before (3/16,
+        // 5/16, 5/16, 3/16 from 3584 tokens on, two or three equal ones below) / these: 8192 tokens 2288 / 2187, 6000 1734 / 1684, 4096
+        // 1209 / 1139, 3400 1082 / 958, 2500 944 / 773, 2000 710 / 678; two of 512 443 at 1024 tokens, three 482.
+        n_chunks = T >= 3328 ? 4 : T >= 1536 ? 3 : 2;
+        auto round256 = [](int v) { return v < 384 ? 256 : (v + 128) / 256 * 256; };
+        first = n_chunks == 2 ? d2d_cdiv(d2d_cdiv(T, 2), 128) * 128 : round256((n_chunks == 4 ? 7 : 10) * (T / 32));
+        middle = n_chunks == 2 ? first : round256((T - 2 * first) / (n_chunks - 2));
+    } else {
+        // The copies: equal chunks, as many as pay for their launches.  us with 2 / 3 / 4, GPT-2-medium-shaped layer: 2048 tokens 192 /
+        // 207 / 215, 3000 256 / 245 / 258, 4096 331 / 304 / 293, 6000 464 / 423 / 390 (sizes of before: 441); BERT-shaped: 3000 203 / 201
+        // / 216, 4096 256 / 236 / 247, 6000 364 / 328 / 307 (327).
+        n_chunks = row_bytes >= (size_t)7500000 ? 4 : T >= 2560 ? 3 : 2;
+        first = middle = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
+    }
+    for (int c = 1; c < n_chunks; ++c) bounds[c] = first + (c - 1) * middle < T ? first + (c - 1) * middle : T;
+    return n_chunks;
+}
+
 d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_t T, float tau, void *y_host,
                               void *ws, size_t ws_bytes, void *stream)
 {
@@ -1063,31 +1094,8 @@ d2d_status d2d_layer_fwd_host(const d2d_layer *layer, const void *x_host, int32_
     // chunk c+1 to the device (copy-in stream), the layer on chunk c (`stream`) and the copy of chunk c-1 back to the
     // host (copy-out stream) run at the same time; PCIe carries both directions at once.  The routing buffers and the
     // layer workspace are reused chunk after chunk, which is safe because the layer calls are serial on `stream`.
-    // Which leg is the slowest decides how: a token's FLOP take longer than its bytes over PCIe from 18000 hidden neurons times matrices
-    // on (1.4 PFLOP/s, 54 GB/s).
     int bounds[d2d_layer::kHostChunks + 1] = {0, T, T, T, T};
-    int n_chunks = 1;
-    if (T >= 1024 && row_bytes >= ((size_t)3 << 20)) {
-        int first = 0, middle = 0;                           // sizes: first, middle, .., middle, the rest
-        if ((layer->desc.gated ? 3 : 2) * (int64_t)layer->desc.d_ff >= 18000) {
-            // The layer: the call takes about (copy-in of the first chunk) + (all layer calls) + (copy-out of the last), if a chunk is
-            // copied in while the layer works on the one before and out while it works on the next: sizes may grow and shrink by the
-            // ratio of the two times, 1.3.  Multiples of 256, the rows of a pair's tile.  Llama-shaped layer, us, sizes of before (3/16,
-            // 5/16, 5/16, 3/16 from 3584 tokens on, two or three equal ones below) / these: 8192 tokens 2288 / 2187, 6000 1734 / 1684, 4096
-            // 1209 / 1139, 3400 1082 / 958, 2500 944 / 773, 2000 710 / 678; two of 512 443 at 1024 tokens, three 482.
-            n_chunks = T >= 3328 ? 4 : T >= 1536 ? 3 : 2;
-            auto round256 = [](int v) { return v < 384 ? 256 : (v + 128) / 256 * 256; };
-            first = n_chunks == 2 ? d2d_cdiv(d2d_cdiv(T, 2), 128) * 128 : round256((n_chunks == 4 ? 7 : 10) * (T / 32));
-            middle = n_chunks == 2 ? first : round256((T - 2 * first) / (n_chunks - 2));
-        } else {
-            // The copies: equal chunks, as many as pay for their launches.  us with 2 / 3 / 4, GPT-2-medium-shaped layer: 2048 tokens 192 /
-            // 207 / 215, 3000 256 / 245 / 258, 4096 331 / 304 / 293, 6000 464 / 423 / 390 (sizes of before: 441); BERT-shaped: 3000 203 / 201
-            // / 216, 4096 256 / 236 / 247, 6000 364 / 328 / 307 (327).
-            n_chunks = row_bytes >= (size_t)7500000 ? 4 : T >= 2560 ? 3 : 2;
-            first = middle = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
-        }
-        for (int c = 1; c < n_chunks; ++c) bounds[c] = first + (c - 1) * middle < T ? first + (c - 1) * middle : T;
-    }
+    int n_chunks = cut_host_batch(layer, T, bounds);
     if (const char *e = getenv("D2D_HOST_CHUNKS")) {          // 1 .. 4 equal chunks, for tuning
         const int n = atoi(e);
         if (n >= 1 && n <= d2d_layer::kHostChunks && T >= 128 * n) {
