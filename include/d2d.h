@@ -418,7 +418,7 @@ D2D_API d2d_status d2d_layer_fwd(const d2d_layer *layer, const void *x, int32_t 
  * ([T,d] of desc.dtype).  The call copies x to the device, runs the layer,
  * copies y back and synchronises `stream`; all device memory it needs comes
  * from `ws` (device, at least d2d_layer_fwd_host_workspace_bytes bytes).
- * Batches of 1024 tokens and 3 MB or more are cut into two to four chunks
+ * Batches of 1024 tokens and 3 MB or more, or of 3584 tokens and 2 MB, are cut into two to four chunks
  * (equal ones where the copies take longest, shorter ones at the ends where the
  * layer does: the call then takes about the copy-in of the first chunk + the
  * layer on all of them + the copy-out of the last) and pipelined over

@@ -1046,9 +1046,12 @@ size_t d2d_layer_fwd_host_workspace_bytes(const d2d_layer *layer, int32_t max_to
 static int cut_host_batch(const d2d_layer *L, int T, int *bounds)
 {
     const size_t row_bytes = (size_t)T * L->desc.d * L->elem;
-    if (T < 1024 || row_bytes < ((size_t)3 << 20)) return 1;
+    // Under 3 MB two chunks pay where there are many narrow rows, from 2 MB on (us, one / two chunks: d = 256, 4000 tokens 128 / 115,
+    // 5800 160 / 139; d = 128, 6000 102 / 99, 12000 162 / 143; float32, d = 64, 12000 458 / 420; d = 128, 3600 667 / 717, 6000 1006 / 1031)
+    const bool large = row_bytes >= ((size_t)3 << 20);
+    if (T < 1024 || !(large || (T >= 3584 && row_bytes >= ((size_t)2 << 20)))) return 1;
     int n_chunks = 2, first = 0, middle = 0;                 // sizes: first, middle, .., middle, the rest
-    if (L->desc.dtype == D2D_BF16 && (L->desc.gated ? 3 : 2) * (int64_t)L->desc.d_ff >= 18000) {
+    if (L->desc.dtype == D2D_BF16 && large && (L->desc.gated ? 3 : 2) * (int64_t)L->desc.d_ff >= 18000) {
         // The layer: the call takes about (copy-in of the first chunk) + (all layer calls) + (copy-out of the last), if a chunk is
         // copied in while the layer works on the one before and out while it works on the next: sizes may grow and shrink by the
         // ratio of the two times, 1.3.  Multiples of 256, the rows of a pair's tile.  Llama-shaped layer, us, sizes of before (3/16,
@@ -1062,7 +1065,7 @@ static int cut_host_batch(const d2d_layer *L, int T, int *bounds)
         // The copies: equal chunks, as many as pay for their launches.  us with 2 / 3 / 4, GPT-2-medium-shaped layer: 2048 tokens 192 /
         // 207 / 215, 3000 256 / 245 / 258, 4096 331 / 304 / 293, 6000 464 / 423 / 390 (sizes of before: 441); BERT-shaped: 3000 203 / 201
         // / 216, 4096 256 / 236 / 247, 6000 364 / 328 / 307 (327).
-        n_chunks = row_bytes >= (size_t)7500000 ? 4 : T >= 2560 ? 3 : 2;
+        n_chunks = row_bytes >= (size_t)7500000 ? 4 : large && T >= 2560 ? 3 : 2;
         first = middle = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
     }
     for (int c = 1; c < n_chunks; ++c) bounds[c] = first + (c - 1) * middle < T ? first + (c - 1) * middle : T;

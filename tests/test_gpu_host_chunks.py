@@ -15,6 +15,7 @@ def api():
 
 GATED = dict(d=1536, d_ff=6144, E=96, gated=True, act="silu", b1_shift=None)       # 18432 neurons times matrices: the layer is the slowest leg
 PLAIN = dict(d=1536, d_ff=9216, E=144)
+NARROW = dict(d=256, d_ff=1024, E=64)
 BERT = dict(d=768, d_ff=3072, E=128)
 F32_WIDE = dict(dtype="f32", d=512, d_ff=9216, E=72, d_h=64)
 CASES = [
@@ -24,6 +25,9 @@ CASES = [
     (PLAIN, 1536, (512, 512, 512)), (PLAIN, 3328, (768, 1024, 1024, 512)),
     # equal ones: by tokens, and by the bytes of the rows (3 MB)
     (BERT, 2048, (1024, 1024)), (BERT, 2047, (2047,)), (BERT, 2559, (1280, 1279)), (BERT, 2560, (896, 896, 768)),
+    # narrow rows: two from 2 MB and 3584 tokens on
+    (NARROW, 4095, (4095,)), (NARROW, 4096, (2048, 2048)), (NARROW, 6143, (3072, 3071)), (NARROW, 6144, (2048, 2048, 2048)),
+    (dict(d=320, d_ff=1024, E=64), 3583, (3583,)), (dict(d=320, d_ff=1024, E=64), 3584, (1792, 1792)),
     # float32 takes the equal ones
     (F32_WIDE, 1600, (896, 704)),
 ]
