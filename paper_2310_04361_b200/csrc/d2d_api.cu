@@ -1063,9 +1063,10 @@ static int cut_host_batch(const d2d_layer *L, int T, int *bounds)
         middle = n_chunks == 2 ? first : round256((T - 2 * first) / (n_chunks - 2));
     } else {
         // The copies: equal chunks, as many as pay for their launches.  us with 2 / 3 / 4, GPT-2-medium-shaped layer: 2048 tokens 192 /
-        // 207 / 215, 3000 256 / 245 / 258, 4096 331 / 304 / 293, 6000 464 / 423 / 390 (sizes of before: 441); BERT-shaped: 3000 203 / 201
-        // / 216, 4096 256 / 236 / 247, 6000 364 / 328 / 307 (327).
-        n_chunks = row_bytes >= (size_t)7500000 ? 4 : large && T >= 2560 ? 3 : 2;
+        // 207 / 215, 3000 256 / 245 / 258, 3450 - / 265 / 284, 3600 302 / 290 / 269, 6000 464 / 423 / 390; BERT-shaped: 3000 203 / 201 / 216,
+        // 4096 256 / 236 / 247, 4500 - / 253 / 257, 4800 293 / 268 / 256, 6000 364 / 328 / 307; d = 256: 8000 tokens 179 / 166 / 186, 13000
+        // 264 / 251 / 232.
+        n_chunks = row_bytes > ((size_t)7 << 20) ? 4 : large && T >= 2560 ? 3 : 2;
         first = middle = d2d_cdiv(d2d_cdiv(T, n_chunks), 128) * 128;
     }
     for (int c = 1; c < n_chunks; ++c) bounds[c] = first + (c - 1) * middle < T ? first + (c - 1) * middle : T;

@@ -17,14 +17,16 @@ GATED = dict(d=1536, d_ff=6144, E=96, gated=True, act="silu", b1_shift=None)    
 PLAIN = dict(d=1536, d_ff=9216, E=144)
 NARROW = dict(d=256, d_ff=1024, E=64)
 BERT = dict(d=768, d_ff=3072, E=128)
+GPT2 = dict(d=1024, d_ff=4096, E=256)
 F32_WIDE = dict(dtype="f32", d=512, d_ff=9216, E=72, d_h=64)
 CASES = [
     # sizes by the layer: two, three and four chunks, on both sides of each line, and ragged ends
     (GATED, 1023, (1023,)), (GATED, 1024, (512, 512)), (GATED, 1535, (768, 767)), (GATED, 1536, (512, 512, 512)), (GATED, 2047, (512, 1024, 511)),
     (GATED, 3327, (1024, 1280, 1023)), (GATED, 3328, (768, 1024, 1024, 512)), (GATED, 4099, (1024, 1024, 1024, 1027)),
     (PLAIN, 1536, (512, 512, 512)), (PLAIN, 3328, (768, 1024, 1024, 512)),
-    # equal ones: by tokens, and by the bytes of the rows (3 MB)
+    # equal ones: by tokens, and by the bytes of the rows (3 and 7 MB)
     (BERT, 2048, (1024, 1024)), (BERT, 2047, (2047,)), (BERT, 2559, (1280, 1279)), (BERT, 2560, (896, 896, 768)),
+    (GPT2, 3584, (1280, 1280, 1024)), (GPT2, 3585, (1024, 1024, 1024, 513)),
     # narrow rows: two from 2 MB and 3584 tokens on
     (NARROW, 4095, (4095,)), (NARROW, 4096, (2048, 2048)), (NARROW, 6143, (3072, 3071)), (NARROW, 6144, (2048, 2048, 2048)),
     (dict(d=320, d_ff=1024, E=64), 3583, (3583,)), (dict(d=320, d_ff=1024, E=64), 3584, (1792, 1792)),
