@@ -1060,3 +1060,34 @@ def test_wide_split_down_projections_repeat(api, T, path):
         assert torch.equal(y.view(torch.int16), first.view(torch.int16)), rep
     assert bool(torch.isfinite(first.float()).all())
     layer.close()
+
+
+# batches on both sides of each line up to which the down projection builds the lists: 1600 tokens (before a main loop that is not split),
+# 16384 mask words, 2e10 FLOP
+@pytest.mark.parametrize("shape,last,Ts", [(dict(d=1024, d_ff=4096, E=256), 1600, (1025, 1537, 1599, 1600, 1601)),
+                                           (dict(d=768, d_ff=3072, E=192), 1600, (1300, 1600, 1601)),
+                                           (dict(d=512, d_ff=344 * 16, E=344, d_h=256), 1489, (1489, 1490)),
+                                           (dict(d=4096, d_ff=8192, E=256), 298, (298, 299))])
+def test_lists_ride_up_to_their_limits(api, shape, last, Ts):
+    cfg = wl.LayerConfig("ride", "bf16", **{**dict(d_h=128, act="gelu_erf", token_sigma=0.5, b1_shift=-0.3), **shape}, T=max(Ts), seed=67)
+    layer = api.Layer.from_config(cfg, wl.make_weights(cfg))
+    xd = api.to_device(wl.make_tokens(cfg), cfg.dtype)
+    for T in Ts:
+        launches = []
+        for lists in (False, True):
+            before = api.launch_count()
+            layer.layer_fwd(xd[:T], 0.4, routing=layer.new_routing(T, lists=lists))
+            launches.append(api.launch_count() - before)
+        assert (launches[0] == launches[1]) == (T <= last), (T, launches)      # riding lists need no launch of their own
+        for tau in (0.4, 0.0):
+            r = layer.new_routing(T)
+            _poison(r.perm), _poison(r.counts), _poison(r.offsets)
+            layer.layer_fwd(xd[:T], tau, routing=r)
+            torch.cuda.synchronize()
+            G = oracle.unpack_mask(r.mask_u32(), cfg.E)
+            _check_routing(r, G, dual=False)
+        small = layer.new_routing(T, perm_capacity=int(G.sum()) - 1)
+        layer.layer_fwd(xd[:T], 0.0, routing=small)
+        torch.cuda.synchronize()
+        assert small.status == 7                               # D2D_ERR_CAPACITY
+    layer.close()
