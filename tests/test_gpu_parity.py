@@ -1091,3 +1091,23 @@ def test_lists_ride_up_to_their_limits(api, shape, last, Ts):
         torch.cuda.synchronize()
         assert small.status == 7                               # D2D_ERR_CAPACITY
     layer.close()
+
+
+@pytest.mark.parametrize("T", [1025, 1300, 1589, 1590])
+def test_lists_of_a_group_ride_up_to_their_limit(api, T):
+    """Three layers' lists on one down projection of up to 2e10 FLOP (1589 tokens), on a stream of the group's own above."""
+    cfg = wl.with_tokens(wl.CONFIGS["gpt2_attn"], T)
+    w = wl.make_weights(cfg)
+    layers = [api.Layer.from_config(cfg, w) for _ in range(3)]
+    group = api.LayerGroup(layers)
+    x = api.to_device(wl.make_tokens(cfg), cfg.dtype)
+    for tau in (0.5, 0.0):
+        rs = [layer.new_routing(T) for layer in layers]
+        for r in rs:
+            _poison(r.perm), _poison(r.counts), _poison(r.offsets)
+        group.group_fwd(x, tau, routings=rs)
+        torch.cuda.synchronize()
+        G = oracle.unpack_mask(rs[0].mask_u32(), cfg.E)
+        for r in rs:                                           # equal weights: equal decisions
+            _check_routing(r, G, dual=False)
+    group.close()
