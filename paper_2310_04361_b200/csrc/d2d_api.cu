@@ -261,9 +261,14 @@ static int path_before_launch(const d2d_layer *L, int T, bool counted)
 // log2(T / 128) / h of the E experts and has all of the others in its union, which leaves 1 - (1 - rho) log2(T / 128) / (E h) of
 // the work.  (Independent decisions are the worst case; correlated ones leave less.)  The form is level with the dense pair where 0.73
 // is left: expert step of the paper's shape, us, sorted / dense, a box each: 50432 tokens p = 0.1 175 / 342, 0.2 266 / 348, 0.3 341 /
-// 356, 0.4 396 / 370 (the limit: 0.32); 25000 tokens 0.1 130 / 183, 0.2 172 / 178, 0.3 189 / 178 (0.28); 12608 tokens 0.1 84 / 106, 0.2
-// 104 / 106, 0.3 119 / 106 (0.23); and the choice itself costs 10 where the dense pair runs in the end.
-// in_layer_call: behind a router, which overlaps a dense up projection that is not chosen: only batches that had a choice anyway.
+// 356, 0.4 396 / 370 (the limit: 0.32); 25000 tokens 0.1 130 / 183, 0.2 172 / 178, 0.3 189 / 178 (0.28); and the choice itself costs 10 to
+// 14 where the dense pair runs in the end (p = 0.5: 25000 tokens 222 / 208, 40000 356 / 344, 50432 437 / 424).
+// in_layer_call: behind a router, which overlaps a dense up projection that is not chosen: only batches that had a choice anyway (they
+// paid for the kernels of two other forms).  Layer call, us, with this choice / the dense pair forced / with the fused, gathered and dense
+// forms that were the choice before: 42600 tokens, rho = 0.06 147 / 322 / 268, 0.14 250 / 353 / 381, 0.28 350 / 364 / 415, above the limit
+// 0.33 404 / 373 / 448, 0.51 411 / 390 / 392; 80000 tokens, 0.09 356 / 632 / 658, 0.33 669 / 674 / 812; 32 experts of 64 neurons, d = 1024,
+// 60000 tokens (the limit: 0.235), 0.05 234 / 405 / 341, 0.12 388 / 439 / 469, 0.18 445 / 429 / 528, 0.22 486 / 447 / 487: there the
+// form is level a little earlier, at 0.17.
 static double default_fused_rho_max(int g);
 static long long sorted_n_sel_max(const d2d_layer *L, int T, bool in_layer_call)
 {

@@ -13,7 +13,8 @@
 //   sort_rows_kernel     copies the token rows (and masks) to their places; one CTA lists the work of the two projections
 //   gemm_tc.cu           both projections, from the lists (d2d_gemm_args::sorted)
 // Which place a token gets inside its bucket is left to chance; y is not: a token's sums run over k in
-// ascending order, and the experts its neighbours brought in contribute exact zeros.
+// ascending order, and the experts its neighbours brought in contribute exact zeros (finite weights: an infinity or NaN in W2 of an expert
+// that a token does not keep reaches it where a neighbour keeps that expert; in the dense pair it reaches every token).
 #include "gemm_tc.cuh"
 #include "moe_sorted.cuh"
 #include "tc_common.cuh"

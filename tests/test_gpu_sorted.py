@@ -102,3 +102,47 @@ def test_a_workspace_serves_every_smaller_batch_of_ordered_tokens(api, E, s, d):
         assert all(a <= b for a, b in zip(at, at[1:]))
     group.close()
     layer.close()
+
+
+# tau: few pairs, some, and more than the limit (the dense pair then runs); a ragged last tile of one row, and the last batch without the
+# choice; with and without the lists, which a stream of the layer's own builds beside the four kernels
+@pytest.mark.parametrize("T,tau,ordered", [(43009, 0.9, True), (43009, 0.6, True), (50432, 0.7, True), (43009, 0.4, False), (42300, 0.7, False)])
+def test_sorted_form_behind_a_router(api, T, tau, ordered):
+    cfg = wl.with_tokens(wl.CONFIGS["paper"], T)
+    w, x = wl.make_weights(cfg), wl.make_tokens(cfg)
+    layer = api.Layer.from_config(cfg, w)
+    xd = api.to_device(x, cfg.dtype)
+    used, masks, ys = [], [], []
+    ws = layer.workspace(T)
+    tail = ws[layer.workspace_bytes(T) - 8 * T:layer.workspace_bytes(T)]       # masks and lists of work in the form's scratch
+    for path, lists in (("auto", True), ("auto", True), ("auto", False), ("dense", False)):
+        layer.set_expert_path(path)
+        ws.fill_(0xff)                                         # bf16 NaNs; what a form does not write stays
+        r = layer.new_routing(T, lists=lists)
+        if lists:
+            r.perm.fill_(-1), r.counts.fill_(-1), r.offsets.fill_(-1)
+        y = torch.full((T, cfg.d), float("nan"), dtype=torch.bfloat16, device="cuda")
+        layer.layer_fwd(xd, tau, y=y, routing=r)
+        torch.cuda.synchronize()
+        assert r.status == 0
+        used.append(bool((tail != 0xff).any()))
+        masks.append(r.mask_u32().copy())
+        ys.append(y)
+        G = oracle.unpack_mask(masks[0], cfg.E)
+        if path == "auto":
+            behind_the_choice = 2.0 * T * cfg.d * cfg.d_ff >= 2e11
+            assert (int(G.sum()) <= layer.sorted_limit(T) and behind_the_choice) == ordered
+        if lists:
+            want = oracle.metadata(G)
+            assert np.array_equal(r.k[:T].cpu().numpy(), G.sum(1)) and r.n_sel == want["n_sel"]
+            assert np.array_equal(r.counts.cpu().numpy(), want["counts"]) and np.array_equal(r.offsets.cpu().numpy(), want["offsets"])
+            assert np.array_equal(r.perm[: r.n_sel].cpu().numpy(), want["perm"])
+    assert used == [ordered] * 3 + [False]
+    assert all(np.array_equal(m, masks[0]) for m in masks)
+    # bit for bit what the dense pair gives: the same products in the same order, plus exact zeros
+    assert all(torch.equal(y.view(torch.int16), ys[-1].view(torch.int16)) for y in ys)
+    sample = np.unique(np.concatenate([[0, 127, T - 1], np.random.default_rng(T).integers(0, T, 100)]))
+    ref = oracle.moe_ffn(x[sample], w["w1"], w["b1"], w["w_gate"], w["w2"], w["b2"], oracle.ACT_BY_NAME[cfg.act], G[sample])
+    got = ys[0].float().cpu().numpy()[sample]
+    assert np.isfinite(got).all() and np.abs(got - ref).max() / np.abs(ref).max() <= TOL_Y
+    layer.close()
