@@ -265,7 +265,8 @@ D2D_API d2d_status d2d_decode_plan_for(const d2d_layer_desc *desc, int32_t n_lay
  * sub-chunk counters of the expert kernels).  They reset themselves when a
  * call completes; a call that ended with D2D_ERR_TIMEOUT in the status word
  * may have left them non-zero, and the next call would then skip work.  Enqueue
- * this on the stream after such a call (it is a 1-2 KB memset). */
+ * this on the stream after such a call (a memset of 1 to 2 KB, 9 where the layer
+ * has d2d_layer_get_sorted's form). */
 D2D_API d2d_status d2d_layer_reset_counters(d2d_layer *layer, void *stream);
 
 /* Bytes of device workspace that any call on `layer` with up to max_tokens

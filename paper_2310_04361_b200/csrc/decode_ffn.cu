@@ -18,8 +18,8 @@
 // The last CTA to add to its columns (a ticket per rank) adds b2 and writes y.
 //
 // Measured, whole layer calls back to back (small_batch_ffn.cu or the tensor-core path -> these two kernels): d = 1024,
-// 256 experts of 16: 18.1 -> 12.4 us at 1 token, 38 -> 14.8 us at 13; d = 4096, 344 gated experts of 32: 114 -> 59.6 us at 7
-// tokens, 64 -> 44 us at 1 with 8-bit weights; three d = 1024 layers of 128 experts on 8 shared tokens: 43 -> 16.6 us.
+// 256 experts of 16: 18.1 -> 12.1 us at 1 token, 38 -> 14.7 us at 13; d = 4096, 344 gated experts of 32: 114 -> 56.8 us at 7
+// tokens, 64 -> 37 us at 1 with 8-bit weights; three d = 1024 layers of 128 experts on 8 shared tokens: 43 -> 15.8 us.
 //
 // How many tokens fit is a matter of shared memory: the token rows, the partial sums and the hidden values grow with them, and
 // the ring beside them needs three stages.  One layer of bf16 weights: 32 tokens with d = 512 or 640, 16 with 768, 1024 or 2048, 8
@@ -418,8 +418,8 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
     } else if (warp > NCW) {
         // ------------------------------------------------------------------ talks to the cluster: sends the hidden values, and tells
         // the others that a round's have been read.  A release at cluster scope takes 0.6 us, sending as much: a consumer warp would
-        // hold up all others with it (Llama-shaped layer, tau = 0.2, us, with the sends by consumer warps / here: 37.7 / 35.4 at 1 token and
-        // 52.9 / 50.6 at 6, 8-bit weights; 59.4 / 56.6 at 7 tokens.  A warp for each other CTA: the same with clusters of two, and 43.7
+        // hold up all others with it (Llama-shaped layer, tau = 0.2, us, with the sends by consumer warps / here: 37.7 / 35.4 at 1 token (163
+        // experts kept) and 52.9 / 50.6 at 6, 8-bit weights; 59.4 / 56.7 at 7 tokens.  A warp for each other CTA: the same with clusters of two, and 43.7
         // instead of 40.9 at 1 token, where they are of four.)
         bool ok = d2d_tc::mbar_wait_warp(smem_addr(&bar_go), 0, P.status);
         __syncwarp();
@@ -673,7 +673,7 @@ decode_ffn_kernel(const __nv_bfloat16 *__restrict__ x, const FfnShape S, const _
                 float *z = zs + (size_t)place * 3 * 16 * T8 + tid;
                 float v[2] = {0.0f, 0.0f};
                 // (codes: scales only when both sums are there, and without ldexpf: 34.5 instead of 35.6 us for the Llama-shaped layer at 1
-                // token, 45.7 instead of 47.1 at 2, tau = 0.2)
+                // token that keeps 163 experts, 45.7 instead of 47.1 at 2, tau = 0.2)
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     if (m == 1 && !S.gated) break;
